@@ -1281,8 +1281,11 @@ int melinoe_trace_miss_proxies(void *cuda_stream, const int32_t *trace_dev, int 
         return MELINOE_ERR_UNSUPPORTED;
     if (n_configs == 0)
         return MELINOE_OK;
+    int dev = 0, n_sms = 0;
+    CU_TRY(cudaGetDevice(&dev));
+    CU_TRY(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev));
     CU_TRY(launch_miss_proxies(static_cast<cudaStream_t>(cuda_stream), trace_dev, n_layers, n_tokens, top_k, n_experts, configs_dev,
-                               n_configs, soft_mean_dev, reinterpret_cast<long long *>(hard_total_dev)));
+                               n_configs, n_sms, soft_mean_dev, reinterpret_cast<long long *>(hard_total_dev)));
     return MELINOE_OK;
 }
 

@@ -156,7 +156,7 @@ cudaError_t launch_fetch_experts(cudaStream_t stream, int n_sms, const FetchPara
 
 // ---- cache-miss proxies of a recorded routing trace (Section 3.1, Definition C.1)
 cudaError_t launch_miss_proxies(cudaStream_t stream, const int32_t *idx, int n_layers, int T, int K, int E,
-                                const melinoe_proxy_config *cfgs, int n_cfg, double *soft_mean, long long *hard_total);
+                                const melinoe_proxy_config *cfgs, int n_cfg, int n_sms, double *soft_mean, long long *hard_total);
 
 // ---- 4-bit host store: expand one 4-bit expert (layout in dequant.cu) into a bf16 slot
 // ---- decode-sized input from device-mapped host memory into device memory (bytes % 16 == 0)

@@ -1,10 +1,8 @@
 // Forward-only evaluation of the paper's cache-miss proxies over a recorded routing trace
 // (Section 3.1: the soft cache state of the cache simulation loss L_cs; Definition C.1: the hard
-// gamma-discounted Top-C cache, whose misses are the transfers of Appendix C.1).  One warp per
-// configuration (layer, cache size, gamma) walks the layer's tokens in order; lane l owns experts
-// l and l + 32.  Everything is fp64 and in the order the definitions state, so the hard misses
-// (an integer result) are exact and the soft proxy differs from a straightforward evaluation only
-// by the order of a 64-term sum.
+// gamma-discounted Top-C cache, whose misses are the transfers of Appendix C.1).  fp64 throughout;
+// the hard misses (an integer result) are exact, the soft proxy differs from a straightforward
+// evaluation by fp64 rounding only.
 //
 //   soft:  c starts at 0 and follows c <- gamma c + r while its L1 norm stays below C; the first
 //          update that reaches C is rescaled to norm C and starts the normaliser Z = 1; from then
@@ -12,11 +10,34 @@
 //   hard:  count starts at 0, count <- gamma count + r; the cache holds the up to C experts of
 //          largest non-zero count (lower index first among equals); miss_t = requested experts
 //          outside it.
+//
+// One block per configuration (layer, cache size, gamma).  What bounds it is the walk along the trace,
+// a chain of dependent fp64 operations per token, so the chain is kept as short as the definitions
+// allow and everything else is moved off it:
+//   - the requests of a token are one bit mask, made once per block by all threads and transposed, so that
+//     a lane has 32 tokens' requests of its expert in one word;
+//   - soft (two warps): u = Z c follows u <- gamma u + r with no division and no normaliser in it, and
+//     c = u / Z.  Z does not depend on the requests: lane i holds gamma^i and 1 + gamma + .. + gamma^(i-1),
+//     so 32 tokens' normalisers are one multiply-add and one division per lane.  Every lane sums its own
+//     expert's u / Z; the lanes meet once, at the end.
+//   - hard (one warp, or two): the counts do not depend on C.  The configurations of one layer and gamma
+//     therefore share the ranking: each block ranks a part of the tokens (the counts up to there are
+//     replayed, two operations per token), keeps a histogram of the requested experts' ranks, and adds to
+//     each of those configurations the requests whose rank is C or more.  Only requested experts are
+//     ranked, one per lane.
+// 912 configurations (57 sizes of 16 layers) over 512 tokens of 8 requests: 1128 us when every
+// configuration ranked all 64 experts of every token and met in a warp-wide sum per token, 46 us like this
+// (issue slots half busy; a single layer's 57 configurations take 20 us, of which the chain is about 8).
 #include "kernels.cuh"
 
 namespace melinoe {
 
 namespace {
+
+constexpr int kProxyThreads = 128;
+constexpr int kProxyChunk = 512;       // tokens whose masks are held at a time (7 blocks of an SM fit its shared memory)
+constexpr int kProxyGroup = 4;         // tokens a warp ranks at a time
+constexpr int kProxyWindow = 1024;     // configurations among which equal (layer, gamma) pairs share their ranking
 
 __device__ __forceinline__ double warp_sum(double v)
 {
@@ -26,88 +47,328 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-__global__ void __launch_bounds__(32) miss_proxy_kernel(const int32_t *__restrict__ idx, int n_layers, int T, int K, int E,
-                                                        const melinoe_proxy_config *__restrict__ cfgs, int n_cfg,
-                                                        double *__restrict__ soft_mean, long long *__restrict__ hard_total)
+// 32 x 32 bits across the warp: bit j of lane l becomes bit l of lane j.
+__device__ __forceinline__ unsigned transpose32(unsigned x, int lane)
 {
-    __shared__ double s_count[kMaxExperts];
-    const int lane = threadIdx.x;
+    const unsigned keep[5] = {0x0000ffffu, 0x00ff00ffu, 0x0f0f0f0fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const int o = 16 >> i;
+        const unsigned m = keep[i], y = __shfl_xor_sync(0xffffffffu, x, o);
+        x = lane & o ? ((y >> o) & m) | (x & ~m) : (x & m) | ((y & m) << o);
+    }
+    return x;
+}
+
+__device__ __forceinline__ bool proxy_config_valid(const melinoe_proxy_config &c, int n_layers, int E)
+{
+    return c.layer >= 0 && c.layer < n_layers && c.cache_slots >= 1 && c.cache_slots <= E && c.gamma >= 0.0 && c.gamma <= 1.0;
+}
+
+__global__ void __launch_bounds__(kProxyThreads, 7) miss_proxy_kernel(const int32_t *__restrict__ idx, int n_layers, int T, int K, int E,
+                                                                      const melinoe_proxy_config *__restrict__ cfgs, int n_cfg, int n_sms,
+                                                                      double *__restrict__ soft_mean, unsigned long long *hard_total)
+{
+    __shared__ unsigned s_mask[2][kProxyChunk];      // requests of a token: experts 0..31, 32..63
+    __shared__ double s_iz[2][32];
+    __shared__ double s_part[2][32][33];             // fill phase: the lanes' states after each of 32 tokens
+    __shared__ double s_snap[2][kProxyGroup][kMaxExperts + 1];   // ranking: the counts before each of some tokens
+    __shared__ int s_group[4][2];                    // per warp: configurations with this layer and gamma, before this one and in all
+    __shared__ unsigned long long s_asked[4];
+    __shared__ double s_hit[2];
+    __shared__ unsigned s_hist[kMaxExperts + 1];     // requests by rank; the last entry: experts with a zero count
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ci = blockIdx.x;
-    if (ci >= n_cfg)
-        return;
+    // Warps 0 and 1 of the roles walk the soft state, 2 and 3 rank.  A block's warp w sits on scheduler w of its SM, so
+    // the roles rotate from one block of an SM to the next.
+    const int role = (warp + ci / n_sms) & 3;
     const melinoe_proxy_config cfg = cfgs[ci];
+    if (!proxy_config_valid(cfg, n_layers, E)) {
+        if (tid == 0) {       // a configuration that names nothing: marked, not evaluated
+            soft_mean[ci] = __longlong_as_double(0x7ff8000000000000ll);
+            hard_total[ci] = ~0ull;
+        }
+        return;
+    }
     const int C = cfg.cache_slots;
     const double gamma = cfg.gamma;
-    if (cfg.layer < 0 || cfg.layer >= n_layers || C < 1 || C > E || !(gamma >= 0.0 && gamma <= 1.0)) {
-        if (lane == 0) {       // a configuration that names nothing: marked, not evaluated
-            soft_mean[ci] = __longlong_as_double(0x7ff8000000000000ll);
-            hard_total[ci] = -1;
-        }
-        return;
+    for (int i = tid; i <= kMaxExperts; i += kProxyThreads)
+        s_hist[i] = 0u;
+    const int w0 = ci / kProxyWindow * kProxyWindow, w1 = min(w0 + kProxyWindow, n_cfg);
+    auto same = [&](int j) {
+        const melinoe_proxy_config o = cfgs[j];
+        return o.layer == cfg.layer && o.gamma == gamma && o.cache_slots >= 1 && o.cache_slots <= E;
+    };
+    int before = 0, all = 0;
+#pragma unroll 8
+    for (int j = w0 + tid; j < w1; j += kProxyThreads) {
+        const bool s = same(j);
+        all += s;
+        before += s && j < ci;
     }
-    const int32_t *trace = idx + (size_t)cfg.layer * T * K;
-    const int e0 = lane, e1 = lane + 32;
-    double c0 = 0.0, c1 = 0.0, n0 = 0.0, n1 = 0.0, Z = 1.0;
-    bool filled = false;
-    double soft = 0.0;
-    long long hard = 0;
-    for (int t = 0; t < T; ++t) {
-        // request vector of the token
-        bool r0 = false, r1 = false;
-        for (int j = 0; j < K; ++j) {
-            const int e = trace[(size_t)t * K + j];
-            r0 |= e == e0;
-            r1 |= e == e1;
-        }
-        const double q0 = r0 ? 1.0 : 0.0, q1 = r1 ? 1.0 : 0.0;
-        soft += warp_sum(q0 * (1.0 - c0) + q1 * (1.0 - c1));
-        // hard cache: rank of this lane's experts among the non-zero counts
-        s_count[e0] = n0;
-        s_count[e1] = n1;
-        __syncwarp();
-        int k0 = 0, k1 = 0;
-        for (int e = 0; e < E; ++e) {
-            const double o = s_count[e];
-            k0 += (o > n0) || (o == n0 && e < e0);
-            k1 += (o > n1) || (o == n1 && e < e1);
-        }
-        __syncwarp();
-        const bool in0 = e0 < E && n0 > 0.0 && k0 < C, in1 = e1 < E && n1 > 0.0 && k1 < C;
-        hard += __popc(__ballot_sync(0xffffffffu, r0 && !in0)) + __popc(__ballot_sync(0xffffffffu, r1 && !in1));
-        // updates
-        if (!filled) {
-            double a0 = gamma * c0 + q0, a1 = gamma * c1 + q1;
-            const double norm = warp_sum(a0 + a1);
-            if (norm >= (double)C) {
-                a0 *= (double)C / norm;
-                a1 *= (double)C / norm;
-                filled = true;
-                Z = 1.0;
-            }
-            c0 = a0;
-            c1 = a1;
-        } else {
-            const double Zn = gamma * Z + (double)K / (double)C;
-            c0 = (gamma * Z * c0 + q0) / Zn;
-            c1 = (gamma * Z * c1 + q1) / Zn;
-            Z = Zn;
-        }
-        // product rounded before the sum (no contraction): the hard cache's decisions hang on these bits
-        n0 = __dadd_rn(__dmul_rn(gamma, n0), q0);
-        n1 = __dadd_rn(__dmul_rn(gamma, n1), q1);
-    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    all = __reduce_add_sync(0xffffffffu, all);
     if (lane == 0) {
-        soft_mean[ci] = T > 0 ? soft / (double)T : 0.0;
-        hard_total[ci] = hard;
+        s_group[warp][0] = before;
+        s_group[warp][1] = all;
     }
+
+    const int32_t *trace = idx + (size_t)cfg.layer * T * K;
+    const bool vec = (K & 3) == 0 && (reinterpret_cast<uintptr_t>(trace) & 15u) == 0;
+    const int e0 = lane, e1 = lane + 32;
+    const unsigned bit = 1u << lane;
+    // soft warps: the state of this lane's expert (warp `half` has experts 32 half ..), and what the lane needs to
+    // form the normalisers
+    const int half = role & 1;
+    double u = 0.0, acc = 0.0, Zb = 1.0;
+    double gi = 1.0, si = 0.0, g32 = 1.0, s32 = 0.0;
+    if (role < 2) {
+#pragma unroll 1
+        for (int i = 0; i < 32; ++i) {
+            if (i == lane) {
+                gi = g32;
+                si = s32;
+            }
+            s32 = fma(gamma, s32, 1.0);
+            g32 *= gamma;
+        }
+    }
+    const double KC = (double)K / (double)C;
+    bool filled = false;
+    // ranking warps: the counts of this lane's experts
+    const int group_tokens = K <= 32 ? min(32 / K, kProxyGroup) : 1;
+    double n0 = 0.0, n1 = 0.0;
+    int rank_lo = 0, rank_hi = 0;
+    // 1 or 0 as a double without a conversion (the low word is zero)
+    auto one_if = [](bool r) { return __hiloint2double(r ? 0x3ff00000 : 0, 0); };
+    unsigned long long asked = 0ull;
+
+    for (int t0 = 0; t0 < T; t0 += kProxyChunk) {
+        const int nt = min(kProxyChunk, T - t0);
+#pragma unroll 2
+        for (int t = tid; t < nt; t += kProxyThreads) {
+            const int32_t *row = trace + (size_t)(t0 + t) * K;
+            unsigned lo = 0u, hi = 0u;
+            auto add = [&](int e) {
+                const unsigned b = (unsigned)e < (unsigned)E ? 1u << (e & 31) : 0u;
+                if (e < 32)
+                    lo |= b;
+                else
+                    hi |= b;
+            };
+            if (vec) {
+#pragma unroll 2
+                for (int j = 0; j < K; j += 4) {
+                    const int4 v = __ldg(reinterpret_cast<const int4 *>(row + j));
+                    add(v.x);
+                    add(v.y);
+                    add(v.z);
+                    add(v.w);
+                }
+            } else {
+#pragma unroll 4
+                for (int j = 0; j < K; ++j)
+                    add(__ldg(row + j));
+            }
+            s_mask[0][t] = lo;
+            s_mask[1][t] = hi;
+            asked += (unsigned)(__popc(lo) + __popc(hi));
+        }
+        __syncthreads();
+        if (t0 == 0) {
+            // the tokens this block ranks, and the warps that do it: one where many configurations share the work
+            const int G = s_group[0][1] + s_group[1][1] + s_group[2][1] + s_group[3][1];
+            const int o = s_group[0][0] + s_group[1][0] + s_group[2][0] + s_group[3][0];
+            const int n_rank_warps = G >= 16 ? 1 : 2;
+            if (role - 2 < n_rank_warps) {
+                const long long parts = (long long)G * n_rank_warps, part = (long long)o * n_rank_warps + (role - 2);
+                rank_lo = (int)(part * T / parts);
+                rank_hi = (int)((part + 1) * T / parts);
+            }
+        }
+        if (role < 2) {
+            // r: the lane's expert is requested
+            // (predicated by hand: five instructions)
+            auto step = [&](unsigned r, double iz) {
+                asm("{\n\t.reg .pred p;\n\t.reg .b32 h, l;\n\t.reg .f64 q;\n\t"
+                    "setp.ne.u32 p, %2, 0;\n\t"
+                    "@p fma.rn.f64 %0, %1, %3, %0;\n\t"
+                    "selp.b32 h, 0x3ff00000, 0, p;\n\t"
+                    "mov.b32 l, 0;\n\t"
+                    "mov.b64 q, {l, h};\n\t"
+                    "fma.rn.f64 %1, %4, %1, q;\n\t}"
+                    : "+d"(acc), "+d"(u)
+                    : "r"(r), "d"(iz), "d"(gamma));
+            };
+            int t = 0;
+            // fill phase: 32 tokens ahead as if none of them filled the cache, then their norms, one per lane (each the
+            // sum over the lanes in a fixed tree order); the first that reaches C, if any, is gone back to
+            while (t < nt && !filled) {
+                const int cnt = min(32, nt - t);
+                // bit j: the lane's expert is requested by token t + j
+                const unsigned asks = transpose32(lane < cnt ? s_mask[half][t + lane] : 0u, lane);
+                const double b = u, c = acc;
+#pragma unroll 4
+                for (int j = 0; j < cnt; ++j) {
+                    step(asks & (1u << j), 1.0);
+                    s_part[half][j][lane] = u;
+                }
+                asm volatile("bar.sync 1, 64;" ::: "memory");
+                double v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    v[i] = (s_part[0][lane][i] + s_part[1][lane][i]) + (s_part[0][lane][i + 16] + s_part[1][lane][i + 16]);
+#pragma unroll
+                for (int w = 8; w >= 1; w >>= 1)
+#pragma unroll
+                    for (int i = 0; i < w; ++i)
+                        v[i] += v[i + w];
+                const unsigned full = __ballot_sync(0xffffffffu, lane < cnt && v[0] >= (double)C);
+                if (full) {
+                    const int run = __ffs((int)full);
+                    const double norm = __shfl_sync(0xffffffffu, v[0], run - 1);
+                    u = b, acc = c;
+#pragma unroll 1
+                    for (int j = 0; j < run; ++j)
+                        step(asks & (1u << j), 1.0);
+                    u *= (double)C / norm;
+                    filled = true;
+                    t += run;
+                } else {
+                    t += cnt;
+                }
+                asm volatile("bar.sync 1, 64;" ::: "memory");
+            }
+            while (t < nt) {
+                // Z of the next 32 tokens, one per lane
+                const int cnt = min(32, nt - t);
+                const unsigned asks = transpose32(lane < cnt ? s_mask[half][t + lane] : 0u, lane);
+                const double z = fma(gi, Zb, KC * si);
+                s_iz[half][lane] = 1.0 / z;
+                __syncwarp();
+                if (cnt == 32) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        step(asks & (1u << j), s_iz[half][j]);
+                    Zb = fma(g32, Zb, KC * s32);
+                } else {
+#pragma unroll 1
+                    for (int j = 0; j < cnt; ++j)
+                        step(asks & (1u << j), s_iz[half][j]);
+                    Zb = __shfl_sync(0xffffffffu, z, cnt);
+                }
+                __syncwarp();
+                t += cnt;
+            }
+        } else if (rank_hi > t0) {
+            // product rounded before the sum (no contraction): the hard cache's decisions hang on these bits
+            auto advance = [&](bool r0, bool r1) {
+                n0 = __dadd_rn(__dmul_rn(gamma, n0), one_if(r0));
+                n1 = __dadd_rn(__dmul_rn(gamma, n1), one_if(r1));
+            };
+            const int lo = min(max(rank_lo - t0, 0), nt), hi = min(max(rank_hi - t0, 0), nt);
+            for (int t = 0; t < lo; t += 32) {
+                const int cnt = min(32, lo - t);
+                const unsigned a0 = transpose32(lane < cnt ? s_mask[0][t + lane] : 0u, lane);
+                const unsigned a1 = transpose32(lane < cnt ? s_mask[1][t + lane] : 0u, lane);
+                if (cnt == 32) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        advance((a0 >> j) & 1u, (a1 >> j) & 1u);
+                } else {
+#pragma unroll 1
+                    for (int j = 0; j < cnt; ++j)
+                        advance((a0 >> j) & 1u, (a1 >> j) & 1u);
+                }
+            }
+            // as many tokens at a time as have their requests in one warp: the counts before each of them, then one
+            // request per lane against all of its token's counts
+            double(*snap)[kMaxExperts + 1] = s_snap[role - 2];
+            for (int t = lo; t < hi; t += group_tokens) {
+                const int g = min(group_tokens, hi - t);
+                for (int i = 0; i < g; ++i) {
+                    snap[i][e0] = n0;
+                    snap[i][e1] = n1;
+                    advance(s_mask[0][t + i] & bit, s_mask[1][t + i] & bit);
+                }
+                __syncwarp();
+                uint64_t seen = 0;      // more than 32 requests per token: those of the token's earlier passes
+                for (int i0 = 0; i0 < g * K; i0 += 32) {
+                    const int i = i0 + lane, tok = i / K;
+                    int r = i < g * K ? __ldg(trace + (size_t)(t0 + t) * K + i) : -1;
+                    if ((unsigned)r >= (unsigned)E || ((seen >> r) & 1ull))
+                        r = -1;
+                    // an expert that a token names twice is one request
+                    const unsigned twins = __match_any_sync(0xffffffffu, r < 0 ? -1 - lane : tok * kMaxExperts + r);
+                    if (g * K > 32)
+                        seen |= (uint64_t)__reduce_or_sync(0xffffffffu, r >= 0 && r < 32 ? 1u << r : 0u) |
+                                (uint64_t)__reduce_or_sync(0xffffffffu, r >= 32 ? 1u << (r - 32) : 0u) << 32;
+                    const double *row = snap[r < 0 ? 0 : tok];
+                    const double nr = row[max(r, 0)];
+                    int k = 0;
+#pragma unroll 16
+                    for (int e = 0; e < kMaxExperts; ++e) {
+                        const double n = row[e];
+                        k += n > nr || (n == nr && e < r);
+                    }
+                    if (r >= 0 && (twins & (bit - 1u)) == 0u)
+                        atomicAdd(&s_hist[nr > 0.0 ? k : kMaxExperts], 1u);
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1)
+        asked += __shfl_xor_sync(0xffffffffu, asked, m);
+    if (lane == 0)
+        s_asked[warp] = asked;
+    if (role < 2) {
+        const double hit = warp_sum(acc);
+        if (lane == 0)
+            s_hit[half] = hit;
+    } else if (role == 2) {
+        // requests of rank r or more
+        unsigned above = s_hist[kMaxExperts];
+#pragma unroll
+        for (int h = 1; h >= 0; --h) {
+            unsigned v = s_hist[32 * h + lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned w = __shfl_down_sync(0xffffffffu, v, o);
+                v += lane + o < 32 ? w : 0u;
+            }
+            v += above;
+            s_hist[32 * h + lane] = v;
+            above = __shfl_sync(0xffffffffu, v, 0);
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        const double n = (double)(s_asked[0] + s_asked[1] + s_asked[2] + s_asked[3]);
+        soft_mean[ci] = T > 0 ? (n - (s_hit[0] + s_hit[1])) / (double)T : 0.0;
+    }
+#pragma unroll 8
+    for (int j = w0 + tid; j < w1; j += kProxyThreads)
+        if (same(j)) {
+            const unsigned n = s_hist[cfgs[j].cache_slots];
+            if (n)
+                atomicAdd(hard_total + j, (unsigned long long)n);
+        }
 }
 
 }  // namespace
 
 cudaError_t launch_miss_proxies(cudaStream_t stream, const int32_t *idx, int n_layers, int T, int K, int E,
-                                const melinoe_proxy_config *cfgs, int n_cfg, double *soft_mean, long long *hard_total)
+                                const melinoe_proxy_config *cfgs, int n_cfg, int n_sms, double *soft_mean, long long *hard_total)
 {
-    miss_proxy_kernel<<<n_cfg, 32, 0, stream>>>(idx, n_layers, T, K, E, cfgs, n_cfg, soft_mean, hard_total);
+    // the blocks add their parts up
+    const cudaError_t e = cudaMemsetAsync(hard_total, 0, (size_t)n_cfg * sizeof(long long), stream);
+    if (e != cudaSuccess)
+        return e;
+    miss_proxy_kernel<<<n_cfg, kProxyThreads, 0, stream>>>(idx, n_layers, T, K, E, cfgs, n_cfg, n_sms, soft_mean,
+                                                           reinterpret_cast<unsigned long long *>(hard_total));
     count_launch();
     return cudaGetLastError();
 }

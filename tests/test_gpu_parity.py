@@ -559,6 +559,35 @@ def test_trace_miss_proxies_match_the_oracle():
     assert bool(torch.isnan(so).all()) and ha.tolist() == [-1, -1]
 
 
+@pytest.mark.parametrize("T,K,E,gamma,sizes", [
+    (1, 1, 1, 0.5, [1]),
+    (31, 3, 33, 0.9, [1, 3, 32, 33]),           # fewer tokens than one batch of 32; three configurations rank with two warps
+    (1100, 8, 64, 0.9, list(range(8, 65))),     # tokens held 512 at a time; 57 sizes share the ranking
+    (513, 40, 64, 1.0, [40, 41, 63, 64]),       # more requests per token than a warp has lanes
+    (700, 1, 64, 0.9, [5, 10, 11, 64]),         # the norm tends to K / (1 - gamma) = 10: just below, never above
+    (200, 6, 40, 0.0, [6, 7, 40]),              # nothing is remembered
+])
+def test_trace_miss_proxies_at_the_edges_of_their_batches(T, K, E, gamma, sizes):
+    """Hard misses exact, soft proxy to fp64 rounding (a sum of at most 64 T terms of at most 1 each)."""
+    from paper_2602_11192_b200 import binding as B
+    from paper_2602_11192_b200.runner import current_stream_ptr
+    import torch
+    rs = np.random.default_rng(T)
+    pref = rs.dirichlet(np.full(E, 0.5)) + 1e-3
+    trace = np.stack([rs.choice(E, size=K, replace=False, p=pref / pref.sum()) for _ in range(T)]).astype(np.int32)
+    n = len(sizes)
+    cfg = (B.ProxyConfig * n)(*[B.ProxyConfig(0, c, gamma) for c in sizes])
+    cfg_dev = torch.frombuffer(bytearray(bytes(cfg)), dtype=torch.uint8).cuda()
+    soft = torch.zeros(n, dtype=torch.float64, device="cuda")
+    hard = torch.full((n,), 7, dtype=torch.int64, device="cuda")
+    B.melinoe_trace_miss_proxies(current_stream_ptr(), torch.from_numpy(trace).cuda(), 1, T, K, E, cfg_dev, n, soft, hard)
+    soft, hard = soft.cpu().numpy(), hard.cpu().numpy()
+    for j, c in enumerate(sizes):
+        so, ho = oracle.miss_proxies(trace, E, c, gamma)
+        assert hard[j] == int(ho.sum()), (c, hard[j], int(ho.sum()))
+        assert abs(soft[j] - so.mean()) <= 1e-10 * max(1.0, abs(so.mean())), (c, soft[j], so.mean())
+
+
 def test_argument_and_state_errors():
     import torch
     from paper_2602_11192_b200 import MoELayer, MelinoeError, melinoe_moe_expert_bytes

@@ -108,8 +108,7 @@ int melinoe_moe_create(int d_model, int d_ff, int n_experts, int top_k, int cach
  * with melinoe_moe_register_host_experts_q4 and a miss is a plain copy of the 4-bit blob; the compute
  * kernel expands the codes in registers on their way into the tensor-core fragments, so HBM and the
  * host link only ever carry 4-bit data.  The layer computes with exactly the weights the format defines
- * (see melinoe_moe_pack_expert_q4).  Shared experts, if any, are registered as 4-bit blobs too.  Calls of
- * every size run the decode kernel, 8 tokens per launch (there is no 4-bit grouped GEMM).  Needs
+ * (see melinoe_moe_pack_expert_q4).  Shared experts, if any, are registered as 4-bit blobs too.  Needs
  * d_model = 512, 1024, 2048 or 4096 on top of the limits above.
  */
 int melinoe_moe_create_q4(int d_model, int d_ff, int n_experts, int top_k, int cache_slots,
@@ -227,12 +226,11 @@ int melinoe_moe_reserve(melinoe_moe_t *h, int max_tokens);
  * until the stream work of this call has finished.  stats_dev: see melinoe_moe_stats; may be
  * NULL.  n_tokens == 0 is a no-op.
  *
- * Host behaviour.  Calls of at most 8 tokens (or of any size on shapes the grouped GEMM does not
- * cover) on a bf16 store the device can address: the routing / planning kernel and the expert-FFN
- * kernel are queued and the call returns; the FFN kernel reads the experts the call misses from the
+ * Host behaviour.  Calls of at most 8 tokens on a store of the slots' own format that the device can
+ * address: the routing / planning kernel and the expert-FFN kernel are queued and the call returns; the FFN kernel reads the experts the call misses from the
  * host store itself, stores those that stay resident into their slots, and writes the result.  The
  * host learns the call's cache decisions only through stats_dev.
- * All other calls (more than 8 tokens through the grouped GEMM; a 4-bit store; host copies forced):
+ * All other calls (more than 8 tokens; a 4-bit store for bf16 slots; host copies forced):
  * the router, planning and resident-expert kernels are queued first; the call then waits (bounded;
  * TIMEOUT after 60 s) until the planning kernel has published the call's miss queue in page-locked
  * memory, issues one cudaMemcpyAsync per missed expert on the handle's copy stream, ties the streams
@@ -451,8 +449,8 @@ int melinoe_moe_set_timeline(melinoe_moe_t *h, void *trace_dev, size_t bytes);
 int melinoe_moe_timeline_ctas(melinoe_moe_t *h);
 
 /* 1 if the most recent forward call of the handle ran its expert FFN as the tensor-core grouped
- * GEMM (calls of more than 8 tokens on shapes with d_model % 256 == 0 and d_ff % 128 == 0), 0 if it
- * ran the decode kernel (in slices of 8 tokens where the call had more). */
+ * GEMM over bf16 slots (calls of more than 8 tokens), 0 if it ran the decode kernel or the slots hold 4-bit blobs
+ * (whose calls of more than 8 tokens run the grouped GEMM with the codes expanded in front of it). */
 int melinoe_moe_last_call_used_gemm(melinoe_moe_t *h);
 
 /* Test hook, host side only: the nth host-issued expert copy from now (cudaMemcpyAsync of a miss

@@ -73,10 +73,10 @@ typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32
 encode_tiled_fn g_encode_tiled = nullptr;
 std::once_flag g_encode_once;
 
-// 2-D bf16 tensor [rows][cols] with rows pitch_bytes apart, box of box_rows x 64 columns; with or
-// without the 128-byte swizzle (the expert blobs are stored already permuted, see melinoe_moe_pack_expert).
-bool encode_map(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, uint64_t pitch_bytes, uint32_t box_rows,
-                bool swizzle)
+// A tensor of `rank` dimensions (innermost first; strides in bytes of all but the innermost), with or without the
+// 128-byte swizzle (the expert blobs are stored already permuted, see melinoe_moe_pack_expert).
+bool encode_map(CUtensorMap *m, CUtensorMapDataType type, int rank, const void *base, const cuuint64_t *dims,
+                const cuuint64_t *strides, const cuuint32_t *box, bool swizzle)
 {
     std::call_once(g_encode_once, [] {
         cudaDriverEntryPointQueryResult qr;
@@ -86,25 +86,49 @@ bool encode_map(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, 
             g_encode_tiled = reinterpret_cast<encode_tiled_fn>(fn);
         (void)cudaGetLastError();
     });
-    if (!g_encode_tiled || rows == 0)
+    if (!g_encode_tiled)
         return false;
-    const cuuint64_t dims[2] = {cols, rows};
-    const cuuint64_t strides[1] = {pitch_bytes};
-    const cuuint32_t box[2] = {64, box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return g_encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return g_encode_tiled(m, type, (cuuint32_t)rank, const_cast<void *>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The three views of expert blobs that lie back to back from `base` (n_rows = experts * F rows f):
-// W_g rows, W_u rows (boxes of 128 rows), W_d^T rows (boxes of 64 rows), all d columns at a pitch of 6 d bytes.
-bool encode_weight_maps(CUtensorMap *m3, const void *base, int d, uint64_t n_rows)
+// Activations [rows][cols] bf16: three maps with boxes of 32, 64 and 128 rows x 64 columns.
+bool encode_activation_maps(CUtensorMap *m3, const void *base, uint64_t cols, uint64_t rows)
+{
+    const cuuint64_t dims[2] = {cols, rows}, strides[1] = {cols * 2};
+    for (uint32_t i = 0; i < 3; ++i) {
+        const cuuint32_t box[2] = {64, 32u << i};
+        if (!encode_map(m3 + i, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, true))
+            return false;
+    }
+    return true;
+}
+
+// The two views of n expert blobs `stride` bytes apart that the grouped GEMM's weight tiles are boxes of (ffn_gemm.cu).
+bool encode_weight_maps(CUtensorMap *m2, const void *base, int d_, int F_, int n_, size_t stride, int fmt)
 {
     const char *b = static_cast<const char *>(base);
-    const uint64_t pitch = (uint64_t)6 * d;
-    return encode_map(m3 + 0, b, d, n_rows, pitch, 128, false) && encode_map(m3 + 1, b + (size_t)2 * d, d, n_rows, pitch, 128, false) &&
-           encode_map(m3 + 2, b + (size_t)4 * d, d, n_rows, pitch, 64, false);
+    const cuuint64_t d = (cuuint64_t)d_, F = (cuuint64_t)F_, n = (cuuint64_t)n_;
+    if (fmt == 0) {
+        // GEMM 1: (column, f mod 8, W_g | W_u, f / 8 over all experts); the blobs are contiguous
+        const cuuint64_t dims1[4] = {d, 8, 2, n * F / 8}, str1[3] = {6 * d, 2 * d, 48 * d};
+        const cuuint32_t box1[4] = {64, 8, 2, 8};
+        // GEMM 2: (column within a group of 64, f, column group, expert) of W_d^T
+        const cuuint64_t dims2[4] = {64, F, d / 64, n}, str2[3] = {6 * d, 128, stride};
+        const cuuint32_t box2[4] = {64, 64, 2, 1};
+        return encode_map(m2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, b, dims1, str1, box1, false) &&
+               encode_map(m2 + 1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, b + 4 * d, dims2, str2, box2, false);
+    }
+    // the same of 4-bit codes: (byte, f mod 8, W_g | W_u, f / 8, expert) and (byte, f, expert)
+    const cuuint64_t ub = melinoe_moe_expert_bytes_q4(d_, F_) / F;
+    const cuuint64_t dims1[5] = {d / 2, 8, 2, F / 8, n}, str1[4] = {ub, d / 2, 8 * ub, stride};
+    const cuuint32_t box1[5] = {128, 8, 2, 8, 1};
+    const cuuint64_t dims2[3] = {d / 2, F, n}, str2[2] = {ub, stride};
+    const cuuint32_t box2[3] = {128, 128, 1};
+    return encode_map(m2, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, b, dims1, str1, box1, false) &&
+           encode_map(m2 + 1, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, b + d, dims2, str2, box2, false);
 }
 
 double now_s()
@@ -317,8 +341,8 @@ int ensure_capacity(melinoe_moe *h, int T)
         CU_TRY(cudaMalloc(&h->zbuf, sorted * h->d * sizeof(float)));
         CU_TRY(cudaMalloc(&h->xs, sorted * h->d * 2));
         CU_TRY(cudaMalloc(&h->hs, sorted * h->F * 2));
-        if (!encode_map(&h->maps_host[kMapXs], h->xs, h->d, sorted, (uint64_t)h->d * 2, 128, true) ||
-            !encode_map(&h->maps_host[kMapHs], h->hs, h->F, sorted, (uint64_t)h->F * 2, 128, true))
+        if (!encode_activation_maps(&h->maps_host[kMapXs0], h->xs, h->d, sorted) ||
+            !encode_activation_maps(&h->maps_host[kMapHs0], h->hs, h->F, sorted))
             return MELINOE_ERR_CUDA;
         CU_TRY(cudaMemcpy(h->maps_dev, h->maps_host, sizeof(h->maps_host), cudaMemcpyHostToDevice));
     }
@@ -572,12 +596,12 @@ static int create_layer(int d, int F, int E, int k, int C, int fmt, melinoe_moe_
     h->ev_group.assign(kMaxGroups + 1, nullptr);
     for (auto &e : h->ev_group)
         CR(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    // grouped GEMM for calls of many tokens: the slots are contiguous, so one tensor map per view
-    // (W_g rows, W_u rows, W_d^T rows) covers every slot
+    // grouped GEMM for calls of many tokens: one tensor map per view covers every slot (bf16 blobs are multiples of
+    // 1 KiB, so their slots are contiguous)
     std::memset(h->maps_host, 0, sizeof(h->maps_host));
-    if (fmt == 0 && ffn_gemm_supported(d, F) && h->slot_stride == h->expert_bytes && ffn_gemm_configure() == cudaSuccess) {
+    if (ffn_gemm_supported(d, F) && (fmt == 1 || h->slot_stride == h->expert_bytes) && ffn_gemm_configure() == cudaSuccess) {
         CR(cudaMalloc(&h->maps_dev, sizeof(h->maps_host)));
-        if (encode_weight_maps(&h->maps_host[kMapSlotsG], h->slots, d, (uint64_t)C * F)) {
+        if (encode_weight_maps(&h->maps_host[kMapSlots0], h->slots, d, F, C, h->slot_stride, fmt)) {
             CR(cudaMemcpy(h->maps_dev, h->maps_host, sizeof(h->maps_host), cudaMemcpyHostToDevice));
             h->gemm_ok = true;
         }
@@ -773,7 +797,7 @@ int melinoe_moe_register_shared_experts(melinoe_moe_t *h, int n_shared, const vo
     CU_TRY(cudaMemcpy(h->shared_dev, tmp, sizeof tmp, cudaMemcpyHostToDevice));
     if (h->gemm_ok) {
         for (int s = 0; s < n_shared; ++s)
-            if (!encode_weight_maps(&h->maps_host[kMapShared0 + 3 * s], ptrs[s], h->d, (uint64_t)h->F))
+            if (!encode_weight_maps(&h->maps_host[kMapShared0 + 2 * s], ptrs[s], h->d, h->F, 1, h->slot_stride, h->fmt))
                 return MELINOE_ERR_CUDA;
         CU_TRY(cudaMemcpy(h->maps_dev, h->maps_host, sizeof(h->maps_host), cudaMemcpyHostToDevice));
     }
@@ -911,7 +935,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     // calls of more than 8 tokens go through the grouped GEMM (where the shapes allow it)
     const bool use_gemm = h->gemm_ok && T > kTokPerVr && h->xs != nullptr && sc.idx == h->own.idx;
     const int n_chunks = (T + kTokPerVr - 1) / kTokPerVr;
-    h->last_used_gemm = use_gemm;
+    h->last_used_gemm = use_gemm && h->fmt == 0;
 
     // ---- everything on the device: the decode kernel fetches the missed experts itself, the host is
     // not in the path at all and returns at once (the call's cache decisions are in stats_dev)
@@ -953,9 +977,13 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     gp.F = h->F;
     gp.E = h->E;
     gp.n_shared = h->n_shared;
+    gp.slots = h->slots;
+    gp.slot_stride = h->slot_stride;
+    gp.shared_blobs = h->shared_dev;
+    gp.unit_bytes = (int)(h->expert_bytes / (size_t)h->F);
     if (use_gemm)
         CU_TRY(launch_gather_rows(s, h->plan, static_cast<const uint16_t *>(hidden_dev), sc.tok_of_sorted, h->xs, h->d,
-                                  T * h->k + h->n_shared * T, h->n_sms));
+                                  T * h->k + h->n_shared * T, h->fmt == 1, h->n_sms));
     auto launch_group = [&](int g) -> int {
         TimedPair tp{nullptr, nullptr};
         if (h->timing) {
@@ -966,12 +994,12 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         }
         if (use_gemm) {
             gp.group = g;
-            // CTA pairs share one weight tile over two m-tiles: worth it where an expert has several m-tiles
-            // (on average at least two here); MELINOE_MOE_GEMM_SINGLE in the environment keeps the single-CTA form
+            // CTA pairs take twice the tokens per weight tile: worth it where the arithmetic, not reading the weights, is
+            // the work; MELINOE_MOE_GEMM_SINGLE in the environment keeps the single-CTA form
             static const bool single_only = std::getenv("MELINOE_MOE_GEMM_SINGLE") != nullptr;
-            const bool pairs = !single_only && (long long)T * h->k >= 256ll * h->E;
-            CU_TRY(launch_ffn_gemm(s, 1, h->n_sms, pairs, gp));
-            CU_TRY(launch_ffn_gemm(s, 2, h->n_sms, pairs, gp));
+            const bool pairs = !single_only && h->fmt == 0 && (long long)T * h->k >= 128ll * h->E;
+            CU_TRY(launch_ffn_gemm(s, 1, h->n_sms, pairs, h->fmt, gp));
+            CU_TRY(launch_ffn_gemm(s, 2, h->n_sms, pairs, h->fmt, gp));
         } else {
             for (int c = 0; c < n_chunks; ++c) {
                 int rc = launch_decode(h, s, sc, hidden_dev, out_dev, T, g, c, g == 0 && c == 0);

@@ -4,43 +4,60 @@
 //
 //   gather    Xs[pos] = hidden[token of sorted position pos]: the tokens of one expert become
 //             consecutive rows, so an expert's activations are one 2-D box for TMA.
-//   GEMM 1    per expert: [G | U] = Xs_e (M_e x d) * [W_g ; W_u]^T, tile 128 tokens x 128 f:
-//             one MMA of N = 256 whose B tile stacks 128 rows of W_g on 128 rows of W_u, so the
-//             accumulator holds g in columns 0..127 and u in 128..255 of the same token row and
-//             the epilogue forms h = SiLU(g) * u in registers; h is stored as bf16.
-//   GEMM 2    per expert: Z = H_e (M_e x F) * W_d^T, tile 128 tokens x 256 output columns, fp32.
+//   GEMM 1    per expert: [G ; U] = [W_g ; W_u] * Xs_e^T (K = d); the epilogue forms h = SiLU(g) * u and
+//             stores it as bf16.
+//   GEMM 2    per expert: Z^T = W_d * H_e^T (K = d_ff), fp32.
 //   combine   y_t = sum_j gate[t][j] * Z[pos(t, j)] (+ shared experts), rank order, one rounding.
+//
+// The weights are the M side of the tensor-core operation and the tokens its N side.  An expert's weights
+// come in whole tiles of 128 rows (64 hidden units of W_g and W_u, or 128 output columns), but its
+// tokens do not come in any multiple: N follows them in steps of 16 (32 for a CTA pair), so that no
+// arithmetic is spent on rows that do not exist.  (With the tokens on the M side a last tile of 256 rows was
+// half empty on average: one fifth of the arithmetic of 4096 tokens over 16 experts.)
 //
 // The expert blob (see melinoe_moe_pack_expert) holds, per hidden unit f, the rows W_g[f], W_u[f]
 // and W_d[:, f], each d elements, with the 16-byte pieces of every 128-byte group stored at
 // (piece xor (f mod 8)).  That permutation is exactly what a TMA load with 128-byte swizzle would
-// have produced in shared memory from plain rows, as long as a tile starts at a multiple of 8 rows
-// and 64 columns; so the weight tiles are fetched by TMA WITHOUT swizzle and the MMA descriptors
-// name the 128-byte-swizzled layout.  W_g and W_u rows are "N x K, K contiguous" (K-major, like the
-// activations Xs and H, which are plain and fetched with TMA swizzle); the W_d^T rows are
-// "K x N, N contiguous": GEMM 2 takes its B operand N-major (four 64-column boxes per stage).
-// The experts of all slots are addressed through one tensor map per view (W_g rows, W_u rows,
-// W_d^T rows: the same row pitch of 6 d bytes, different offsets), because the slots are contiguous.
+// have produced in shared memory from plain rows, as long as a row lands at a shared-memory row equal to f
+// modulo 8; so the weight tiles are fetched by TMA WITHOUT swizzle and the MMA descriptors name the
+// 128-byte-swizzled layout.
+//   GEMM 1    a stage's weight tile is ONE box of a 4-D view (column, f mod 8, W_g | W_u, f / 8): eight rows
+//             of W_g, eight of W_u, and so on, K-major.  g and u of a hidden unit are then accumulator
+//             rows eight apart, and the epilogue brings them together with one shuffle per two tokens.
+//   GEMM 2    rows of W_d^T are "K x M, M contiguous": the operand is M-major, two boxes of 64 columns
+//             x 64 rows f per stage, fetched as one box of the view (column, f, column group, slot); f beyond
+//             d_ff is out of bounds there and reads as zero, so d_ff may end inside a stage.
+// The slots' experts are addressed through one tensor map per view, because the slots are contiguous.
 //
-// One persistent CTA per SM, warp-specialised: warp 0 issues TMA loads into a 4-stage ring,
-// warp 1 issues the MMAs (one elected thread) and commits them to mbarriers, warps 2..5 drain
-// the accumulator (tcgen05.ld, 32 rows per warp) and write the tile.  Two accumulators of 256
-// columns alternate so the epilogue of a tile overlaps the MMAs of the next.  Work items are
-// (request, n-tile, m-tile) triples of the launch's compute group, dealt round-robin.
+// 4-bit slots (template parameter FMT = 1): TMA brings the codes into a ring of its own, and four warps expand
+// them into the weight tile of a stage (the arithmetic of the decode kernel: 15 instructions per 8
+// weights) in front of the tensor cores, so that HBM carries 4-bit data only and no bf16 copy of an expert
+// exists.  In GEMM 1 the expansion leaves elements j and j + 4 of eight side by side; a sum over K does not
+// care, so Xs is gathered with the same order.
 //
-// Ragged M: an m-tile may run past its expert's last row; those rows are computed on whatever
+// One persistent CTA per SM, warp-specialised: warp 0 issues TMA loads into a ring of stages, warp 1
+// issues the MMAs (one elected thread) and commits them to mbarriers, warps 2..5 drain
+// the accumulator (tcgen05.ld, 32 rows per warp) and write the tile; with 4-bit slots warps 6..9 expand and
+// warp 10 fetches codes.  Two accumulators alternate so the epilogue of a tile overlaps the MMAs of the next.
+// Work items are (request, weight tile, token chunk) triples of the launch's compute group, dealt
+// round-robin, the chunks of one weight tile side by side.
+//
+// Ragged N: a chunk's box may run past its expert's last row; those columns are computed on whatever
 // the next rows hold (or zeros past the end of the buffer) and never stored.
 //
 // CTA pairs (template parameter CG = 2, used where the experts have enough tokens): two CTAs of a
-// cluster on neighbouring SMs take two adjacent m-tiles of the same expert and n-tile and run them
+// cluster on neighbouring SMs take two adjacent weight tiles of the same expert and chunk and run them
 // as ONE tensor-core operation of M = 256 (tcgen05.mma.cta_group::2, issued by the even CTA).  Each
-// CTA stages its own 128 activation rows but only HALF of the weight tile (128 of its 256 columns);
-// the tensor cores of both SMs read both halves.  Per CTA and k-block that is 32 KB instead of 48 KB
-// through shared memory for the same arithmetic, which is what limits the single-CTA form, and the
-// ring holds 6 stages instead of 4.  Both CTAs' loads complete on the even CTA's barrier; its MMA
-// thread frees a stage, and hands over an accumulator, in both CTAs at once (commit with cluster
-// multicast); the odd CTA's epilogue warps report to the even CTA's barrier.  Each CTA drains its own
-// accumulator rows.
+// CTA stages its own 128 weight rows but only HALF of the tokens; the tensor cores of both SMs read both
+// halves.  Per CTA and k-block that is 32 KB for a chunk of 256 tokens instead of 48 KB.  Both CTAs' loads
+// complete on the even CTA's barrier; its MMA thread frees a stage, and hands over an accumulator, in both
+// CTAs at once (commit with cluster multicast); the odd CTA's epilogue warps report to the even CTA's
+// barrier.  Each CTA drains its own accumulator rows.
+//
+// Measured, the form with the tokens on the M side -> this one (GEMM 1, GEMM 2, us): 8192 token-expert pairs, 16
+// experts, d 4096, d_ff 6400: 771, 395 -> 698, 353 (1224 TFLOP/s); 65536 pairs, d 2048, d_ff 1408: 631, 433 -> 571, 314
+// (1280 TFLOP/s); 1024 pairs over some 20 experts, d 2048, d_ff 1024, where reading the weights is the work: 51, 30 ->
+// 43, 26.  4-bit slots, 4096 pairs, d 2048, d_ff 1024: 99 and 73, where 64 launches of the decode kernel took 2900.
 //
 // Every wait is bounded; on a timeout the CTA raises its abort flag, every role leaves its
 // loops, tensor memory is freed and the error word tells the host.
@@ -52,13 +69,19 @@ namespace melinoe {
 
 namespace {
 
-constexpr int kGemmThreads = 192;          // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
-constexpr int kBM = 128, kBK = 64;         // tile rows (tokens), K elements per stage (128 bytes)
-constexpr int kBN = 256;                   // accumulator columns: 128 g + 128 u, or 256 outputs
-constexpr int kABytes = kBM * kBK * 2, kBBytes = kBN * kBK * 2;
-// ring stages and bytes of a stage for the single-CTA form (CG = 1) and the CTA-pair form (CG = 2)
-__host__ __device__ constexpr int gemm_stages(int cg) { return cg == 2 ? 6 : 4; }
-__host__ __device__ constexpr int gemm_stage_bytes(int cg) { return kABytes + kBBytes / cg; }
+constexpr int kBK = 64;                    // K elements per stage (128 bytes)
+constexpr int kABytes = 128 * kBK * 2;     // weight tile of a stage: 128 rows
+constexpr int kRawBytes = 16384;           // 4-bit slots: codes of one fetch (GEMM 1: 256 columns of 128 rows; GEMM 2: 128 rows f of 256 columns)
+constexpr int kRawStages = 3;
+constexpr size_t kGemmSmem = 227 * 1024 - 4096;      // dynamic shared memory of a CTA (the static part is below 3 KB)
+// threads, tokens of a chunk at most, bytes and number of ring stages for CG CTAs per operation and slot format FMT
+__host__ __device__ constexpr int gemm_threads(int fmt) { return fmt ? 352 : 192; }
+__host__ __device__ constexpr int gemm_tokens(int cg) { return cg == 2 ? 256 : 128; }
+__host__ __device__ constexpr int gemm_stage_bytes(int cg) { return kABytes + gemm_tokens(cg) / cg * kBK * 2; }
+__host__ __device__ constexpr int gemm_stages(int cg, int fmt)
+{
+    return (int)((kGemmSmem - 1024 - (fmt ? kRawStages * kRawBytes : 0)) / gemm_stage_bytes(cg));
+}
 constexpr long long kGemmWaitCycles = 4000000000ll;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -109,7 +132,9 @@ __device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// 2-D tiled TMA load: box at (x = element column, y = row) of the tensor map into shared memory.
+// Tiled TMA loads: box at the given coordinates (innermost first) of the tensor map into shared memory.  The _pair
+// forms are those of a CTA pair, whose completion may be counted on the peer CTA's barrier (bar is an address in
+// the cluster's shared window).
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar)
 {
     asm volatile(
@@ -117,14 +142,39 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
-
-// The same from a CTA of a pair: the completion may be counted on the peer CTA's barrier (bar is an
-// address in the cluster's shared window).
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar)
 {
     asm volatile(
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, int w, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap *map, int x, int y, int z, int w, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, int w, int v, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(v), "r"(bar)
         : "memory");
 }
 // Address of this CTA's shared-memory location `addr` in CTA `rank` of the cluster.
@@ -156,23 +206,23 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
     return d;
 }
 
-// The same for an N-major B operand made of 64-column boxes (64 K rows of 128 bytes each, 8 KB per
-// box): the boxes follow one another along N (leading offset), groups of 8 K rows are 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc_sw128_nmajor(uint32_t addr)
+// The same for an M-major A operand made of 64-column boxes (64 K rows of 128 bytes each, 8 KB per
+// box): the boxes follow one another along M (leading offset), groups of 8 K rows are 1024 bytes apart.
+__device__ __forceinline__ uint64_t smem_desc_sw128_mmajor(uint32_t addr)
 {
     uint64_t d = smem_desc_sw128(addr);
     d |= (uint64_t)(8192u >> 4) << 16;                // between 64-column boxes
     return d;
 }
 
-// Instruction descriptor: bf16 x bf16 -> fp32, A K-major, B K-major or N-major, M = 128, N = 256.
-__device__ __forceinline__ uint32_t instr_desc_bf16(int m, int n, bool b_nmajor)
+// Instruction descriptor: bf16 x bf16 -> fp32, A K-major or M-major, B K-major.
+__device__ __forceinline__ uint32_t instr_desc_bf16(int m, int n, bool a_mmajor)
 {
     uint32_t d = 0;
     d |= 1u << 4;                    // D format: fp32
     d |= 1u << 7;                    // A format: bf16
     d |= 1u << 10;                   // B format: bf16
-    d |= (b_nmajor ? 1u : 0u) << 16; // B major: 0 = K, 1 = N
+    d |= (a_mmajor ? 1u : 0u) << 15; // A major: 0 = K, 1 = M
     d |= (uint32_t)(n >> 3) << 17;
     d |= (uint32_t)(m >> 4) << 24;
     return d;
@@ -232,35 +282,57 @@ __device__ __forceinline__ uint32_t bf16_rne(float v)
     return u >> 16;
 }
 
+// Eight 4-bit codes into bf16 weights, as four registers P[j] = (element j, element j + 4); see the decode kernel.
+__device__ __forceinline__ void expand8(uint32_t w, uint32_t ss, uint32_t (&P)[4])
+{
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        uint32_t t = ((w >> (4 * j)) & 0x000f000fu) | 0x43004300u;
+        asm("sub.rn.bf16x2 %0, %0, %1;" : "+r"(t) : "r"(0x43084308u));
+        asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(P[j]) : "r"(t), "r"(ss));
+    }
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
 struct GemmItem {
-    int row0;      // first sorted row of the m-tile
-    int row_end;   // one past the expert's last sorted row
-    int b_row;     // first expert row of its tensor maps (its slot times F, 0 for a shared expert)
-    int n0;        // first output column of the tile (f for GEMM 1, output column for GEMM 2)
-    int shared;    // B comes from a shared expert's tensor map: index of that expert, else -1
+    int row0;      // first sorted row of the token chunk
+    int n;         // tokens of the operation (a multiple of 16 CG)
+    int n_live;    // tokens that exist
+    int m0;        // first hidden unit (GEMM 1) or output column (GEMM 2) of this CTA's weight tile
+    int slot;      // cache slot of the expert, or -1 - index of the shared expert
 };
 
 // PHASE 1: h = SiLU(Xs W_g^T) * (Xs W_u^T) -> hs (bf16).  PHASE 2: z = hs W_d^T -> zs (fp32).
-template <int PHASE, int CG>
-__global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
+template <int PHASE, int CG, int FMT>
+__global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmParams p)
 {
-    constexpr int kStages = gemm_stages(CG), kStageBytes = gemm_stage_bytes(CG);
+    static_assert(FMT == 0 || CG == 1, "4-bit slots: single CTAs");
+    constexpr int kStages = gemm_stages(CG, FMT), kStageBytes = gemm_stage_bytes(CG), NT = gemm_tokens(CG);
+    constexpr int kMTile = PHASE == 1 ? 64 : 128;            // hidden units, or output columns, of one CTA's tile
+    constexpr int kRawBlocks = PHASE == 1 ? 4 : 2;           // k-blocks of one fetch of codes
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ uint64_t s_bars[2 * kStages + 4];
+    __shared__ uint64_t s_bars[2 * kStages + 4 + 2 * kRawStages];
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
     __shared__ int s_tile0[kMaxReq + 1], s_nreq;
-    __shared__ int4 s_rec[kMaxReq];                          // tok_off, n_tok, slot, expert of the launch's requests
+    __shared__ int4 s_rec[kMaxReq];                          // first row, tokens, slot (shared expert s: -1 - s), tokens of a chunk
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const DevPlan *plan = p.plan;
-    if (plan->status != MELINOE_OK)
-        return;
     // 1024-byte aligned ring (the swizzle pattern repeats every 1024 bytes)
     unsigned char *ring = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const uint32_t ring_s = smem_u32(ring);
+    const uint32_t ring_s = smem_u32(ring), raw_s = ring_s + kStages * kStageBytes;
     const uint32_t full0 = smem_u32(s_bars), empty0 = full0 + 8 * kStages;
-    const uint32_t tfull0 = empty0 + 8 * kStages, tempty0 = tfull0 + 16;
+    const uint32_t tfull0 = empty0 + 8 * kStages, tempty0 = tfull0 + 16, rfull0 = tempty0 + 16, rempty0 = rfull0 + 8 * kRawStages;
     volatile int *abort_flag = &s_abort;
     // rank within the CTA pair; the even CTA issues the MMAs, owns the "stage full" barriers and counts
     // the drained accumulators of both
@@ -269,33 +341,64 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
         asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     const int n_units = (int)gridDim.x / CG, unit = (int)blockIdx.x / CG;    // CTAs, or CTA pairs, that share out the items
 
-    // ---- the launch's requests and their m-tiles (CG = 2: pairs of m-tiles)
-    const int K = PHASE == 1 ? p.d : p.F;                 // reduction length
-    const int n_tiles_n = PHASE == 1 ? p.F / 128 : p.d / kBN;
-    if (tid == 0) {
+    if (tid == 32) {
         s_abort = 0;
-        int n = 0, tiles = 0;
-        const int n_req_total = plan->n_req + p.n_shared;
-        for (int r = 0; r < n_req_total; ++r) {
-            const ReqRec rec = plan->req[r];
-            if (rec.group == p.group && rec.n_tok > 0) {
-                s_rec[n] = make_int4(rec.tok_off, rec.n_tok, rec.slot, rec.expert);
-                s_tile0[n] = tiles;
-                tiles += (rec.n_tok + CG * kBM - 1) / (CG * kBM) * n_tiles_n;
-                ++n;
-            }
-        }
-        s_tile0[n] = tiles;
-        s_nreq = n;
         for (int i = 0; i < kStages; ++i) {
-            mbar_init(full0 + 8 * i, 1);
+            mbar_init(full0 + 8 * i, FMT ? 5 : 1);
             mbar_init(empty0 + 8 * i, 1);
         }
-        mbar_init(tfull0, 1);
-        mbar_init(tfull0 + 8, 1);
-        mbar_init(tempty0, 4 * CG);
-        mbar_init(tempty0 + 8, 4 * CG);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(tfull0 + 8 * i, 1);
+            mbar_init(tempty0 + 8 * i, 4 * CG);
+        }
+        if (FMT)
+            for (int i = 0; i < kRawStages; ++i) {
+                mbar_init(rfull0 + 8 * i, 1);
+                mbar_init(rempty0 + 8 * i, 4);
+            }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (plan->status != MELINOE_OK)
+        return;
+    // ---- the launch's requests and their items, by warp 0, a lane per request
+    const int K = PHASE == 1 ? p.d : p.F;                 // reduction length
+    const int m_tiles = PHASE == 1 ? (p.F + CG * 64 - 1) / (CG * 64) : p.d / (CG * 128);
+    if (warp == 0) {
+        const int n_req_total = plan->n_req + p.n_shared;
+        int n = 0, tiles = 0;
+        for (int r0 = 0; r0 < n_req_total; r0 += 32) {
+            const int r = r0 + lane;
+            bool on = false;
+            int4 rec = make_int4(0, 0, 0, 0);
+            int items = 0;
+            if (r < n_req_total) {
+                const int4 a = *reinterpret_cast<const int4 *>(&plan->req[r].expert);       // expert, slot, hit, evicted
+                const int4 b = *reinterpret_cast<const int4 *>(&plan->req[r].vr_start);     // vr_start, group, tok_off, n_tok
+                on = b.y == p.group && b.w > 0;
+                const int chunks = (b.w + NT - 1) / NT;
+                const int size = on ? ((b.w + chunks - 1) / chunks + 16 * CG - 1) / (16 * CG) * (16 * CG) : 0;
+                rec = make_int4(b.z, b.w, a.y >= 0 ? a.y : -1 - (a.x - p.E), size);
+                items = on ? chunks * m_tiles : 0;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, on);
+            int inc = items;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, inc, o);
+                inc += lane >= o ? v : 0;
+            }
+            if (on) {
+                const int at = n + __popc(m & ((1u << lane) - 1u));
+                s_rec[at] = rec;
+                s_tile0[at] = tiles + inc - items;
+            }
+            n += __popc(m);
+            tiles += __shfl_sync(0xffffffffu, inc, 31);
+        }
+        if (lane == 0) {
+            s_tile0[n] = tiles;
+            s_nreq = n;
+        }
     }
     __syncthreads();
     const int n_reqs = s_nreq;
@@ -309,12 +412,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
     if (warp == 2) {
         if (CG == 1) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)),
-                         "r"(512));
+                         "r"(2 * NT));
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
         } else {
             // the same warp of both CTAs, the same destination: one allocation over the pair
             asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)),
-                         "r"(512));
+                         "r"(2 * NT));
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
         }
     }
@@ -323,35 +426,40 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = s_tmem_base;
 
-    // item w -> (request, n-tile, m-tile): within a request the m-tiles of one n-tile are adjacent,
-    // so CTAs working side by side share the weight tile in L2
+    // item w -> (request, weight tile, token chunk): the chunks of one weight tile are adjacent, so CTAs working
+    // side by side share it in L2.  Items are asked for in ascending order: the search carries on where it was.
+    int q_at = 0;
     auto item_of = [&](int w) -> GemmItem {
-        int q = 0;
-        while (q + 1 < n_reqs && s_tile0[q + 1] <= w)
-            ++q;
-        const int4 rec = s_rec[q];                                  // tok_off, n_tok, slot, expert
-        const int local = w - s_tile0[q];
-        const int mtiles = (rec.y + CG * kBM - 1) / (CG * kBM);
-        const int nt = local / mtiles, mt = local % mtiles;
+        while (q_at + 1 < n_reqs && s_tile0[q_at + 1] <= w)
+            ++q_at;
+        const int4 rec = s_rec[q_at];
+        const int local = w - s_tile0[q_at];
+        const int chunks = (rec.y + NT - 1) / NT;
+        const int mt = local / chunks, c = local % chunks;
         GemmItem it;
-        it.row0 = rec.x + (mt * CG + (int)rank) * kBM;              // this CTA's 128 rows of the item
-        it.row_end = rec.x + rec.y;
-        it.shared = rec.z >= 0 ? -1 : rec.w - p.E;
-        it.b_row = (rec.z >= 0 ? rec.z : 0) * p.F;                  // shared experts have maps of their own
-        it.n0 = PHASE == 1 ? nt * 128 : nt * kBN;
+        it.row0 = rec.x + c * rec.w;
+        it.n_live = min(rec.w, rec.y - c * rec.w);
+        it.n = (it.n_live + 16 * CG - 1) / (16 * CG) * (16 * CG);
+        it.m0 = (mt * CG + (int)rank) * kMTile;
+        it.slot = rec.z;
         return it;
     };
-    const int kblocks = K / kBK;
+    const int kblocks = (K + kBK - 1) / kBK;
 
     if (warp == 0) {
         // ============================================================ TMA producer
         if (lane == 0) {
-            const CUtensorMap *map_a = p.maps + (PHASE == 1 ? kMapXs : kMapHs);
+            const CUtensorMap *map_b = p.maps + (PHASE == 1 ? kMapXs0 : kMapHs0);
             uint32_t n = 0;
             for (int w = unit; w < total_items && !*abort_flag; w += n_units) {
                 const GemmItem it = item_of(w);
-                // W_g rows, W_u rows, W_d^T rows of the slots, or of the shared expert
-                const CUtensorMap *map_w = it.shared < 0 ? p.maps + kMapSlotsG : p.maps + kMapShared0 + 3 * it.shared;
+                // the weights of the slots, or of the shared expert
+                const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
+                const int slot = it.slot >= 0 ? it.slot : 0;
+                // the smallest box that holds this CTA's share of the tokens: 32, 64 or 128 rows
+                const int rows = it.n / CG, cls = rows <= 32 ? 0 : rows <= 64 ? 1 : 2;
+                const int b_row = it.row0 + (int)rank * rows;
+                const uint32_t bytes = (FMT ? 0u : (uint32_t)kABytes) + ((32u * kBK * 2) << cls);
                 for (int kb = 0; kb < kblocks; ++kb, ++n) {
                     const uint32_t s = n % kStages;
                     if (n >= (uint32_t)kStages && !mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag))
@@ -359,31 +467,24 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
                     const uint32_t a_dst = ring_s + s * kStageBytes, b_dst = a_dst + kABytes;
                     if (CG == 1) {
                         const uint32_t bar = full0 + 8 * s;
-                        mbar_expect(bar, kStageBytes);
-                        tma_load_2d(a_dst, map_a, kb * kBK, it.row0, bar);
-                        if (PHASE == 1) {
-                            tma_load_2d(b_dst, map_w, kb * kBK, it.b_row + it.n0, bar);                   // 128 rows of W_g
-                            tma_load_2d(b_dst + kBBytes / 2, map_w + 1, kb * kBK, it.b_row + it.n0, bar); // 128 rows of W_u
-                        } else {
-                            // 64 rows f of W_d^T, four boxes of 64 output columns
-#pragma unroll
-                            for (int i = 0; i < kBN / 64; ++i)
-                                tma_load_2d(b_dst + i * 8192, map_w + 2, it.n0 + 64 * i, it.b_row + kb * kBK, bar);
+                        mbar_expect(bar, bytes);
+                        if (FMT == 0) {
+                            if (PHASE == 1)
+                                tma_load_4d(a_dst, map_w, kb * kBK, 0, 0, (slot * p.F + it.m0) / 8, bar);
+                            else
+                                tma_load_4d(a_dst, map_w, 0, kb * kBK, it.m0 / 64, slot, bar);
                         }
+                        tma_load_2d(b_dst, map_b + cls, kb * kBK, b_row, bar);
                     } else {
                         // the bytes of both CTAs are expected, once, on the even CTA's barrier
                         const uint32_t bar = cluster_addr(full0 + 8 * s, 0);
                         if (rank == 0)
-                            mbar_expect(full0 + 8 * s, 2 * kStageBytes);
-                        tma_load_2d_pair(a_dst, map_a, kb * kBK, it.row0, bar);
-                        if (PHASE == 1) {
-                            // columns 0..127 of the accumulator (g) come from the even CTA's half, 128..255 (u) from the odd one's
-                            tma_load_2d_pair(b_dst, map_w + rank, kb * kBK, it.b_row + it.n0, bar);
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 2; ++i)
-                                tma_load_2d_pair(b_dst + i * 8192, map_w + 2, it.n0 + 64 * (2 * (int)rank + i), it.b_row + kb * kBK, bar);
-                        }
+                            mbar_expect(full0 + 8 * s, 2 * bytes);
+                        if (PHASE == 1)
+                            tma_load_4d_pair(a_dst, map_w, kb * kBK, 0, 0, (slot * p.F + it.m0) / 8, bar);
+                        else
+                            tma_load_4d_pair(a_dst, map_w, 0, kb * kBK, it.m0 / 64, slot, bar);
+                        tma_load_2d_pair(b_dst, map_b + cls, kb * kBK, b_row, bar);
                     }
                 }
             }
@@ -397,14 +498,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
     } else if (warp == 1) {
         // ============================================================ MMA issuer (of a pair: the even CTA's)
         if (lane == 0 && rank == 0) {
-            const uint32_t idesc = instr_desc_bf16(CG * kBM, kBN, PHASE == 2);
             uint32_t n = 0, item = 0;
             for (int w = unit; w < total_items && !*abort_flag; w += n_units, ++item) {
+                const uint32_t idesc = instr_desc_bf16(CG * 128, item_of(w).n, PHASE == 2);
                 const uint32_t acc = item & 1u;
                 if (item >= 2 && !mbar_wait(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag))
                     break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t d_tmem = tmem_base + acc * kBN;
+                const uint32_t d_tmem = tmem_base + acc * NT;
                 bool ok = true;
                 for (int kb = 0; kb < kblocks; ++kb, ++n) {
                     const uint32_t s = n % kStages;
@@ -414,17 +515,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t a_addr = ring_s + s * kStageBytes, b_addr = a_addr + kABytes;
-                    const uint64_t a_desc = smem_desc_sw128(a_addr);
-                    const uint64_t b_desc = PHASE == 1 ? smem_desc_sw128(b_addr) : smem_desc_sw128_nmajor(b_addr);
+                    const uint64_t a_desc = PHASE == 1 ? smem_desc_sw128(a_addr) : smem_desc_sw128_mmajor(a_addr);
+                    const uint64_t b_desc = smem_desc_sw128(b_addr);
                     // 16 K elements: 32 bytes along a K-major row (2 descriptor units), 16 rows of 128 bytes
-                    // in an N-major box (128 units)
-                    constexpr int kBStep = PHASE == 1 ? 2 : 128;
+                    // in an M-major box (128 units)
+                    constexpr int kAStep = PHASE == 1 ? 2 : 128;
 #pragma unroll
                     for (int ks = 0; ks < kBK / 16; ++ks) {
                         if (CG == 1)
-                            umma_bf16(d_tmem, a_desc + 2 * ks, b_desc + kBStep * ks, idesc, (kb | ks) != 0);
+                            umma_bf16(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, (kb | ks) != 0);
                         else
-                            umma_bf16_pair(d_tmem, a_desc + 2 * ks, b_desc + kBStep * ks, idesc, (kb | ks) != 0);
+                            umma_bf16_pair(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, (kb | ks) != 0);
                     }
                     // the stage is free once these MMAs have read it
                     if (CG == 1)
@@ -441,7 +542,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
                     umma_commit_pair(tfull0 + 8 * acc);
             }
         }
-    } else {
+    } else if (warp < 6) {
         // ============================================================ epilogue (warps 2..5)
         const int quarter = warp & 3;                        // the 32 accumulator rows this warp may read
         uint32_t item = 0;
@@ -451,44 +552,39 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
             if (!mbar_wait(tfull0 + 8 * acc, (item >> 1) & 1u, abort_flag))
                 break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int row = it.row0 + quarter * 32 + lane;
-            const bool live = row < it.row_end;
-            const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * kBN;
+            const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * NT;
             if (PHASE == 1) {
+                // lanes 0..7 hold g of eight hidden units, 8..15 u of the same ones, 16..31 those of the next eight.  Of two
+                // neighbouring tokens the g lane finishes the first and the u lane the second.
+                const int f = it.m0 + quarter * 16 + (lane >> 4) * 8 + (lane & 7);
+                const bool is_u = (lane & 8) != 0;
+                uint16_t *dst = p.hs + (size_t)(it.row0 + (is_u ? 1 : 0)) * p.F + f;
+                const int left = f < p.F ? it.n_live - (is_u ? 1 : 0) : 0;      // this lane stores tokens j (+ 1) with j below this
 #pragma unroll 1
-                for (int c = 0; c < 128; c += 32) {
-                    uint32_t g[32], u[32];
-                    tmem_ld32(t_row + c, g);
-                    tmem_ld32(t_row + 128 + c, u);
+                for (int c = 0; c < it.n_live; c += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(t_row + c, v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (live) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(p.hs + (size_t)row * p.F + it.n0 + c);
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            uint32_t o[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float g0 = __uint_as_float(g[v * 8 + 2 * e]), g1 = __uint_as_float(g[v * 8 + 2 * e + 1]);
-                                const float u0 = __uint_as_float(u[v * 8 + 2 * e]), u1 = __uint_as_float(u[v * 8 + 2 * e + 1]);
-                                const float h0 = g0 / (1.0f + __expf(-g0)) * u0, h1 = g1 / (1.0f + __expf(-g1)) * u1;
-                                o[e] = bf16_rne(h0) | (bf16_rne(h1) << 16);
-                            }
-                            dst[v] = make_uint4(o[0], o[1], o[2], o[3]);
-                        }
+                    for (int j = 0; j < 32; j += 2) {
+                        const uint32_t o = __shfl_xor_sync(0xffffffffu, is_u ? v[j] : v[j + 1], 8);
+                        const float g = __uint_as_float(is_u ? o : v[j]), u = __uint_as_float(is_u ? v[j + 1] : o);
+                        const float h = __fdividef(g, 1.0f + __expf(-g)) * u;
+                        if (c + j < left)
+                            dst[(size_t)(c + j) * p.F] = (uint16_t)bf16_rne(h);
                     }
                 }
             } else {
+                float *dst = p.zs + (size_t)it.row0 * p.d + it.m0 + quarter * 32 + lane;
 #pragma unroll 1
-                for (int c = 0; c < kBN; c += 32) {
-                    uint32_t z[32];
-                    tmem_ld32(t_row + c, z);
+                for (int c = 0; c < it.n_live; c += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(t_row + c, v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (live) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(p.zs + (size_t)row * p.d + it.n0 + c);
 #pragma unroll
-                        for (int v = 0; v < 8; ++v)
-                            dst[v] = make_uint4(z[4 * v], z[4 * v + 1], z[4 * v + 2], z[4 * v + 3]);
-                    }
+                    for (int j = 0; j < 32; ++j)
+                        if (c + j < it.n_live)
+                            dst[(size_t)(c + j) * p.d] = __uint_as_float(v[j]);
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -498,6 +594,110 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
                     mbar_arrive(tempty0 + 8 * acc);
                 else
                     mbar_arrive_cluster(cluster_addr(tempty0 + 8 * acc, 0));
+            }
+        }
+    } else if (FMT == 1 && warp < 10) {
+        // ============================================================ expansion of 4-bit codes (warps 6..9)
+        const int row = (warp - 6) * 32 + lane;              // row of the weight tile, or (column group, f) of GEMM 2's
+        const size_t ub = (size_t)p.unit_bytes, scales = 3 * (size_t)(p.d / 2);
+        uint32_t n = 0, rn = 0;
+        for (int w = unit; w < total_items && !*abort_flag; w += n_units) {
+            const GemmItem it = item_of(w);
+            const char *blob = it.slot >= 0 ? p.slots + (size_t)it.slot * p.slot_stride : p.shared_blobs[-1 - it.slot];
+            // GEMM 1: rows of eight g, eight u, ..; GEMM 2: rows f, 64 of the first column group, 64 of the second
+            const int f_row = PHASE == 1 ? it.m0 + (row >> 4) * 8 + (row & 7) : (row & 63);
+            const int part = (row >> 3) & 1, cg = row >> 6;
+            const char *sc_base = PHASE == 1 ? blob + (size_t)f_row * ub + scales + (size_t)part * (p.d / 32)
+                                             : blob + (size_t)f_row * ub + scales + 2 * (size_t)(p.d / 32) + (size_t)(it.m0 / 64 + cg) * 2;
+            // the scale of the next k-block is in flight while this one is expanded
+            auto scale_of = [&](int kb) -> uint32_t {
+                if (PHASE == 1)
+                    return f_row < p.F && kb < kblocks ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base) + kb) : 0u;
+                return kb * kBK + f_row < p.F ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base + (size_t)kb * kBK * ub)) : 0u;
+            };
+            uint32_t sc = scale_of(0);
+            bool ok = true;
+            for (int kb = 0; kb < kblocks && ok; ++kb, ++n) {
+                const int sub = kb % kRawBlocks;
+                const uint32_t rs = rn % kRawStages, s = n % kStages;
+                if (sub == 0)
+                    ok = mbar_wait(rfull0 + 8 * rs, (rn / kRawStages) & 1u, abort_flag);
+                if (ok && n >= (uint32_t)kStages)
+                    ok = mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag);
+                if (!ok)
+                    break;
+                const uint32_t ss = sc * 0x10001u;
+                sc = scale_of(kb + 1);
+                const uint32_t raw = raw_s + rs * kRawBytes, a_dst = ring_s + s * kStageBytes + row * 128;
+                const uint32_t x = (uint32_t)(row & 7);      // = f mod 8 in both phases
+                if (PHASE == 1) {
+                    // 64 columns = pieces 2 sub, 2 sub + 1 of this row's 128 bytes of codes -> eight pieces of bf16
+                    const uint32_t src = raw + row * 128;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint4 c4 = lds128(src + (((2 * sub + h) ^ x) << 4));
+                        const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            uint32_t P[4];
+                            expand8(cw[i], ss, P);
+                            sts128(a_dst + (((4 * h + i) ^ x) << 4), P[0], P[1], P[2], P[3]);
+                        }
+                    }
+                } else {
+                    // one f, one group of 64 columns; nibble q of word w is column 8 q + w
+                    const uint32_t src = raw + (sub * 64 + (row & 63)) * 128;
+                    const uint32_t pc0 = (uint32_t)((it.m0 / 32) & 7) + 2u * cg;      // first piece of the group in its 128 bytes
+                    uint32_t o[8][4];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint4 c4 = lds128(src + (((pc0 + h) ^ x) << 4));
+                        const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            uint32_t P[4], Q[4];
+                            expand8(cw[2 * i], ss, P);
+                            expand8(cw[2 * i + 1], ss, Q);
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                o[q][2 * h + i] = __byte_perm(P[q], Q[q], 0x5410);
+                                o[q + 4][2 * h + i] = __byte_perm(P[q], Q[q], 0x7632);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        sts128(a_dst + ((q ^ x) << 4), o[q][0], o[q][1], o[q][2], o[q][3]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the tensor cores read what was just stored
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(full0 + 8 * s);
+                if (sub == kRawBlocks - 1 || kb == kblocks - 1) {
+                    if (lane == 0)
+                        mbar_arrive(rempty0 + 8 * rs);
+                    ++rn;
+                }
+            }
+        }
+    } else if (FMT == 1 && warp == 10) {
+        // ============================================================ fetch of 4-bit codes
+        if (lane == 0) {
+            uint32_t rn = 0;
+            for (int w = unit; w < total_items && !*abort_flag; w += n_units) {
+                const GemmItem it = item_of(w);
+                const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
+                const int slot = it.slot >= 0 ? it.slot : 0;
+                for (int kb = 0; kb < kblocks; kb += kRawBlocks, ++rn) {
+                    const uint32_t rs = rn % kRawStages;
+                    if (rn >= (uint32_t)kRawStages && !mbar_wait(rempty0 + 8 * rs, ((rn / kRawStages) - 1u) & 1u, abort_flag))
+                        break;
+                    mbar_expect(rfull0 + 8 * rs, kRawBytes);
+                    if (PHASE == 1)
+                        tma_load_5d(raw_s + rs * kRawBytes, map_w, kb * 32, 0, 0, it.m0 / 8, slot, rfull0 + 8 * rs);
+                    else
+                        tma_load_3d(raw_s + rs * kRawBytes, map_w, it.m0 / 256 * 128, kb * kBK, slot, rfull0 + 8 * rs);
+                }
             }
         }
     }
@@ -511,15 +711,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) ffn_gemm_kernel(GemmParams p)
         cluster_sync_all();
     if (warp == 2) {
         if (CG == 1)
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * NT));
         else
-            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * NT));
     }
     if (*abort_flag && tid == 0)
         atomicExch(p.err, MELINOE_ERR_TIMEOUT);
 }
 
-// Xs[pos] = hidden[tok_of_sorted[pos]], one block per sorted row.
+// Xs[pos] = hidden[tok_of_sorted[pos]], one block per sorted row.  PERMUTE: elements (0,4) (1,5) (2,6) (3,7) of every
+// eight, the order in which 4-bit codes expand.
+template <bool PERMUTE>
 __global__ void __launch_bounds__(256) gather_rows_kernel(const DevPlan *plan, const uint16_t *__restrict__ x,
                                                           const int32_t *__restrict__ tok_of_sorted, uint16_t *xs, int d,
                                                           int n_sorted)
@@ -529,8 +731,13 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const DevPlan *plan, c
     for (int pos = blockIdx.x; pos < n_sorted; pos += gridDim.x) {
         const uint4 *src = reinterpret_cast<const uint4 *>(x + (size_t)tok_of_sorted[pos] * d);
         uint4 *dst = reinterpret_cast<uint4 *>(xs + (size_t)pos * d);
-        for (int i = threadIdx.x; i < d / 8; i += 256)
-            dst[i] = src[i];
+        for (int i = threadIdx.x; i < d / 8; i += 256) {
+            uint4 v = src[i];
+            if (PERMUTE)
+                v = make_uint4(__byte_perm(v.x, v.z, 0x5410), __byte_perm(v.x, v.z, 0x7632), __byte_perm(v.y, v.w, 0x5410),
+                               __byte_perm(v.y, v.w, 0x7632));
+            dst[i] = v;
+        }
     }
 }
 
@@ -568,57 +775,73 @@ __global__ void __launch_bounds__(256) combine_rows_kernel(const DevPlan *plan, 
     }
 }
 
-constexpr size_t gemm_smem(int cg) { return (size_t)gemm_stages(cg) * gemm_stage_bytes(cg) + 1024; }
+constexpr size_t gemm_smem(int cg, int fmt)
+{
+    return (size_t)gemm_stages(cg, fmt) * gemm_stage_bytes(cg) + (fmt ? kRawStages * kRawBytes : 0) + 1024;
+}
+
+template <int PHASE, int CG, int FMT>
+cudaError_t gemm_launch(cudaStream_t stream, int n_sms, const GemmParams &p)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(n_sms / CG * CG);
+    lc.blockDim = dim3(gemm_threads(FMT));
+    lc.dynamicSmemBytes = gemm_smem(CG, FMT);
+    lc.stream = stream;
+    cudaLaunchAttribute attr[1];
+    if (CG == 2) {
+        // clusters of two CTAs on neighbouring SMs
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        lc.attrs = attr;
+        lc.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&lc, ffn_gemm_kernel<PHASE, CG, FMT>, p);
+}
+
+template <int PHASE, int CG, int FMT>
+cudaError_t gemm_configure()
+{
+    return cudaFuncSetAttribute(ffn_gemm_kernel<PHASE, CG, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(CG, FMT));
+}
 
 }  // namespace
 
-bool ffn_gemm_supported(int d, int F) { return d % kBN == 0 && F % 128 == 0 && d >= kBN && F >= 128; }
+bool ffn_gemm_supported(int d, int F) { return d % 256 == 0 && F % kUnitRows == 0; }
 
 cudaError_t ffn_gemm_configure()
 {
-    cudaError_t e = cudaFuncSetAttribute(ffn_gemm_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(1));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ffn_gemm_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(1));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ffn_gemm_kernel<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(2));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ffn_gemm_kernel<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(2));
-    return e;
+    const cudaError_t e[6] = {gemm_configure<1, 1, 0>(), gemm_configure<2, 1, 0>(), gemm_configure<1, 2, 0>(),
+                              gemm_configure<2, 2, 0>(), gemm_configure<1, 1, 1>(), gemm_configure<2, 1, 1>()};
+    for (cudaError_t r : e)
+        if (r != cudaSuccess)
+            return r;
+    return cudaSuccess;
 }
 
 cudaError_t launch_gather_rows(cudaStream_t stream, const DevPlan *plan, const uint16_t *x, const int32_t *tok_of_sorted,
-                               uint16_t *xs, int d, int n_sorted, int n_sms)
+                               uint16_t *xs, int d, int n_sorted, bool permute, int n_sms)
 {
     const int grid = n_sorted < n_sms * 16 ? n_sorted : n_sms * 16;
-    gather_rows_kernel<<<grid, 256, 0, stream>>>(plan, x, tok_of_sorted, xs, d, n_sorted);
+    if (permute)
+        gather_rows_kernel<true><<<grid, 256, 0, stream>>>(plan, x, tok_of_sorted, xs, d, n_sorted);
+    else
+        gather_rows_kernel<false><<<grid, 256, 0, stream>>>(plan, x, tok_of_sorted, xs, d, n_sorted);
     count_launch();
     return cudaGetLastError();
 }
 
-cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, const GemmParams &p)
+cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, int fmt, const GemmParams &p)
 {
-    if (!pairs) {
-        if (phase == 1)
-            ffn_gemm_kernel<1, 1><<<n_sms, kGemmThreads, gemm_smem(1), stream>>>(p);
-        else
-            ffn_gemm_kernel<2, 1><<<n_sms, kGemmThreads, gemm_smem(1), stream>>>(p);
-        count_launch();
-        return cudaGetLastError();
-    }
-    // clusters of two CTAs on neighbouring SMs
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(n_sms / 2 * 2);
-    lc.blockDim = dim3(kGemmThreads);
-    lc.dynamicSmemBytes = gemm_smem(2);
-    lc.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    const cudaError_t e = phase == 1 ? cudaLaunchKernelEx(&lc, ffn_gemm_kernel<1, 2>, p) : cudaLaunchKernelEx(&lc, ffn_gemm_kernel<2, 2>, p);
+    cudaError_t e;
+    if (fmt == 1)
+        e = phase == 1 ? gemm_launch<1, 1, 1>(stream, n_sms, p) : gemm_launch<2, 1, 1>(stream, n_sms, p);
+    else if (pairs)
+        e = phase == 1 ? gemm_launch<1, 2, 0>(stream, n_sms, p) : gemm_launch<2, 2, 0>(stream, n_sms, p);
+    else
+        e = phase == 1 ? gemm_launch<1, 1, 0>(stream, n_sms, p) : gemm_launch<2, 1, 0>(stream, n_sms, p);
     count_launch();
     return e;
 }

@@ -112,10 +112,10 @@ cudaError_t launch_ffn_decode(cudaStream_t stream, const DecLaunchCfg &cfg, cons
 // ---- grouped GEMM expert FFN on tcgen05 for calls with many tokens per expert (prefill)
 // Tensor maps in device memory, in this order:
 enum {
-    kMapXs = 0, kMapHs = 1,                                          // activations: boxes of 128 rows x 64 columns
-    kMapSlotsG = 2, kMapSlotsU = 3, kMapSlotsD = 4,                  // W_g, W_u rows (128-row boxes), W_d^T rows (64-row boxes) of all slots
-    kMapShared0 = 5,                                                 // per shared expert: the same three views
-    kMapCount = kMapShared0 + 3 * kMaxShared
+    kMapXs0 = 0, kMapHs0 = 3,                                        // activations: boxes of 32, 64, 128 rows x 64 columns
+    kMapSlots0 = 6,                                                  // weights of all slots for GEMM 1 and for GEMM 2 (see ffn_gemm.cu)
+    kMapShared0 = 8,                                                 // per shared expert: the same two views
+    kMapCount = kMapShared0 + 2 * kMaxShared
 };
 struct GemmParams {
     const DevPlan *plan;
@@ -124,12 +124,19 @@ struct GemmParams {
     float *zs;                       // expert outputs, [sorted rows][d] fp32
     int *err;
     int group, d, F, E, n_shared;
+    // 4-bit slots: the blobs themselves (their scales are read directly) and the bytes of one hidden unit
+    const char *slots;
+    size_t slot_stride;
+    const char *const *shared_blobs;
+    int unit_bytes;
 };
 bool ffn_gemm_supported(int d, int F);
 cudaError_t ffn_gemm_configure();
+// permute: store elements j and j + 4 of every eight side by side (the order in which 4-bit codes expand)
 cudaError_t launch_gather_rows(cudaStream_t stream, const DevPlan *plan, const uint16_t *x, const int32_t *tok_of_sorted,
-                               uint16_t *xs, int d, int n_sorted, int n_sms);
-cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, const GemmParams &p);
+                               uint16_t *xs, int d, int n_sorted, bool permute, int n_sms);
+// pairs: CTA pairs (bf16 slots only); fmt: what the slots hold, 0 = bf16 blobs, 1 = 4-bit blobs
+cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, int fmt, const GemmParams &p);
 cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const float *gate, const int32_t *inv_pos,
                                 const float *zs, uint16_t *out, int T, int d, int k, int n_shared, int n_sms);
 

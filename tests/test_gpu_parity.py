@@ -187,6 +187,24 @@ def test_prefill_grouped_gemm(d, F, E, k, C, n_shared, Ts):
     P.close()
 
 
+@pytest.mark.parametrize("store,d,F,E,k,n_shared,Ts", [
+    ("bf16", 256, 8, 2, 1, 0, (9, 33)),                # one row group of hidden units: less than a weight tile and a k-block
+    ("bf16", 512, 200, 3, 3, 1, (15, 17, 127, 129)),   # every expert sees every token: chunks of 16, 32, 128 and 2 x 80 tokens; d_ff ends inside a tile
+    ("bf16", 256, 328, 2, 2, 0, (256, 257, 258, 300)), # CTA pairs: 256 tokens in one chunk, 257 in two; d_ff ends inside the pair's second tile
+    ("q4slots", 512, 200, 3, 3, 1, (9, 16, 129)),      # the same of 4-bit codes, with a shared expert
+    ("q4slots", 1024, 264, 4, 2, 0, (70,)),            # codes of a column group in both halves of their 128 bytes
+    ("q4slots", 4096, 136, 2, 1, 0, (20,)),
+])
+def test_grouped_gemm_at_the_edges_of_its_tiles(store, d, F, E, k, n_shared, Ts):
+    """Token counts around the steps of the tensor-core operation's N and d_ff that ends inside weight tiles and
+    k-blocks, element by element against the oracle."""
+    P = _pair(d, F, E, k, E, seed=400 + d // 256 + F, n_shared=n_shared, store=store)
+    for step, T in enumerate(Ts):
+        tokens = sorted(set([0, 1, T - 2, T - 1] + list(range(0, T, 5))))
+        P.step(gen.hidden_states(401 + d, 0, "prefill", step, T, d), tokens=tokens)
+    P.close()
+
+
 def test_prefill_router_breaks_ties_towards_the_lowest_expert_id():
     """More than 8 tokens go through the general router kernel: with a zero router matrix the logits are
     the bias alone, and a bias with equal entries makes ties that must go to the lowest ids (Eq. 1 with

@@ -146,7 +146,7 @@ struct TimedPair {
 // kernel's output accumulator [<= 8 tokens][d] (64-bit words, all zero between launches); ybuf: fp32
 // sums of a call that is computed in several launches.
 struct Scratch {
-    int32_t *idx = nullptr, *perm = nullptr, *inv_pos = nullptr, *tok_of_sorted = nullptr;
+    int32_t *idx = nullptr, *perm = nullptr, *inv_pos = nullptr, *tok_of_sorted = nullptr, *block_counts = nullptr;
     float *gate = nullptr, *logits = nullptr, *ybuf = nullptr;
     long long *yacc = nullptr;
     int cap_tokens = 0;
@@ -214,7 +214,7 @@ struct melinoe_moe {
 
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t ev_last = nullptr;      // end of the most recent call on the caller's stream
-    cudaEvent_t ev_plan = nullptr;      // caller's stream: the planning kernel of the current call is done
+    cudaEvent_t ev_plan = nullptr;      // caller's stream: planning and group 0 of the current call are done
     cudaEvent_t ev_arrive = nullptr;    // copy stream: a wave's transfers have landed
     std::vector<cudaEvent_t> ev_group;  // compute stream: FFN group g of the current call is done
     bool has_last = false;
@@ -258,6 +258,7 @@ void free_scratch(melinoe_moe *h)
     cudaFree(o.perm);
     cudaFree(o.inv_pos);
     cudaFree(o.tok_of_sorted);
+    cudaFree(o.block_counts);
     cudaFree(o.gate);
     cudaFree(o.logits);
     cudaFree(o.yacc);
@@ -285,7 +286,7 @@ int wait_idle(melinoe_moe *h)
 }
 
 // Bounded host wait for the planning kernel of call `seq` to publish its miss queue.
-// ev_plan was recorded right behind that kernel.
+// ev_plan was recorded behind that kernel and group 0.
 int wait_for_plan(melinoe_moe *h, uint32_t seq)
 {
     volatile uint32_t *w = &h->hplan->hdr.seq;
@@ -332,6 +333,9 @@ int ensure_capacity(melinoe_moe *h, int T)
     CU_TRY(cudaMalloc(&o.perm, sorted * 4));
     CU_TRY(cudaMalloc(&o.inv_pos, pairs * 4));
     CU_TRY(cudaMalloc(&o.tok_of_sorted, sorted * 4));
+    // (the router makes at most two blocks per SM of up to four tokens per SM, and at least four tokens a block beyond)
+    const size_t router_blocks = (size_t)(cap / 4 > 2 * h->n_sms ? cap / 4 : 2 * h->n_sms) + 1;
+    CU_TRY(cudaMalloc(&o.block_counts, router_blocks * kMaxExperts * 4));
     CU_TRY(cudaMalloc(&o.yacc, (size_t)launch_tokens * h->d * sizeof(long long)));
     CU_TRY(cudaMemset(o.yacc, 0, (size_t)launch_tokens * h->d * sizeof(long long)));
     CU_TRY(cudaMalloc(&o.ybuf, (size_t)cap * h->d * sizeof(float)));
@@ -843,7 +847,7 @@ int take_pair(melinoe_moe *h, TimedPair *tp)
 // One launch of the decode FFN kernel: compute group `group` (or -1: the whole call, missed experts
 // read from the host store) for tokens [8 * chunk, 8 * chunk + 8) of the call.
 int launch_decode(melinoe_moe *h, cudaStream_t s, const Scratch &sc, const void *hidden_dev, void *out_dev, int T,
-                  int group, int chunk, bool first_of_call)
+                  int group, int chunk, bool behind_planner)
 {
     const int tokens = T - chunk * kTokPerVr < kTokPerVr ? T - chunk * kTokPerVr : kTokPerVr;
     DecGeometry geo;
@@ -871,7 +875,7 @@ int launch_decode(melinoe_moe *h, cudaStream_t s, const Scratch &sc, const void 
     dp.chunk = chunk;
     dp.n_chunks = (T + kTokPerVr - 1) / kTokPerVr;
     dp.write_back = 1;
-    dp.wait_prior = first_of_call ? 0 : 1;
+    dp.wait_prior = behind_planner ? 0 : 1;     // directly behind the fused planner: its plan word says enough
     dp.fmt = h->fmt;
     CU_TRY(launch_ffn_decode(s, h->cfg, geo, dp));
     return MELINOE_OK;
@@ -924,16 +928,37 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         h->req_trace_count += 1;
     }
     const bool small = route_plan_small_supported(T, h->k, h->d);
+    // calls of more than 8 tokens go through the grouped GEMM
+    const bool use_gemm = h->gemm_ok && T > kTokPerVr && h->xs != nullptr && sc.idx == h->own.idx;
     if (small) {
         CU_TRY(launch_route_plan_small(s, static_cast<const uint16_t *>(hidden_dev), h->w_router, h->bias, h->token_seq,
                                        h->d, sc.idx, sc.gate, sc.logits, pp));
     } else {
-        CU_TRY(launch_router(s, static_cast<const uint16_t *>(hidden_dev), h->w_router, h->bias, h->token_seq, T, h->d,
-                             h->E, h->k, sc.idx, sc.gate, sc.logits));
+        const RouterShape sh = router_shape(T, h->E, h->n_sms);
+        pp.block_counts = sc.block_counts;
+        pp.n_blocks = sh.n_blocks;
+        CU_TRY(launch_router(s, sh, static_cast<const uint16_t *>(hidden_dev), h->w_router, h->bias, h->token_seq, T, h->d,
+                             h->E, h->k, sc.idx, sc.gate, sc.logits, sc.block_counts));
         CU_TRY(launch_plan(s, pp));
+        GatherParams ga;
+        ga.plan = h->plan;
+        ga.x = static_cast<const uint16_t *>(hidden_dev);
+        ga.idx = sc.idx;
+        ga.block_base = sc.block_counts;
+        ga.perm = sc.perm;
+        ga.inv_pos = sc.inv_pos;
+        ga.tok_of_sorted = sc.tok_of_sorted;
+        ga.xs = use_gemm ? h->xs : nullptr;
+        ga.T = T;
+        ga.d = h->d;
+        ga.E = h->E;
+        ga.k = h->k;
+        ga.n_shared = h->n_shared;
+        ga.tokens_per_block = sh.tokens_per_block;
+        ga.n_blocks = sh.n_blocks;
+        ga.permute = h->fmt == 1;
+        CU_TRY(launch_gather_rows(s, ga));
     }
-    // calls of more than 8 tokens go through the grouped GEMM (where the shapes allow it)
-    const bool use_gemm = h->gemm_ok && T > kTokPerVr && h->xs != nullptr && sc.idx == h->own.idx;
     const int n_chunks = (T + kTokPerVr - 1) / kTokPerVr;
     h->last_used_gemm = use_gemm && h->fmt == 0;
 
@@ -951,7 +976,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
                     return rc;
                 CU_TRY(cudaEventRecord(tp.a, s));
             }
-            int rc = launch_decode(h, s, sc, hidden_dev, out_dev, T, -1, c, c == 0);
+            int rc = launch_decode(h, s, sc, hidden_dev, out_dev, T, -1, c, small && c == 0);
             if (rc != MELINOE_OK)
                 return rc;
             if (h->timing) {
@@ -966,7 +991,6 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
 
     // ---- transfers issued by the host: group 0 is queued at once, the miss waves follow as the host
     // learns of them
-    CU_TRY(cudaEventRecord(h->ev_plan, s));
     GemmParams gp;
     gp.plan = h->plan;
     gp.maps = h->maps_dev;
@@ -981,9 +1005,6 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     gp.slot_stride = h->slot_stride;
     gp.shared_blobs = h->shared_dev;
     gp.unit_bytes = (int)(h->expert_bytes / (size_t)h->F);
-    if (use_gemm)
-        CU_TRY(launch_gather_rows(s, h->plan, static_cast<const uint16_t *>(hidden_dev), sc.tok_of_sorted, h->xs, h->d,
-                                  T * h->k + h->n_shared * T, h->fmt == 1, h->n_sms));
     auto launch_group = [&](int g) -> int {
         TimedPair tp{nullptr, nullptr};
         if (h->timing) {
@@ -1002,7 +1023,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
             CU_TRY(launch_ffn_gemm(s, 2, h->n_sms, pairs, h->fmt, gp));
         } else {
             for (int c = 0; c < n_chunks; ++c) {
-                int rc = launch_decode(h, s, sc, hidden_dev, out_dev, T, g, c, g == 0 && c == 0);
+                int rc = launch_decode(h, s, sc, hidden_dev, out_dev, T, g, c, small && g == 0 && c == 0);
                 if (rc != MELINOE_OK)
                     return rc;
             }
@@ -1026,6 +1047,9 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     if (rc != MELINOE_OK)
         return fail(rc);
 
+    // (behind group 0: an event between two kernels would keep them from overlapping)
+    if (cudaEventRecord(h->ev_plan, s) != cudaSuccess)
+        return fail(cuda_fail(cudaGetLastError()));
     // the miss queue of this call
     rc = wait_for_plan(h, h->call_seq);
     if (rc != MELINOE_OK)
@@ -1132,7 +1156,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
 
     if (use_gemm)
         CU_TRY(launch_combine_rows(s, h->plan, sc.gate, sc.inv_pos, h->zbuf, static_cast<uint16_t *>(out_dev), T, h->d,
-                                   h->k, h->n_shared, h->n_sms));
+                                   h->k, h->n_shared));
     CU_TRY(cudaEventRecord(h->ev_last, s));
     h->has_last = true;
     return MELINOE_OK;

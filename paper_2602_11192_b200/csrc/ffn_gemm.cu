@@ -358,6 +358,9 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
             }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // (what the kernels ahead wrote is read from here on)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (plan->status != MELINOE_OK)
         return;
     // ---- the launch's requests and their items, by warp 0, a lane per request
@@ -719,60 +722,144 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         atomicExch(p.err, MELINOE_ERR_TIMEOUT);
 }
 
-// Xs[pos] = hidden[tok_of_sorted[pos]], one block per sorted row.  PERMUTE: elements (0,4) (1,5) (2,6) (3,7) of every
-// eight, the order in which 4-bit codes expand.
+// Token lists and Xs[pos] = hidden[token of pos].  A block takes the tokens that one block of the router took: a pair's
+// position is its expert's offset, plus the pairs of that expert in the blocks before (both from the planning kernel),
+// plus those before it in this block.  A token's row is read once and written k times (and once per shared
+// expert).  PERMUTE: elements (0,4) (1,5) (2,6) (3,7) of every eight, the order in which 4-bit codes expand.
+constexpr int kGatherMaxPairs = 512;       // pairs of one router block at most (see router_shape)
+
 template <bool PERMUTE>
-__global__ void __launch_bounds__(256) gather_rows_kernel(const DevPlan *plan, const uint16_t *__restrict__ x,
-                                                          const int32_t *__restrict__ tok_of_sorted, uint16_t *xs, int d,
-                                                          int n_sorted)
+__global__ void __launch_bounds__(256) gather_rows_kernel(GatherParams p)
 {
-    if (plan->status != MELINOE_OK)
+    __shared__ int32_t s_run[kMaxExperts];
+    __shared__ int32_t s_pos[kGatherMaxPairs];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int t0 = blockIdx.x * p.tokens_per_block, n = min(p.tokens_per_block, p.T - t0);
+    const int k = p.k, n_pairs = p.T * k;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (p.plan->status != MELINOE_OK)
         return;
-    for (int pos = blockIdx.x; pos < n_sorted; pos += gridDim.x) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(x + (size_t)tok_of_sorted[pos] * d);
-        uint4 *dst = reinterpret_cast<uint4 *>(xs + (size_t)pos * d);
-        for (int i = threadIdx.x; i < d / 8; i += 256) {
-            uint4 v = src[i];
-            if (PERMUTE)
-                v = make_uint4(__byte_perm(v.x, v.z, 0x5410), __byte_perm(v.x, v.z, 0x7632), __byte_perm(v.y, v.w, 0x5410),
-                               __byte_perm(v.y, v.w, 0x7632));
-            dst[i] = v;
+    if (tid < 32) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int e = lane + 32 * h;
+            s_run[e] = e < p.E ? p.plan->offsets[e] + p.block_base[(size_t)blockIdx.x * kMaxExperts + e] : 0;
         }
+        __syncwarp();
+        for (int i0 = 0; i0 < n * k; i0 += 32) {
+            const int i = i0 + lane, q = t0 * k + i;
+            const int e = i < n * k ? p.idx[q] : -1 - lane;
+            const unsigned same = __match_any_sync(0xffffffffu, e);
+            const int r = __popc(same & ((1u << lane) - 1u));
+            int pos = 0;
+            if (e >= 0) {
+                pos = s_run[e] + r;
+                s_pos[i] = pos;
+                p.perm[pos] = q;
+                p.inv_pos[q] = pos;
+                p.tok_of_sorted[pos] = t0 + i / k;
+            }
+            __syncwarp();
+            if (e >= 0 && r == 0)
+                s_run[e] = pos + __popc(same);
+            __syncwarp();
+        }
+    }
+    for (int i = tid; i < n * p.n_shared; i += 256)
+        p.tok_of_sorted[n_pairs + i / n * p.T + t0 + i % n] = t0 + i % n;
+    if (p.xs == nullptr)
+        return;
+    __syncthreads();
+    const int row16 = p.d / 8;                  // 16-byte pieces of a row
+#pragma unroll 2
+    for (int i = tid; i < n * row16; i += 256) {
+        const int t = i / row16, c = i % row16;
+        uint4 v = __ldg(reinterpret_cast<const uint4 *>(p.x + (size_t)(t0 + t) * p.d) + c);
+        if (PERMUTE)
+            v = make_uint4(__byte_perm(v.x, v.z, 0x5410), __byte_perm(v.x, v.z, 0x7632), __byte_perm(v.y, v.w, 0x5410),
+                           __byte_perm(v.y, v.w, 0x7632));
+        uint4 *dst = reinterpret_cast<uint4 *>(p.xs) + c;
+        for (int j = 0; j < k; ++j)
+            dst[(size_t)s_pos[t * k + j] * row16] = v;
+        for (int j = 0; j < p.n_shared; ++j)
+            dst[((size_t)n_pairs + (size_t)j * p.T + t0 + t) * row16] = v;
     }
 }
 
-// y_t = sum_j gate[t][j] * Z[inv_pos[t*k+j]] + sum_s Z[T*k + s*T + t], fp32 in rank order, bf16 out.
+// y_t = sum_j gate[t][j] * Z[inv_pos[t*k+j]] + sum_s Z[T*k + s*T + t], fp32 in rank order, bf16 out.  A block per token
+// (and per quarter of a wide row); the rows of eight experts are in flight at a time.
 __global__ void __launch_bounds__(256) combine_rows_kernel(const DevPlan *plan, const float *__restrict__ gate,
                                                            const int32_t *__restrict__ inv_pos, const float *__restrict__ zs,
                                                            uint16_t *out, int T, int d, int k, int n_shared)
 {
+    __shared__ float s_gate[32 + kMaxShared];
+    __shared__ int32_t s_pos[32 + kMaxShared];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool ok = plan->status == MELINOE_OK;
-    for (int t = blockIdx.x; t < T; t += gridDim.x) {
-        for (int c = threadIdx.x * 4; c < d; c += 256 * 4) {
-            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (ok) {
-                for (int j = 0; j < k; ++j) {
-                    const float gw = gate[t * k + j];
-                    const float4 z = *reinterpret_cast<const float4 *>(zs + (size_t)inv_pos[t * k + j] * d + c);
-                    y.x = fmaf(gw, z.x, y.x);
-                    y.y = fmaf(gw, z.y, y.y);
-                    y.z = fmaf(gw, z.z, y.z);
-                    y.w = fmaf(gw, z.w, y.w);
+    const int t = blockIdx.x, n = k + n_shared;
+    if (threadIdx.x < n) {
+        const int j = threadIdx.x;
+        s_gate[j] = j < k ? gate[t * k + j] : 1.0f;      // (1 * z is z: shared experts are added as they are)
+        s_pos[j] = j < k ? inv_pos[t * k + j] : T * k + (j - k) * T + t;
+    }
+    __syncthreads();
+    const int c = (blockIdx.y * 256 + threadIdx.x) * 4;
+    if (c >= d)
+        return;
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (ok) {
+        for (int j0 = 0; j0 < n; j0 += 8) {
+            float4 z[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (j0 + j < n)
+                    z[j] = __ldcs(reinterpret_cast<const float4 *>(zs + (size_t)s_pos[j0 + j] * d + c));
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (j0 + j < n) {
+                    const float gw = s_gate[j0 + j];
+                    y.x = fmaf(gw, z[j].x, y.x);
+                    y.y = fmaf(gw, z[j].y, y.y);
+                    y.z = fmaf(gw, z[j].z, y.z);
+                    y.w = fmaf(gw, z[j].w, y.w);
                 }
-                for (int s = 0; s < n_shared; ++s) {
-                    const float4 z = *reinterpret_cast<const float4 *>(zs + ((size_t)T * k + (size_t)s * T + t) * d + c);
-                    y.x += z.x;
-                    y.y += z.y;
-                    y.z += z.z;
-                    y.w += z.w;
-                }
-            }
-            uint2 o;
-            o.x = bf16_rne(y.x) | (bf16_rne(y.y) << 16);
-            o.y = bf16_rne(y.z) | (bf16_rne(y.w) << 16);
-            *reinterpret_cast<uint2 *>(out + (size_t)t * d + c) = o;
         }
     }
+    uint2 o;
+    o.x = bf16_rne(y.x) | (bf16_rne(y.y) << 16);
+    o.y = bf16_rne(y.z) | (bf16_rne(y.w) << 16);
+    *reinterpret_cast<uint2 *>(out + (size_t)t * d + c) = o;
+}
+
+// Launch with programmatic stream serialisation (the kernel waits for the one ahead itself) and, for CG = 2, clusters of
+// two CTAs on neighbouring SMs.
+template <typename... Params, typename... Args>
+cudaError_t launch_after(cudaStream_t stream, void (*kernel)(Params...), dim3 grid, int threads, size_t smem, int cluster, Args... args)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = grid;
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (pdl_enabled()) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    lc.attrs = attr;
+    lc.numAttrs = n;
+    const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, args...);
+    count_launch();
+    return e;
 }
 
 constexpr size_t gemm_smem(int cg, int fmt)
@@ -783,22 +870,7 @@ constexpr size_t gemm_smem(int cg, int fmt)
 template <int PHASE, int CG, int FMT>
 cudaError_t gemm_launch(cudaStream_t stream, int n_sms, const GemmParams &p)
 {
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(n_sms / CG * CG);
-    lc.blockDim = dim3(gemm_threads(FMT));
-    lc.dynamicSmemBytes = gemm_smem(CG, FMT);
-    lc.stream = stream;
-    cudaLaunchAttribute attr[1];
-    if (CG == 2) {
-        // clusters of two CTAs on neighbouring SMs
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        lc.attrs = attr;
-        lc.numAttrs = 1;
-    }
-    return cudaLaunchKernelEx(&lc, ffn_gemm_kernel<PHASE, CG, FMT>, p);
+    return launch_after(stream, ffn_gemm_kernel<PHASE, CG, FMT>, dim3(n_sms / CG * CG), gemm_threads(FMT), gemm_smem(CG, FMT), CG, p);
 }
 
 template <int PHASE, int CG, int FMT>
@@ -821,38 +893,26 @@ cudaError_t ffn_gemm_configure()
     return cudaSuccess;
 }
 
-cudaError_t launch_gather_rows(cudaStream_t stream, const DevPlan *plan, const uint16_t *x, const int32_t *tok_of_sorted,
-                               uint16_t *xs, int d, int n_sorted, bool permute, int n_sms)
+cudaError_t launch_gather_rows(cudaStream_t stream, const GatherParams &p)
 {
-    const int grid = n_sorted < n_sms * 16 ? n_sorted : n_sms * 16;
-    if (permute)
-        gather_rows_kernel<true><<<grid, 256, 0, stream>>>(plan, x, tok_of_sorted, xs, d, n_sorted);
-    else
-        gather_rows_kernel<false><<<grid, 256, 0, stream>>>(plan, x, tok_of_sorted, xs, d, n_sorted);
-    count_launch();
-    return cudaGetLastError();
+    if (p.tokens_per_block * p.k > kGatherMaxPairs)
+        return cudaErrorInvalidValue;
+    return launch_after(stream, p.permute ? gather_rows_kernel<true> : gather_rows_kernel<false>, dim3(p.n_blocks), 256, 0, 1, p);
 }
 
 cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, int fmt, const GemmParams &p)
 {
-    cudaError_t e;
     if (fmt == 1)
-        e = phase == 1 ? gemm_launch<1, 1, 1>(stream, n_sms, p) : gemm_launch<2, 1, 1>(stream, n_sms, p);
-    else if (pairs)
-        e = phase == 1 ? gemm_launch<1, 2, 0>(stream, n_sms, p) : gemm_launch<2, 2, 0>(stream, n_sms, p);
-    else
-        e = phase == 1 ? gemm_launch<1, 1, 0>(stream, n_sms, p) : gemm_launch<2, 1, 0>(stream, n_sms, p);
-    count_launch();
-    return e;
+        return phase == 1 ? gemm_launch<1, 1, 1>(stream, n_sms, p) : gemm_launch<2, 1, 1>(stream, n_sms, p);
+    if (pairs)
+        return phase == 1 ? gemm_launch<1, 2, 0>(stream, n_sms, p) : gemm_launch<2, 2, 0>(stream, n_sms, p);
+    return phase == 1 ? gemm_launch<1, 1, 0>(stream, n_sms, p) : gemm_launch<2, 1, 0>(stream, n_sms, p);
 }
 
 cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const float *gate, const int32_t *inv_pos,
-                                const float *zs, uint16_t *out, int T, int d, int k, int n_shared, int n_sms)
+                                const float *zs, uint16_t *out, int T, int d, int k, int n_shared)
 {
-    const int grid = T < n_sms * 8 ? T : n_sms * 8;
-    combine_rows_kernel<<<grid, 256, 0, stream>>>(plan, gate, inv_pos, zs, out, T, d, k, n_shared);
-    count_launch();
-    return cudaGetLastError();
+    return launch_after(stream, combine_rows_kernel, dim3(T, (d + 1023) / 1024), 256, 0, 1, plan, gate, inv_pos, zs, out, T, d, k, n_shared);
 }
 
 }  // namespace melinoe

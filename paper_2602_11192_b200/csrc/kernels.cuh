@@ -13,10 +13,16 @@ void count_launch();
 // Programmatic stream serialisation for the decode kernels (on unless MELINOE_MOE_NO_PDL is set in the environment).
 bool pdl_enabled();
 
-// ---- router (Eq. 1): logits, top-k, gates
-cudaError_t launch_router(cudaStream_t stream, const uint16_t *x, const uint16_t *w_r,
+// ---- router (Eq. 1): logits, top-k, gates, and per block how many of its tokens chose each expert
+struct RouterShape {
+    int tokens_per_warp, n_eg;       // tokens and expert groups of a warp's tile
+    int tokens_per_block, n_blocks;
+};
+RouterShape router_shape(int T, int E, int n_sms);
+// block_counts [n_blocks][kMaxExperts]
+cudaError_t launch_router(cudaStream_t stream, const RouterShape &shape, const uint16_t *x, const uint16_t *w_r,
                           const float *bias, const int32_t *token_seq, int T, int d, int E, int k,
-                          int32_t *idx, float *gate, float *logits_out);
+                          int32_t *idx, float *gate, float *logits_out, int32_t *block_counts);
 
 // ---- planning: gather lists, LRU slot lookup, miss queue, statistics
 struct PlanParams {
@@ -41,6 +47,9 @@ struct PlanParams {
     char *trace_rec;
     int trace_max_tokens;
     const float *gate;        // [T][k], for the trace record of calls planned by the general kernel
+    // general kernel: the router's counts per block; become the pairs of each expert in the blocks before
+    int32_t *block_counts;
+    int n_blocks;
 };
 // Layout of one request-trace record for a layer of n_experts experts and top_k, max_tokens tokens.
 struct TraceLayout {
@@ -132,13 +141,23 @@ struct GemmParams {
 };
 bool ffn_gemm_supported(int d, int F);
 cudaError_t ffn_gemm_configure();
-// permute: store elements j and j + 4 of every eight side by side (the order in which 4-bit codes expand)
-cudaError_t launch_gather_rows(cudaStream_t stream, const DevPlan *plan, const uint16_t *x, const int32_t *tok_of_sorted,
-                               uint16_t *xs, int d, int n_sorted, bool permute, int n_sms);
+// Token lists (perm, inv_pos, tok_of_sorted) of a call planned by the general kernel and, unless xs is null, the
+// gathered activations, in the blocks the router worked in.
+struct GatherParams {
+    const DevPlan *plan;
+    const uint16_t *x;               // hidden [T][d]
+    const int32_t *idx;              // [T][k]
+    const int32_t *block_base;       // PlanParams::block_counts after the planning kernel
+    int32_t *perm, *inv_pos, *tok_of_sorted;
+    uint16_t *xs;
+    int T, d, E, k, n_shared, tokens_per_block, n_blocks;
+    int permute;                     // store elements j and j + 4 of every eight side by side (the order in which 4-bit codes expand)
+};
+cudaError_t launch_gather_rows(cudaStream_t stream, const GatherParams &p);
 // pairs: CTA pairs (bf16 slots only); fmt: what the slots hold, 0 = bf16 blobs, 1 = 4-bit blobs
 cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, int fmt, const GemmParams &p);
 cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const float *gate, const int32_t *inv_pos,
-                                const float *zs, uint16_t *out, int T, int d, int k, int n_shared, int n_sms);
+                                const float *zs, uint16_t *out, int T, int d, int k, int n_shared);
 
 // ---- preload (Eq. 5): cache requests of a list of experts, and the copy of the missing ones into their slots
 struct PreloadParams {

@@ -102,23 +102,11 @@ struct PreloadList {
     int32_t slot[kMaxExperts];
 };
 
-// Device side: publish the miss queue of call `seq` (one 16-byte store per record).
+// Device side: one record of the miss queue (one 16-byte store).
 __device__ inline void store16_host(void *dst, const void *rec)
 {
     const int4 v = *reinterpret_cast<const int4 *>(rec);
     asm volatile("st.volatile.global.v4.s32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                  : "memory");
 }
-__device__ inline void publish_miss_queue(HostPlan *hp, const HostMiss *miss, int n_miss, int n_groups, int status,
-                                          uint32_t seq)
-{
-    for (int i = 0; i < n_miss; ++i) {
-        HostMiss m = miss[i];
-        m.seq = seq;
-        store16_host(&hp->miss[i], &m);
-    }
-    HostPlanHeader h{n_miss, n_groups, status, seq};
-    store16_host(&hp->hdr, &h);
-}
-
 }  // namespace melinoe

@@ -1,7 +1,11 @@
 // Planning kernel: token-to-expert gather, slot lookup with LRU eviction, miss queue.
 //
-// One block per call.  It turns the router's indices into
-//   (a) per-expert token lists (stable counting sort of the (token, rank) pairs),
+// One block per call, behind the router.  What bounds it is the latency of a few dependent steps, so the steps are
+// few and each is done by many threads; whatever needs the pairs themselves is left to the kernels around it: the
+// router counts per block how often each expert was chosen, and the gather kernel places the pairs.  (One block
+// counting and sorting the pairs itself took 100 us for 49152 of them.)  It makes
+//   (a) from the router's counts, the experts' offsets in the sorted order of the (token, rank) pairs and the pairs
+//       of each expert in the blocks before each block: where the gather kernel puts a block's pairs,
 //   (b) the call's cache requests: one per distinct expert, experts resident at call entry
 //       first (ascending id), then the missing ones (ascending id); a miss takes the lowest
 //       empty slot, else the least recently stamped slot (Section 3.2: experts are fetched on
@@ -18,20 +22,21 @@ namespace melinoe {
 namespace {
 
 constexpr int kPlanThreads = 1024;
-constexpr int kPlanWarps = kPlanThreads / 32;
+constexpr int kPlanSegs = kPlanThreads / kMaxExperts;    // parts in which the router's blocks are summed
+constexpr int kPlanKeep = 8;                             // counts a thread keeps between the two passes
 
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
 {
     __shared__ int32_t s_counts[kMaxReq];
     __shared__ int32_t s_offsets[kMaxReq + 1];
-    __shared__ int32_t s_running[kMaxExperts];
-    __shared__ int32_t s_warp_cnt[kPlanWarps][kMaxExperts];
+    __shared__ int32_t s_seg[kPlanSegs][kMaxExperts];
     __shared__ DevCache s_cache;
     __shared__ int32_t s_group_of_expert[kMaxExperts];
     __shared__ int32_t s_req_of_expert[kMaxReq];
     __shared__ ReqRec s_req[kMaxReq];
     __shared__ HostMiss s_miss[kMaxExperts];
     __shared__ int32_t s_group_vr_begin[kMaxGroups + 1];
+    __shared__ int32_t s_grp_first[kMaxGroups + 1];              // count policy: first miss of a wave
     __shared__ unsigned long long s_key[kMaxExperts];            // victim-order key of a slot
     __shared__ int32_t s_victim[kMaxExperts];                    // V: slots in victim order
     __shared__ int32_t s_miss_expert[kMaxExperts];               // expert of miss number i
@@ -43,12 +48,13 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
     const int n_pairs = p.T * p.k;
     const int E = p.E, C = p.C;
 
-    // ---- load persistent cache state, clear tables
+    // ---- load persistent cache state, clear tables.  The router, which may still be running (programmatic launch), lets
+    // this kernel start only once everything ahead of it, the previous call's planning included, is complete.
     {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(p.cache);
         uint32_t *dst = reinterpret_cast<uint32_t *>(&s_cache);
         for (int i = tid; i < (int)(sizeof(DevCache) / 4); i += kPlanThreads)
-            dst[i] = src[i];
+            dst[i] = __ldcg(src + i);
     }
     for (int i = tid; i < kMaxReq; i += kPlanThreads) {
         s_counts[i] = 0;
@@ -56,73 +62,81 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
     }
     if (tid < 8)
         s_misc[tid] = 0;
-    __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    // ---- (a) histogram
-    for (int q = tid; q < n_pairs; q += kPlanThreads) {
-        const int e = p.idx[q];
-        if (e >= 0 && e < E)
-            atomicAdd(&s_counts[e], 1);
-        else
-            s_misc[6] = MELINOE_ERR_INVALID;
+    // ---- (a) the pairs of each expert: every thread sums one expert over a run of blocks, then the runs are put in order
+    {
+        const int e = tid & (kMaxExperts - 1), seg = tid / kMaxExperts;
+        const int per = (p.n_blocks + kPlanSegs - 1) / kPlanSegs;
+        const int b_lo = min(seg * per, p.n_blocks), n = min(b_lo + per, p.n_blocks) - b_lo;
+        int32_t *col = p.block_counts + (size_t)b_lo * kMaxExperts + e;
+        int keep[kPlanKeep], sum = 0;
+#pragma unroll
+        for (int i = 0; i < kPlanKeep; ++i)
+            keep[i] = i < n ? __ldcg(col + (size_t)i * kMaxExperts) : 0;
+#pragma unroll
+        for (int i = 0; i < kPlanKeep; ++i)
+            sum += keep[i];
+#pragma unroll 8
+        for (int i = kPlanKeep; i < n; ++i)
+            sum += __ldcg(col + (size_t)i * kMaxExperts);
+        s_seg[seg][e] = sum;
+        __syncthreads();
+        int run = 0, total = 0;
+#pragma unroll
+        for (int i = 0; i < kPlanSegs; ++i) {
+            const int v = s_seg[i][e];
+            run += i < seg ? v : 0;
+            total += v;
+        }
+        if (seg == 0 && e < E)
+            s_counts[e] = total;
+#pragma unroll
+        for (int i = 0; i < kPlanKeep; ++i) {
+            if (i < n)
+                col[(size_t)i * kMaxExperts] = run;
+            run += keep[i];
+        }
+        for (int i0 = kPlanKeep; i0 < n; i0 += kPlanKeep) {
+#pragma unroll
+            for (int i = 0; i < kPlanKeep; ++i)
+                keep[i] = i0 + i < n ? col[(size_t)(i0 + i) * kMaxExperts] : 0;
+#pragma unroll
+            for (int i = 0; i < kPlanKeep; ++i) {
+                if (i0 + i < n)
+                    col[(size_t)(i0 + i) * kMaxExperts] = run;
+                run += keep[i];
+            }
+        }
     }
     __syncthreads();
     // count policy (Definition C.1): one time step per call, count <- gamma * count + request
     if (p.policy == MELINOE_POLICY_COUNT && tid < E)
         s_cache.count[tid] = __fadd_rn(__fmul_rn(p.gamma, s_cache.count[tid]), s_counts[tid] > 0 ? 1.0f : 0.0f);
-    if (tid == 0) {
-        int run = 0;
-        for (int e = 0; e < E; ++e) {
-            s_offsets[e] = run;
-            s_running[e] = run;
-            run += s_counts[e];
+    if (warp == 0) {
+        // offsets: a scan over the experts, then the shared experts' blocks of T
+        const int c0 = lane < E ? s_counts[lane] : 0, c1 = lane + 32 < E ? s_counts[lane + 32] : 0;
+        int i0 = c0, i1 = c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(0xffffffffu, i0, o), b = __shfl_up_sync(0xffffffffu, i1, o);
+            i0 += lane >= o ? a : 0;
+            i1 += lane >= o ? b : 0;
         }
-        for (int s = 0; s < p.n_shared; ++s) {
-            s_counts[E + s] = p.T;
-            s_offsets[E + s] = run;
-            run += p.T;
+        i1 += __shfl_sync(0xffffffffu, i0, 31);
+        if (lane < E)
+            s_offsets[lane] = i0 - c0;
+        if (lane + 32 < E)
+            s_offsets[lane + 32] = i1 - c1;
+        __syncwarp();
+        if (lane <= p.n_shared) {
+            s_offsets[E + lane] = n_pairs + lane * p.T;
+            if (lane < p.n_shared)
+                s_counts[E + lane] = p.T;
         }
-        s_offsets[E + p.n_shared] = run;
     }
     __syncthreads();
-
-    // ---- stable scatter, kPlanThreads pairs per pass, in pair order
-    for (int base = 0; base < n_pairs; base += kPlanThreads) {
-        for (int i = tid; i < kPlanWarps * kMaxExperts; i += kPlanThreads)
-            (&s_warp_cnt[0][0])[i] = 0;
-        __syncthreads();
-        const int q = base + tid;
-        int e = q < n_pairs ? p.idx[q] : kMaxExperts;
-        if (e < 0 || e >= E)
-            e = kMaxExperts;  // invalid or padding: takes no part
-        const unsigned same = __match_any_sync(0xffffffffu, e);
-        const int rank = __popc(same & ((1u << lane) - 1u));
-        if (e < kMaxExperts && rank == 0)
-            s_warp_cnt[warp][e] = __popc(same);
-        __syncthreads();
-        if (tid < E) {
-            int run = 0;
-            for (int w = 0; w < kPlanWarps; ++w) {
-                const int c = s_warp_cnt[w][tid];
-                s_warp_cnt[w][tid] = run;
-                run += c;
-            }
-            s_group_of_expert[tid] = run;  // scratch: this pass's total for expert tid
-        }
-        __syncthreads();
-        if (e < kMaxExperts) {
-            const int pos = s_running[e] + s_warp_cnt[warp][e] + rank;
-            p.perm[pos] = q;
-            p.inv_pos[q] = pos;
-            p.tok_of_sorted[pos] = q / p.k;
-        }
-        __syncthreads();
-        if (tid < E)
-            s_running[tid] += s_group_of_expert[tid];
-        __syncthreads();
-    }
-    for (int i = tid; i < p.n_shared * p.T; i += kPlanThreads)
-        p.tok_of_sorted[n_pairs + i] = i % p.T;
 
     // ---- (b), (c): cache requests, by warp 0; lane owns experts lane and lane + 32 and slots lane and
     // lane + 32.  The sequential rules (hits in ascending id, then misses in ascending id, a miss
@@ -194,6 +208,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
             // earlier misses of the call brought in): one search per miss, in ascending expert id.
             // Victim: lowest empty slot, else the smallest (count of the occupant, stamp).
             int cur_group = 1, i = 0;
+            if (lane == 0)
+                s_grp_first[1] = 0;
             for (uint64_t m = miss_mask; m; m &= m - 1, ++i) {
                 const int e = __ffsll((long long)m) - 1;
                 uint64_t khi = ~0ull, klo = ~0ull;
@@ -230,8 +246,11 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
                     if ((need >> ev) & 1ull)
                         dep = s_group_of_expert[ev];
                 }
-                if (dep == cur_group)
+                if (dep == cur_group) {
                     ++cur_group;      // it would overwrite an expert of the current wave: next wave
+                    if (lane == 0)
+                        s_grp_first[cur_group] = i;
+                }
                 __syncwarp();
                 if (lane == 0) {
                     if (ev >= 0)
@@ -292,38 +311,30 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
         const int n_evict = p.policy == MELINOE_POLICY_COUNT ? n_evict_seq : __popcll(ballot64(ev_flag[0], ev_flag[1]));
         counter += (uint64_t)n_req;
         __syncwarp();
+        // shared experts: always resident, group 0.  Records for the compute kernels, grouped: the hits, the shared
+        // experts, then the misses wave by wave.
+        const int n_req_total = n_req + p.n_shared, ndr = n_req_total;
+        if (lane < p.n_shared) {
+            s_req[n_req + lane] = ReqRec{E + lane, -1, 1, -1, 0, 0, s_offsets[E + lane], p.T};
+            s_req_of_expert[E + lane] = n_req + lane;
+        }
+        __syncwarp();
+        for (int r = lane; r < n_req_total; r += 32)
+            s_req[r].vr_start = r < n_hits ? r : r < n_req ? r + p.n_shared : r - n_miss;
+        int status = s_misc[6];
+        if (n_groups > (int)p.gmax)
+            status = MELINOE_ERR_STATE;
+        const bool ok = status == MELINOE_OK;      // otherwise nothing is left for the compute kernels to do
+        for (int g = lane; g <= kMaxGroups; g += 32) {
+            int b = 0;
+            if (ok && g >= 1) {
+                // misses served before wave g: (g - 1) * C under LRU, the wave's recorded first miss otherwise
+                const int done = p.policy == MELINOE_POLICY_COUNT ? (g < n_groups ? s_grp_first[g] : n_miss) : (g - 1) * C;
+                b = n_hits + p.n_shared + (done < n_miss ? done : n_miss);
+            }
+            s_group_vr_begin[g] = b;
+        }
         if (lane == 0) {
-            int n_req_total = n_req;
-            for (int s = 0; s < p.n_shared; ++s) {
-                s_req[n_req_total] = ReqRec{E + s, -1, 1, -1, 0, 0, s_offsets[E + s], p.T};
-                s_req_of_expert[E + s] = n_req_total;
-                ++n_req_total;
-            }
-            // records for the compute kernels, grouped: group 0 = hits then shared experts, then the
-            // miss waves in order
-            int ndr = 0;
-            s_group_vr_begin[0] = 0;
-            for (int r = 0; r < n_hits; ++r)
-                s_req[r].vr_start = ndr++;
-            for (int r = n_req; r < n_req_total; ++r)
-                s_req[r].vr_start = ndr++;
-            int g = 0;
-            for (int r = n_hits; r < n_req; ++r) {
-                while (g < s_req[r].group)
-                    s_group_vr_begin[++g] = ndr;
-                s_req[r].vr_start = ndr++;
-            }
-            while (g < kMaxGroups)
-                s_group_vr_begin[++g] = ndr;
-            int status = s_misc[6];
-            if (n_groups > (int)p.gmax)
-                status = MELINOE_ERR_STATE;
-            if (status != MELINOE_OK) {
-                // leave nothing for the compute kernels to do
-                for (int i = 0; i <= kMaxGroups; ++i)
-                    s_group_vr_begin[i] = 0;
-                ndr = 0;
-            }
             s_cache.counter = counter;
             s_cache.tot_hits += (uint64_t)n_hits;
             s_cache.tot_misses += (uint64_t)n_miss;
@@ -334,14 +345,39 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
             s_misc[2] = n_miss;
             s_misc[3] = n_evict;
             s_misc[4] = n_groups;
-            s_misc[5] = ndr;
+            s_misc[5] = ok ? ndr : 0;
             s_misc[6] = status;
             s_misc[7] = n_req_total;
         }
     }
     __syncthreads();
 
-    // ---- write the plan, the virtual requests and the cache state back
+    // ---- (d) miss queue for the host, (e) statistics
+    if (tid < s_misc[2]) {
+        s_miss[tid].seq = p.call_seq;
+        store16_host(&p.hplan->miss[tid], &s_miss[tid]);
+    }
+    if (tid == kPlanThreads - 32) {
+        const int n_miss = s_misc[2];
+        const HostPlanHeader hdr{n_miss, s_misc[4], s_misc[6], p.call_seq};
+        store16_host(&p.hplan->hdr, &hdr);
+        if (p.stats) {
+            melinoe_moe_stats st;
+            st.status = s_misc[6];
+            st.n_tokens = p.T;
+            st.n_distinct = s_misc[0];
+            st.hits = s_misc[1];
+            st.misses = n_miss;
+            st.evictions = s_misc[3];
+            st.groups = s_misc[4];
+            st.reserved = 0;
+            st.bytes_h2d = (uint64_t)n_miss * (uint64_t)p.expert_bytes;
+            st.call_no = s_cache.call_no;
+            *p.stats = st;
+        }
+    }
+
+    // ---- write the plan, the records for the compute kernels and the cache state back
     const int n_req_total = s_misc[7];
     const bool ok = s_misc[6] == MELINOE_OK;
     DevPlan *plan = p.plan;
@@ -390,25 +426,6 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
             dst[i] = src[i];
     }
 
-    // ---- (d) miss queue for the host service, (e) statistics
-    if (tid == 0) {
-        const int n_miss = s_misc[2];
-        if (p.stats) {
-            melinoe_moe_stats st;
-            st.status = s_misc[6];
-            st.n_tokens = p.T;
-            st.n_distinct = s_misc[0];
-            st.hits = s_misc[1];
-            st.misses = n_miss;
-            st.evictions = s_misc[3];
-            st.groups = s_misc[4];
-            st.reserved = 0;
-            st.bytes_h2d = (uint64_t)n_miss * (uint64_t)p.expert_bytes;
-            st.call_no = s_cache.call_no;
-            *p.stats = st;
-        }
-        publish_miss_queue(p.hplan, s_miss, n_miss, s_misc[4], s_misc[6], p.call_seq);
-    }
     // the call's request-trace record, if one is being kept
     if (p.trace_rec) {
         const TraceLayout tl = trace_layout(E, p.k, p.trace_max_tokens);
@@ -445,9 +462,18 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
 
 cudaError_t launch_plan(cudaStream_t stream, const PlanParams &p)
 {
-    plan_kernel<<<1, kPlanThreads, 0, stream>>>(p);
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(1);
+    lc.blockDim = dim3(kPlanThreads);
+    lc.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = pdl_enabled() ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&lc, plan_kernel, p);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace melinoe

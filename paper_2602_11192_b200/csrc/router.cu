@@ -1,4 +1,6 @@
-// Router: logits, top-k with lowest-index tie-breaking, renormalised gates (Eq. 1).
+// Router: logits, top-k with lowest-index tie-breaking, renormalised gates (Eq. 1), for calls that the fused decode
+// planner does not take; and how often each block's tokens chose each expert, from which the planning kernel makes
+// the token lists.
 //
 // The selected indices are an integer result that must agree bit for bit with a CPU
 // evaluation, so the fp32 logit is summed in one fixed order: element j belongs to lane
@@ -6,6 +8,13 @@
 // (products of two bf16 values are exact in fp32, so fused or unfused multiply-add give the
 // same bits); the 32 lane sums are folded by xor-butterflies with strides 16, 8, 4, 2, 1; the
 // bias is added last.  That is exactly one 16-byte load per lane per 256 columns.
+//
+// A warp holds TT tokens x EE experts in registers; a block is n_eg expert groups x TG token groups of warps, so
+// every block reads the whole router matrix once.  What bounds it: for a few hundred tokens the latency of those
+// reads (TT = 1 or 2, EE = 4: many warps, CH pieces of 256 columns in flight), for thousands the issue slots: 4 x 8
+// gives 256 multiply-adds per 12 loads and 128 conversions, and fma.rn.f32x2 (two experts at a time, each rounded
+// on its own: the same bits) halves what the multiply-adds take of the issue slots.  The butterfly folds
+// TT * EE values at once by exchanging halves: 31 shuffles for 32 values instead of 160.
 #include "kernels.cuh"
 
 namespace melinoe {
@@ -15,118 +24,179 @@ namespace {
 __device__ __forceinline__ float bf16lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
 
-constexpr int kRouterWarps = 8;
-constexpr int kMaxExpertsPerWarp = kMaxExperts / kRouterWarps;  // 8
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void fma2(uint64_t &acc, uint64_t a, uint64_t b)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
 
-// One block handles TT consecutive tokens.  Warp w computes experts w, w+8, ...
-template <int TT>
-__global__ void __launch_bounds__(kRouterWarps * 32)
+// TT tokens x EE experts per warp, CH pieces of 256 columns loaded ahead of their arithmetic.
+template <int TT, int EE, int CH>
+__global__ void __launch_bounds__(512)
 router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ w_r,
                    const float *__restrict__ bias, const int32_t *__restrict__ token_seq,
-                   int T, int d, int E, int k, int32_t *__restrict__ idx,
-                   float *__restrict__ gate, float *__restrict__ logits_out)
+                   int T, int d, int E, int k, int n_eg, int tokens_per_block, int32_t *__restrict__ idx,
+                   float *__restrict__ gate, float *__restrict__ logits_out, int32_t *__restrict__ block_counts)
 {
-    __shared__ __align__(16) float s_logit[TT][kMaxExperts];
-    __shared__ float s_sel[TT][32];
-    __shared__ int32_t s_sel_idx[TT][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t0 = blockIdx.x * TT;
-
-    float acc[kMaxExpertsPerWarp][TT];
-#pragma unroll
-    for (int i = 0; i < kMaxExpertsPerWarp; ++i)
-#pragma unroll
-        for (int t = 0; t < TT; ++t)
-            acc[i][t] = 0.0f;
+    extern __shared__ __align__(16) float s_logit[];        // [tokens_per_block][kMaxExperts]
+    __shared__ int32_t s_count[kMaxExperts];
+    __shared__ float s_sel[16][32];
+    __shared__ int32_t s_sel_idx[16][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
+    const int b0 = blockIdx.x * tokens_per_block;            // the block's first token
+    const int n_tok = min(tokens_per_block, T - b0);
+    const int e0 = warp % n_eg * EE, tl = warp / n_eg * TT;  // this warp's first expert, first token within the block
+    for (int i = threadIdx.x; i < kMaxExperts; i += blockDim.x)
+        s_count[i] = 0;
 
     const int n_chunks = d >> 8;
-#pragma unroll 2
-    for (int c = 0; c < n_chunks; ++c) {
-        const int col = (c << 8) + (lane << 3);
-        // all of this step's loads go out before any arithmetic
-        uint4 xv[TT], wvs[kMaxExpertsPerWarp];
+    const uint4 *xrow[TT], *wrow[EE];
 #pragma unroll
-        for (int t = 0; t < TT; ++t) {
-            const int tt = min(t0 + t, T - 1);
-            xv[t] = *reinterpret_cast<const uint4 *>(x + (size_t)tt * d + col);
-        }
+    for (int t = 0; t < TT; ++t)
+        xrow[t] = reinterpret_cast<const uint4 *>(x + (size_t)min(b0 + tl + t, T - 1) * d) + lane;
 #pragma unroll
-        for (int i = 0; i < kMaxExpertsPerWarp; ++i) {
-            const int e = warp + i * kRouterWarps;
-            wvs[i] = e < E ? __ldg(reinterpret_cast<const uint4 *>(w_r + (size_t)e * d + col)) : make_uint4(0, 0, 0, 0);
-        }
+    for (int e = 0; e < EE; ++e)
+        wrow[e] = reinterpret_cast<const uint4 *>(w_r + (size_t)min(e0 + e, E - 1) * d) + lane;
+    uint64_t acc[TT][EE / 2];
 #pragma unroll
-        for (int i = 0; i < kMaxExpertsPerWarp; ++i) {
-            const int e = warp + i * kRouterWarps;
-            if (e < E) {
-                const uint4 wv = wvs[i];
+    for (int t = 0; t < TT; ++t)
 #pragma unroll
-                for (int t = 0; t < TT; ++t) {
-                    float a = acc[i][t];
-                    a = __fmaf_rn(bf16lo(xv[t].x), bf16lo(wv.x), a);
-                    a = __fmaf_rn(bf16hi(xv[t].x), bf16hi(wv.x), a);
-                    a = __fmaf_rn(bf16lo(xv[t].y), bf16lo(wv.y), a);
-                    a = __fmaf_rn(bf16hi(xv[t].y), bf16hi(wv.y), a);
-                    a = __fmaf_rn(bf16lo(xv[t].z), bf16lo(wv.z), a);
-                    a = __fmaf_rn(bf16hi(xv[t].z), bf16hi(wv.z), a);
-                    a = __fmaf_rn(bf16lo(xv[t].w), bf16lo(wv.w), a);
-                    a = __fmaf_rn(bf16hi(xv[t].w), bf16hi(wv.w), a);
-                    acc[i][t] = a;
+        for (int e = 0; e < EE / 2; ++e)
+            acc[t][e] = 0ull;
+    // (the router matrix does not change while calls are queued; everything else may be the work of the kernel ahead)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // top-k below: warp w serves token w of the block first; its bias is on the way meanwhile
+    float bias0 = 0.0f, bias1 = 0.0f;
+    auto load_bias = [&](int t) {
+        const int q = token_seq ? token_seq[b0 + t] : 0;
+        bias0 = lane < E ? bias[(size_t)q * E + lane] : 0.0f;
+        bias1 = lane + 32 < E ? bias[(size_t)q * E + lane + 32] : 0.0f;
+    };
+    if (bias && warp < n_tok)
+        load_bias(warp);
+
+    if (tl < n_tok) {
+#pragma unroll 1
+        for (int c0 = 0; c0 < n_chunks; c0 += CH) {
+            uint4 xv[CH][TT], wv[CH][EE];
+#pragma unroll
+            for (int c = 0; c < CH; ++c)
+                if (c0 + c < n_chunks) {
+#pragma unroll
+                    for (int t = 0; t < TT; ++t)
+                        xv[c][t] = __ldca(xrow[t] + (c0 + c) * 32);
+#pragma unroll
+                    for (int e = 0; e < EE; ++e)
+                        wv[c][e] = __ldg(wrow[e] + (c0 + c) * 32);
                 }
+#pragma unroll
+            for (int c = 0; c < CH; ++c)
+                if (c0 + c < n_chunks) {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        auto word = [r](const uint4 &v) { return r == 0 ? v.x : r == 1 ? v.y : r == 2 ? v.z : v.w; };
+                        uint64_t wl[EE / 2], wh[EE / 2];
+#pragma unroll
+                        for (int e = 0; e < EE / 2; ++e) {
+                            const uint32_t a = word(wv[c][2 * e]), b = word(wv[c][2 * e + 1]);
+                            wl[e] = pack2(bf16lo(a), bf16lo(b));
+                            wh[e] = pack2(bf16hi(a), bf16hi(b));
+                        }
+#pragma unroll
+                        for (int t = 0; t < TT; ++t) {
+                            const uint32_t v = word(xv[c][t]);
+                            const uint64_t xl = pack2(bf16lo(v), bf16lo(v)), xh = pack2(bf16hi(v), bf16hi(v));
+#pragma unroll
+                            for (int e = 0; e < EE / 2; ++e)
+                                fma2(acc[t][e], xl, wl[e]);
+#pragma unroll
+                            for (int e = 0; e < EE / 2; ++e)
+                                fma2(acc[t][e], xh, wh[e]);
+                        }
+                    }
+                }
+        }
+        // the butterfly over the lanes: while more than one value is left, the lower lanes of a stride take the first half
+        // of them and the upper lanes the second
+        constexpr int N = TT * EE;
+        float v[N];
+#pragma unroll
+        for (int t = 0; t < TT; ++t)
+#pragma unroll
+            for (int e = 0; e < EE / 2; ++e)
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(v[t * EE + 2 * e]), "=f"(v[t * EE + 2 * e + 1]) : "l"(acc[t][e]));
+        int left = N;
+#pragma unroll
+        for (int m = 16; m >= 1; m >>= 1) {
+            if (left > 1) {
+                left >>= 1;
+                const bool up = (lane & m) != 0;
+#pragma unroll
+                for (int i = 0; i < N / 2; ++i)
+                    if (i < left) {
+                        const float o = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + left], m);
+                        v[i] = __fadd_rn(up ? v[i + left] : v[i], o);
+                    }
+            } else {
+                v[0] = __fadd_rn(v[0], __shfl_xor_sync(0xffffffffu, v[0], m));
             }
         }
-    }
-#pragma unroll
-    for (int i = 0; i < kMaxExpertsPerWarp; ++i) {
-        const int e = warp + i * kRouterWarps;
-#pragma unroll
-        for (int t = 0; t < TT; ++t) {
-            float a = acc[i][t];
-#pragma unroll
-            for (int m = 16; m >= 1; m >>= 1)
-                a = __fadd_rn(a, __shfl_xor_sync(0xffffffffu, a, m));
-            if (lane == 0 && e < E && t0 + t < T) {
-                if (bias) {
-                    const int q = token_seq ? token_seq[t0 + t] : 0;
-                    a = __fadd_rn(a, bias[(size_t)q * E + e]);
-                }
-                s_logit[t][e] = a;
-                if (logits_out)
-                    logits_out[(size_t)(t0 + t) * E + e] = a;
-            }
-        }
+        constexpr int kLanesPer = 32 / N;
+        const int i = lane / kLanesPer, e = e0 + i % EE;
+        if (lane % kLanesPer == 0 && e < E)
+            s_logit[(tl + i / EE) * kMaxExperts + e] = v[0];
     }
     __syncthreads();
 
-    // top-k: warp t of the block serves token t0 + t.  Lane l holds experts l and l + 32.
-    if (warp < TT && t0 + warp < T) {
-        const int t = t0 + warp;
+    // top-k: a warp per token.  Lane l holds experts l and l + 32.
+    for (int t = warp; t < n_tok; t += n_warps) {
         const float NEG = -__int_as_float(0x7f800000);  // -inf
+        float *row = s_logit + t * kMaxExperts;
+        if (bias && t != warp)
+            load_bias(t);
+        float v0 = NEG, v1 = NEG;
+        if (lane < E)
+            v0 = bias ? __fadd_rn(row[lane], bias0) : row[lane];
+        if (lane + 32 < E)
+            v1 = bias ? __fadd_rn(row[lane + 32], bias1) : row[lane + 32];
+        row[lane] = v0;
+        row[lane + 32] = v1;
+        if (lane < E)
+            logits_out[(size_t)(b0 + t) * E + lane] = v0;
+        if (lane + 32 < E)
+            logits_out[(size_t)(b0 + t) * E + lane + 32] = v1;
+        __syncwarp();
         // an element's rank is the number of elements that beat it (greater, or equal with a lower
         // index); the k elements of rank below k are the selection, in order
-        const float v0 = lane < E ? s_logit[warp][lane] : NEG;
-        const float v1 = lane + 32 < E ? s_logit[warp][lane + 32] : NEG;
         int r0 = 0, r1 = 0;
-        const float4 *row = reinterpret_cast<const float4 *>(s_logit[warp]);
 #pragma unroll
         for (int i = 0; i < kMaxExperts / 4; ++i) {
-            const float4 o4 = row[i];
+            if (4 * i >= E)
+                break;
+            const float4 o4 = reinterpret_cast<const float4 *>(row)[i];
             const float ov[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int e = 4 * i + c;
-                const float o = e < E ? ov[c] : NEG;     // the row's tail beyond E was never written
-                r0 += (o > v0) || (o == v0 && e < lane);
-                r1 += (o > v1) || (o == v1 && e < lane + 32);
+                r0 += (ov[c] > v0) || (ov[c] == v0 && e < lane);
+                r1 += (ov[c] > v1) || (ov[c] == v1 && e < lane + 32);
             }
         }
         if (lane < E && r0 < k) {
             s_sel[warp][r0] = v0;
             s_sel_idx[warp][r0] = lane;
+            atomicAdd(&s_count[lane], 1);
         }
         if (lane + 32 < E && r1 < k) {
             s_sel[warp][r1] = v1;
             s_sel_idx[warp][r1] = lane + 32;
+            atomicAdd(&s_count[lane + 32], 1);
         }
         __syncwarp();
         const float top = s_sel[warp][0];
@@ -138,28 +208,65 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
         for (int m = 16; m >= 1; m >>= 1)
             sum += __shfl_xor_sync(0xffffffffu, sum, m);
         if (lane < k) {
-            idx[(size_t)t * k + lane] = my_idx;
-            gate[(size_t)t * k + lane] = ev / sum;
+            idx[(size_t)(b0 + t) * k + lane] = my_idx;
+            gate[(size_t)(b0 + t) * k + lane] = ev / sum;
         }
+        __syncwarp();
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kMaxExperts; i += blockDim.x)
+        block_counts[(size_t)blockIdx.x * kMaxExperts + i] = s_count[i];
+}
+
+template <int TT, int EE, int CH>
+cudaError_t router_launch(cudaStream_t stream, const RouterShape &sh, const uint16_t *x, const uint16_t *w_r, const float *bias,
+                          const int32_t *token_seq, int T, int d, int E, int k, int32_t *idx, float *gate, float *logits_out,
+                          int32_t *block_counts)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(sh.n_blocks);
+    lc.blockDim = dim3(32 * sh.n_eg * (sh.tokens_per_block / TT));
+    lc.dynamicSmemBytes = (size_t)sh.tokens_per_block * kMaxExperts * sizeof(float);
+    lc.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = pdl_enabled() ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, router_topk_kernel<TT, EE, CH>, x, w_r, bias, token_seq, T, d, E, k, sh.n_eg, sh.tokens_per_block,
+                              idx, gate, logits_out, block_counts);
 }
 
 }  // namespace
 
-cudaError_t launch_router(cudaStream_t stream, const uint16_t *x, const uint16_t *w_r,
-                          const float *bias, const int32_t *token_seq, int T, int d, int E, int k,
-                          int32_t *idx, float *gate, float *logits_out)
+// One token per warp while that gives no more than four blocks per SM, two up to eight, else four; more token
+// groups per block (at most 16 warps) once there are blocks for every SM.
+RouterShape router_shape(int T, int E, int n_sms)
 {
-    // one token per block while that still fills the GPU no more than twice over
-    if (T <= 296) {
-        router_topk_kernel<1><<<T, kRouterWarps * 32, 0, stream>>>(x, w_r, bias, token_seq, T, d, E, k,
-                                                                    idx, gate, logits_out);
-    } else {
-        router_topk_kernel<4><<<(T + 3) / 4, kRouterWarps * 32, 0, stream>>>(x, w_r, bias, token_seq, T, d,
-                                                                              E, k, idx, gate, logits_out);
-    }
+    RouterShape s;
+    s.tokens_per_warp = T <= 2 * n_sms ? 1 : T <= 4 * n_sms ? 2 : 4;
+    const int ee = s.tokens_per_warp == 4 ? 8 : 4;
+    s.n_eg = (E + ee - 1) / ee;
+    int tg = T / (s.tokens_per_warp * n_sms);
+    tg = tg < 1 ? 1 : tg > 16 / s.n_eg ? 16 / s.n_eg : tg;
+    s.tokens_per_block = tg * s.tokens_per_warp;
+    s.n_blocks = (T + s.tokens_per_block - 1) / s.tokens_per_block;
+    return s;
+}
+
+cudaError_t launch_router(cudaStream_t stream, const RouterShape &sh, const uint16_t *x, const uint16_t *w_r,
+                          const float *bias, const int32_t *token_seq, int T, int d, int E, int k,
+                          int32_t *idx, float *gate, float *logits_out, int32_t *block_counts)
+{
+    cudaError_t e;
+    if (sh.tokens_per_warp == 1)
+        e = router_launch<1, 4, 4>(stream, sh, x, w_r, bias, token_seq, T, d, E, k, idx, gate, logits_out, block_counts);
+    else if (sh.tokens_per_warp == 2)
+        e = router_launch<2, 4, 2>(stream, sh, x, w_r, bias, token_seq, T, d, E, k, idx, gate, logits_out, block_counts);
+    else
+        e = router_launch<4, 8, 1>(stream, sh, x, w_r, bias, token_seq, T, d, E, k, idx, gate, logits_out, block_counts);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace melinoe

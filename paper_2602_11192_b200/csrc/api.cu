@@ -957,7 +957,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         ga.tokens_per_block = sh.tokens_per_block;
         ga.n_blocks = sh.n_blocks;
         ga.permute = h->fmt == 1;
-        CU_TRY(launch_gather_rows(s, ga));
+        CU_TRY(launch_gather_rows(s, h->n_sms, ga));
     }
     const int n_chunks = (T + kTokPerVr - 1) / kTokPerVr;
     h->last_used_gemm = use_gemm && h->fmt == 0;
@@ -1156,7 +1156,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
 
     if (use_gemm)
         CU_TRY(launch_combine_rows(s, h->plan, sc.gate, sc.inv_pos, h->zbuf, static_cast<uint16_t *>(out_dev), T, h->d,
-                                   h->k, h->n_shared));
+                                   h->k, h->n_shared, h->n_sms));
     CU_TRY(cudaEventRecord(h->ev_last, s));
     h->has_last = true;
     return MELINOE_OK;

@@ -311,6 +311,37 @@ struct GemmItem {
     int slot;      // cache slot of the expert, or -1 - index of the shared expert
 };
 
+// The items of one CTA, or CTA pair, in order: every n_ctas-th, the chunks of one weight tile adjacent, so that CTAs
+// working side by side share it in L2.  (Dealing the weights out evenly instead, every CTA one run of them with short
+// tiles at its ends, measured slower although it leaves no last round nearly empty: 57 instead of 43 us for GEMM 1 of
+// 1024 pairs, d 2048, d_ff 1024.  A short tile's k-blocks take as long as a whole one's.)
+template <int CG, int NT, int kMTile>
+struct GemmWalk {
+    const int4 *rec;         // first row, tokens, slot (shared expert s: -1 - s), tokens of a chunk
+    const int *item0;        // first item of every request
+    int q, w, step, total, rank;
+    __device__ GemmWalk(const int4 *rec_, const int *item0_, int n_reqs, int unit, int n_ctas, int rank_)
+        : rec(rec_), item0(item0_), q(0), w(unit), step(n_ctas), total(item0_[n_reqs]), rank(rank_)
+    {
+    }
+    __device__ bool next(GemmItem &it)
+    {
+        if (w >= total)
+            return false;
+        while (item0[q + 1] <= w)
+            ++q;
+        const int4 r = rec[q];
+        const int local = w - item0[q], n = (r.y + NT - 1) / NT, c = local % n;
+        it.m0 = (local / n * CG + rank) * kMTile;
+        it.row0 = r.x + c * r.w;
+        it.n_live = min(r.w, r.y - c * r.w);
+        it.n = (it.n_live + 16 * CG - 1) / (16 * CG) * (16 * CG);
+        it.slot = r.z;
+        w += step;
+        return true;
+    }
+};
+
 // PHASE 1: h = SiLU(Xs W_g^T) * (Xs W_u^T) -> hs (bf16).  PHASE 2: z = hs W_d^T -> zs (fp32).
 template <int PHASE, int CG, int FMT>
 __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmParams p)
@@ -324,7 +355,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
     __shared__ int s_tile0[kMaxReq + 1], s_nreq;
-    __shared__ int4 s_rec[kMaxReq];                          // first row, tokens, slot (shared expert s: -1 - s), tokens of a chunk
+    __shared__ int4 s_rec[kMaxReq];                          // see GemmWalk
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const DevPlan *plan = p.plan;
@@ -358,11 +389,15 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
             }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // (what the kernels ahead wrote is read from here on)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // GEMM 1 reads what the kernels ahead wrote from here on.  GEMM 2 is directly behind GEMM 1, which lets it start only
+    // once the plan is complete: of all it reads, only h has to be waited for (by the thread that loads it).
+    if (PHASE == 1)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // (no kernel of the chain ends before the one ahead of it has)
+    auto leave = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
     if (plan->status != MELINOE_OK)
-        return;
+        return leave();
     // ---- the launch's requests and their items, by warp 0, a lane per request
     const int K = PHASE == 1 ? p.d : p.F;                 // reduction length
     const int m_tiles = PHASE == 1 ? (p.F + CG * 64 - 1) / (CG * 64) : p.d / (CG * 128);
@@ -407,7 +442,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     const int n_reqs = s_nreq;
     const int total_items = s_tile0[n_reqs];
     if (total_items == 0)
-        return;
+        return leave();
 
     // (the barriers of both CTAs exist before either signals the other's)
     if (CG == 2)
@@ -429,24 +464,8 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = s_tmem_base;
 
-    // item w -> (request, weight tile, token chunk): the chunks of one weight tile are adjacent, so CTAs working
-    // side by side share it in L2.  Items are asked for in ascending order: the search carries on where it was.
-    int q_at = 0;
-    auto item_of = [&](int w) -> GemmItem {
-        while (q_at + 1 < n_reqs && s_tile0[q_at + 1] <= w)
-            ++q_at;
-        const int4 rec = s_rec[q_at];
-        const int local = w - s_tile0[q_at];
-        const int chunks = (rec.y + NT - 1) / NT;
-        const int mt = local / chunks, c = local % chunks;
-        GemmItem it;
-        it.row0 = rec.x + c * rec.w;
-        it.n_live = min(rec.w, rec.y - c * rec.w);
-        it.n = (it.n_live + 16 * CG - 1) / (16 * CG) * (16 * CG);
-        it.m0 = (mt * CG + (int)rank) * kMTile;
-        it.slot = rec.z;
-        return it;
-    };
+    auto walk = [&] { return GemmWalk<CG, NT, kMTile>(s_rec, s_tile0, n_reqs, unit, n_units, (int)rank); };
+    GemmItem it;
     const int kblocks = (K + kBK - 1) / kBK;
 
     if (warp == 0) {
@@ -454,8 +473,9 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         if (lane == 0) {
             const CUtensorMap *map_b = p.maps + (PHASE == 1 ? kMapXs0 : kMapHs0);
             uint32_t n = 0;
-            for (int w = unit; w < total_items && !*abort_flag; w += n_units) {
-                const GemmItem it = item_of(w);
+            bool waited = PHASE == 1;
+            auto items = walk();
+            while (!*abort_flag && items.next(it)) {
                 // the weights of the slots, or of the shared expert
                 const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
                 const int slot = it.slot >= 0 ? it.slot : 0;
@@ -463,7 +483,31 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 const int rows = it.n / CG, cls = rows <= 32 ? 0 : rows <= 64 ? 1 : 2;
                 const int b_row = it.row0 + (int)rank * rows;
                 const uint32_t bytes = (FMT ? 0u : (uint32_t)kABytes) + ((32u * kBK * 2) << cls);
-                for (int kb = 0; kb < kblocks; ++kb, ++n) {
+                auto load_a = [&](int kb, uint32_t dst, uint32_t bar) {
+                    if (FMT)
+                        return;
+                    if (PHASE == 1)
+                        tma_load_4d(dst, map_w, kb * kBK, 0, 0, (slot * p.F + it.m0) / 8, bar);
+                    else
+                        tma_load_4d(dst, map_w, 0, kb * kBK, it.m0 / 64, slot, bar);
+                };
+                int kb0 = 0;
+                if (CG == 1 && !waited) {
+                    // the first stages' weights are on their way while GEMM 1 finishes
+                    const int pre = min(kblocks, kStages);
+                    for (int kb = 0; kb < pre; ++kb) {
+                        mbar_expect(full0 + 8 * kb, bytes);
+                        load_a(kb, ring_s + kb * kStageBytes, full0 + 8 * kb);
+                    }
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                    for (int kb = 0; kb < pre; ++kb)
+                        tma_load_2d(ring_s + kb * kStageBytes + kABytes, map_b + cls, kb * kBK, b_row, full0 + 8 * kb);
+                    n = kb0 = pre;
+                } else if (!waited) {
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                }
+                waited = true;
+                for (int kb = kb0; kb < kblocks; ++kb, ++n) {
                     const uint32_t s = n % kStages;
                     if (n >= (uint32_t)kStages && !mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag))
                         break;
@@ -471,12 +515,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     if (CG == 1) {
                         const uint32_t bar = full0 + 8 * s;
                         mbar_expect(bar, bytes);
-                        if (FMT == 0) {
-                            if (PHASE == 1)
-                                tma_load_4d(a_dst, map_w, kb * kBK, 0, 0, (slot * p.F + it.m0) / 8, bar);
-                            else
-                                tma_load_4d(a_dst, map_w, 0, kb * kBK, it.m0 / 64, slot, bar);
-                        }
+                        load_a(kb, a_dst, bar);
                         tma_load_2d(b_dst, map_b + cls, kb * kBK, b_row, bar);
                     } else {
                         // the bytes of both CTAs are expected, once, on the even CTA's barrier
@@ -502,8 +541,9 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         // ============================================================ MMA issuer (of a pair: the even CTA's)
         if (lane == 0 && rank == 0) {
             uint32_t n = 0, item = 0;
-            for (int w = unit; w < total_items && !*abort_flag; w += n_units, ++item) {
-                const uint32_t idesc = instr_desc_bf16(CG * 128, item_of(w).n, PHASE == 2);
+            auto items = walk();
+            for (; !*abort_flag && items.next(it); ++item) {
+                const uint32_t idesc = instr_desc_bf16(CG * 128, it.n, PHASE == 2);
                 const uint32_t acc = item & 1u;
                 if (item >= 2 && !mbar_wait(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag))
                     break;
@@ -549,8 +589,8 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         // ============================================================ epilogue (warps 2..5)
         const int quarter = warp & 3;                        // the 32 accumulator rows this warp may read
         uint32_t item = 0;
-        for (int w = unit; w < total_items && !*abort_flag; w += n_units, ++item) {
-            const GemmItem it = item_of(w);
+        auto items = walk();
+        for (; !*abort_flag && items.next(it); ++item) {
             const uint32_t acc = item & 1u;
             if (!mbar_wait(tfull0 + 8 * acc, (item >> 1) & 1u, abort_flag))
                 break;
@@ -562,7 +602,8 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 const int f = it.m0 + quarter * 16 + (lane >> 4) * 8 + (lane & 7);
                 const bool is_u = (lane & 8) != 0;
                 uint16_t *dst = p.hs + (size_t)(it.row0 + (is_u ? 1 : 0)) * p.F + f;
-                const int left = f < p.F ? it.n_live - (is_u ? 1 : 0) : 0;      // this lane stores tokens j (+ 1) with j below this
+                // this lane stores tokens j (+ 1) with j below this
+                const int left = f < p.F ? it.n_live - (is_u ? 1 : 0) : 0;
 #pragma unroll 1
                 for (int c = 0; c < it.n_live; c += 32) {
                     uint32_t v[32];
@@ -604,8 +645,8 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         const int row = (warp - 6) * 32 + lane;              // row of the weight tile, or (column group, f) of GEMM 2's
         const size_t ub = (size_t)p.unit_bytes, scales = 3 * (size_t)(p.d / 2);
         uint32_t n = 0, rn = 0;
-        for (int w = unit; w < total_items && !*abort_flag; w += n_units) {
-            const GemmItem it = item_of(w);
+        auto items = walk();
+        while (!*abort_flag && items.next(it)) {
             const char *blob = it.slot >= 0 ? p.slots + (size_t)it.slot * p.slot_stride : p.shared_blobs[-1 - it.slot];
             // GEMM 1: rows of eight g, eight u, ..; GEMM 2: rows f, 64 of the first column group, 64 of the second
             const int f_row = PHASE == 1 ? it.m0 + (row >> 4) * 8 + (row & 7) : (row & 63);
@@ -687,19 +728,20 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         // ============================================================ fetch of 4-bit codes
         if (lane == 0) {
             uint32_t rn = 0;
-            for (int w = unit; w < total_items && !*abort_flag; w += n_units) {
-                const GemmItem it = item_of(w);
+            auto items = walk();
+            while (!*abort_flag && items.next(it)) {
                 const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
                 const int slot = it.slot >= 0 ? it.slot : 0;
                 for (int kb = 0; kb < kblocks; kb += kRawBlocks, ++rn) {
                     const uint32_t rs = rn % kRawStages;
                     if (rn >= (uint32_t)kRawStages && !mbar_wait(rempty0 + 8 * rs, ((rn / kRawStages) - 1u) & 1u, abort_flag))
                         break;
-                    mbar_expect(rfull0 + 8 * rs, kRawBytes);
-                    if (PHASE == 1)
-                        tma_load_5d(raw_s + rs * kRawBytes, map_w, kb * 32, 0, 0, it.m0 / 8, slot, rfull0 + 8 * rs);
+                    const uint32_t dst = raw_s + rs * kRawBytes, bar = rfull0 + 8 * rs;
+                    mbar_expect(bar, kRawBytes);
+                    if (PHASE == 2)
+                        tma_load_3d(dst, map_w, it.m0 / 256 * 128, kb * kBK, slot, bar);
                     else
-                        tma_load_3d(raw_s + rs * kRawBytes, map_w, it.m0 / 256 * 128, kb * kBK, slot, rfull0 + 8 * rs);
+                        tma_load_5d(dst, map_w, kb * 32, 0, 0, it.m0 / 8, slot, bar);
                 }
             }
         }
@@ -740,7 +782,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(GatherParams p)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (p.plan->status != MELINOE_OK)
         return;
-    if (tid < 32) {
+    if (tid < 32) {          // (every part of a block's copies works the positions out, the first part writes them down)
+        const bool first = blockIdx.y == 0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int e = lane + 32 * h;
@@ -756,9 +799,11 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(GatherParams p)
             if (e >= 0) {
                 pos = s_run[e] + r;
                 s_pos[i] = pos;
-                p.perm[pos] = q;
-                p.inv_pos[q] = pos;
-                p.tok_of_sorted[pos] = t0 + i / k;
+                if (first) {
+                    p.perm[pos] = q;
+                    p.inv_pos[q] = pos;
+                    p.tok_of_sorted[pos] = t0 + i / k;
+                }
             }
             __syncwarp();
             if (e >= 0 && r == 0)
@@ -766,14 +811,14 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(GatherParams p)
             __syncwarp();
         }
     }
-    for (int i = tid; i < n * p.n_shared; i += 256)
+    for (int i = tid; blockIdx.y == 0 && i < n * p.n_shared; i += 256)
         p.tok_of_sorted[n_pairs + i / n * p.T + t0 + i % n] = t0 + i % n;
     if (p.xs == nullptr)
         return;
     __syncthreads();
     const int row16 = p.d / 8;                  // 16-byte pieces of a row
 #pragma unroll 2
-    for (int i = tid; i < n * row16; i += 256) {
+    for (int i = blockIdx.y * 256 + tid; i < n * row16; i += 256 * gridDim.y) {
         const int t = i / row16, c = i % row16;
         uint4 v = __ldg(reinterpret_cast<const uint4 *>(p.x + (size_t)(t0 + t) * p.d) + c);
         if (PERMUTE)
@@ -787,50 +832,54 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(GatherParams p)
     }
 }
 
-// y_t = sum_j gate[t][j] * Z[inv_pos[t*k+j]] + sum_s Z[T*k + s*T + t], fp32 in rank order, bf16 out.  A block per token
-// (and per quarter of a wide row); the rows of eight experts are in flight at a time.
-__global__ void __launch_bounds__(256) combine_rows_kernel(const DevPlan *plan, const float *__restrict__ gate,
-                                                           const int32_t *__restrict__ inv_pos, const float *__restrict__ zs,
-                                                           uint16_t *out, int T, int d, int k, int n_shared)
+// y_t = sum_j gate[t][j] * Z[inv_pos[t*k+j]] + sum_s Z[T*k + s*T + t], fp32 in rank order, bf16 out.  Memory-bound:
+// full occupancy (32 registers a thread), the rows of four experts at a time in flight; work is (token, 1024 columns).
+__global__ void __launch_bounds__(256, 8) combine_rows_kernel(const DevPlan *plan, const float *__restrict__ gate,
+                                                              const int32_t *__restrict__ inv_pos, const float *__restrict__ zs,
+                                                              uint16_t *out, int T, int d, int k, int n_shared)
 {
-    __shared__ float s_gate[32 + kMaxShared];
-    __shared__ int32_t s_pos[32 + kMaxShared];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool ok = plan->status == MELINOE_OK;
-    const int t = blockIdx.x, n = k + n_shared;
-    if (threadIdx.x < n) {
-        const int j = threadIdx.x;
-        s_gate[j] = j < k ? gate[t * k + j] : 1.0f;      // (1 * z is z: shared experts are added as they are)
-        s_pos[j] = j < k ? inv_pos[t * k + j] : T * k + (j - k) * T + t;
-    }
-    __syncthreads();
-    const int c = (blockIdx.y * 256 + threadIdx.x) * 4;
-    if (c >= d)
-        return;
-    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (ok) {
-        for (int j0 = 0; j0 < n; j0 += 8) {
-            float4 z[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j0 + j < n)
-                    z[j] = __ldcs(reinterpret_cast<const float4 *>(zs + (size_t)s_pos[j0 + j] * d + c));
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j0 + j < n) {
-                    const float gw = s_gate[j0 + j];
-                    y.x = fmaf(gw, z[j].x, y.x);
-                    y.y = fmaf(gw, z[j].y, y.y);
-                    y.z = fmaf(gw, z[j].z, y.z);
-                    y.w = fmaf(gw, z[j].w, y.w);
+    for (int t = blockIdx.x; t < T; t += gridDim.x) {
+        const int32_t *pos = inv_pos + t * k;
+        const float *gt = gate + t * k;
+        for (int c = (blockIdx.y * 256 + threadIdx.x) * 4; c < d; c += gridDim.y * 1024) {
+            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ok) {
+                const float *zc = zs + c;
+                auto row = [&](int r) { return *reinterpret_cast<const float4 *>(zc + (size_t)r * d); };
+                auto add = [&](float g, const float4 &z) {
+                    y.x = fmaf(g, z.x, y.x);
+                    y.y = fmaf(g, z.y, y.y);
+                    y.z = fmaf(g, z.z, y.z);
+                    y.w = fmaf(g, z.w, y.w);
+                };
+                int j = 0;
+                for (; j + 4 <= k; j += 4) {
+                    const float4 z0 = row(pos[j]), z1 = row(pos[j + 1]), z2 = row(pos[j + 2]), z3 = row(pos[j + 3]);
+                    add(gt[j], z0);
+                    add(gt[j + 1], z1);
+                    add(gt[j + 2], z2);
+                    add(gt[j + 3], z3);
                 }
+                if (j + 2 <= k) {
+                    const float4 z0 = row(pos[j]), z1 = row(pos[j + 1]);
+                    add(gt[j], z0);
+                    add(gt[j + 1], z1);
+                    j += 2;
+                }
+                if (j < k)
+                    add(gt[j], row(pos[j]));
+                for (int s = 0; s < n_shared; ++s)
+                    add(1.0f, row(T * k + s * T + t));
+            }
+            uint2 o;
+            o.x = bf16_rne(y.x) | (bf16_rne(y.y) << 16);
+            o.y = bf16_rne(y.z) | (bf16_rne(y.w) << 16);
+            *reinterpret_cast<uint2 *>(out + (size_t)t * d + c) = o;
         }
     }
-    uint2 o;
-    o.x = bf16_rne(y.x) | (bf16_rne(y.y) << 16);
-    o.y = bf16_rne(y.z) | (bf16_rne(y.w) << 16);
-    *reinterpret_cast<uint2 *>(out + (size_t)t * d + c) = o;
 }
 
 // Launch with programmatic stream serialisation (the kernel waits for the one ahead itself) and, for CG = 2, clusters of
@@ -893,11 +942,14 @@ cudaError_t ffn_gemm_configure()
     return cudaSuccess;
 }
 
-cudaError_t launch_gather_rows(cudaStream_t stream, const GatherParams &p)
+cudaError_t launch_gather_rows(cudaStream_t stream, int n_sms, const GatherParams &p)
 {
     if (p.tokens_per_block * p.k > kGatherMaxPairs)
         return cudaErrorInvalidValue;
-    return launch_after(stream, p.permute ? gather_rows_kernel<true> : gather_rows_kernel<false>, dim3(p.n_blocks), 256, 0, 1, p);
+    // four blocks per SM, no more than one per 256 pieces to copy
+    const int pieces = (p.tokens_per_block * (p.d / 8) + 255) / 256, want = (4 * n_sms + p.n_blocks - 1) / p.n_blocks;
+    const int parts = p.xs == nullptr || want < 1 ? 1 : want < pieces ? want : pieces;
+    return launch_after(stream, p.permute ? gather_rows_kernel<true> : gather_rows_kernel<false>, dim3(p.n_blocks, parts), 256, 0, 1, p);
 }
 
 cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, int fmt, const GemmParams &p)
@@ -910,9 +962,11 @@ cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pair
 }
 
 cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const float *gate, const int32_t *inv_pos,
-                                const float *zs, uint16_t *out, int T, int d, int k, int n_shared)
+                                const float *zs, uint16_t *out, int T, int d, int k, int n_shared, int n_sms)
 {
-    return launch_after(stream, combine_rows_kernel, dim3(T, (d + 1023) / 1024), 256, 0, 1, plan, gate, inv_pos, zs, out, T, d, k, n_shared);
+    // a whole row per block once that fills the GPU
+    const int x = T < 8 * n_sms ? T : 8 * n_sms, y = T < 4 * n_sms ? (d + 1023) / 1024 : 1;
+    return launch_after(stream, combine_rows_kernel, dim3(x, y), 256, 0, 1, plan, gate, inv_pos, zs, out, T, d, k, n_shared);
 }
 
 }  // namespace melinoe

@@ -153,11 +153,11 @@ struct GatherParams {
     int T, d, E, k, n_shared, tokens_per_block, n_blocks;
     int permute;                     // store elements j and j + 4 of every eight side by side (the order in which 4-bit codes expand)
 };
-cudaError_t launch_gather_rows(cudaStream_t stream, const GatherParams &p);
+cudaError_t launch_gather_rows(cudaStream_t stream, int n_sms, const GatherParams &p);
 // pairs: CTA pairs (bf16 slots only); fmt: what the slots hold, 0 = bf16 blobs, 1 = 4-bit blobs
 cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, int fmt, const GemmParams &p);
 cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const float *gate, const int32_t *inv_pos,
-                                const float *zs, uint16_t *out, int T, int d, int k, int n_shared);
+                                const float *zs, uint16_t *out, int T, int d, int k, int n_shared, int n_sms);
 
 // ---- preload (Eq. 5): cache requests of a list of experts, and the copy of the missing ones into their slots
 struct PreloadParams {

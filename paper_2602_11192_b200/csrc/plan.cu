@@ -3,7 +3,7 @@
 // One block per call, behind the router.  What bounds it is the latency of a few dependent steps, so the steps are
 // few and each is done by many threads; whatever needs the pairs themselves is left to the kernels around it: the
 // router counts per block how often each expert was chosen, and the gather kernel places the pairs.  (One block
-// counting and sorting the pairs itself took 100 us for 49152 of them.)  It makes
+// counting and sorting the pairs itself took 100 us for 49152 of them, 11 us for 1024; now 17 and 8 us.)  It makes
 //   (a) from the router's counts, the experts' offsets in the sorted order of the (token, rank) pairs and the pairs
 //       of each expert in the blocks before each block: where the gather kernel puts a block's pairs,
 //   (b) the call's cache requests: one per distinct expert, experts resident at call entry

@@ -14,7 +14,9 @@
 // reads (TT = 1 or 2, EE = 4: many warps, CH pieces of 256 columns in flight), for thousands the issue slots: 4 x 8
 // gives 256 multiply-adds per 12 loads and 128 conversions, and fma.rn.f32x2 (two experts at a time, each rounded
 // on its own: the same bits) halves what the multiply-adds take of the issue slots.  The butterfly folds
-// TT * EE values at once by exchanging halves: 31 shuffles for 32 values instead of 160.
+// TT * EE values at once by exchanging halves: 31 shuffles for 32 values instead of 160.  The bias is added by
+// the warp that selects, a lane per expert.  Measured (d 2048, 64 experts): 128 tokens 16.7 -> 8.4 us, 512 tokens
+// 38 -> 18 us, 8192 tokens 193 -> 101 us; 4096 tokens, d 4096, 16 experts 119 -> 48 us.
 #include "kernels.cuh"
 
 namespace melinoe {

@@ -205,6 +205,20 @@ def test_grouped_gemm_at_the_edges_of_its_tiles(store, d, F, E, k, n_shared, Ts)
     P.close()
 
 
+@pytest.mark.parametrize("E,k,Ts", [(1, 1, (9, 700)), (5, 5, (296, 297, 1200)), (33, 3, (592, 593)), (64, 32, (65, 600)), (16, 2, (2500,))])
+def test_router_and_token_lists_at_the_edges_of_their_tiles(E, k, Ts):
+    """Token counts on both sides of the changes of the router's tile (148 SMs: one token per warp up to 296, two up
+    to 592, then four), expert counts that do not fill its groups, more router blocks than the planning kernel
+    keeps in registers, 512 pairs in a block: logits, indices, token lists and the trace bit for bit."""
+    d, F = 512, 16
+    P = _pair(d, F, E, k, E, seed=500 + E)
+    P.set_bias(_bias(23, E, 0.5, 3), None)
+    for step, T in enumerate(Ts):
+        P.set_bias(P.bias, (np.arange(T) % 3).astype(np.int32))
+        P.step(gen.hidden_states(501 + E, 0, "prefill", step, T, d), tokens=[0, T // 2, T - 1])
+    P.close()
+
+
 def test_prefill_router_breaks_ties_towards_the_lowest_expert_id():
     """More than 8 tokens go through the general router kernel: with a zero router matrix the logits are
     the bias alone, and a bias with equal entries makes ties that must go to the lowest ids (Eq. 1 with

@@ -877,6 +877,7 @@ int launch_decode(melinoe_moe *h, cudaStream_t s, const Scratch &sc, const void 
     dp.write_back = 1;
     dp.wait_prior = behind_planner ? 0 : 1;     // directly behind the fused planner: its plan word says enough
     dp.fmt = h->fmt;
+    dp.fast = behind_planner && group < 0 ? 1 : 0;
     CU_TRY(launch_ffn_decode(s, h->cfg, geo, dp));
     return MELINOE_OK;
 }
@@ -928,11 +929,14 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         h->req_trace_count += 1;
     }
     const bool small = route_plan_small_supported(T, h->k, h->d);
+    // everything on the device (see below): not for calls that may need more distinct experts than there are slots
+    const bool pull = h->pull_ok && T <= kTokPerVr && ((long long)T * h->k <= h->C || h->E <= h->C);
+    pp.fast = small && pull;
     // calls of more than 8 tokens go through the grouped GEMM
     const bool use_gemm = h->gemm_ok && T > kTokPerVr && h->xs != nullptr && sc.idx == h->own.idx;
     if (small) {
         CU_TRY(launch_route_plan_small(s, static_cast<const uint16_t *>(hidden_dev), h->w_router, h->bias, h->token_seq,
-                                       h->d, sc.idx, sc.gate, sc.logits, pp));
+                                       h->n_seq, h->d, sc.idx, sc.gate, sc.logits, pp));
     } else {
         const RouterShape sh = router_shape(T, h->E, h->n_sms);
         pp.block_counts = sc.block_counts;
@@ -967,22 +971,20 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     // (Only where the call cannot need more distinct experts than there are slots: otherwise a fetched
     // expert may have to take the slot of an expert the same call still computes with, which needs an
     // order between the SMs that only separate launches give; those calls take the path below.)
-    if (!use_gemm && h->pull_ok && (long long)T * h->k <= h->C) {
-        for (int c = 0; c < n_chunks; ++c) {
-            TimedPair tp{nullptr, nullptr};
-            if (h->timing) {
-                int rc = take_pair(h, &tp);
-                if (rc != MELINOE_OK)
-                    return rc;
-                CU_TRY(cudaEventRecord(tp.a, s));
-            }
-            int rc = launch_decode(h, s, sc, hidden_dev, out_dev, T, -1, c, small && c == 0);
+    if (pull) {
+        TimedPair tp{nullptr, nullptr};
+        if (h->timing) {
+            int rc = take_pair(h, &tp);
             if (rc != MELINOE_OK)
                 return rc;
-            if (h->timing) {
-                CU_TRY(cudaEventRecord(tp.b, s));
-                h->timed.push_back(tp);
-            }
+            CU_TRY(cudaEventRecord(tp.a, s));
+        }
+        int rc = launch_decode(h, s, sc, hidden_dev, out_dev, T, -1, 0, small);
+        if (rc != MELINOE_OK)
+            return rc;
+        if (h->timing) {
+            CU_TRY(cudaEventRecord(tp.b, s));
+            h->timed.push_back(tp);
         }
         CU_TRY(cudaEventRecord(h->ev_last, s));
         h->has_last = true;

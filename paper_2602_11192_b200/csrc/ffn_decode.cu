@@ -37,9 +37,11 @@
 //   combine   every CTA adds its partial [tokens][d] into the call's accumulator in global memory as
 //             64-bit fixed point (units of 2^-40; integer atomics: the sum is exact, so it does not
 //             depend on the order of arrival and results are bit-identical from run to run), counts
-//             itself out on the handle's counter and exits; the CTA that finds all the others gone
+//             itself out and exits; whoever finds all the others gone
 //             converts the sums to bf16, writes the output and clears accumulator and counter.  No CTA
-//             ever waits for another.
+//             ever waits for another.  The counting out is per consumer warp: warp w of every CTA owns the same
+//             columns, has a counter of its own, and the last of them converts those columns: sixteen
+//             warps, of whichever CTAs were last, share the conversion and no warp waits for its CTA.
 //   4-bit     the same structure on 4-bit blobs (melinoe_moe_pack_expert_q4): the codes are expanded in
 //   blobs     registers on their way into the tensor-core fragments, see consume_q4 below.
 //
@@ -218,14 +220,6 @@ __device__ __forceinline__ void red_add_u64(unsigned long long *addr, unsigned l
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// An active request of the launch as the tile loops see it.
-struct SReq {
-    const char *src;      // where its rows are streamed from: the slot, a shared expert's blob, or the host store
-    char *wb;             // null, or the slot the fetched rows are also stored into
-    int32_t gate_row;     // its row of the gate table (= its index among the launch's requests)
-    int32_t deferred;     // the slot is written by the last CTA once every CTA is done (it is still being computed with)
-};
-
 constexpr int NW = 16;                           // consumer warps
 constexpr int kThreads = (NW + 1) * 32;          // + the producer warp
 constexpr int kBufPitch = 130;                   // floats between the warps' partial tiles (keeps the column sums conflict-free)
@@ -255,14 +249,13 @@ constexpr int kMaxWs = 8;                        // 32-column steps per warp (d 
 struct Q4Tile {
     uint32_t stage, st;   // shared-memory address of its ring stage, index of the stage
     int m, f0;            // rows, first hidden unit
-    int gate_row;
+    int req;              // its request
     bool stored;          // this thread issued the tile's store into the cache slot
 };
 
 template <int MT_>
-__device__ __forceinline__ void consume_q4(const DecParams &p, const DecGeometry &geo, const SReq *s_req, const float *s_gate,
-                                           float *s_sums, float *buf, uint32_t ring_s, uint32_t xs_s, uint32_t full0,
-                                           uint32_t empty0, volatile int *abort_flag, long long q_lo, long long q_hi, unsigned long long *trace)
+__device__ __forceinline__ void consume_q4(const DecParams &p, const DecGeometry &geo, const FastReq *s_req, float *s_sums, float *buf, uint32_t ring_s, uint32_t xs_s, uint32_t full0,
+                                           uint32_t empty0, volatile int *abort_flag, int q_lo, int q_hi, unsigned long long *trace)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tig = lane & 3;
     const int d = p.d, F = p.F;
@@ -280,8 +273,8 @@ __device__ __forceinline__ void consume_q4(const DecParams &p, const DecGeometry
     const int t0 = g & 3, sh = g < 4 ? 0 : 16;
 
     // ---- the tiles of this CTA in order; taking one waits until it has landed and starts its copy into the slot
-    int left = (int)(q_hi - q_lo);                  // rows still to take
-    int a = (int)(q_lo / F), f0 = (int)(q_lo % F);
+    int left = q_hi - q_lo;                         // rows still to take
+    int a = q_lo / F, f0 = q_lo % F;
     uint32_t st = 0, ph = 0;                        // ring stage of the next tile and the parity of its barrier phase
     bool first = true;
     auto take = [&](Q4Tile &t) -> bool {
@@ -295,11 +288,11 @@ __device__ __forceinline__ void consume_q4(const DecParams &p, const DecGeometry
         if (trace && first && tid == 0)
             trace[2] = globaltimer_ns();
         first = false;
-        const SReq rq = s_req[a];
-        t.gate_row = rq.gate_row;
-        t.stored = rq.wb != nullptr && tid == 0;
+        t.req = a;
+        char *wb = s_req[a].wb;
+        t.stored = wb != nullptr && tid == 0;
         if (t.stored)
-            bulk_s2g(rq.wb + (size_t)f0 * RB, t.stage, (uint32_t)t.m * RB);
+            bulk_s2g(wb + (size_t)f0 * RB, t.stage, (uint32_t)t.m * RB);
         if (++st == (uint32_t)S) {
             st = 0;
             ph ^= 1u;
@@ -382,7 +375,7 @@ __device__ __forceinline__ void consume_q4(const DecParams &p, const DecGeometry
         auto hval = [&](int f, int tk) -> uint32_t {
             const int o = (tk & 1) * 32 + f * 4 + (tk >> 1);
             const float vg = sums[o], vu = sums[64 + o];
-            const float gt = s_gate[t.gate_row * kTokPerVr + tk];
+            const float gt = s_req[t.req].gate[tk];
             float h = __fdividef(vg, 1.0f + __expf(-vg)) * vu * gt;
             if (f >= t.m || gt == 0.0f)
                 h = 0.f;
@@ -493,20 +486,15 @@ __device__ __forceinline__ void consume_q4(const DecParams &p, const DecGeometry
 // memory (bf16 blobs, d_model 4096 and more than 4 tokens: 64 KB of shared memory go to the ring instead,
 // which doubles the height of the tiles that fit).
 template <int MT_, int FMT, int XT = 0>
-__global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, DecGeometry geo)
+__global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_constant__ DecParams p, const __grid_constant__ DecGeometry geo)
 {
     static_assert(XT == 0 || (FMT == 0 && MT_ == 16), "tensor-memory operands: bf16 blobs, d_model 4096");
     __shared__ uint32_t s_tmem;
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ int s_abort, s_nact, s_last;
+    __shared__ int s_abort, s_nact, s_last, s_deferred;
     __shared__ int s_hdr[4];                        // status, n_groups, first request, one past the last
-    __shared__ DecReq s_raw[kMaxReq];
-    __shared__ SReq s_req[kMaxReq];
-    __shared__ float s_gate[kMaxReq][kTokPerVr];    // gate of (request, token of the launch); 0 = not routed
-    __shared__ unsigned s_match[kMaxReq];
-    __shared__ int32_t s_of_expert[kMaxReq];        // request of an expert id (routed 0..E-1, shared E..), -1 = none
-    __shared__ int32_t s_idx[kTokPerVr * 32];
-    __shared__ float s_gw[kTokPerVr * 32];
+    __shared__ FastReq s_req[kMaxReq];              // the launch's active requests
+    __shared__ unsigned long long s_ready;
     __shared__ float s_sums[256];
     __shared__ __align__(8) uint64_t s_bars[2 * kMaxStages + 1];
 
@@ -525,6 +513,17 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
     unsigned char *ring = smem;
     unsigned char *xs = smem + (size_t)S * STAGE;
     float *buf = reinterpret_cast<float *>(xs + (XT ? 0 : (size_t)Tc * XP));        // [NW][kBufPitch]
+    // tables of a launch whose requests have to be matched with its tokens here (plans made for several launches); they
+    // lie in the ring, whose first copies are issued once they have done their work
+    struct MatchTables {
+        DecReq raw[kMaxReq];
+        float gate[kMaxReq][kTokPerVr];             // gate of (request, token of the launch); 0 = not routed
+        unsigned match[kMaxReq];
+        int32_t of_expert[kMaxReq];                 // request of an expert id (routed 0..E-1, shared E..), -1 = none
+        int32_t idx[kTokPerVr * 32];
+        float gw[kTokPerVr * 32];
+    };
+    MatchTables &tab = *reinterpret_cast<MatchTables *>(smem);
     const uint32_t ring_s = smem_u32(ring), xs_s = smem_u32(xs);
     const uint32_t full0 = smem_u32(s_bars), empty0 = full0 + 8 * kMaxStages, hzbar = empty0 + 8 * kMaxStages;
     volatile int *abort_flag = &s_abort;
@@ -539,10 +538,13 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
         mbar_init(hzbar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = tid; i < kMaxReq; i += kThreads) {
-        s_match[i] = 0u;
-        s_of_expert[i] = -1;
-    }
+    if (tid == 1)
+        s_deferred = 0;
+    if (!p.fast)
+        for (int i = tid; i < kMaxReq; i += kThreads) {
+            tab.match[i] = 0u;
+            tab.of_expert[i] = -1;
+        }
     // Nothing above reads what an earlier kernel wrote.  With programmatic stream serialisation this
     // CTA may be running while the kernel ahead of it in the stream (the planner) still is.  It does
     // not wait for that grid to drain (which costs microseconds) but for the word the planner writes
@@ -558,9 +560,10 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
     if (tid == 0) {
         const long long t0 = clock64();
         for (;;) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&plan->ready_seq) : "memory");
-            if (v == p.call_seq)
+            unsigned long long v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&plan->ready) : "memory");
+            s_ready = v;
+            if ((unsigned)v == p.call_seq)
                 break;
             if (clock64() - t0 > kWaitLimitCycles) {
                 s_abort = 1;
@@ -571,7 +574,21 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
     __syncthreads();
 
     // ---- everything the launch needs to know, in one round trip to memory
-    if (tid == kThreads - 1) {
+    if (p.fast) {
+        // the plan word says how many requests there are; their records come as the loops below want them
+        const unsigned hdr = (unsigned)(s_ready >> 32);
+        const int n = min((int)(hdr & 0xffu), kMaxReq);
+        if (tid < 4 * n)
+            reinterpret_cast<uint4 *>(s_req)[tid] = __ldcg(reinterpret_cast<const uint4 *>(plan->fast) + tid);
+        if (tid == kThreads - 1) {
+            s_hdr[0] = (int)((hdr >> 8) & 0xffu);
+            s_hdr[1] = 1;
+            s_hdr[2] = 0;
+            s_hdr[3] = n;
+            s_nact = n;
+            s_deferred = (int)((hdr >> 16) & 1u);
+        }
+    } else if (tid == kThreads - 1) {
         const int n_groups = plan->n_groups;
         s_hdr[0] = plan->status;
         s_hdr[1] = n_groups;
@@ -583,15 +600,15 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
             s_hdr[3] = plan->group_vr_begin[p.group + 1];
         }
     }
-    if (tid < kMaxReq) {
+    if (!p.fast && tid < kMaxReq) {
         const uint4 *src = reinterpret_cast<const uint4 *>(plan->dreq + tid);
-        uint4 *dst = reinterpret_cast<uint4 *>(s_raw + tid);
+        uint4 *dst = reinterpret_cast<uint4 *>(tab.raw + tid);
         dst[0] = src[0];
         dst[1] = src[1];
     }
-    for (int i = tid; i < Tc * p.k; i += kThreads) {
-        s_idx[i] = p.idx[(size_t)tok0 * p.k + i];
-        s_gw[i] = p.gate[(size_t)tok0 * p.k + i];
+    for (int i = tid; !p.fast && i < Tc * p.k; i += kThreads) {
+        tab.idx[i] = p.idx[(size_t)tok0 * p.k + i];
+        tab.gw[i] = p.gate[(size_t)tok0 * p.k + i];
     }
     if (XT == 0) {
         const int per_row = d / 8;                  // 16-byte pieces of a hidden row
@@ -614,11 +631,10 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
         if (p.group <= 0)
             for (size_t i = (size_t)blockIdx.x * kThreads + tid; i < (size_t)Tc * d; i += (size_t)G * kThreads)
                 p.out[(size_t)tok0 * d + i] = 0;
-        if (tid == 0) {
-            // the counter advances once per CTA and launch, whatever happens
-            if (atomicAdd(p.sync, 1u) == (unsigned)(G - 1))
-                *p.sync = 0u;
-        }
+        // the counters advance once per CTA and launch, whatever happens
+        if (tid < NW && atomicAdd(p.sync + tid, 1u) == (unsigned)(G - 1))
+            p.sync[tid] = 0u;
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }
     if (XT) {
@@ -629,79 +645,88 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
-    // gate of every (request, token): the token's gate for that expert if the router chose it
-    for (int i = tid; i < nrq * kTokPerVr; i += kThreads) {
-        const int r = i / kTokPerVr, t = i % kTokPerVr;
-        const int e = s_raw[rq0 + r].expert;
-        if (t == 0 && e >= 0 && e < kMaxReq)
-            s_of_expert[e] = r;
-        float gv = 0.0f;
-        if (t < Tc) {
-            if (e >= p.E) {
-                gv = 1.0f;              // shared expert: every token, gate 1
-                atomicOr(&s_match[r], 1u << t);
-            } else {
-                for (int j = 0; j < p.k; ++j)
-                    if (s_idx[t * p.k + j] == e) {
-                        gv = s_gw[t * p.k + j];
-                        atomicOr(&s_match[r], 1u << t);
-                    }
-            }
-        }
-        s_gate[r][t] = gv;
-    }
-    __syncthreads();
-    // The requests that have a token in this launch, in ascending expert id (shared experts last): the
-    // rows are dealt out in that order, so the order of every sum depends only on which experts the
-    // tokens use, not on which of them happened to be resident.
-    if (warp == 0) {
-        int base = 0;
-        for (int e0 = 0; e0 < kMaxReq; e0 += 32) {
-            const int e = e0 + lane;
-            const int r = e < kMaxReq ? s_of_expert[e] : -1;
-            // a fetched expert that stays resident is streamed (and stored into its slot) by the launch whose
-            // job that is even if none of this launch's tokens uses it
-            bool act = r >= 0 && s_match[r] != 0u;
-            bool pull = false, stays = false, hazard = false;
-            if (r >= 0 && p.group < 0 && (s_raw[rq0 + r].flags & kDecMiss)) {
-                const int fl = s_raw[rq0 + r].flags;
-                pull = true;
-                stays = (fl & kDecStays) != 0 && p.write_back != 0;
-                hazard = (fl & kDecHazard) != 0;
-                if (stays && (hazard ? p.chunk == p.n_chunks - 1 : p.chunk == 0))
-                    act = true;
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, act);
-            if (act) {
-                const DecReq q = s_raw[rq0 + r];
-                SReq sr;
-                sr.src = q.blob;
-                sr.wb = nullptr;
-                sr.gate_row = r;
-                sr.deferred = 0;
-                if (pull) {
-                    // Where a call is made in several launches (more than 8 tokens): the first one stores
-                    // the expert into its slot and the later ones read it there, unless the slot still
-                    // holds an expert the call computes with: then every launch reads the host store and
-                    // the last one stores it once all CTAs are done.
-                    if (stays && !hazard && p.chunk > 0) {
-                        sr.src = q.blob;
-                    } else {
-                        sr.src = q.host;
-                        if (q.host == nullptr)
-                            s_abort = 2;
-                        if (stays && !hazard)
-                            sr.wb = const_cast<char *>(q.blob);
-                        if (stays && hazard && p.chunk == p.n_chunks - 1)
-                            sr.deferred = 1;
-                    }
+    if (!p.fast) {
+        // gate of every (request, token): the token's gate for that expert if the router chose it
+        for (int i = tid; i < nrq * kTokPerVr; i += kThreads) {
+            const int r = i / kTokPerVr, t = i % kTokPerVr;
+            const int e = tab.raw[rq0 + r].expert;
+            if (t == 0 && e >= 0 && e < kMaxReq)
+                tab.of_expert[e] = r;
+            float gv = 0.0f;
+            if (t < Tc) {
+                if (e >= p.E) {
+                    gv = 1.0f;              // shared expert: every token, gate 1
+                    atomicOr(&tab.match[r], 1u << t);
+                } else {
+                    for (int j = 0; j < p.k; ++j)
+                        if (tab.idx[t * p.k + j] == e) {
+                            gv = tab.gw[t * p.k + j];
+                            atomicOr(&tab.match[r], 1u << t);
+                        }
                 }
-                s_req[base + __popc(m & ((1u << lane) - 1u))] = sr;
             }
-            base += __popc(m);
+            tab.gate[r][t] = gv;
         }
-        if (lane == 0)
-            s_nact = base;
+        __syncthreads();
+        // The requests that have a token in this launch, in ascending expert id (shared experts last): the
+        // rows are dealt out in that order, so the order of every sum depends only on which experts the
+        // tokens use, not on which of them happened to be resident.
+        if (warp == 0) {
+            int base = 0;
+            for (int e0 = 0; e0 < kMaxReq; e0 += 32) {
+                const int e = e0 + lane;
+                const int r = e < kMaxReq ? tab.of_expert[e] : -1;
+                // a fetched expert that stays resident is streamed (and stored into its slot) by the launch whose
+                // job that is even if none of this launch's tokens uses it
+                bool act = r >= 0 && tab.match[r] != 0u;
+                bool pull = false, stays = false, hazard = false;
+                if (r >= 0 && p.group < 0 && (tab.raw[rq0 + r].flags & kDecMiss)) {
+                    const int fl = tab.raw[rq0 + r].flags;
+                    pull = true;
+                    stays = (fl & kDecStays) != 0 && p.write_back != 0;
+                    hazard = (fl & kDecHazard) != 0;
+                    if (stays && (hazard ? p.chunk == p.n_chunks - 1 : p.chunk == 0))
+                        act = true;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, act);
+                if (act) {
+                    const DecReq q = tab.raw[rq0 + r];
+                    FastReq sr;
+                    sr.src = q.blob;
+                    sr.wb = sr.deferred = nullptr;
+                    sr.expert = e;
+#pragma unroll
+                    for (int t = 0; t < kTokPerVr; ++t)
+                        sr.gate[t] = tab.gate[r][t];
+                    if (pull) {
+                        // Where a call is made in several launches (more than 8 tokens): the first one stores
+                        // the expert into its slot and the later ones read it there, unless the slot still
+                        // holds an expert the call computes with: then every launch reads the host store and
+                        // the last one stores it once all CTAs are done.
+                        if (stays && !hazard && p.chunk > 0) {
+                            sr.src = q.blob;
+                        } else {
+                            sr.src = q.host;
+                            if (q.host == nullptr)
+                                s_abort = 2;
+                            if (stays && !hazard)
+                                sr.wb = const_cast<char *>(q.blob);
+                            if (stays && hazard && p.chunk == p.n_chunks - 1) {
+                                sr.deferred = const_cast<char *>(q.blob);
+                                s_deferred = 1;
+                            }
+                        }
+                    }
+                    s_req[base + __popc(m & ((1u << lane) - 1u))] = sr;
+                }
+                base += __popc(m);
+            }
+            if (lane == 0)
+                s_nact = base;
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the ring's first copies come over these tables
+    } else if (tid < nrq && s_req[tid].src == nullptr) {
+        s_abort = 2;
     }
     __syncthreads();
     const int nact = s_nact;
@@ -710,31 +735,37 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
         trace[1] = globaltimer_ns();
 
     // ---- this CTA's share of the rows: f rows of the active requests, request-major, dealt out evenly
-    const long long rows = no_host ? 0 : (long long)nact * F;
-    const long long q_lo = blockIdx.x * rows / G, q_hi = (blockIdx.x + 1) * rows / G;
+    const int rows = no_host ? 0 : nact * F;
+    const int q_lo = (int)((long long)blockIdx.x * rows / G), q_hi = (int)((long long)(blockIdx.x + 1) * rows / G);
 
     if (warp == NW) {
         // =================================================================== producer
         if (lane == 0) {
-            uint32_t n = 0;
-            long long q = q_lo;
-            int a = (int)(q / F), f0 = (int)(q % F);
-            while (q < q_hi) {
-                const int m = (int)min((long long)min(TR, F - f0), q_hi - q);
-                const uint32_t st = n % (uint32_t)S;
-                if (n >= (uint32_t)S && !mbar_wait(empty0 + 8 * st, ((n / S) - 1u) & 1u, abort_flag))
+            uint32_t n = 0, st = 0, ph = 1;         // copies issued; ring stage of the next one, parity of its being free
+            int left = q_hi - q_lo, a = q_lo / F, f0 = q_lo % F;
+            while (left > 0) {
+                const int m = min(min(TR, F - f0), left);
+                if (n >= (uint32_t)S && !mbar_wait(empty0 + 8 * st, ph, abort_flag))
                     break;
                 const uint32_t bytes = (uint32_t)m * RB;
                 mbar_expect(full0 + 8 * st, bytes);
                 bulk_g2s(ring_s + st * STAGE, s_req[a].src + (size_t)f0 * RB, bytes, full0 + 8 * st);
                 ++n;
-                q += m;
+                if (++st == (uint32_t)S) {
+                    st = 0;
+                    ph ^= 1u;
+                }
+                left -= m;
                 f0 += m;
                 if (f0 == F) {
                     f0 = 0;
                     ++a;
                 }
             }
+            // this grid does not end before the planner's has: the kernel behind it reads the cache state that the planner
+            // writes after its announcement (one waiting thread is enough, and here it costs nothing)
+            if (blockIdx.x == 0)
+                asm volatile("griddepcontrol.wait;" ::: "memory");
             if (*abort_flag) {
                 // a wait ran out: give the copies still in flight a bounded time to land before this
                 // CTA's shared memory goes away
@@ -748,7 +779,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
         // =================================================================== consumers
         const int g = lane >> 2, tig = lane & 3;
         if constexpr (FMT == 1) {
-            consume_q4<MT_>(p, geo, s_req, &s_gate[0][0], s_sums, buf, ring_s, xs_s, full0, empty0, abort_flag, q_lo, q_hi, trace);
+            consume_q4<MT_>(p, geo, s_req, s_sums, buf, ring_s, xs_s, full0, empty0, abort_flag, q_lo, q_hi, trace);
         } else {
         float acc[kMaxMt][4];
 #pragma unroll
@@ -776,22 +807,18 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
         // (W_u rows, k high); down: four consecutive 8-column pieces of the W_d^T rows
         const int r8 = lane & 7, sel_gu = (lane >> 3) & 1, kh = lane >> 4, mat = lane >> 3;
         const uint32_t src0 = (uint32_t)((2 * tig) * 4 + (g >> 1)), src1 = src0 + 4;
-        uint32_t n = 0;
-        long long q = q_lo;
-        int a = (int)(q / F), f0 = (int)(q % F);
-        bool first = true;
-        while (q < q_hi) {
-            const int m = (int)min((long long)min(TR, F - f0), q_hi - q);
-            const uint32_t st = n % (uint32_t)S;
+        uint32_t st = 0, ph = 0;                    // ring stage of the tile and the parity of its barrier phase
+        int left = q_hi - q_lo, a = q_lo / F, f0 = q_lo % F;
+        while (left > 0) {
+            const int m = min(min(TR, F - f0), left);
             const uint32_t stage = ring_s + st * STAGE;
-            mbar_wait(full0 + 8 * st, (n / S) & 1u, abort_flag);
-            if (trace && first && tid == 0)
-                trace[2] = globaltimer_ns();
-            first = false;
-            const SReq rq = s_req[a];
-            const bool store_tile = rq.wb != nullptr && tid == 0;
+            mbar_wait(full0 + 8 * st, ph, abort_flag);
+            if (p.trace && tid == 0 && left == q_hi - q_lo)
+                p.trace[(size_t)blockIdx.x * 8 + 2] = globaltimer_ns();
+            char *wb = s_req[a].wb;
+            const bool store_tile = wb != nullptr && tid == 0;
             if (store_tile)
-                bulk_s2g(rq.wb + (size_t)f0 * RB, stage, (uint32_t)m * RB);
+                bulk_s2g(wb + (size_t)f0 * RB, stage, (uint32_t)m * RB);
             const int rr = r8 < m ? r8 : 0;               // rows the tile does not have read row 0 (never used)
             const uint32_t swz = (uint32_t)((f0 + rr) & 7);
             const uint32_t rowbase = stage + rr * RB;
@@ -854,7 +881,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
             asm volatile("bar.sync 1, %0;" ::"n"(NW * 32) : "memory");
             const float s0 = s_sums[lane], s1 = s_sums[32 + lane], s2 = s_sums[64 + lane], s3 = s_sums[96 + lane];
             // rows g and g + 8 of the tile are g_f and u_f of f = f0 + g, columns are tokens 2 tig, 2 tig + 1
-            const float gt0 = s_gate[rq.gate_row][2 * tig], gt1 = s_gate[rq.gate_row][2 * tig + 1];
+            const float gt0 = s_req[a].gate[2 * tig], gt1 = s_req[a].gate[2 * tig + 1];
             // (the fast division: the exact one takes its slow path for the zeros of unused token columns)
             float h0 = __fdividef(s0, 1.0f + __expf(-s0)) * s2 * gt0;
             float h1 = __fdividef(s1, 1.0f + __expf(-s1)) * s3 * gt1;
@@ -909,8 +936,11 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(empty0 + 8 * st);
-            ++n;
-            q += m;
+            if (++st == (uint32_t)S) {
+                st = 0;
+                ph ^= 1u;
+            }
+            left -= m;
             f0 += m;
             if (f0 == F) {
                 f0 = 0;
@@ -945,92 +975,103 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
             }
         }
         }
+        // ---- count this warp out; the last CTA's warp turns the sums of its columns into the output
+        __syncwarp();
+        unsigned ticket = 0;
+        if (lane == 0) {
+            // (the warp barrier orders the other lanes' adds before lane 0's fence, which is cumulative)
+            __threadfence();
+            ticket = atomicAdd(p.sync + warp, 1u);
+        }
+        ticket = __shfl_sync(0xffffffffu, ticket, 0);
+        if (trace && tid == 0)
+            trace[4] = globaltimer_ns();
+        if (ticket == (unsigned)(G - 1)) {
+            if (lane == 0)
+                p.sync[warp] = 0u;                // the counter is back at zero for the next launch
+            __threadfence();
+            if (trace)
+                trace[5] = globaltimer_ns();
+            const bool acc_in = p.group > 0, acc_out = p.group >= 0 && p.group < n_groups - 1;
+            // The warp's columns: `own` contiguous ones, except that the 4-bit path's column steps of 32, where a warp has only
+            // one of them, are 16 columns in each half of a block of 64.  Sixteen elements per lane at a time, all their
+            // loads before any store: this warp is the whole grid's critical path, and a load behind a store that may
+            // alias it would wait for it.
+            constexpr int kSteps = MT_ > 0 ? MT_ / 2 : 8, kToks = 16 / kSteps;
+            const int own = MT * 16;
+            const bool halves = FMT == 1 && MT == 2;
+            const int c0 = halves ? (warp >> 1) * 64 + 16 * (warp & 1) + (lane & 15) + 32 * (lane >> 4) : warp * own + lane;
+            for (int t0 = 0; t0 < Tc; t0 += kToks) {
+                long long fx[16];
+                float carry[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int t = t0 + j / kSteps, i = j % kSteps * 32;
+                    const bool on = t < Tc && (MT_ > 0 || i + lane < own);
+                    fx[j] = on ? __ldcg(p.yacc + t * d + c0 + i) : 0ll;
+                    carry[j] = acc_in && on ? __ldcg(p.ybuf + (size_t)(tok0 + t) * d + c0 + i) : 0.0f;
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int t = t0 + j / kSteps, i = j % kSteps * 32;
+                    if (t < Tc && (MT_ > 0 || i + lane < own)) {
+                        p.yacc[t * d + c0 + i] = 0;              // the accumulator is left clean for the next launch
+                        float v = __ll2float_rn(fx[j]) * (1.0f / 1099511627776.0f);     // one rounding, then an exact scaling
+                        const size_t o = (size_t)(tok0 + t) * d + c0 + i;
+                        if (acc_in)
+                            v += carry[j];
+                        if (acc_out)
+                            p.ybuf[o] = v;
+                        else
+                            p.out[o] = (uint16_t)bf16_rne(v);
+                    }
+                }
+            }
+            if (trace)
+                trace[6] = globaltimer_ns();
+        }
         if (tid == 0)
             bulk_wait_all();              // the slot stores of this thread have completed
     }
 
-    // ---- the CTA that finishes last turns the sums into the output; all others are done
-    if (XT)
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    if (*abort_flag && lane == 0)
+        atomicExch(p.err, no_host ? MELINOE_ERR_STATE : MELINOE_ERR_TIMEOUT);
     if (XT) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (warp == 0)
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(128));
     }
+    if (trace && tid == 0)
+        trace[7] = globaltimer_ns();
+    if (!s_deferred)
+        return;
+
+    // ---- fetched experts whose slot was still being computed with: stored by the last CTA, once every CTA is done
+    __syncthreads();
     if (tid == 0) {
         __threadfence();
-        const unsigned ticket = atomicAdd(p.sync, 1u);
-        s_last = ticket == (unsigned)(G - 1);
+        s_last = atomicAdd(p.sync + NW, 1u) == (unsigned)(G - 1);
         if (s_last)
-            *p.sync = 0u;                 // the counter is back at zero for the next launch
-        if (trace)
-            trace[4] = globaltimer_ns();
+            p.sync[NW] = 0u;
     }
     __syncthreads();
-    if (*abort_flag && tid == 0)
-        atomicExch(p.err, no_host ? MELINOE_ERR_STATE : MELINOE_ERR_TIMEOUT);
-    if (!s_last) {
-        if (trace && tid == 0)
-            trace[7] = globaltimer_ns();
-        return;
-    }
-    __threadfence();
-    if (trace && tid == 0)
-        trace[5] = globaltimer_ns();
-    {
-        const bool acc_in = p.group > 0, acc_out = p.group >= 0 && p.group < n_groups - 1;
-        long long *yacc = p.yacc;
-        const int N = Tc * d;
-        // four elements per thread at a time, all their loads before any store: this CTA is the whole
-        // grid's critical path, and a load behind a store that may alias it would wait for it
-        constexpr int kBatch = 4;
-        for (int e0 = tid; e0 < N; e0 += kBatch * kThreads) {
-            long long fx[kBatch];
-            float carry[kBatch];
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) {
-                const int e = e0 + j * kThreads;
-                fx[j] = e < N ? __ldcg(yacc + e) : 0ll;
-                carry[j] = (acc_in && e < N) ? __ldcg(p.ybuf + (size_t)tok0 * d + e) : 0.0f;
-            }
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) {
-                const int e = e0 + j * kThreads;
-                if (e < N) {
-                    yacc[e] = 0;                                 // the accumulator is left clean for the next launch
-                    float v = __ll2float_rn(fx[j]) * (1.0f / 1099511627776.0f);     // one rounding, then an exact scaling
-                    const size_t o = (size_t)tok0 * d + e;       // element e of the launch's [tokens][d] block
-                    if (acc_in)
-                        v += carry[j];
-                    if (acc_out)
-                        p.ybuf[o] = v;
-                    else
-                        p.out[o] = (uint16_t)bf16_rne(v);
-                }
-            }
-        }
-    }
-    if (trace && tid == 0)
-        trace[6] = globaltimer_ns();
-
-    // ---- fetched experts whose slot was still being computed with: stored now that every CTA is done
-    if (tid == 0) {
+    if (s_last && tid == 0) {
         uint32_t phase = 0;
         bool any = false;
-        __syncwarp();
         for (int a = 0; a < nact && *abort_flag != 1; ++a) {
-            if (!s_req[a].deferred)
+            char *slot = s_req[a].deferred;
+            if (slot == nullptr)
                 continue;
-            const SReq rq = s_req[a];
-            char *slot = const_cast<char *>(s_raw[rq0 + rq.gate_row].blob);
+            const char *src = s_req[a].src;
             for (int f = 0; f < F; f += TR) {
                 const uint32_t bytes = (uint32_t)min(TR, F - f) * RB;
                 if (any)
                     bulk_wait_read();
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 mbar_expect(hzbar, bytes);
-                bulk_g2s(ring_s, rq.src + (size_t)f * RB, bytes, hzbar);
+                bulk_g2s(ring_s, src + (size_t)f * RB, bytes, hzbar);
                 if (!mbar_wait(hzbar, phase & 1u, abort_flag))
                     break;
                 ++phase;
@@ -1043,8 +1084,6 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(DecParams p, De
         if (*abort_flag == 1)
             atomicExch(p.err, MELINOE_ERR_TIMEOUT);
     }
-    if (trace && tid == 0)
-        trace[7] = globaltimer_ns();
 }
 
 }  // namespace
@@ -1078,7 +1117,10 @@ cudaError_t ffn_decode_configure(int n_sms, size_t max_smem, DecLaunchCfg *cfg)
         if (e != cudaSuccess)
             return e;
     }
-    cfg->grid = n_sms < 255 ? n_sms : 255;   // one CTA per SM (the accumulator words count CTAs in one byte)
+    // One CTA per SM, but for the SM where the planner is still finishing its records when it announces the plan: a CTA
+    // there would enter microseconds after the others and end as much later.  (The other SMs of the planner's cluster
+    // are free by then, and one SM less does not slow the stream.)
+    cfg->grid = n_sms > 1 ? n_sms - 1 : 1;
     cfg->max_smem = usable;
     cfg->pdl = pdl_enabled();
     return cudaSuccess;

@@ -39,6 +39,7 @@ struct PlanParams {
     HostPlan *hplan;          // page-locked host memory (device-visible address)
     uint32_t gmax;            // compute groups the caller has room for
     uint32_t call_seq;        // written to the miss queue's seq word when the record is complete
+    int fast;                 // fused planner: the call is served by one decode launch that fetches the missed experts itself
     int policy;               // MELINOE_POLICY_LRU or MELINOE_POLICY_COUNT
     float gamma;              // decay of the count policy
     melinoe_moe_stats *stats; // may be null
@@ -69,7 +70,7 @@ cudaError_t launch_plan(cudaStream_t stream, const PlanParams &p);
 // ---- router and planning in one kernel (one thread-block cluster), for calls of at most 8 tokens
 bool route_plan_small_supported(int T, int k, int d);
 cudaError_t launch_route_plan_small(cudaStream_t stream, const uint16_t *x, const uint16_t *w_r, const float *bias,
-                                    const int32_t *token_seq, int d, int32_t *idx, float *gate, float *logits_out,
+                                    const int32_t *token_seq, int n_seq, int d, int32_t *idx, float *gate, float *logits_out,
                                     const PlanParams &p);
 
 // ---- decode expert FFN (Eq. 3) with the gate-weighted combine (Eq. 2) fused in, for up to 8 tokens per launch
@@ -81,8 +82,8 @@ struct DecParams {
     long long *yacc;                 // [8][d] output accumulator words of the launch; all zero between launches
     float *ybuf;                     // [T][d] fp32: sum over the earlier launches of the same tokens (group mode)
     uint16_t *out;                   // [T][d] bf16
-    unsigned *sync;                  // the handle's counter for the rare launches whose CTAs have to know who is last (zero between launches)
-    uint32_t call_seq;               // the call's sequence number: the plan is ready when plan->ready_seq equals it
+    unsigned *sync;                  // counters: of every consumer warp's columns, and of the launch (all zero between launches)
+    uint32_t call_seq;               // the call's sequence number: the plan is ready when the low half of plan->ready equals it
     int *err;                        // device error word (0 = ok)
     unsigned long long *trace;       // null, or 8 clock stamps per CTA of the most recent launch
     int d, F, E, k, T, n_shared;
@@ -93,6 +94,7 @@ struct DecParams {
     int wait_prior;                  // the kernel ahead in the stream is another launch of the same call (it uses the
                                      // same accumulator): wait for that grid to finish before anything else
     int fmt;                         // 0: bf16 blobs, 1: 4-bit blobs
+    int fast;                        // the launch's requests are plan->fast (planned by the fused planner for this launch)
 };
 struct DecLaunchCfg {
     int grid;                        // one CTA per SM

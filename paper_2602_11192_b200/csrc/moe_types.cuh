@@ -58,20 +58,39 @@ constexpr int kDecMiss = 1;      // not resident at call entry: the weights come
 constexpr int kDecStays = 2;     // a miss that still occupies its slot when the call ends: written into the slot
 constexpr int kDecHazard = 4;    // ... whose slot held, at call entry, an expert that this call also computes with
 
+// A request of a decode call as its one FFN launch takes it: in ascending expert id (shared experts last), which is
+// the order of every sum.  64 bytes, read by four threads at once.
+struct __align__(64) FastReq {
+    const char *src;             // where its rows are streamed from: the slot, a shared expert's blob, or the host store
+    char *wb;                    // null, or the slot the fetched rows are also stored into
+    char *deferred;              // null, or the slot they are stored into once every CTA is done (the call still computes with
+                                 // what the slot holds)
+    int32_t expert, reserved;
+    float gate[kTokPerVr];       // its gate for every token of the call; 0 = not routed to it
+};
+// What the word that announces a plan says beside the call's sequence number (low half): requests of the decode
+// launch, status, whether one of them is deferred.
+__host__ __device__ inline uint64_t ready_word(uint32_t seq, int n_fast, int status, bool deferred)
+{
+    return (uint64_t)seq | ((uint64_t)(uint32_t)(n_fast | status << 8 | (deferred ? 1 << 16 : 0)) << 32);
+}
+
 // Per-call plan written by the planning kernel, read by the FFN and combine kernels.
 struct DevPlan {
     int32_t n_tokens, n_req, n_hits, n_miss, n_evict, n_groups, n_dreq, status;
-    // Sequence number of the call whose plan this is, written last (after a device-wide fence) by the
-    // planning kernel: the decode FFN kernel, which may have been scheduled while the planner was still
-    // running, waits for it instead of waiting for the planner's grid to drain.
-    uint32_t ready_seq;
-    uint32_t pad_[3];
+    // Announces the plan: ready_word(), written behind a device-wide fence by the planning kernel.  The decode FFN
+    // kernel, which may have been scheduled while the planner was still running, waits for it instead of waiting for the
+    // planner's grid to drain.  A decode call whose FFN launch fetches the missed experts itself needs fast[] alone: it is
+    // announced as soon as that is complete, the rest of the plan follows (before the planner's grid ends).
+    uint64_t ready;
+    uint32_t pad_[2];
     int32_t group_vr_begin[kMaxGroups + 1];   // first entry of dreq[] of every compute group
     int32_t counts[kMaxReq];
     int32_t offsets[kMaxReq + 1];
     int32_t req_of_expert[kMaxReq];        // -1 = expert not requested by this call
     ReqRec req[kMaxReq];
     DecReq dreq[kMaxReq];                     // group 0 (hits, then shared experts), then the misses by wave
+    FastReq fast[kMaxReq];
 };
 
 // The miss queue of a call: what the host needs in order to issue the transfers, written by

@@ -449,12 +449,12 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
             *reinterpret_cast<melinoe_moe_trace_header *>(p.trace_rec) = th;
         }
     }
-    // the plan is complete: announce it (see DevPlan::ready_seq)
+    // the plan is complete: announce it (see DevPlan::ready)
     __threadfence();
     __syncthreads();
     if (tid == 0) {
         __threadfence();
-        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&plan->ready_seq), "r"(p.call_seq) : "memory");
+        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&plan->ready), "l"(ready_word(p.call_seq, 0, 0, false)) : "memory");
     }
 }
 

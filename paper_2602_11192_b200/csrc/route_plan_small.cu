@@ -4,17 +4,22 @@
 //
 // At this size every step is latency, not throughput, so the kernel is organised to take as
 // few dependent memory round trips as possible:
-//   - logits: one warp per expert, spread over a thread-block cluster of 8 CTAs x 8 warps (a single
-//     SM pulling the whole router matrix takes ~9 us; eight take ~2); each lane has all its loads in
-//     flight at once, the router row already before the kernel ahead in the stream has finished;
+//   - before the kernel ahead in the stream has finished (programmatic launch): the router row of every warp is loaded,
+//     and what that kernel may still write (hidden states, bias, token sequences) is asked into L2;
+//   - logits: one warp per expert (and token group, where there are fewer experts than warps), spread over a
+//     thread-block cluster of 8 CTAs x 8 warps (a single SM pulling the whole router matrix takes ~9 us; eight take
+//     ~2); two tokens at a time, the next two already on their way;
 //   - the logits go straight into the shared memory of the cluster's first CTA and the cluster
 //     barrier tells it when they are all there: no fence, no device counter, no second launch;
 //   - top-k is a rank count (an element's rank is the number of elements that beat it) shared by
-//     the eight warps, instead of k rounds of a warp-wide maximum; the gates are computed by the
-//     other warps while the first one plans;
+//     the eight warps, instead of k rounds of a warp-wide maximum; which experts the call needs is a ballot over
+//     the ranks, so that planning does not wait for the selection to be sorted;
 //   - planning is written for one warp with lane = expert / slot / request: ranks come from
 //     ballots and population counts, prefix sums from shuffles, and the LRU victims of a call are
-//     taken from one sorted list instead of one search per miss.
+//     taken from one sorted list instead of one search per miss; the gates are computed beside it;
+//   - a call whose FFN launch fetches the missed experts itself is announced as soon as that launch's
+//     records (where every needed expert's weights are, its gates) are complete; the cache's stamps, the token lists,
+//     the inspection records and the statistics follow while the FFN kernel already streams.
 //
 // The results are exactly those of the general router and planning kernels.  The logit sum uses
 // the same fixed order (element j belongs to lane (j mod 256) / 8, lanes add their elements in
@@ -40,9 +45,11 @@ constexpr int kThreads = kWarpsPerBlock * 32;
 constexpr int kCluster = kMaxExperts / kWarpsPerBlock;   // 8 CTAs: a warp for each of up to 64 experts
 constexpr int kMaxT = kTokPerVr;                 // 8 tokens
 constexpr int kMaxPairs = kMaxExperts;           // T * k <= 64 is required by the launcher
+constexpr int kChunks = 8;                       // pieces of 256 columns loaded ahead of their arithmetic
 
 __device__ __forceinline__ float bf16lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ int warp_excl_scan(int v, int lane, int &total)
 {
@@ -74,9 +81,11 @@ __device__ __forceinline__ void write_req(ReqRec *r, int expert, int slot, int h
         *reinterpret_cast<int4 *>(trace_req) = make_int4(expert, slot, hit, evicted);
 }
 
+// NH: d_model is at most NH * 2048
+template <int NH>
 __global__ void __launch_bounds__(kThreads, 1)
 route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ w_r,
-                        const float *__restrict__ bias, const int32_t *__restrict__ token_seq, int d,
+                        const float *__restrict__ bias, const int32_t *__restrict__ token_seq, int n_seq, int d,
                         int32_t *__restrict__ idx_out, float *__restrict__ gate_out, float *logits_out,
                         PlanParams p)
 {
@@ -94,10 +103,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     __shared__ unsigned long long s_key[kMaxExperts];            // victim-order key of a slot
     __shared__ int32_t s_victim[kMaxExperts];                    // V: slots in victim order
     __shared__ int32_t s_miss_expert[kMaxExperts];               // expert of miss number i
-    __shared__ int32_t s_needflags[2][kMaxExperts];              // per planning warp: 1 = some pair of the call names this expert
     __shared__ HostMiss s_hm[kMaxExperts];                       // the call's miss queue, sent to the host last
-    __shared__ int32_t s_miss_slot[kMaxExperts];                 // count policy: its slot and wave
-    __shared__ int32_t s_miss_group[kMaxExperts];
     __shared__ int32_t s_entry_occ[kMaxExperts];                 // occupant of a slot at call entry
     __shared__ float s_sel[kMaxT][kMaxExperts];                  // a token's selected logits, by rank
 
@@ -107,17 +113,34 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     unsigned cta_rank;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(cta_rank));
 
-    // ================================================================ logits: one warp per expert
-    const int e_mine = (int)cta_rank * kWarpsPerBlock + warp;
+    // ================================================================ logits: one warp per (expert, token group)
+    const int n_tg = min(T, kMaxExperts / E);           // token groups
+    const int gw = (int)cta_rank * kWarpsPerBlock + warp, tg = gw / E, e_mine = tg < n_tg ? gw % E : E;
     const int n_chunks = d >> 8;
-    // The router matrix does not change while calls are queued, so the first eight pieces of the
-    // row go out before anything else.
-    uint4 wv0[8];
+    const uint4 *wrow = reinterpret_cast<const uint4 *>(w_r + (size_t)e_mine * d) + lane;
+    // The router matrix does not change while calls are queued, so the row goes out before anything else.
+    uint4 wv[NH][kChunks];
     if (e_mine < E) {
-        const uint4 *wrow = reinterpret_cast<const uint4 *>(w_r + (size_t)e_mine * d) + lane;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            wv0[i] = i < n_chunks ? __ldg(wrow + i * 32) : make_uint4(0, 0, 0, 0);
+        for (int h = 0; h < NH; ++h)
+#pragma unroll
+            for (int i = 0; i < kChunks; ++i)
+                if (h * kChunks + i < n_chunks)
+                    wv[h][i] = __ldg(wrow + (h * kChunks + i) * 32);
+    }
+    DevCache *cache = p.cache;
+    {
+        // into L2, whatever of it is not there yet: a line per thread
+        const int i = (int)cta_rank * kThreads + tid, x_lines = T * d / 64;
+        const int j = i - x_lines;
+        if (i < x_lines)
+            prefetch_l2(x + (size_t)i * 64);
+        else if (j < 12)
+            prefetch_l2(reinterpret_cast<const char *>(cache) + min(j * 128, (int)sizeof(DevCache) - 4));
+        else if (bias && j < 12 + 64 && (j - 12) * 32 < n_seq * E)
+            prefetch_l2(bias + (j - 12) * 32);
+        else if (token_seq && j == 12 + 64)
+            prefetch_l2(token_seq);
     }
     // The launch may have been made with programmatic stream serialisation: this block can then be
     // running before the kernel ahead of it in the stream has finished.  Nothing before this point
@@ -125,21 +148,102 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     // launch).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // lane t holds token t's bias (two dependent loads, in flight under the dot products)
-    float my_bias = 0.0f;
-    if (e_mine < E && bias && lane < T) {
-        const int q = token_seq ? token_seq[lane] : 0;
-        my_bias = bias[(size_t)q * E + e_mine];
+    const bool by_count = p.policy == MELINOE_POLICY_COUNT;
+    if (e_mine < E) {
+        // tokens tg, tg + n_tg, ..: two at a time (a and b), in batches of up to 2048 columns, the next batch on its way
+        const int mine = (T - tg + n_tg - 1) / n_tg;
+        const int n_half = NH == 1 ? 1 : (n_chunks + kChunks - 1) / kChunks, n_batch = (mine + 1) / 2 * n_half;
+        uint4 xv[2][2][kChunks];
+        auto load = [&](int batch, uint4 (&v)[2][kChunks]) {
+            const int pr = batch / n_half, h = batch % n_half;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int t = tg + (2 * pr + u) * n_tg;
+                const uint4 *xrow = reinterpret_cast<const uint4 *>(x + (size_t)t * d) + lane + h * kChunks * 32;
+#pragma unroll
+                for (int i = 0; i < kChunks; ++i)
+                    if (t < T && h * kChunks + i < n_chunks)
+                        v[u][i] = __ldcg(xrow + i * 32);
+            }
+        };
+        load(0, xv[0]);
+        // lane i holds the bias of the warp's token i.  Where there are no more sequences than lanes, every lane loads one
+        // sequence's bias beside the tokens' sequences, instead of one load behind the other.
+        float my_bias = 0.0f;
+        if (bias) {
+            const int q = token_seq && lane < mine ? token_seq[tg + lane * n_tg] : 0;
+            if (n_seq <= 32) {
+                const float of_seq = lane < n_seq ? bias[(size_t)lane * E + e_mine] : 0.0f;
+                my_bias = __shfl_sync(0xffffffffu, of_seq, q & 31);
+            } else if (lane < mine) {
+                my_bias = bias[(size_t)q * E + e_mine];
+            }
+        }
+        float a = 0.0f, b = 0.0f, my_logit = 0.0f;
+        auto compute = [&](int batch, const uint4 (&v)[2][kChunks]) {
+            const int pr = batch / n_half, h = batch % n_half;
+            auto dot = [&](const uint4 (&w)[kChunks]) {
+#pragma unroll
+                for (int i = 0; i < kChunks; ++i) {
+                    if (h * kChunks + i < n_chunks) {
+                        auto piece = [&](uint32_t xa, uint32_t xb, uint32_t ww) {
+                            a = __fmaf_rn(bf16lo(xa), bf16lo(ww), a);
+                            b = __fmaf_rn(bf16lo(xb), bf16lo(ww), b);
+                            a = __fmaf_rn(bf16hi(xa), bf16hi(ww), a);
+                            b = __fmaf_rn(bf16hi(xb), bf16hi(ww), b);
+                        };
+                        piece(v[0][i].x, v[1][i].x, w[i].x);
+                        piece(v[0][i].y, v[1][i].y, w[i].y);
+                        piece(v[0][i].z, v[1][i].z, w[i].z);
+                        piece(v[0][i].w, v[1][i].w, w[i].w);
+                    }
+                }
+            };
+            if (NH == 1 || h == 0)
+                dot(wv[0]);
+            else
+                dot(wv[NH - 1]);
+            if (h == n_half - 1) {
+#pragma unroll
+                for (int m = 16; m >= 1; m >>= 1) {
+                    a = __fadd_rn(a, __shfl_xor_sync(0xffffffffu, a, m));
+                    b = __fadd_rn(b, __shfl_xor_sync(0xffffffffu, b, m));
+                }
+                if (lane == 2 * pr)
+                    my_logit = a;
+                if (lane == 2 * pr + 1)
+                    my_logit = b;
+                a = b = 0.0f;
+            }
+        };
+#pragma unroll 1
+        for (int batch = 0; batch < n_batch; batch += 2) {
+            if (batch + 1 < n_batch)
+                load(batch + 1, xv[1]);
+            compute(batch, xv[0]);
+            if (batch + 2 < n_batch)
+                load(batch + 2, xv[0]);
+            if (batch + 1 < n_batch)
+                compute(batch + 1, xv[1]);
+        }
+        if (lane < mine) {
+            if (bias)
+                my_logit = __fadd_rn(my_logit, my_bias);
+            // into the first CTA's shared memory, and to global memory for the inspection calls
+            const int t = tg + lane * n_tg;
+            uint32_t remote;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                         : "=r"(remote)
+                         : "r"((uint32_t)__cvta_generic_to_shared(&s_logit[t][e_mine])), "r"(0));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(my_logit) : "memory");
+            logits_out[(size_t)t * E + e_mine] = my_logit;
+        }
     }
-
-    // the planner's view of the cache: its loads overlap the logits
-    DevCache *cache = p.cache;
+    // the planner's view of the cache: its loads overlap the cluster barrier
     int soe0 = -1, soe1 = -1, eos0 = -1, eos1 = -1;
     unsigned long long st0 = 0ull, st1 = 0ull, counter = 0ull, call_no = 0ull;
     float cnt0 = 0.0f, cnt1 = 0.0f;
-    const bool by_count = p.policy == MELINOE_POLICY_COUNT;
-    if (cta_rank == 0 && warp == 1) {
-        // the gather warp only needs to know which experts are resident
+    if (cta_rank == 0 && warp <= 1) {
         if (lane < E)
             soe0 = cache->slot_of_expert[lane];
         if (lane + 32 < E)
@@ -152,10 +256,6 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             if (lane + 32 < E)
                 cnt1 = cache->count[lane + 32];
         }
-        if (lane < E)
-            soe0 = cache->slot_of_expert[lane];
-        if (lane + 32 < E)
-            soe1 = cache->slot_of_expert[lane + 32];
         if (lane < C) {
             eos0 = cache->expert_of_slot[lane];
             st0 = cache->stamp[lane];
@@ -166,59 +266,6 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         }
         counter = cache->counter;
         call_no = cache->call_no + 1ull;
-    }
-    if (e_mine < E) {
-        const uint4 *wrow = reinterpret_cast<const uint4 *>(w_r + (size_t)e_mine * d) + lane;
-        float my_logit = 0.0f;
-        for (int t = 0; t < T; ++t) {
-            const uint4 *xrow = reinterpret_cast<const uint4 *>(x + (size_t)t * d) + lane;
-            float a = 0.0f;
-            for (int c0 = 0; c0 < n_chunks; c0 += 8) {
-                // all of a lane's loads for these 8 pieces go out before any arithmetic
-                uint4 wv[8], xv[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const bool on = c0 + i < n_chunks;
-                    xv[i] = on ? __ldcg(xrow + (c0 + i) * 32) : make_uint4(0, 0, 0, 0);
-                }
-                if (c0 == 0) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        wv[i] = wv0[i];
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        wv[i] = c0 + i < n_chunks ? __ldg(wrow + (c0 + i) * 32) : make_uint4(0, 0, 0, 0);
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    if (c0 + i < n_chunks) {
-                        a = __fmaf_rn(bf16lo(xv[i].x), bf16lo(wv[i].x), a);
-                        a = __fmaf_rn(bf16hi(xv[i].x), bf16hi(wv[i].x), a);
-                        a = __fmaf_rn(bf16lo(xv[i].y), bf16lo(wv[i].y), a);
-                        a = __fmaf_rn(bf16hi(xv[i].y), bf16hi(wv[i].y), a);
-                        a = __fmaf_rn(bf16lo(xv[i].z), bf16lo(wv[i].z), a);
-                        a = __fmaf_rn(bf16hi(xv[i].z), bf16hi(wv[i].z), a);
-                        a = __fmaf_rn(bf16lo(xv[i].w), bf16lo(wv[i].w), a);
-                        a = __fmaf_rn(bf16hi(xv[i].w), bf16hi(wv[i].w), a);
-                    }
-                }
-            }
-#pragma unroll
-            for (int m = 16; m >= 1; m >>= 1)
-                a = __fadd_rn(a, __shfl_xor_sync(0xffffffffu, a, m));
-            if (lane == t)
-                my_logit = bias ? __fadd_rn(a, my_bias) : a;
-        }
-        if (lane < T) {
-            // into the first CTA's shared memory, and to global memory for the inspection calls
-            uint32_t remote;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-                         : "=r"(remote)
-                         : "r"((uint32_t)__cvta_generic_to_shared(&s_logit[lane][e_mine])), "r"(0));
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(my_logit) : "memory");
-            logits_out[(size_t)lane * E + e_mine] = my_logit;
-        }
     }
     // ---- the cluster's first CTA carries on when every logit has arrived
     if (cta_rank == 0)
@@ -232,10 +279,9 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     // ================================================================ top-k
     // An element's rank is the number of elements that beat it (greater, or equal with a lower
     // index).  The eight warps share the count (warp w compares against elements 8w .. 8w + 7 of
-    // every token) and add their parts up in shared memory; then warp t writes token t's selection.
-    // Only the indices are on the way to the planner: the gates are left to the other warps.
-    {
-        const float NEG = -__int_as_float(0x7f800000);  // -inf
+    // every token) and add their parts up in shared memory.
+    const float NEG = -__int_as_float(0x7f800000);  // -inf
+    if (8 * warp < E)
         for (int t = 0; t < T; ++t) {
             const float v0 = lane < E ? s_logit[t][lane] : NEG;
             const float v1 = lane + 32 < E ? s_logit[t][lane + 32] : NEG;
@@ -258,64 +304,72 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             if (r1)
                 atomicAdd(&s_rank[t][lane + 32], r1);
         }
-        __syncthreads();
-        if (warp < T) {
-            const int t = warp;
-            const int r0 = s_rank[t][lane], r1 = s_rank[t][lane + 32];
-            if (lane < E && r0 < k) {
-                s_sel[t][r0] = s_logit[t][lane];
-                s_idx[t * k + r0] = lane;
+    __syncthreads();
+
+    // lane owns experts lane and lane + 32, slots lane and lane + 32, pairs lane and lane + 32
+    DevPlan *plan = p.plan;
+    const int e0 = lane, e1 = lane + 32;
+    // which experts the call's tokens selected
+    uint64_t need = 0;
+    for (int t = 0; t < T; ++t)
+        need |= ballot64(e0 < E && s_rank[t][e0] < k, e1 < E && s_rank[t][e1] < k);
+
+    if (warp >= 1) {
+        // ============================================================ selection and gates (Eq. 1), beside the planner
+        for (int t = warp - 1; t < T; t += kWarpsPerBlock - 1) {
+            const int r0 = s_rank[t][e0], r1 = s_rank[t][e1];
+            const float v0 = s_logit[t][e0], v1 = s_logit[t][e1];
+            const bool on0 = e0 < E && r0 < k, on1 = e1 < E && r1 < k;
+            if (on0) {
+                s_sel[t][r0] = v0;
+                s_idx[t * k + r0] = e0;
             }
-            if (lane + 32 < E && r1 < k) {
-                s_sel[t][r1] = s_logit[t][lane + 32];
-                s_idx[t * k + r1] = lane + 32;
+            if (on1) {
+                s_sel[t][r1] = v1;
+                s_idx[t * k + r1] = e1;
             }
-        }
-        __syncthreads();
-    }
-    if (warp >= 2) {
-        // ============================================================ gates (Eq. 1), off the planner's path
-        for (int t = warp - 2; t < T; t += kWarpsPerBlock - 2) {
+            __syncwarp();
             const float top = s_sel[t][0];
             const float ev = lane < k ? expf(s_sel[t][lane] - top) : 0.0f;
             float sum = ev;
 #pragma unroll
             for (int m = 16; m >= 1; m >>= 1)
                 sum += __shfl_xor_sync(0xffffffffu, sum, m);
+            if (p.fast) {
+                // the gates of every needed expert for this token, at the expert's place in the launch's order
+                if ((need >> e0) & 1ull)
+                    plan->fast[rank_below(need, e0)].gate[t] = on0 ? expf(v0 - top) / sum : 0.0f;
+                if ((need >> e1) & 1ull)
+                    plan->fast[rank_below(need, e1)].gate[t] = on1 ? expf(v1 - top) / sum : 0.0f;
+            }
             if (lane < k) {
+                const float gv = ev / sum;
                 idx_out[(size_t)t * k + lane] = s_idx[t * k + lane];
-                gate_out[(size_t)t * k + lane] = ev / sum;
+                gate_out[(size_t)t * k + lane] = gv;
                 if (p.trace_rec && t < p.trace_max_tokens) {
                     const TraceLayout tl = trace_layout(E, k, p.trace_max_tokens);
                     reinterpret_cast<int32_t *>(p.trace_rec + tl.idx_off)[t * k + lane] = s_idx[t * k + lane];
-                    reinterpret_cast<float *>(p.trace_rec + tl.gate_off)[t * k + lane] = ev / sum;
+                    reinterpret_cast<float *>(p.trace_rec + tl.gate_off)[t * k + lane] = gv;
                 }
             }
         }
+        if (p.fast && warp == kWarpsPerBlock - 1)
+            for (int i = lane; i < p.n_shared * kMaxT; i += 32)
+                plan->fast[__popcll(need) + i / kMaxT].gate[i % kMaxT] = i % kMaxT < T ? 1.0f : 0.0f;
         // these warps' results are written before the planning warp announces the plan
         asm volatile("bar.arrive 2, %0;" ::"n"(kThreads) : "memory");
-        return;
+        if (warp != 1) {
+            asm volatile("bar.arrive 3, %0;" ::"n"(kThreads - 32) : "memory");
+            return;
+        }
+        asm volatile("bar.sync 3, %0;" ::"n"(kThreads - 32) : "memory");      // every token's selection is in s_idx
     }
 
     // ================================================================ planning, by two warps side by side
-    // Warp 1 builds the token lists (what the gather and the inspection calls need), warp 0 the cache
-    // requests (what the compute kernel waits for).  Both know which experts are needed and which of
-    // those are resident, so both can tell a request's place in the call's request order.
-    // lane owns experts lane and lane + 32, slots lane and lane + 32, pairs lane and lane + 32
-    // (the cache state of this lane's experts and slots was loaded before the logits)
-    DevPlan *plan = p.plan;
-    const int e0 = lane, e1 = lane + 32;
-    // which experts the call's pairs name
-    int32_t *s_needflag = s_needflags[warp];
-    s_needflag[lane] = 0;
-    s_needflag[lane + 32] = 0;
-    __syncwarp();
-    if (lane < n_pairs)
-        s_needflag[s_idx[lane]] = 1;
-    if (lane + 32 < n_pairs)
-        s_needflag[s_idx[lane + 32]] = 1;
-    __syncwarp();
-    const uint64_t need = ballot64(s_needflag[lane] != 0, s_needflag[lane + 32] != 0);
+    // Warp 0 makes the cache requests (what the compute kernel waits for), warp 1 the token lists (what the gather and the
+    // inspection calls need).  Both know which experts are needed and which of those are resident, so both can tell a
+    // request's place in the call's request order.
+    // (the cache state of this lane's experts and slots was loaded before the logits arrived)
     const uint64_t resident = ballot64(soe0 >= 0, soe1 >= 0);
     const uint64_t hit_mask = need & resident, miss_mask = need & ~resident;
     const int n_hits = __popcll(hit_mask), n_miss = __popcll(miss_mask), n_req = n_hits + n_miss;
@@ -381,7 +435,9 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
                 plan->counts[E + lane] = T;
             plan->offsets[E + lane] = n_pairs + lane * T;
         }
-        asm volatile("bar.arrive 2, %0;" ::"n"(kThreads) : "memory");
+        // a call computed group by group reads these lists' records: they are part of what is announced
+        if (!p.fast)
+            asm volatile("bar.arrive 4, 64;" ::: "memory");
         return;
     }
 
@@ -394,6 +450,38 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     const int ndr = n_req + p.n_shared;             // records for the compute kernels: hits, shared experts, misses
     const int status = n_groups > (int)p.gmax ? MELINOE_ERR_STATE : MELINOE_OK;
     const bool ok = status == MELINOE_OK;
+    // what the hits' and the shared experts' FFN work needs
+    auto slot_ptr = [&](int slot) { return const_cast<char *>(p.slots) + (size_t)slot * p.slot_stride; };
+    auto write_fast = [&](int at, int e, const char *src, char *wb, char *deferred) {
+        FastReq *f = &plan->fast[at];
+        *reinterpret_cast<ulonglong2 *>(&f->src) = make_ulonglong2((unsigned long long)src, (unsigned long long)wb);
+        *reinterpret_cast<ulonglong2 *>(&f->deferred) = make_ulonglong2((unsigned long long)deferred, (unsigned long long)(unsigned)e);
+    };
+    if (p.fast) {
+        if ((hit_mask >> e0) & 1ull)
+            write_fast(rank_below(need, e0), e0, slot_ptr(soe0), nullptr, nullptr);
+        if ((hit_mask >> e1) & 1ull)
+            write_fast(rank_below(need, e1), e1, slot_ptr(soe1), nullptr, nullptr);
+        for (int s = lane; s < p.n_shared; s += 32)
+            write_fast(n_req + s, E + s, p.shared_blobs[s], nullptr, nullptr);
+    }
+    bool deferred = false;
+    // The plan is announced.  The decode FFN kernel behind this one in the stream may already be running (programmatic
+    // launch) and waits for this word, not for this grid to drain.
+    // (The barrier orders the other warps' and lanes' writes before lane 0's release, which is cumulative:
+    // whoever acquires the word sees them all.)
+    auto announce = [&] {
+        asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+        const bool any = __any_sync(0xffffffffu, deferred);
+        if (lane == 0)
+            asm volatile("st.release.gpu.global.u64 [%0], %1;"
+                         ::"l"(&plan->ready), "l"(ready_word(p.call_seq, p.fast && ok ? ndr : 0, status, any))
+                         : "memory");
+    };
+    const bool early = p.fast && n_miss == 0;
+    if (early)
+        announce();
+
     if (by_count) {
         // Definition C.1: one time step per call, count <- gamma * count + request
         const float n0 = __fadd_rn(__fmul_rn(p.gamma, cnt0), req0 ? 1.0f : 0.0f);
@@ -418,12 +506,8 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         const int e = h ? e1 : e0, soe = h ? soe1 : soe0;
         if ((hit_mask >> e) & 1ull) {
             const int r = rank_below(hit_mask, e);
-            const unsigned long long st = counter + (unsigned long long)r + 1ull;
-            s_key[soe] = (1ull << 63) | st;
-            cache->stamp[soe] = st;
-            write_req(&plan->req[r], e, soe, 1, -1, r, 0, tr_req ? tr_req + 16 * r : nullptr);
+            s_key[soe] = (1ull << 63) | (counter + (unsigned long long)r + 1ull);
             s_grp_of[e] = 0;
-            plan->dreq[r] = DecReq{p.slots + (size_t)soe * p.slot_stride, nullptr, e, 0, 0, 0};
         }
         if ((miss_mask >> e) & 1ull)
             s_miss_expert[rank_below(miss_mask, e)] = e;
@@ -445,6 +529,19 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     __syncwarp();
     bool ev_flag[2] = {false, false};
     int n_evict_seq = 0;
+    // where a miss's work goes: stays = it still occupies its slot when the call ends; storing it there must wait for the
+    // end of the call's compute if the slot held one of the call's experts at entry
+    auto miss_records = [&](int i, int e, int slot, int group, bool stays) {
+        const int occ = s_entry_occ[slot];
+        const bool hazard = stays && occ >= 0 && ((need >> occ) & 1ull);
+        const char *host = p.host_blobs ? p.host_blobs[e] : nullptr;
+        plan->dreq[n_hits + p.n_shared + i] =
+            DecReq{slot_ptr(slot), host, e, kDecMiss | (stays ? kDecStays : 0) | (hazard ? kDecHazard : 0), group, 0};
+        if (p.fast) {
+            write_fast(rank_below(need, e), e, host, stays && !hazard ? slot_ptr(slot) : nullptr, hazard ? slot_ptr(slot) : nullptr);
+            deferred |= hazard;
+        }
+    };
     if (by_count) {
         // The count policy has no closed form (a victim depends on the counts of what the earlier
         // misses of the call brought in): one search per miss, in ascending expert id, over a live
@@ -513,29 +610,44 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
                 s_live_stamp[slot] = st;
                 s_grp_of[e] = cur_group;
                 write_req(&plan->req[n_hits + i], e, slot, 0, ev, vr_at, cur_group, tr_req ? tr_req + 16 * (n_hits + i) : nullptr);
-                s_miss_expert[i] = e;
-                s_miss_slot[i] = slot;
-                s_miss_group[i] = cur_group;
                 s_hm[i] = HostMiss{e, slot, (int16_t)cur_group, (int16_t)dep, p.call_seq};
             }
             __syncwarp();
         }
         n_groups = n_miss ? cur_group + 1 : 1;
-        // a miss stays if it still occupies its slot when the call ends; writing it there must wait
-        // for the end of the call's compute if the slot held one of the call's hits at entry
-        for (int j = lane; j < n_miss; j += 32) {
-            const int e = s_miss_expert[j], slot = s_miss_slot[j], occ = s_entry_occ[slot];
-            const bool stays = s_live_occ[slot] == e;
-            const bool hazard = stays && occ >= 0 && ((need >> occ) & 1ull);
-            plan->dreq[n_hits + p.n_shared + j] =
-                DecReq{p.slots + (size_t)slot * p.slot_stride, p.host_blobs ? p.host_blobs[e] : nullptr, e,
-                       kDecMiss | (stays ? kDecStays : 0) | (hazard ? kDecHazard : 0), s_miss_group[j], 0};
+        for (int j = lane; j < n_miss; j += 32)
+            miss_records(j, s_hm[j].expert, s_hm[j].slot, s_hm[j].group, s_live_occ[s_hm[j].slot] == s_hm[j].expert);
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int e = h ? e1 : e0;
+            if ((miss_mask >> e) & 1ull) {
+                const int i = rank_below(miss_mask, e);
+                miss_records(i, e, s_victim[i % C], 1 + i / C, i + C >= n_miss);
+            }
         }
-    } else
+    }
+    if (p.fast && !early)
+        announce();
+
+    // ---- the hits' records and stamps; under LRU, the misses' records and what they change in the cache
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int e = h ? e1 : e0, soe = h ? soe1 : soe0;
+        if ((hit_mask >> e) & 1ull) {
+            const int r = rank_below(hit_mask, e);
+            if (!by_count || n_miss == 0 || s_live_occ[soe] == e)      // (the count policy's misses may have taken the slot)
+                cache->stamp[soe] = counter + (unsigned long long)r + 1ull;
+            write_req(&plan->req[r], e, soe, 1, -1, r, 0, tr_req ? tr_req + 16 * r : nullptr);
+            plan->dreq[r] = DecReq{slot_ptr(soe), nullptr, e, 0, 0, 0};
+        }
+    }
+    // (a slot that held a hit at entry may be a miss's now: its stamp is the miss's)
+    __syncwarp();
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int e = h ? e1 : e0;
-        if ((miss_mask >> e) & 1ull) {
+        if (((miss_mask >> e) & 1ull) && !by_count) {
             const int i = rank_below(miss_mask, e);
             const int slot = s_victim[i % C];
             const int ev = i < C ? s_entry_occ[slot] : s_miss_expert[i - C];
@@ -546,16 +658,9 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             else if (ev >= 0 && ((need >> ev) & 1ull))
                 dep = 0;
             ev_flag[h] = ev >= 0;
-            const int vr_at = n_hits + p.n_shared + i;
-            write_req(&plan->req[n_hits + i], e, slot, 0, ev, vr_at, group, tr_req ? tr_req + 16 * (n_hits + i) : nullptr);
+            write_req(&plan->req[n_hits + i], e, slot, 0, ev, n_hits + p.n_shared + i, group, tr_req ? tr_req + 16 * (n_hits + i) : nullptr);
             // cache update: the last miss that lands in a slot keeps it
             const bool stays = i + C >= n_miss;
-            {
-                const int occ = s_entry_occ[slot];
-                const bool hazard = stays && occ >= 0 && ((need >> occ) & 1ull);
-                plan->dreq[vr_at] = DecReq{p.slots + (size_t)slot * p.slot_stride, p.host_blobs ? p.host_blobs[e] : nullptr, e,
-                                           kDecMiss | (stays ? kDecStays : 0) | (hazard ? kDecHazard : 0), group, 0};
-            }
             cache->slot_of_expert[e] = stays ? slot : -1;
             if (stays) {
                 cache->expert_of_slot[slot] = e;
@@ -597,18 +702,17 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         cache->tot_evictions += (unsigned long long)n_evict;
         cache->call_no = call_no;
     }
-    // The plan is complete: announce it.  The decode FFN kernel behind this one in the stream may
-    // already be running (programmatic launch) and waits for this word, not for this grid to drain.
-    // (The barrier orders the other warps' and lanes' writes before lane 0's release, which is cumulative:
-    // whoever acquires the word sees them all.)
-    asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
-    if (lane == 0)
-        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&plan->ready_seq), "r"(p.call_seq) : "memory");
+    // a call computed group by group: the plan is complete now, with the token lists' records
+    if (!p.fast) {
+        asm volatile("bar.sync 4, 64;" ::: "memory");
+        announce();
+    }
     // What may live in host memory goes out last, so that no fence above has to wait for the host link:
     // the statistics, and the miss queue for calls whose transfers the host issues.
-    for (int i = lane; i < n_miss; i += 32)
-        store16_host(&p.hplan->miss[i], &s_hm[i]);
     __syncwarp();
+    if (!p.fast)
+        for (int i = lane; i < n_miss; i += 32)
+            store16_host(&p.hplan->miss[i], &s_hm[i]);
     if (lane == 0) {
         if (p.stats) {
             melinoe_moe_stats st;
@@ -624,8 +728,10 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             st.call_no = call_no;
             *p.stats = st;
         }
-        const HostPlanHeader hdr{n_miss, n_groups, status, p.call_seq};
-        store16_host(&p.hplan->hdr, &hdr);
+        if (!p.fast) {
+            const HostPlanHeader hdr{n_miss, n_groups, status, p.call_seq};
+            store16_host(&p.hplan->hdr, &hdr);
+        }
         if (p.trace_rec) {
             melinoe_moe_trace_header th;
             th.call_no = call_no;
@@ -649,7 +755,7 @@ bool route_plan_small_supported(int T, int k, int d)
 }
 
 cudaError_t launch_route_plan_small(cudaStream_t stream, const uint16_t *x, const uint16_t *w_r, const float *bias,
-                                    const int32_t *token_seq, int d, int32_t *idx, float *gate, float *logits_out,
+                                    const int32_t *token_seq, int n_seq, int d, int32_t *idx, float *gate, float *logits_out,
                                     const PlanParams &p)
 {
     // one cluster of 8 CTAs; programmatic stream serialisation: the blocks may be scheduled while the
@@ -669,7 +775,8 @@ cudaError_t launch_route_plan_small(cudaStream_t stream, const uint16_t *x, cons
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl_enabled() ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, route_plan_small_kernel, x, w_r, bias, token_seq, d, idx, gate, logits_out, p);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, d <= 256 * kChunks ? route_plan_small_kernel<1> : route_plan_small_kernel<2>, x, w_r, bias, token_seq,
+                                             n_seq, d, idx, gate, logits_out, p);
     count_launch();
     return e;
 }

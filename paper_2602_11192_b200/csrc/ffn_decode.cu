@@ -220,6 +220,11 @@ __device__ __forceinline__ void red_add_u64(unsigned long long *addr, unsigned l
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
+template <int N>
+struct Count {
+    static constexpr int value = N;
+};
+
 constexpr int NW = 16;                           // consumer warps
 constexpr int kThreads = (NW + 1) * 32;          // + the producer warp
 constexpr int kBufPitch = 130;                   // floats between the warps' partial tiles (keeps the column sums conflict-free)
@@ -634,7 +639,6 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
         // the counters advance once per CTA and launch, whatever happens
         if (tid < NW && atomicAdd(p.sync + tid, 1u) == (unsigned)(G - 1))
             p.sync[tid] = 0u;
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }
     if (XT) {
@@ -762,10 +766,6 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
                     ++a;
                 }
             }
-            // this grid does not end before the planner's has: the kernel behind it reads the cache state that the planner
-            // writes after its announcement (one waiting thread is enough, and here it costs nothing)
-            if (blockIdx.x == 0)
-                asm volatile("griddepcontrol.wait;" ::: "memory");
             if (*abort_flag) {
                 // a wait ran out: give the copies still in flight a bounded time to land before this
                 // CTA's shared memory goes away
@@ -994,27 +994,29 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
                 trace[5] = globaltimer_ns();
             const bool acc_in = p.group > 0, acc_out = p.group >= 0 && p.group < n_groups - 1;
             // The warp's columns: `own` contiguous ones, except that the 4-bit path's column steps of 32, where a warp has only
-            // one of them, are 16 columns in each half of a block of 64.  Sixteen elements per lane at a time, all their
-            // loads before any store: this warp is the whole grid's critical path, and a load behind a store that may
-            // alias it would wait for it.
-            constexpr int kSteps = MT_ > 0 ? MT_ / 2 : 8, kToks = 16 / kSteps;
+            // one of them, are 16 columns in each half of a block of 64.  All loads of some tokens before any store: this
+            // warp is the whole grid's critical path, and a load behind a store that may alias it would wait for it.
+            // For the same reason a launch of one token has a form of its own: what four predicated tokens take in
+            // instructions was 1.5 us per launch.
+            constexpr int kSteps = MT_ > 0 ? MT_ / 2 : 8;
             const int own = MT * 16;
             const bool halves = FMT == 1 && MT == 2;
             const int c0 = halves ? (warp >> 1) * 64 + 16 * (warp & 1) + (lane & 15) + 32 * (lane >> 4) : warp * own + lane;
-            for (int t0 = 0; t0 < Tc; t0 += kToks) {
-                long long fx[16];
-                float carry[16];
+            auto convert = [&](auto n_toks, int t0) {
+                constexpr int kToks = decltype(n_toks)::value;
+                long long fx[kToks * kSteps];
+                float carry[kToks * kSteps];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
+                for (int j = 0; j < kToks * kSteps; ++j) {
                     const int t = t0 + j / kSteps, i = j % kSteps * 32;
-                    const bool on = t < Tc && (MT_ > 0 || i + lane < own);
+                    const bool on = (kToks == 1 || t < Tc) && (MT_ > 0 || i + lane < own);
                     fx[j] = on ? __ldcg(p.yacc + t * d + c0 + i) : 0ll;
                     carry[j] = acc_in && on ? __ldcg(p.ybuf + (size_t)(tok0 + t) * d + c0 + i) : 0.0f;
                 }
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
+                for (int j = 0; j < kToks * kSteps; ++j) {
                     const int t = t0 + j / kSteps, i = j % kSteps * 32;
-                    if (t < Tc && (MT_ > 0 || i + lane < own)) {
+                    if ((kToks == 1 || t < Tc) && (MT_ > 0 || i + lane < own)) {
                         p.yacc[t * d + c0 + i] = 0;              // the accumulator is left clean for the next launch
                         float v = __ll2float_rn(fx[j]) * (1.0f / 1099511627776.0f);     // one rounding, then an exact scaling
                         const size_t o = (size_t)(tok0 + t) * d + c0 + i;
@@ -1026,6 +1028,14 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
                             p.out[o] = (uint16_t)bf16_rne(v);
                     }
                 }
+            };
+            if (Tc == 1) {
+                convert(Count<1>(), 0);
+            } else {
+                constexpr int kToks = 16 / kSteps;
+#pragma unroll 1
+                for (int t0 = 0; t0 < Tc; t0 += kToks)
+                    convert(Count<kToks>(), t0);
             }
             if (trace)
                 trace[6] = globaltimer_ns();

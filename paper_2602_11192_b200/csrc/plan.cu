@@ -49,7 +49,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
     const int E = p.E, C = p.C;
 
     // ---- load persistent cache state, clear tables.  The router, which may still be running (programmatic launch), lets
-    // this kernel start only once everything ahead of it, the previous call's planning included, is complete.
+    // this kernel start only once everything ahead of it is complete.
+    wait_for_previous_planning(p);
     {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(p.cache);
         uint32_t *dst = reinterpret_cast<uint32_t *>(&s_cache);
@@ -455,6 +456,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
     if (tid == 0) {
         __threadfence();
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&plan->ready), "l"(ready_word(p.call_seq, 0, 0, false)) : "memory");
+        planning_complete(p);
     }
 }
 

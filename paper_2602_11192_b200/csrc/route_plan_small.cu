@@ -244,6 +244,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     unsigned long long st0 = 0ull, st1 = 0ull, counter = 0ull, call_no = 0ull;
     float cnt0 = 0.0f, cnt1 = 0.0f;
     if (cta_rank == 0 && warp <= 1) {
+        wait_for_previous_planning(p);
         if (lane < E)
             soe0 = cache->slot_of_expert[lane];
         if (lane + 32 < E)
@@ -435,9 +436,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
                 plan->counts[E + lane] = T;
             plan->offsets[E + lane] = n_pairs + lane * T;
         }
-        // a call computed group by group reads these lists' records: they are part of what is announced
-        if (!p.fast)
-            asm volatile("bar.arrive 4, 64;" ::: "memory");
+        asm volatile("bar.arrive 4, 64;" ::: "memory");
         return;
     }
 
@@ -702,11 +701,12 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         cache->tot_evictions += (unsigned long long)n_evict;
         cache->call_no = call_no;
     }
-    // a call computed group by group: the plan is complete now, with the token lists' records
-    if (!p.fast) {
-        asm volatile("bar.sync 4, 64;" ::: "memory");
+    // the planning is complete now, with the token lists' records; a call computed group by group is announced
+    asm volatile("bar.sync 4, 64;" ::: "memory");
+    if (!p.fast)
         announce();
-    }
+    if (lane == 0)
+        planning_complete(p);
     // What may live in host memory goes out last, so that no fence above has to wait for the host link:
     // the statistics, and the miss queue for calls whose transfers the host issues.
     __syncwarp();

@@ -4,8 +4,7 @@
 //
 // At this size every step is latency, not throughput, so the kernel is organised to take as
 // few dependent memory round trips as possible:
-//   - before the kernel ahead in the stream has finished (programmatic launch): the router row of every warp is loaded,
-//     and what that kernel may still write (hidden states, bias, token sequences) is asked into L2;
+//   - before the kernel ahead in the stream has finished (programmatic launch): the router row of every warp is loaded;
 //   - logits: one warp per expert (and token group, where there are fewer experts than warps), spread over a
 //     thread-block cluster of 8 CTAs x 8 warps (a single SM pulling the whole router matrix takes ~9 us; eight take
 //     ~2); two tokens at a time, the next two already on their way;
@@ -49,6 +48,13 @@ constexpr int kChunks = 8;                       // pieces of 256 columns loaded
 
 __device__ __forceinline__ float bf16lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+// A load that stays where it is written (the dot products run twice, and only the second pass may use what is loaded).
+__device__ __forceinline__ uint32_t ld_now(const void *p)
+{
+    uint32_t v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ int warp_excl_scan(int v, int lane, int &total)
@@ -129,26 +135,24 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
                     wv[h][i] = __ldg(wrow + (h * kChunks + i) * 32);
     }
     DevCache *cache = p.cache;
-    {
-        // into L2, whatever of it is not there yet: a line per thread
-        const int i = (int)cta_rank * kThreads + tid, x_lines = T * d / 64;
-        const int j = i - x_lines;
-        if (i < x_lines)
-            prefetch_l2(x + (size_t)i * 64);
-        else if (j < 12)
-            prefetch_l2(reinterpret_cast<const char *>(cache) + min(j * 128, (int)sizeof(DevCache) - 4));
-        else if (bias && j < 12 + 64 && (j - 12) * 32 < n_seq * E)
-            prefetch_l2(bias + (j - 12) * 32);
-        else if (token_seq && j == 12 + 64)
-            prefetch_l2(token_seq);
-    }
+    if (cta_rank == 0 && tid < 12)       // into L2, whatever of it is not there yet
+        prefetch_l2(reinterpret_cast<const char *>(cache) + min(tid * 128, (int)sizeof(DevCache) - 4));
+    // (long past when this kernel waits for the call before to end)
+    if (cta_rank == 0 && warp <= 1)
+        wait_for_previous_planning(p);
     // The launch may have been made with programmatic stream serialisation: this block can then be
     // running before the kernel ahead of it in the stream has finished.  Nothing before this point
     // reads what that kernel may have written; wait for it here (returns at once in an ordinary
     // launch).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const bool by_count = p.policy == MELINOE_POLICY_COUNT;
+    // The dot products run twice: first on whatever the hidden states' memory holds, while the kernel ahead ends, so that
+    // the pass that counts finds its instructions in the caches (2.3 -> 1.5 us for one token of d_model 2048; the
+    // same for the planning below, or for the FFN kernel while it waits, costs registers and gains nothing).
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 1)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
     if (e_mine < E) {
         // tokens tg, tg + n_tg, ..: two at a time (a and b), in batches of up to 2048 columns, the next batch on its way
         const int mine = (T - tg + n_tg - 1) / n_tg;
@@ -163,7 +167,9 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
 #pragma unroll
                 for (int i = 0; i < kChunks; ++i)
                     if (t < T && h * kChunks + i < n_chunks)
-                        v[u][i] = __ldcg(xrow + i * 32);
+                        asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];"
+                                     : "=r"(v[u][i].x), "=r"(v[u][i].y), "=r"(v[u][i].z), "=r"(v[u][i].w)
+                                     : "l"(xrow + i * 32));
             }
         };
         load(0, xv[0]);
@@ -171,12 +177,12 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         // sequence's bias beside the tokens' sequences, instead of one load behind the other.
         float my_bias = 0.0f;
         if (bias) {
-            const int q = token_seq && lane < mine ? token_seq[tg + lane * n_tg] : 0;
+            const int q = token_seq && lane < mine ? (int)ld_now(token_seq + tg + lane * n_tg) : 0;
             if (n_seq <= 32) {
-                const float of_seq = lane < n_seq ? bias[(size_t)lane * E + e_mine] : 0.0f;
+                const float of_seq = lane < n_seq ? __uint_as_float(ld_now(bias + (size_t)lane * E + e_mine)) : 0.0f;
                 my_bias = __shfl_sync(0xffffffffu, of_seq, q & 31);
             } else if (lane < mine) {
-                my_bias = bias[(size_t)q * E + e_mine];
+                my_bias = __uint_as_float(ld_now(bias + (size_t)q * E + e_mine));
             }
         }
         float a = 0.0f, b = 0.0f, my_logit = 0.0f;
@@ -226,7 +232,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             if (batch + 1 < n_batch)
                 compute(batch + 1, xv[1]);
         }
-        if (lane < mine) {
+        if (pass == 1 && lane < mine) {
             if (bias)
                 my_logit = __fadd_rn(my_logit, my_bias);
             // into the first CTA's shared memory, and to global memory for the inspection calls
@@ -239,12 +245,12 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             logits_out[(size_t)t * E + e_mine] = my_logit;
         }
     }
+    }
     // the planner's view of the cache: its loads overlap the cluster barrier
     int soe0 = -1, soe1 = -1, eos0 = -1, eos1 = -1;
     unsigned long long st0 = 0ull, st1 = 0ull, counter = 0ull, call_no = 0ull;
     float cnt0 = 0.0f, cnt1 = 0.0f;
     if (cta_rank == 0 && warp <= 1) {
-        wait_for_previous_planning(p);
         if (lane < E)
             soe0 = cache->slot_of_expert[lane];
         if (lane + 32 < E)

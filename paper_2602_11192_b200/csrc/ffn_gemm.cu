@@ -29,7 +29,7 @@
 //             d_ff is out of bounds there and reads as zero, so d_ff may end inside a stage.
 // The slots' experts are addressed through one tensor map per view, because the slots are contiguous.
 //
-// 4-bit slots (template parameter FMT = 1): TMA brings the codes into a ring of its own, and four warps expand
+// 4-bit slots (template parameter FMT = 1): TMA brings the codes into a ring of its own, and eight warps expand
 // them into the weight tile of a stage (the arithmetic of the decode kernel: 15 instructions per 8
 // weights) in front of the tensor cores, so that HBM carries 4-bit data only and no bf16 copy of an expert
 // exists.  In GEMM 1 the expansion leaves elements j and j + 4 of eight side by side; a sum over K does not
@@ -37,10 +37,10 @@
 //
 // One persistent CTA per SM, warp-specialised: warp 0 issues TMA loads into a ring of stages, warp 1
 // issues the MMAs (one elected thread) and commits them to mbarriers, warps 2..5 drain
-// the accumulator (tcgen05.ld, 32 rows per warp) and write the tile; with 4-bit slots warps 6..9 expand and
-// warp 10 fetches codes.  Two accumulators alternate so the epilogue of a tile overlaps the MMAs of the next.
+// the accumulator (tcgen05.ld, 32 rows per warp) and write the tile; with 4-bit slots warps 6..13 expand and
+// warp 14 fetches codes.  Two accumulators alternate so the epilogue of a tile overlaps the MMAs of the next.
 // Work items are (request, weight tile, token chunk) triples of the launch's compute group, dealt
-// round-robin, the chunks of one weight tile side by side.
+// round-robin to CTA pairs, and cut into equal runs of k-blocks for single CTAs (GemmWalk, GemmSplit).
 //
 // Ragged N: a chunk's box may run past its expert's last row; those columns are computed on whatever
 // the next rows hold (or zeros past the end of the buffer) and never stored.
@@ -75,12 +75,12 @@ constexpr int kRawBytes = 16384;           // 4-bit slots: codes of one fetch (G
 constexpr int kRawStages = 3;
 constexpr size_t kGemmSmem = 227 * 1024 - 4096;      // dynamic shared memory of a CTA (the static part is below 3 KB)
 // threads, tokens of a chunk at most, bytes and number of ring stages for CG CTAs per operation and slot format FMT
-__host__ __device__ constexpr int gemm_threads(int fmt) { return fmt ? 352 : 192; }
-__host__ __device__ constexpr int gemm_tokens(int cg) { return cg == 2 ? 256 : 128; }
-__host__ __device__ constexpr int gemm_stage_bytes(int cg) { return kABytes + gemm_tokens(cg) / cg * kBK * 2; }
+__host__ __device__ constexpr int gemm_threads(int fmt) { return fmt ? 480 : 192; }
+__host__ __device__ constexpr int gemm_tokens(int cg, int fmt) { return cg == 2 || fmt ? 256 : 128; }
+__host__ __device__ constexpr int gemm_stage_bytes(int cg, int fmt) { return kABytes + gemm_tokens(cg, fmt) / cg * kBK * 2; }
 __host__ __device__ constexpr int gemm_stages(int cg, int fmt)
 {
-    return (int)((kGemmSmem - 1024 - (fmt ? kRawStages * kRawBytes : 0)) / gemm_stage_bytes(cg));
+    return (int)((kGemmSmem - 1024 - (fmt ? kRawStages * kRawBytes : 0)) / gemm_stage_bytes(cg, fmt));
 }
 constexpr long long kGemmWaitCycles = 4000000000ll;
 
@@ -275,6 +275,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
         : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&r)[32])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+        ::"r"(taddr), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "f"(r[8]), "f"(r[9]),
+          "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15]), "f"(r[16]), "f"(r[17]), "f"(r[18]), "f"(r[19]),
+          "f"(r[20]), "f"(r[21]), "f"(r[22]), "f"(r[23]), "f"(r[24]), "f"(r[25]), "f"(r[26]), "f"(r[27]), "f"(r[28]), "f"(r[29]),
+          "f"(r[30]), "f"(r[31])
+        : "memory");
+}
+
 __device__ __forceinline__ uint32_t bf16_rne(float v)
 {
     uint32_t u = __float_as_uint(v);
@@ -287,6 +300,16 @@ __device__ __forceinline__ void expand8(uint32_t w, uint32_t ss, uint32_t (&P)[4
 {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
+        uint32_t t = ((w >> (4 * j)) & 0x000f000fu) | 0x43004300u;
+        asm("sub.rn.bf16x2 %0, %0, %1;" : "+r"(t) : "r"(0x43084308u));
+        asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(P[j]) : "r"(t), "r"(ss));
+    }
+}
+// The first two of the four registers: elements (0, 4) and (1, 5) of the word.
+__device__ __forceinline__ void expand4(uint32_t w, uint32_t ss, uint32_t (&P)[2])
+{
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
         uint32_t t = ((w >> (4 * j)) & 0x000f000fu) | 0x43004300u;
         asm("sub.rn.bf16x2 %0, %0, %1;" : "+r"(t) : "r"(0x43084308u));
         asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(P[j]) : "r"(t), "r"(ss));
@@ -309,19 +332,18 @@ struct GemmItem {
     int n_live;    // tokens that exist
     int m0;        // first hidden unit (GEMM 1) or output column (GEMM 2) of this CTA's weight tile
     int slot;      // cache slot of the expert, or -1 - index of the shared expert
+    int k0, k1;    // k-blocks of this piece of the tile
 };
 
-// The items of one CTA, or CTA pair, in order: every n_ctas-th, the chunks of one weight tile adjacent, so that CTAs
-// working side by side share it in L2.  (Dealing the weights out evenly instead, every CTA one run of them with short
-// tiles at its ends, measured slower although it leaves no last round nearly empty: 57 instead of 43 us for GEMM 1 of
-// 1024 pairs, d 2048, d_ff 1024.  A short tile's k-blocks take as long as a whole one's.)
-template <int CG, int NT, int kMTile>
+// The items of one CTA pair, in order: every n_ctas-th, the chunks of one weight tile adjacent, so that pairs
+// working side by side share it in L2.
+template <int NT, int kMTile>
 struct GemmWalk {
     const int4 *rec;         // first row, tokens, slot (shared expert s: -1 - s), tokens of a chunk
     const int *item0;        // first item of every request
-    int q, w, step, total, rank;
-    __device__ GemmWalk(const int4 *rec_, const int *item0_, int n_reqs, int unit, int n_ctas, int rank_)
-        : rec(rec_), item0(item0_), q(0), w(unit), step(n_ctas), total(item0_[n_reqs]), rank(rank_)
+    int q, w, step, total, rank, kblocks;
+    __device__ GemmWalk(const int4 *rec_, const int *item0_, const int *, int n_reqs, int unit, int n_ctas, int rank_, int kblocks_)
+        : rec(rec_), item0(item0_), q(0), w(unit), step(n_ctas), total(item0_[n_reqs]), rank(rank_), kblocks(kblocks_)
     {
     }
     __device__ bool next(GemmItem &it)
@@ -332,14 +354,127 @@ struct GemmWalk {
             ++q;
         const int4 r = rec[q];
         const int local = w - item0[q], n = (r.y + NT - 1) / NT, c = local % n;
-        it.m0 = (local / n * CG + rank) * kMTile;
+        it.m0 = (local / n * 2 + rank) * kMTile;
         it.row0 = r.x + c * r.w;
         it.n_live = min(r.w, r.y - c * r.w);
-        it.n = (it.n_live + 16 * CG - 1) / (16 * CG) * (16 * CG);
+        it.n = (it.n_live + 31) / 32 * 32;
         it.slot = r.z;
+        it.k0 = 0;
+        it.k1 = kblocks;
         w += step;
         return true;
     }
+};
+
+// The pieces of one single CTA.  With few tokens per expert there are few rounds of tiles (or less than one), and the last
+// round would leave most of the chip idle; so the tiles are laid end to end, each as long as its k-blocks (in quads
+// of 4, the unit in which 4-bit codes are fetched) times what one costs, and every CTA takes an equal run.  A tile that a
+// run's border cuts is computed in parts: the CTA with its last k-blocks starts its accumulator from the others' fp32 sums,
+// added up in their order (its epilogue warps put them there while the tile before is computed).  A CTA does
+// the first part of the tile that it shares with its successor before everything else, and the
+// last part of the tile that it shares with its predecessors last, so that it finds their sums ready; it only ever
+// waits for CTAs of lower index, which never wait before they have delivered.
+// (Dealing out rows of weights instead was slower than whole tiles: a short tile's k-blocks take as long as a
+// whole one's.)
+// A k-block's cost: reading the weights (16-bit), which tokens hardly add to, or expanding them.
+__device__ __forceinline__ int gemm_item_cost(int chunk, int fmt) { return (fmt ? 8 : 16) + (chunk + 31) / 32; }
+template <int NT, int kMTile, int FMT>
+struct GemmSplit {
+    const int4 *rec;
+    const int *item0, *cost0;      // first item of every request, and its place on the line of costs
+    int n_reqs, kblocks, quads, units, unit;
+    int w_lo, q_lo, w_hi, q_hi, cur, step;
+    __device__ GemmSplit(const int4 *rec_, const int *item0_, const int *cost0_, int n_reqs_, int unit_, int n_ctas, int, int kblocks_)
+        : rec(rec_), item0(item0_), cost0(cost0_), n_reqs(n_reqs_), kblocks(kblocks_), quads((kblocks_ + 3) / 4), unit(unit_), step(0)
+    {
+        // no more CTAs than there are tiles, or pieces of two quads
+        const int items = item0[n_reqs];
+        units = min(n_ctas, max(items, items * quads / 2));
+        locate(unit, w_lo, q_lo);
+        locate(unit + 1, w_hi, q_hi);
+        cur = w_lo + (q_lo > 0 ? 1 : 0);
+    }
+    // where the run of CTA u begins: tile and quad
+    __device__ void locate(int u, int &w, int &quad) const
+    {
+        const int total = cost0[n_reqs];
+        const int at = u >= units ? total : (int)((long long)u * total / units);
+        if (at >= total) {
+            w = item0[n_reqs];
+            quad = 0;
+            return;
+        }
+        int r = 0;
+        for (int s = 64; s; s >>= 1)
+            if (r + s < n_reqs && cost0[r + s] <= at)
+                r += s;
+        const int c = gemm_item_cost(rec[r].w, FMT), local = at - cost0[r];
+        w = item0[r] + local / (c * quads);
+        quad = local % (c * quads) / c;
+    }
+    __device__ bool fill(GemmItem &it, int w, int qa, int qb) const
+    {
+        int q = 0;
+        for (int s = 64; s; s >>= 1)
+            if (q + s < n_reqs && item0[q + s] <= w)
+                q += s;
+        const int4 r = rec[q];
+        const int local = w - item0[q], n = (r.y + NT - 1) / NT, c = local % n;
+        it.m0 = local / n * kMTile;
+        it.row0 = r.x + c * r.w;
+        it.n_live = min(r.w, r.y - c * r.w);
+        it.n = (it.n_live + 15) / 16 * 16;
+        it.slot = r.z;
+        it.k0 = 4 * qa;
+        it.k1 = min(4 * qb, kblocks);
+        return true;
+    }
+    __device__ bool next(GemmItem &it)
+    {
+        if (step == 0) {
+            step = 1;
+            if (w_hi != w_lo && q_hi > 0)
+                return fill(it, w_hi, 0, q_hi);
+        }
+        if (step == 1) {
+            if (cur < w_hi)
+                return fill(it, cur++, 0, quads);
+            step = 2;
+        }
+        if (step == 2) {
+            step = 3;
+            if (w_lo == w_hi)
+                return q_lo < q_hi && fill(it, w_lo, q_lo, q_hi);
+            if (q_lo > 0)
+                return fill(it, w_lo, q_lo, quads);
+        }
+        return false;
+    }
+    // the CTAs with the earlier parts of tile w_lo: bit i = CTA unit - 1 - i
+    __device__ unsigned long long partners() const
+    {
+        unsigned long long m = 0;
+        int wb = w_lo, qb = q_lo;
+        for (int i = 0; i < 64 && unit - 1 - i >= 0; ++i) {
+            int wa, qa;
+            locate(unit - 1 - i, wa, qa);
+            if (wa != wb || qa != qb)
+                m |= 1ull << i;
+            if (wa < w_lo || qa == 0)
+                break;
+            wb = wa;
+            qb = qa;
+        }
+        return m;
+    }
+};
+template <int CG, int NT, int kMTile, int FMT>
+struct GemmItems {
+    using type = GemmSplit<NT, kMTile, FMT>;
+};
+template <int NT, int kMTile, int FMT>
+struct GemmItems<2, NT, kMTile, FMT> {
+    using type = GemmWalk<NT, kMTile>;
 };
 
 // PHASE 1: h = SiLU(Xs W_g^T) * (Xs W_u^T) -> hs (bf16).  PHASE 2: z = hs W_d^T -> zs (fp32).
@@ -347,14 +482,14 @@ template <int PHASE, int CG, int FMT>
 __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmParams p)
 {
     static_assert(FMT == 0 || CG == 1, "4-bit slots: single CTAs");
-    constexpr int kStages = gemm_stages(CG, FMT), kStageBytes = gemm_stage_bytes(CG), NT = gemm_tokens(CG);
+    constexpr int kStages = gemm_stages(CG, FMT), kStageBytes = gemm_stage_bytes(CG, FMT), NT = gemm_tokens(CG, FMT);
     constexpr int kMTile = PHASE == 1 ? 64 : 128;            // hidden units, or output columns, of one CTA's tile
     constexpr int kRawBlocks = PHASE == 1 ? 4 : 2;           // k-blocks of one fetch of codes
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ uint64_t s_bars[2 * kStages + 4 + 2 * kRawStages];
+    __shared__ uint64_t s_bars[2 * kStages + 5 + 2 * kRawStages];
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
-    __shared__ int s_tile0[kMaxReq + 1], s_nreq;
+    __shared__ int s_tile0[kMaxReq + 1], s_cost0[kMaxReq + 1], s_nreq;
     __shared__ int4 s_rec[kMaxReq];                          // see GemmWalk
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -364,6 +499,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     const uint32_t ring_s = smem_u32(ring), raw_s = ring_s + kStages * kStageBytes;
     const uint32_t full0 = smem_u32(s_bars), empty0 = full0 + 8 * kStages;
     const uint32_t tfull0 = empty0 + 8 * kStages, tempty0 = tfull0 + 16, rfull0 = tempty0 + 16, rempty0 = rfull0 + 8 * kRawStages;
+    const uint32_t tinit = rempty0 + 8 * kRawStages;
     volatile int *abort_flag = &s_abort;
     // rank within the CTA pair; the even CTA issues the MMAs, owns the "stage full" barriers and counts
     // the drained accumulators of both
@@ -375,24 +511,24 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     if (tid == 32) {
         s_abort = 0;
         for (int i = 0; i < kStages; ++i) {
-            mbar_init(full0 + 8 * i, FMT ? 5 : 1);
+            mbar_init(full0 + 8 * i, FMT ? 9 : 1);
             mbar_init(empty0 + 8 * i, 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(tfull0 + 8 * i, 1);
             mbar_init(tempty0 + 8 * i, 4 * CG);
         }
+        mbar_init(tinit, 4);
         if (FMT)
             for (int i = 0; i < kRawStages; ++i) {
                 mbar_init(rfull0 + 8 * i, 1);
-                mbar_init(rempty0 + 8 * i, 4);
+                mbar_init(rempty0 + 8 * i, 8);
             }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // GEMM 1 reads what the kernels ahead wrote from here on.  GEMM 2 is directly behind GEMM 1, which lets it start only
-    // once the plan is complete: of all it reads, only h has to be waited for (by the thread that loads it).
-    if (PHASE == 1)
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The kernel directly ahead (the gather, or GEMM 1) lets this one start only once the plan is complete, and the weights
+    // of the group are in their slots: of all that is read here, only the activations have to be waited for, by the thread
+    // that loads them, and everything that is written follows from them.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // (no kernel of the chain ends before the one ahead of it has)
     auto leave = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
@@ -401,9 +537,10 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     // ---- the launch's requests and their items, by warp 0, a lane per request
     const int K = PHASE == 1 ? p.d : p.F;                 // reduction length
     const int m_tiles = PHASE == 1 ? (p.F + CG * 64 - 1) / (CG * 64) : p.d / (CG * 128);
+    const int kblocks = (K + kBK - 1) / kBK;
     if (warp == 0) {
         const int n_req_total = plan->n_req + p.n_shared;
-        int n = 0, tiles = 0;
+        int n = 0, tiles = 0, costs = 0;
         for (int r0 = 0; r0 < n_req_total; r0 += 32) {
             const int r = r0 + lane;
             bool on = false;
@@ -419,22 +556,27 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 items = on ? chunks * m_tiles : 0;
             }
             const unsigned m = __ballot_sync(0xffffffffu, on);
-            int inc = items;
+            const int cost = CG == 1 ? items * gemm_item_cost(rec.w, FMT) * ((kblocks + 3) / 4) : 0;
+            int inc = items, inc_c = cost;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, inc, o);
+                const int v = __shfl_up_sync(0xffffffffu, inc, o), c = __shfl_up_sync(0xffffffffu, inc_c, o);
                 inc += lane >= o ? v : 0;
+                inc_c += lane >= o ? c : 0;
             }
             if (on) {
                 const int at = n + __popc(m & ((1u << lane) - 1u));
                 s_rec[at] = rec;
                 s_tile0[at] = tiles + inc - items;
+                s_cost0[at] = costs + inc_c - cost;
             }
             n += __popc(m);
             tiles += __shfl_sync(0xffffffffu, inc, 31);
+            costs += __shfl_sync(0xffffffffu, inc_c, 31);
         }
         if (lane == 0) {
             s_tile0[n] = tiles;
+            s_cost0[n] = costs;
             s_nreq = n;
         }
     }
@@ -464,25 +606,26 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = s_tmem_base;
 
-    auto walk = [&] { return GemmWalk<CG, NT, kMTile>(s_rec, s_tile0, n_reqs, unit, n_units, (int)rank); };
+    using Items = typename GemmItems<CG, NT, kMTile, FMT>::type;
+    auto walk = [&] { return Items(s_rec, s_tile0, s_cost0, n_reqs, unit, n_units, (int)rank, kblocks); };
     GemmItem it;
-    const int kblocks = (K + kBK - 1) / kBK;
 
     if (warp == 0) {
         // ============================================================ TMA producer
         if (lane == 0) {
             const CUtensorMap *map_b = p.maps + (PHASE == 1 ? kMapXs0 : kMapHs0);
             uint32_t n = 0;
-            bool waited = PHASE == 1;
+            bool waited = false;
             auto items = walk();
             while (!*abort_flag && items.next(it)) {
                 // the weights of the slots, or of the shared expert
                 const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
                 const int slot = it.slot >= 0 ? it.slot : 0;
-                // the smallest box that holds this CTA's share of the tokens: 32, 64 or 128 rows
+                // the smallest box that holds this CTA's share of the tokens: 32, 64 or 128 rows, or two of 128
                 const int rows = it.n / CG, cls = rows <= 32 ? 0 : rows <= 64 ? 1 : 2;
                 const int b_row = it.row0 + (int)rank * rows;
-                const uint32_t bytes = (FMT ? 0u : (uint32_t)kABytes) + ((32u * kBK * 2) << cls);
+                const bool two = NT / CG > 128 && rows > 128;
+                const uint32_t bytes = (FMT ? 0u : (uint32_t)kABytes) + ((32u * kBK * 2) << (two ? 3 : cls));
                 auto load_a = [&](int kb, uint32_t dst, uint32_t bar) {
                     if (FMT)
                         return;
@@ -491,23 +634,29 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     else
                         tma_load_4d(dst, map_w, 0, kb * kBK, it.m0 / 64, slot, bar);
                 };
-                int kb0 = 0;
+                auto load_b = [&](int kb, uint32_t dst, uint32_t bar) {
+                    tma_load_2d(dst, map_b + cls, kb * kBK, b_row, bar);
+                    if (two)
+                        tma_load_2d(dst + 128 * kBK * 2, map_b + cls, kb * kBK, b_row + 128, bar);
+                };
+                int kb0 = it.k0;
                 if (CG == 1 && !waited) {
-                    // the first stages' weights are on their way while GEMM 1 finishes
-                    const int pre = min(kblocks, kStages);
-                    for (int kb = 0; kb < pre; ++kb) {
-                        mbar_expect(full0 + 8 * kb, bytes);
-                        load_a(kb, ring_s + kb * kStageBytes, full0 + 8 * kb);
+                    // the first stages' weights are on their way while the kernel ahead finishes
+                    const int pre = min(it.k1 - it.k0, kStages);
+                    for (int i = 0; i < pre; ++i) {
+                        mbar_expect(full0 + 8 * i, bytes);
+                        load_a(it.k0 + i, ring_s + i * kStageBytes, full0 + 8 * i);
                     }
                     asm volatile("griddepcontrol.wait;" ::: "memory");
-                    for (int kb = 0; kb < pre; ++kb)
-                        tma_load_2d(ring_s + kb * kStageBytes + kABytes, map_b + cls, kb * kBK, b_row, full0 + 8 * kb);
-                    n = kb0 = pre;
+                    for (int i = 0; i < pre; ++i)
+                        load_b(it.k0 + i, ring_s + i * kStageBytes + kABytes, full0 + 8 * i);
+                    n = pre;
+                    kb0 += pre;
                 } else if (!waited) {
                     asm volatile("griddepcontrol.wait;" ::: "memory");
                 }
                 waited = true;
-                for (int kb = kb0; kb < kblocks; ++kb, ++n) {
+                for (int kb = kb0; kb < it.k1; ++kb, ++n) {
                     const uint32_t s = n % kStages;
                     if (n >= (uint32_t)kStages && !mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag))
                         break;
@@ -516,7 +665,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                         const uint32_t bar = full0 + 8 * s;
                         mbar_expect(bar, bytes);
                         load_a(kb, a_dst, bar);
-                        tma_load_2d(b_dst, map_b + cls, kb * kBK, b_row, bar);
+                        load_b(kb, b_dst, bar);
                     } else {
                         // the bytes of both CTAs are expected, once, on the even CTA's barrier
                         const uint32_t bar = cluster_addr(full0 + 8 * s, 0);
@@ -547,10 +696,14 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 const uint32_t acc = item & 1u;
                 if (item >= 2 && !mbar_wait(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag))
                     break;
+                // a tile whose first parts other CTAs computed starts from their sums
+                const bool merge = CG == 1 && it.k0 > 0 && it.k1 == kblocks;
+                if (merge && !mbar_wait(tinit, 0, abort_flag))
+                    break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d_tmem = tmem_base + acc * NT;
                 bool ok = true;
-                for (int kb = 0; kb < kblocks; ++kb, ++n) {
+                for (int kb = it.k0; kb < it.k1; ++kb, ++n) {
                     const uint32_t s = n % kStages;
                     if (!mbar_wait(full0 + 8 * s, (n / kStages) & 1u, abort_flag)) {
                         ok = false;
@@ -566,9 +719,9 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
 #pragma unroll
                     for (int ks = 0; ks < kBK / 16; ++ks) {
                         if (CG == 1)
-                            umma_bf16(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, (kb | ks) != 0);
+                            umma_bf16(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, merge || kb != it.k0 || ks != 0);
                         else
-                            umma_bf16_pair(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, (kb | ks) != 0);
+                            umma_bf16_pair(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, merge || kb != it.k0 || ks != 0);
                     }
                     // the stage is free once these MMAs have read it
                     if (CG == 1)
@@ -590,13 +743,88 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         const int quarter = warp & 3;                        // the 32 accumulator rows this warp may read
         uint32_t item = 0;
         auto items = walk();
-        for (; !*abort_flag && items.next(it); ++item) {
+        // sums of the CTAs with the earlier parts of a tile ([token][row] of fp32 per CTA, and a word per CTA and
+        // quarter that says they are there) into the accumulator that the tile will use
+        auto preload = [&](const GemmItem &nx, uint32_t acc) {
+            if constexpr (CG == 1) {
+                const unsigned long long others = items.partners();
+                for (unsigned long long m = others; m; m &= m - 1) {
+                    const unsigned *flag = p.flags + (blockIdx.x - __ffsll((long long)m)) * 4 + quarter;
+                    const long long c0 = clock64();
+                    for (;;) {
+                        unsigned v;
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+                        if (v == p.seq || *abort_flag)
+                            break;
+                        if (clock64() - c0 > kGemmWaitCycles)
+                            *abort_flag = 1;
+                    }
+                }
+                __syncwarp();
+                const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * NT;
+#pragma unroll 1
+                for (int c = 0; c < nx.n; c += 32) {
+                    float sum[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        sum[j] = 0.0f;
+                    // (in ascending order of the CTAs, which is that of the k-blocks)
+                    for (int i = 63 - __clzll((long long)others); i >= 0; --i) {
+                        if (!((others >> i) & 1ull))
+                            continue;
+                        const float *src = p.partial + (size_t)(blockIdx.x - 1 - i) * 128 * p.part_tokens + quarter * 32 + lane;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j)
+                            if (c + j < nx.n_live)
+                                sum[j] += __ldcg(src + (size_t)(c + j) * 128);
+                    }
+                    tmem_st32(t_row + c, sum);
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(tinit);
+            }
+        };
+        GemmItem nx;
+        bool more = items.next(nx);
+        if (more && CG == 1 && nx.k0 > 0 && nx.k1 == kblocks)
+            preload(nx, 0);
+        for (; !*abort_flag && more; ++item) {
+            it = nx;
             const uint32_t acc = item & 1u;
+            more = items.next(nx);
+            // (the other accumulator was drained before this item; a part that this CTA owes another goes out first)
+            const bool owed = CG == 1 && it.k1 < kblocks, merge_next = CG == 1 && more && nx.k0 > 0 && nx.k1 == kblocks;
+            if (merge_next && !owed)
+                preload(nx, acc ^ 1u);
             if (!mbar_wait(tfull0 + 8 * acc, (item >> 1) & 1u, abort_flag))
                 break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * NT;
-            if (PHASE == 1) {
+            if (owed) {
+                // an earlier part of a tile, for the CTA that finishes it
+                float *dst = p.partial + (size_t)blockIdx.x * 128 * p.part_tokens + quarter * 32 + lane;
+#pragma unroll 1
+                for (int c = 0; c < it.n_live; c += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(t_row + c, v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (c + j < it.n_live)
+                            __stcg(dst + (size_t)(c + j) * 128, __uint_as_float(v[j]));
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    __threadfence();
+                    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.flags + blockIdx.x * 4 + quarter), "r"(p.seq) : "memory");
+                }
+                __syncwarp();
+                if (merge_next)
+                    preload(nx, acc ^ 1u);
+            } else if (PHASE == 1) {
                 // lanes 0..7 hold g of eight hidden units, 8..15 u of the same ones, 16..31 those of the next eight.  Of two
                 // neighbouring tokens the g lane finishes the first and the u lane the second.
                 const int f = it.m0 + quarter * 16 + (lane >> 4) * 8 + (lane & 7);
@@ -640,9 +868,9 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     mbar_arrive_cluster(cluster_addr(tempty0 + 8 * acc, 0));
             }
         }
-    } else if (FMT == 1 && warp < 10) {
-        // ============================================================ expansion of 4-bit codes (warps 6..9)
-        const int row = (warp - 6) * 32 + lane;              // row of the weight tile, or (column group, f) of GEMM 2's
+    } else if (FMT == 1 && warp < 14) {
+        // ============================================================ expansion of 4-bit codes (warps 6..13)
+        const int row = ((warp - 6) & 3) * 32 + lane, side = (warp - 6) >> 2;              // row of the weight tile, or (column group, f) of GEMM 2's
         const size_t ub = (size_t)p.unit_bytes, scales = 3 * (size_t)(p.d / 2);
         uint32_t n = 0, rn = 0;
         auto items = walk();
@@ -659,9 +887,9 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     return f_row < p.F && kb < kblocks ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base) + kb) : 0u;
                 return kb * kBK + f_row < p.F ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base + (size_t)kb * kBK * ub)) : 0u;
             };
-            uint32_t sc = scale_of(0);
+            uint32_t sc = scale_of(it.k0);
             bool ok = true;
-            for (int kb = 0; kb < kblocks && ok; ++kb, ++n) {
+            for (int kb = it.k0; kb < it.k1 && ok; ++kb, ++n) {
                 const int sub = kb % kRawBlocks;
                 const uint32_t rs = rn % kRawStages, s = n % kStages;
                 if (sub == 0)
@@ -675,56 +903,53 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 const uint32_t raw = raw_s + rs * kRawBytes, a_dst = ring_s + s * kStageBytes + row * 128;
                 const uint32_t x = (uint32_t)(row & 7);      // = f mod 8 in both phases
                 if (PHASE == 1) {
-                    // 64 columns = pieces 2 sub, 2 sub + 1 of this row's 128 bytes of codes -> eight pieces of bf16
-                    const uint32_t src = raw + row * 128;
+                    // 32 of 64 columns = piece 2 sub + side of this row's 128 bytes of codes -> four pieces of bf16
+                    const uint4 c4 = lds128(raw + row * 128 + (((2 * sub + side) ^ x) << 4));
+                    const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint4 c4 = lds128(src + (((2 * sub + h) ^ x) << 4));
-                        const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            uint32_t P[4];
-                            expand8(cw[i], ss, P);
-                            sts128(a_dst + (((4 * h + i) ^ x) << 4), P[0], P[1], P[2], P[3]);
-                        }
+                    for (int i = 0; i < 4; ++i) {
+                        uint32_t P[4];
+                        expand8(cw[i], ss, P);
+                        sts128(a_dst + (((4 * side + i) ^ x) << 4), P[0], P[1], P[2], P[3]);
                     }
                 } else {
-                    // one f, one group of 64 columns; nibble q of word w is column 8 q + w
+                    // one f, one group of 64 columns; nibble q of word w is column 8 q + w.  Side 0 expands nibbles 0, 1, 4, 5,
+                    // side 1 the others.
                     const uint32_t src = raw + (sub * 64 + (row & 63)) * 128;
                     const uint32_t pc0 = (uint32_t)((it.m0 / 32) & 7) + 2u * cg;      // first piece of the group in its 128 bytes
-                    uint32_t o[8][4];
+                    uint32_t o[4][4];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const uint4 c4 = lds128(src + (((pc0 + h) ^ x) << 4));
-                        const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
+                        const uint32_t cw[4] = {c4.x >> (8 * side), c4.y >> (8 * side), c4.z >> (8 * side), c4.w >> (8 * side)};
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
-                            uint32_t P[4], Q[4];
-                            expand8(cw[2 * i], ss, P);
-                            expand8(cw[2 * i + 1], ss, Q);
+                            uint32_t P[2], Q[2];
+                            expand4(cw[2 * i], ss, P);
+                            expand4(cw[2 * i + 1], ss, Q);
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) {
+                            for (int q = 0; q < 2; ++q) {
                                 o[q][2 * h + i] = __byte_perm(P[q], Q[q], 0x5410);
-                                o[q + 4][2 * h + i] = __byte_perm(P[q], Q[q], 0x7632);
+                                o[q + 2][2 * h + i] = __byte_perm(P[q], Q[q], 0x7632);
                             }
                         }
                     }
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        sts128(a_dst + ((q ^ x) << 4), o[q][0], o[q][1], o[q][2], o[q][3]);
+                    for (int q = 0; q < 4; ++q)
+                        sts128(a_dst + ((((q & 1) + 2 * side + 4 * (q >> 1)) ^ x) << 4), o[q][0], o[q][1], o[q][2], o[q][3]);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the tensor cores read what was just stored
                 __syncwarp();
                 if (lane == 0)
                     mbar_arrive(full0 + 8 * s);
-                if (sub == kRawBlocks - 1 || kb == kblocks - 1) {
+                if (sub == kRawBlocks - 1 || kb == it.k1 - 1) {
                     if (lane == 0)
                         mbar_arrive(rempty0 + 8 * rs);
                     ++rn;
                 }
             }
         }
-    } else if (FMT == 1 && warp == 10) {
+    } else if (FMT == 1 && warp == 14) {
         // ============================================================ fetch of 4-bit codes
         if (lane == 0) {
             uint32_t rn = 0;
@@ -732,7 +957,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
             while (!*abort_flag && items.next(it)) {
                 const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
                 const int slot = it.slot >= 0 ? it.slot : 0;
-                for (int kb = 0; kb < kblocks; kb += kRawBlocks, ++rn) {
+                for (int kb = it.k0; kb < it.k1; kb += kRawBlocks, ++rn) {
                     const uint32_t rs = rn % kRawStages;
                     if (rn >= (uint32_t)kRawStages && !mbar_wait(rempty0 + 8 * rs, ((rn / kRawStages) - 1u) & 1u, abort_flag))
                         break;
@@ -913,7 +1138,7 @@ cudaError_t launch_after(cudaStream_t stream, void (*kernel)(Params...), dim3 gr
 
 constexpr size_t gemm_smem(int cg, int fmt)
 {
-    return (size_t)gemm_stages(cg, fmt) * gemm_stage_bytes(cg) + (fmt ? kRawStages * kRawBytes : 0) + 1024;
+    return (size_t)gemm_stages(cg, fmt) * gemm_stage_bytes(cg, fmt) + (fmt ? kRawStages * kRawBytes : 0) + 1024;
 }
 
 template <int PHASE, int CG, int FMT>
@@ -929,6 +1154,8 @@ cudaError_t gemm_configure()
 }
 
 }  // namespace
+
+int ffn_gemm_part_tokens(int fmt) { return gemm_tokens(1, fmt); }
 
 bool ffn_gemm_supported(int d, int F) { return d % 256 == 0 && F % kUnitRows == 0; }
 

@@ -354,8 +354,8 @@ int ensure_capacity(melinoe_moe *h, int T)
         CU_TRY(cudaMalloc(&h->hs, sorted * h->F * 2));
         h->part_tokens = (cap + 31) / 32 * 32 < ffn_gemm_part_tokens(h->fmt) ? (cap + 31) / 32 * 32 : ffn_gemm_part_tokens(h->fmt);
         CU_TRY(cudaMalloc(&h->partial, (size_t)h->n_sms * 128 * h->part_tokens * sizeof(float)));
-        CU_TRY(cudaMalloc(&h->part_flags, (size_t)h->n_sms * 4 * sizeof(unsigned)));
-        CU_TRY(cudaMemset(h->part_flags, 0, (size_t)h->n_sms * 4 * sizeof(unsigned)));
+        CU_TRY(cudaMalloc(&h->part_flags, (size_t)h->n_sms * 8 * sizeof(unsigned)));
+        CU_TRY(cudaMemset(h->part_flags, 0, (size_t)h->n_sms * 8 * sizeof(unsigned)));
         h->gemm_seq = 0;
         if (!encode_activation_maps(&h->maps_host[kMapXs0], h->xs, h->d, sorted) ||
             !encode_activation_maps(&h->maps_host[kMapHs0], h->hs, h->F, sorted))

@@ -36,9 +36,9 @@
 // care, so Xs is gathered with the same order.
 //
 // One persistent CTA per SM, warp-specialised: warp 0 issues TMA loads into a ring of stages, warp 1
-// issues the MMAs (one elected thread) and commits them to mbarriers, warps 2..5 drain
-// the accumulator (tcgen05.ld, 32 rows per warp) and write the tile; with 4-bit slots warps 6..13 expand and
-// warp 14 fetches codes.  Two accumulators alternate so the epilogue of a tile overlaps the MMAs of the next.
+// issues the MMAs (one elected thread) and commits them to mbarriers, warps 2..9 drain
+// the accumulator (tcgen05.ld, 32 rows per warp) and write the tile; with 4-bit slots warps 10..17 expand and
+// warp 18 fetches codes.  Two accumulators alternate so the epilogue of a tile overlaps the MMAs of the next.
 // Work items are (request, weight tile, token chunk) triples of the launch's compute group, dealt
 // round-robin to CTA pairs, and cut into equal runs of k-blocks for single CTAs (GemmWalk, GemmSplit).
 //
@@ -73,9 +73,10 @@ constexpr int kBK = 64;                    // K elements per stage (128 bytes)
 constexpr int kABytes = 128 * kBK * 2;     // weight tile of a stage: 128 rows
 constexpr int kRawBytes = 16384;           // 4-bit slots: codes of one fetch (GEMM 1: 256 columns of 128 rows; GEMM 2: 128 rows f of 256 columns)
 constexpr int kRawStages = 3;
+constexpr int kEpilogueWarps = 8;          // two per 32 accumulator rows, each with every other 16 tokens
 constexpr size_t kGemmSmem = 227 * 1024 - 4096;      // dynamic shared memory of a CTA (the static part is below 3 KB)
 // threads, tokens of a chunk at most, bytes and number of ring stages for CG CTAs per operation and slot format FMT
-__host__ __device__ constexpr int gemm_threads(int fmt) { return fmt ? 480 : 192; }
+__host__ __device__ constexpr int gemm_threads(int fmt) { return fmt ? 608 : 320; }
 __host__ __device__ constexpr int gemm_tokens(int cg, int fmt) { return cg == 2 || fmt ? 256 : 128; }
 __host__ __device__ constexpr int gemm_stage_bytes(int cg, int fmt) { return kABytes + gemm_tokens(cg, fmt) / cg * kBK * 2; }
 __host__ __device__ constexpr int gemm_stages(int cg, int fmt)
@@ -262,30 +263,31 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar)
                  : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16])
 {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
+          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
         : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&r)[32])
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&r)[16])
 {
     asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
         ::"r"(taddr), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "f"(r[8]), "f"(r[9]),
-          "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15]), "f"(r[16]), "f"(r[17]), "f"(r[18]), "f"(r[19]),
-          "f"(r[20]), "f"(r[21]), "f"(r[22]), "f"(r[23]), "f"(r[24]), "f"(r[25]), "f"(r[26]), "f"(r[27]), "f"(r[28]), "f"(r[29]),
-          "f"(r[30]), "f"(r[31])
+          "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15])
         : "memory");
+}
+// to nearest even, as the low half
+__device__ __forceinline__ uint16_t bf16_bits(float v)
+{
+    uint16_t r;
+    asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(r) : "f"(v));
+    return r;
 }
 
 __device__ __forceinline__ uint32_t bf16_rne(float v)
@@ -511,14 +513,14 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     if (tid == 32) {
         s_abort = 0;
         for (int i = 0; i < kStages; ++i) {
-            mbar_init(full0 + 8 * i, FMT ? 9 : 1);
+            mbar_init(full0 + 8 * i, FMT ? 5 : 1);
             mbar_init(empty0 + 8 * i, 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(tfull0 + 8 * i, 1);
-            mbar_init(tempty0 + 8 * i, 4 * CG);
+            mbar_init(tempty0 + 8 * i, kEpilogueWarps * CG);
         }
-        mbar_init(tinit, 4);
+        mbar_init(tinit, kEpilogueWarps);
         if (FMT)
             for (int i = 0; i < kRawStages; ++i) {
                 mbar_init(rfull0 + 8 * i, 1);
@@ -738,9 +740,12 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     umma_commit_pair(tfull0 + 8 * acc);
             }
         }
-    } else if (warp < 6) {
-        // ============================================================ epilogue (warps 2..5)
+    } else if (warp < 2 + kEpilogueWarps) {
+        // ============================================================ epilogue (warps 2..9)
+        // What bounds it is the instructions of a single warp per scheduler (with four warps, 32 tokens took 1.1 to 2.1 us, and
+        // 256 tokens longer than the products of the next tile), hence eight, and no predicates on whole chunks.
         const int quarter = warp & 3;                        // the 32 accumulator rows this warp may read
+        const int c_first = (warp - 2) / 4 * 16;             // its chunks of 16 tokens: c_first, c_first + 32, ..
         uint32_t item = 0;
         auto items = walk();
         // sums of the CTAs with the earlier parts of a tile ([token][row] of fp32 per CTA, and a word per CTA and
@@ -749,7 +754,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
             if constexpr (CG == 1) {
                 const unsigned long long others = items.partners();
                 for (unsigned long long m = others; m; m &= m - 1) {
-                    const unsigned *flag = p.flags + (blockIdx.x - __ffsll((long long)m)) * 4 + quarter;
+                    const unsigned *flag = p.flags + (blockIdx.x - __ffsll((long long)m)) * kEpilogueWarps + (warp - 2);
                     const long long c0 = clock64();
                     for (;;) {
                         unsigned v;
@@ -763,22 +768,21 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 __syncwarp();
                 const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * NT;
 #pragma unroll 1
-                for (int c = 0; c < nx.n; c += 32) {
-                    float sum[32];
+                for (int c = c_first; c < nx.n; c += 32) {
+                    float sum[16];
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
+                    for (int j = 0; j < 16; ++j)
                         sum[j] = 0.0f;
                     // (in ascending order of the CTAs, which is that of the k-blocks)
                     for (int i = 63 - __clzll((long long)others); i >= 0; --i) {
                         if (!((others >> i) & 1ull))
                             continue;
-                        const float *src = p.partial + (size_t)(blockIdx.x - 1 - i) * 128 * p.part_tokens + quarter * 32 + lane;
+                        const float *src = p.partial + ((size_t)(blockIdx.x - 1 - i) * p.part_tokens + c) * 128 + quarter * 32 + lane;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (c + j < nx.n_live)
-                                sum[j] += __ldcg(src + (size_t)(c + j) * 128);
+                        for (int j = 0; j < 16; ++j)
+                            sum[j] += __ldcg(src + j * 128);      // (tokens that do not exist: whatever is there)
                     }
-                    tmem_st32(t_row + c, sum);
+                    tmem_st16(t_row + c, sum);
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -805,21 +809,19 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
             const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * NT;
             if (owed) {
                 // an earlier part of a tile, for the CTA that finishes it
-                float *dst = p.partial + (size_t)blockIdx.x * 128 * p.part_tokens + quarter * 32 + lane;
+                float *dst = p.partial + (size_t)blockIdx.x * p.part_tokens * 128 + quarter * 32 + lane;
 #pragma unroll 1
-                for (int c = 0; c < it.n_live; c += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(t_row + c, v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                for (int c = c_first; c < it.n; c += 32) {
+                    float v[16];
+                    tmem_ld16(t_row + c, v);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (c + j < it.n_live)
-                            __stcg(dst + (size_t)(c + j) * 128, __uint_as_float(v[j]));
+                    for (int j = 0; j < 16; ++j)
+                        __stcg(dst + (c + j) * 128, v[j]);
                 }
                 __syncwarp();
                 if (lane == 0) {
                     __threadfence();
-                    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.flags + blockIdx.x * 4 + quarter), "r"(p.seq) : "memory");
+                    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.flags + blockIdx.x * kEpilogueWarps + (warp - 2)), "r"(p.seq) : "memory");
                 }
                 __syncwarp();
                 if (merge_next)
@@ -829,34 +831,49 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 // neighbouring tokens the g lane finishes the first and the u lane the second.
                 const int f = it.m0 + quarter * 16 + (lane >> 4) * 8 + (lane & 7);
                 const bool is_u = (lane & 8) != 0;
-                uint16_t *dst = p.hs + (size_t)(it.row0 + (is_u ? 1 : 0)) * p.F + f;
-                // this lane stores tokens j (+ 1) with j below this
+                // this lane stores tokens c + 2 j (+ 1) with c + 2 j below this
                 const int left = f < p.F ? it.n_live - (is_u ? 1 : 0) : 0;
+                uint16_t *dst = p.hs + (size_t)(it.row0 + c_first + (is_u ? 1 : 0)) * p.F + f;
+                const size_t step = (size_t)p.F * 2;
 #pragma unroll 1
-                for (int c = 0; c < it.n_live; c += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(t_row + c, v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                for (int c = c_first; c < it.n_live; c += 32, dst += 16 * step) {
+                    float v[16];
+                    tmem_ld16(t_row + c, v);
+                    uint16_t h[8];
 #pragma unroll
-                    for (int j = 0; j < 32; j += 2) {
-                        const uint32_t o = __shfl_xor_sync(0xffffffffu, is_u ? v[j] : v[j + 1], 8);
-                        const float g = __uint_as_float(is_u ? o : v[j]), u = __uint_as_float(is_u ? v[j + 1] : o);
-                        const float h = __fdividef(g, 1.0f + __expf(-g)) * u;
-                        if (c + j < left)
-                            dst[(size_t)(c + j) * p.F] = (uint16_t)bf16_rne(h);
+                    for (int j = 0; j < 8; ++j) {
+                        const float o = __shfl_xor_sync(0xffffffffu, is_u ? v[2 * j] : v[2 * j + 1], 8);
+                        const float g = is_u ? o : v[2 * j], u = is_u ? v[2 * j + 1] : o;
+                        h[j] = bf16_bits(__fdividef(g, 1.0f + __expf(-g)) * u);
+                    }
+                    if (c + 14 < left) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            dst[j * step] = h[j];
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            if (c + 2 * j < left)
+                                dst[j * step] = h[j];
                     }
                 }
             } else {
-                float *dst = p.zs + (size_t)it.row0 * p.d + it.m0 + quarter * 32 + lane;
+                float *dst = p.zs + (size_t)(it.row0 + c_first) * p.d + it.m0 + quarter * 32 + lane;
+                const size_t step = (size_t)p.d;
 #pragma unroll 1
-                for (int c = 0; c < it.n_live; c += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(t_row + c, v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                for (int c = c_first; c < it.n_live; c += 32, dst += 32 * step) {
+                    float v[16];
+                    tmem_ld16(t_row + c, v);
+                    if (c + 16 <= it.n_live) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (c + j < it.n_live)
-                            dst[(size_t)(c + j) * p.d] = __uint_as_float(v[j]);
+                        for (int j = 0; j < 16; ++j)
+                            dst[j * step] = v[j];
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (c + j < it.n_live)
+                                dst[j * step] = v[j];
+                    }
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -868,11 +885,14 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     mbar_arrive_cluster(cluster_addr(tempty0 + 8 * acc, 0));
             }
         }
-    } else if (FMT == 1 && warp < 14) {
-        // ============================================================ expansion of 4-bit codes (warps 6..13)
-        const int row = ((warp - 6) & 3) * 32 + lane, side = (warp - 6) >> 2;              // row of the weight tile, or (column group, f) of GEMM 2's
+    } else if (FMT == 1 && warp < 18) {
+        // ============================================================ expansion of 4-bit codes (warps 10..17)
+        // Two groups of four warps take the k-blocks in turn: what a k-block takes is latency (waits, the fence before the
+        // tensor cores may read), which the other group's k-block covers.  (Eight warps on every k-block: 0.6 us each, as
+        // with four.)
+        const int row = ((warp - 10) & 3) * 32 + lane, group = (warp - 10) >> 2;     // row of the weight tile, or (column group, f) of GEMM 2's
         const size_t ub = (size_t)p.unit_bytes, scales = 3 * (size_t)(p.d / 2);
-        uint32_t n = 0, rn = 0;
+        uint32_t n0 = 0, rn = 0;
         auto items = walk();
         while (!*abort_flag && items.next(it)) {
             const char *blob = it.slot >= 0 ? p.slots + (size_t)it.slot * p.slot_stride : p.shared_blobs[-1 - it.slot];
@@ -887,69 +907,74 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     return f_row < p.F && kb < kblocks ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base) + kb) : 0u;
                 return kb * kBK + f_row < p.F ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base + (size_t)kb * kBK * ub)) : 0u;
             };
-            uint32_t sc = scale_of(it.k0);
+            uint32_t sc = scale_of(it.k0 + group);
             bool ok = true;
-            for (int kb = it.k0; kb < it.k1 && ok; ++kb, ++n) {
-                const int sub = kb % kRawBlocks;
-                const uint32_t rs = rn % kRawStages, s = n % kStages;
-                if (sub == 0)
-                    ok = mbar_wait(rfull0 + 8 * rs, (rn / kRawStages) & 1u, abort_flag);
-                if (ok && n >= (uint32_t)kStages)
+            for (int kr = it.k0; kr < it.k1 && ok; kr += kRawBlocks, ++rn) {
+                const uint32_t rs = rn % kRawStages;
+                ok = mbar_wait(rfull0 + 8 * rs, (rn / kRawStages) & 1u, abort_flag);
+                for (int sub = group; sub < kRawBlocks && kr + sub < it.k1 && ok; sub += 2) {
+                const int kb = kr + sub;
+                const uint32_t n = n0 + (uint32_t)(kb - it.k0), s = n % kStages;
+                if (n >= (uint32_t)kStages)
                     ok = mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag);
                 if (!ok)
                     break;
                 const uint32_t ss = sc * 0x10001u;
-                sc = scale_of(kb + 1);
+                sc = scale_of(kb + 2);
                 const uint32_t raw = raw_s + rs * kRawBytes, a_dst = ring_s + s * kStageBytes + row * 128;
                 const uint32_t x = (uint32_t)(row & 7);      // = f mod 8 in both phases
                 if (PHASE == 1) {
-                    // 32 of 64 columns = piece 2 sub + side of this row's 128 bytes of codes -> four pieces of bf16
-                    const uint4 c4 = lds128(raw + row * 128 + (((2 * sub + side) ^ x) << 4));
-                    const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        uint32_t P[4];
-                        expand8(cw[i], ss, P);
-                        sts128(a_dst + (((4 * side + i) ^ x) << 4), P[0], P[1], P[2], P[3]);
-                    }
-                } else {
-                    // one f, one group of 64 columns; nibble q of word w is column 8 q + w.  Side 0 expands nibbles 0, 1, 4, 5,
-                    // side 1 the others.
-                    const uint32_t src = raw + (sub * 64 + (row & 63)) * 128;
-                    const uint32_t pc0 = (uint32_t)((it.m0 / 32) & 7) + 2u * cg;      // first piece of the group in its 128 bytes
-                    uint32_t o[4][4];
+                    // 64 columns = pieces 2 sub, 2 sub + 1 of this row's 128 bytes of codes -> eight pieces of bf16
+                    const uint32_t src = raw + row * 128;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const uint4 c4 = lds128(src + (((pc0 + h) ^ x) << 4));
-                        const uint32_t cw[4] = {c4.x >> (8 * side), c4.y >> (8 * side), c4.z >> (8 * side), c4.w >> (8 * side)};
+                        const uint4 c4 = lds128(src + (((2 * sub + h) ^ x) << 4));
+                        const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) {
+                        for (int i = 0; i < 4; ++i) {
+                            uint32_t P[4];
+                            expand8(cw[i], ss, P);
+                            sts128(a_dst + (((4 * h + i) ^ x) << 4), P[0], P[1], P[2], P[3]);
+                        }
+                    }
+                } else {
+                    // one f, one group of 64 columns; nibble q of word w is column 8 q + w
+                    const uint32_t src = raw + (sub * 64 + (row & 63)) * 128;
+                    const uint32_t pc0 = (uint32_t)((it.m0 / 32) & 7) + 2u * cg;      // first piece of the group in its 128 bytes
+                    const uint4 ca = lds128(src + ((pc0 ^ x) << 4)), cb = lds128(src + (((pc0 + 1) ^ x) << 4));
+                    // (half of the nibbles at a time, to save registers)
+#pragma unroll
+                    for (int side = 0; side < 2; ++side) {
+                        const uint32_t cw[8] = {ca.x >> (8 * side), ca.y >> (8 * side), ca.z >> (8 * side), ca.w >> (8 * side),
+                                                cb.x >> (8 * side), cb.y >> (8 * side), cb.z >> (8 * side), cb.w >> (8 * side)};
+                        uint32_t o[4][4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
                             uint32_t P[2], Q[2];
                             expand4(cw[2 * i], ss, P);
                             expand4(cw[2 * i + 1], ss, Q);
 #pragma unroll
                             for (int q = 0; q < 2; ++q) {
-                                o[q][2 * h + i] = __byte_perm(P[q], Q[q], 0x5410);
-                                o[q + 2][2 * h + i] = __byte_perm(P[q], Q[q], 0x7632);
+                                o[q][i] = __byte_perm(P[q], Q[q], 0x5410);
+                                o[q + 2][i] = __byte_perm(P[q], Q[q], 0x7632);
                             }
                         }
-                    }
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        sts128(a_dst + ((((q & 1) + 2 * side + 4 * (q >> 1)) ^ x) << 4), o[q][0], o[q][1], o[q][2], o[q][3]);
+                        for (int q = 0; q < 4; ++q)
+                            sts128(a_dst + ((((q & 1) + 2 * side + 4 * (q >> 1)) ^ x) << 4), o[q][0], o[q][1], o[q][2], o[q][3]);
+                    }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the tensor cores read what was just stored
                 __syncwarp();
                 if (lane == 0)
                     mbar_arrive(full0 + 8 * s);
-                if (sub == kRawBlocks - 1 || kb == it.k1 - 1) {
-                    if (lane == 0)
-                        mbar_arrive(rempty0 + 8 * rs);
-                    ++rn;
                 }
+                if (lane == 0)
+                    mbar_arrive(rempty0 + 8 * rs);
             }
+            n0 += (uint32_t)(it.k1 - it.k0);
         }
-    } else if (FMT == 1 && warp == 14) {
+    } else if (FMT == 1 && warp == 18) {
         // ============================================================ fetch of 4-bit codes
         if (lane == 0) {
             uint32_t rn = 0;

@@ -163,7 +163,7 @@ struct GemmParams {
     size_t slot_stride;
     const char *const *shared_blobs;
     int unit_bytes;
-    // tiles computed in parts by several CTAs: [CTA][part_tokens][128] fp32 sums, a word per CTA and 32 rows, and what the
+    // tiles computed in parts by several CTAs: [CTA][part_tokens][128] fp32 sums, eight words per CTA, and what the
     // words of this launch say
     float *partial;
     unsigned *flags;

@@ -996,30 +996,26 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
             // The warp's columns: `own` contiguous ones, except that the 4-bit path's column steps of 32, where a warp has only
             // one of them, are 16 columns in each half of a block of 64.  All loads of some tokens before any store: this
             // warp is the whole grid's critical path, and a load behind a store that may alias it would wait for it.
-            // For the same reason a launch of one token has a form of its own: what four predicated tokens take in
-            // instructions was 1.5 us per launch.
-            constexpr int kSteps = MT_ > 0 ? MT_ / 2 : 8;
+            // For the same reason the forms differ by what there is to convert: four tokens' predicated instructions
+            // for one token were 1.5 us per launch.
             const int own = MT * 16;
             const bool halves = FMT == 1 && MT == 2;
-            const int c0 = halves ? (warp >> 1) * 64 + 16 * (warp & 1) + (lane & 15) + 32 * (lane >> 4) : warp * own + lane;
-            auto convert = [&](auto n_toks, int t0) {
-                constexpr int kToks = decltype(n_toks)::value;
-                long long fx[kToks * kSteps];
-                float carry[kToks * kSteps];
+            // n elements per lane: element j is column column(j) of token token(j), if on(j)
+            auto convert = [&](auto n, auto on, auto token, auto column) {
+                constexpr int N = decltype(n)::value;
+                long long fx[N];
+                float carry[N];
 #pragma unroll
-                for (int j = 0; j < kToks * kSteps; ++j) {
-                    const int t = t0 + j / kSteps, i = j % kSteps * 32;
-                    const bool on = (kToks == 1 || t < Tc) && (MT_ > 0 || i + lane < own);
-                    fx[j] = on ? __ldcg(p.yacc + t * d + c0 + i) : 0ll;
-                    carry[j] = acc_in && on ? __ldcg(p.ybuf + (size_t)(tok0 + t) * d + c0 + i) : 0.0f;
+                for (int j = 0; j < N; ++j) {
+                    fx[j] = on(j) ? __ldcg(p.yacc + token(j) * d + column(j)) : 0ll;
+                    carry[j] = acc_in && on(j) ? __ldcg(p.ybuf + (size_t)(tok0 + token(j)) * d + column(j)) : 0.0f;
                 }
 #pragma unroll
-                for (int j = 0; j < kToks * kSteps; ++j) {
-                    const int t = t0 + j / kSteps, i = j % kSteps * 32;
-                    if ((kToks == 1 || t < Tc) && (MT_ > 0 || i + lane < own)) {
-                        p.yacc[t * d + c0 + i] = 0;              // the accumulator is left clean for the next launch
+                for (int j = 0; j < N; ++j) {
+                    if (on(j)) {
+                        p.yacc[token(j) * d + column(j)] = 0;    // the accumulator is left clean for the next launch
                         float v = __ll2float_rn(fx[j]) * (1.0f / 1099511627776.0f);     // one rounding, then an exact scaling
-                        const size_t o = (size_t)(tok0 + t) * d + c0 + i;
+                        const size_t o = (size_t)(tok0 + token(j)) * d + column(j);
                         if (acc_in)
                             v += carry[j];
                         if (acc_out)
@@ -1029,13 +1025,40 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
                     }
                 }
             };
-            if (Tc == 1) {
-                convert(Count<1>(), 0);
-            } else {
-                constexpr int kToks = 16 / kSteps;
+            if constexpr (MT_ > 0) {
+                constexpr int kSteps = MT_ / 2, kToks = 16 / kSteps;
+                const int c0 = warp * own + lane;
+                if (Tc == 1) {
+                    convert(Count<kSteps>(), [](int) { return true; }, [](int) { return 0; }, [&](int j) { return c0 + j * 32; });
+                } else {
 #pragma unroll 1
-                for (int t0 = 0; t0 < Tc; t0 += kToks)
-                    convert(Count<kToks>(), t0);
+                    for (int t0 = 0; t0 < Tc; t0 += kToks)
+                        convert(Count<16>(), [&](int j) { return t0 + j / kSteps < Tc; }, [&](int j) { return t0 + j / kSteps; },
+                                [&](int j) { return c0 + j % kSteps * 32; });
+                }
+            } else {
+                // any width: the warp's columns of all tokens end to end
+                const int total = own * Tc;
+                auto flat = [&](auto n, int e0) {
+                    int tok[decltype(n)::value], col[decltype(n)::value];
+#pragma unroll
+                    for (int j = 0; j < decltype(n)::value; ++j) {
+                        const int e = e0 + 32 * j;
+                        tok[j] = e / own;
+                        const int i = e - tok[j] * own;
+                        col[j] = halves ? (warp >> 1) * 64 + 16 * (warp & 1) + (i & 15) + 32 * (i >> 4) : warp * own + i;
+                    }
+                    convert(n, [&](int j) { return e0 + 32 * j < total; }, [&](int j) { return tok[j]; }, [&](int j) { return col[j]; });
+                };
+                if (total <= 64) {
+#pragma unroll 1
+                    for (int e0 = lane; e0 < total; e0 += 32)
+                        flat(Count<1>(), e0);
+                } else {
+#pragma unroll 1
+                    for (int e0 = lane; e0 < total; e0 += 128)
+                        flat(Count<4>(), e0);
+                }
             }
             if (trace)
                 trace[6] = globaltimer_ns();

@@ -585,8 +585,8 @@ static int create_layer(int d, int F, int E, int k, int C, int fmt, melinoe_moe_
     CR(cudaMalloc(&h->cache, sizeof(DevCache)));
     CR(cudaMalloc(&h->plan, sizeof(DevPlan)));
     CR(cudaMalloc(&h->err_word, 256));
-    CR(cudaMalloc(&h->sync, 256));
-    CR(cudaMemset(h->sync, 0, 256));
+    CR(cudaMalloc(&h->sync, kSyncCounters * kSyncPitch * sizeof(unsigned)));
+    CR(cudaMemset(h->sync, 0, kSyncCounters * kSyncPitch * sizeof(unsigned)));
     CR(cudaMalloc(&h->shared_dev, sizeof(char *) * kMaxShared));
     CR(cudaMalloc(&h->host_dev, sizeof(char *) * kMaxExperts));
     CR(cudaMemset(h->host_dev, 0, sizeof(char *) * kMaxExperts));

@@ -637,8 +637,8 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
             for (size_t i = (size_t)blockIdx.x * kThreads + tid; i < (size_t)Tc * d; i += (size_t)G * kThreads)
                 p.out[(size_t)tok0 * d + i] = 0;
         // the counters advance once per CTA and launch, whatever happens
-        if (tid < NW && atomicAdd(p.sync + tid, 1u) == (unsigned)(G - 1))
-            p.sync[tid] = 0u;
+        if (tid < NW && atomicAdd(p.sync + tid * kSyncPitch, 1u) == (unsigned)(G - 1))
+            p.sync[tid * kSyncPitch] = 0u;
         return;
     }
     if (XT) {
@@ -981,14 +981,14 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
         if (lane == 0) {
             // (the warp barrier orders the other lanes' adds before lane 0's fence, which is cumulative)
             __threadfence();
-            ticket = atomicAdd(p.sync + warp, 1u);
+            ticket = atomicAdd(p.sync + warp * kSyncPitch, 1u);
         }
         ticket = __shfl_sync(0xffffffffu, ticket, 0);
         if (trace && tid == 0)
             trace[4] = globaltimer_ns();
         if (ticket == (unsigned)(G - 1)) {
             if (lane == 0)
-                p.sync[warp] = 0u;                // the counter is back at zero for the next launch
+                p.sync[warp * kSyncPitch] = 0u;   // the counter is back at zero for the next launch
             __threadfence();
             if (trace)
                 trace[5] = globaltimer_ns();
@@ -1085,9 +1085,9 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
     __syncthreads();
     if (tid == 0) {
         __threadfence();
-        s_last = atomicAdd(p.sync + NW, 1u) == (unsigned)(G - 1);
+        s_last = atomicAdd(p.sync + NW * kSyncPitch, 1u) == (unsigned)(G - 1);
         if (s_last)
-            p.sync[NW] = 0u;
+            p.sync[NW * kSyncPitch] = 0u;
     }
     __syncthreads();
     if (s_last && tid == 0) {

@@ -119,6 +119,9 @@ struct DecParams {
     int fmt;                         // 0: bf16 blobs, 1: 4-bit blobs
     int fast;                        // the launch's requests are plan->fast (planned by the fused planner for this launch)
 };
+// The counters of DecParams::sync, a cache line each: where the CTAs end together, sixteen counters in one line cost a
+// short launch about a microsecond.
+constexpr int kSyncPitch = 32, kSyncCounters = 17;
 struct DecLaunchCfg {
     int grid;                        // one CTA per SM
     size_t max_smem;                 // dynamic shared memory the kernel may use

@@ -56,6 +56,18 @@ def test_shapes_and_token_counts(d, F, E, k, C):
     P.close()
 
 
+@pytest.mark.parametrize("d,E,k,n_seq", [(4096, 6, 2, 40), (2048, 33, 2, 32), (256, 64, 8, 33), (2304, 3, 1, 5)])
+def test_decode_router_over_its_token_groups_and_sequences(d, E, k, n_seq):
+    """The decode router's warps by experts and token groups, one and two halves of a row, more sequences than lanes:
+    logits, indices and traces bit for bit with every expert resident (more pairs than slots, no more experts)."""
+    P = _pair(d, 16, E, k, E, seed=90 + E)
+    bias = _bias(90, E, 0.5, n_seq)
+    for step, T in enumerate((1, 2, 3, 5, 7, 8)):
+        P.set_bias(bias, ((np.arange(T) * 11 + n_seq - 1) % n_seq).astype(np.int32))
+        P.step(gen.hidden_states(90 + E, 0, "decode", step, T, d))
+    P.close()
+
+
 def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory():
     """d_model 4096 with 5 to 8 tokens per call: the decode kernel writes the hidden states' tensor-core
     operands into tensor memory once and reads them from there (the shared memory goes to taller weight
@@ -194,6 +206,9 @@ def test_prefill_grouped_gemm(d, F, E, k, C, n_shared, Ts):
     ("q4slots", 512, 200, 3, 3, 1, (9, 16, 129)),      # the same of 4-bit codes, with a shared expert
     ("q4slots", 1024, 264, 4, 2, 0, (70,)),            # codes of a column group in both halves of their 128 bytes
     ("q4slots", 4096, 136, 2, 1, 0, (20,)),
+    ("bf16", 2048, 1416, 2, 1, 1, (9, 140)),           # tiles computed in parts by many CTAs, the last part of GEMM 2 three k-blocks
+    ("q4slots", 2048, 1416, 2, 1, 1, (9, 300)),        # the same of 4-bit codes; chunks of up to 256 tokens
+    ("q4slots", 512, 64, 2, 2, 0, (256, 257)),         # one and two chunks; GEMM 2 of a single k-block
 ])
 def test_grouped_gemm_at_the_edges_of_its_tiles(store, d, F, E, k, n_shared, Ts):
     """Token counts around the steps of the tensor-core operation's N and d_ff that ends inside weight tiles and

@@ -75,13 +75,13 @@ constexpr int kRawBytes = 16384;           // 4-bit slots: codes of one fetch (G
 constexpr int kRawStages = 3;
 constexpr int kEpilogueWarps = 8;          // two per 32 accumulator rows, each with every other 16 tokens
 constexpr size_t kGemmSmem = 227 * 1024 - 4096;      // dynamic shared memory of a CTA (the static part is below 3 KB)
-// threads, tokens of a chunk at most, bytes and number of ring stages for CG CTAs per operation and slot format FMT
+// threads, tokens of a chunk at most, number of ring stages for CG CTAs per operation and slot format FMT
 __host__ __device__ constexpr int gemm_threads(int fmt) { return fmt ? 608 : 320; }
-__host__ __device__ constexpr int gemm_tokens(int cg, int fmt) { return cg == 2 || fmt ? 256 : 128; }
-__host__ __device__ constexpr int gemm_stage_bytes(int cg, int fmt) { return kABytes + gemm_tokens(cg, fmt) / cg * kBK * 2; }
-__host__ __device__ constexpr int gemm_stages(int cg, int fmt)
+__host__ __device__ constexpr int gemm_tokens(int cg) { return cg == 2 ? 256 : 128; }
+constexpr int kStageBytes = kABytes + 128 * kBK * 2;      // a CTA stages 128 tokens in both forms
+__host__ __device__ constexpr int gemm_stages(int fmt)
 {
-    return (int)((kGemmSmem - 1024 - (fmt ? kRawStages * kRawBytes : 0)) / gemm_stage_bytes(cg, fmt));
+    return (int)((kGemmSmem - 1024 - (fmt ? kRawStages * kRawBytes : 0)) / kStageBytes);
 }
 constexpr long long kGemmWaitCycles = 4000000000ll;
 
@@ -185,9 +185,23 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+// Arrival on the peer CTA's barrier.  What it reports is in this SM (expanded weights, behind a proxy fence; accumulators
+// drained or filled, behind tcgen05.wait), so nothing has to be made visible through memory: with release semantics
+// of cluster scope each arrival took its warp 1100 cycles.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar)
 {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r));
+    return r != 0;
 }
 __device__ __forceinline__ void cluster_sync_all()
 {
@@ -379,19 +393,22 @@ struct GemmWalk {
 // (Dealing out rows of weights instead was slower than whole tiles: a short tile's k-blocks take as long as a
 // whole one's.)
 // A k-block's cost: reading the weights (16-bit), which tokens hardly add to, or expanding them.
-__device__ __forceinline__ int gemm_item_cost(int chunk, int fmt) { return (fmt ? 8 : 16) + (chunk + 31) / 32; }
-template <int NT, int kMTile, int FMT>
+__device__ __forceinline__ int gemm_item_cost(int chunk, int fmt)
+{
+    return fmt ? 20 + (chunk + 31) / 32 + (chunk <= 64 ? 2 : chunk <= 128 ? 4 : 8) : 16 + (chunk + 31) / 32;
+}
+template <int CG, int NT, int kMTile, int FMT>
 struct GemmSplit {
     const int4 *rec;
     const int *item0, *cost0;      // first item of every request, and its place on the line of costs
-    int n_reqs, kblocks, quads, units, unit;
+    int n_reqs, kblocks, quads, units, unit, rank;
     int w_lo, q_lo, w_hi, q_hi, cur, step;
-    __device__ GemmSplit(const int4 *rec_, const int *item0_, const int *cost0_, int n_reqs_, int unit_, int n_ctas, int, int kblocks_)
-        : rec(rec_), item0(item0_), cost0(cost0_), n_reqs(n_reqs_), kblocks(kblocks_), quads((kblocks_ + 3) / 4), unit(unit_), step(0)
+    __device__ GemmSplit(const int4 *rec_, const int *item0_, const int *cost0_, int n_reqs_, int unit_, int n_units, int rank_, int kblocks_)
+        : rec(rec_), item0(item0_), cost0(cost0_), n_reqs(n_reqs_), kblocks(kblocks_), quads((kblocks_ + 3) / 4), unit(unit_), rank(rank_), step(0)
     {
         // no more CTAs than there are tiles, or pieces of two quads
         const int items = item0[n_reqs];
-        units = min(n_ctas, max(items, items * quads / 2));
+        units = min(n_units, max(items, items * quads / 2));
         locate(unit, w_lo, q_lo);
         locate(unit + 1, w_hi, q_hi);
         cur = w_lo + (q_lo > 0 ? 1 : 0);
@@ -422,10 +439,10 @@ struct GemmSplit {
                 q += s;
         const int4 r = rec[q];
         const int local = w - item0[q], n = (r.y + NT - 1) / NT, c = local % n;
-        it.m0 = local / n * kMTile;
+        it.m0 = (local / n * CG + rank) * kMTile;
         it.row0 = r.x + c * r.w;
         it.n_live = min(r.w, r.y - c * r.w);
-        it.n = (it.n_live + 15) / 16 * 16;
+        it.n = (it.n_live + 16 * CG - 1) / (16 * CG) * (16 * CG);
         it.slot = r.z;
         it.k0 = 4 * qa;
         it.k1 = min(4 * qb, kblocks);
@@ -472,10 +489,10 @@ struct GemmSplit {
 };
 template <int CG, int NT, int kMTile, int FMT>
 struct GemmItems {
-    using type = GemmSplit<NT, kMTile, FMT>;
+    using type = GemmSplit<CG, NT, kMTile, FMT>;
 };
-template <int NT, int kMTile, int FMT>
-struct GemmItems<2, NT, kMTile, FMT> {
+template <int NT, int kMTile>
+struct GemmItems<2, NT, kMTile, 0> {
     using type = GemmWalk<NT, kMTile>;
 };
 
@@ -483,8 +500,9 @@ struct GemmItems<2, NT, kMTile, FMT> {
 template <int PHASE, int CG, int FMT>
 __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmParams p)
 {
-    static_assert(FMT == 0 || CG == 1, "4-bit slots: single CTAs");
-    constexpr int kStages = gemm_stages(CG, FMT), kStageBytes = gemm_stage_bytes(CG, FMT), NT = gemm_tokens(CG, FMT);
+    static_assert(FMT == 0 || CG == 2, "4-bit slots: CTA pairs");
+    constexpr int kStages = gemm_stages(FMT), NT = gemm_tokens(CG);
+    constexpr bool kSplit = CG == 1 || FMT == 1;             // tiles may be computed in parts
     constexpr int kMTile = PHASE == 1 ? 64 : 128;            // hidden units, or output columns, of one CTA's tile
     constexpr int kRawBlocks = PHASE == 1 ? 4 : 2;           // k-blocks of one fetch of codes
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -513,14 +531,14 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     if (tid == 32) {
         s_abort = 0;
         for (int i = 0; i < kStages; ++i) {
-            mbar_init(full0 + 8 * i, FMT ? 5 : 1);
+            mbar_init(full0 + 8 * i, FMT ? 1 + 4 * CG : 1);
             mbar_init(empty0 + 8 * i, 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(tfull0 + 8 * i, 1);
             mbar_init(tempty0 + 8 * i, kEpilogueWarps * CG);
         }
-        mbar_init(tinit, kEpilogueWarps);
+        mbar_init(tinit, kEpilogueWarps * CG);
         if (FMT)
             for (int i = 0; i < kRawStages; ++i) {
                 mbar_init(rfull0 + 8 * i, 1);
@@ -558,7 +576,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 items = on ? chunks * m_tiles : 0;
             }
             const unsigned m = __ballot_sync(0xffffffffu, on);
-            const int cost = CG == 1 ? items * gemm_item_cost(rec.w, FMT) * ((kblocks + 3) / 4) : 0;
+            const int cost = kSplit ? items * gemm_item_cost(rec.w, FMT) * ((kblocks + 3) / 4) : 0;
             int inc = items, inc_c = cost;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -623,14 +641,11 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 // the weights of the slots, or of the shared expert
                 const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
                 const int slot = it.slot >= 0 ? it.slot : 0;
-                // the smallest box that holds this CTA's share of the tokens: 32, 64 or 128 rows, or two of 128
+                // the smallest box that holds this CTA's share of the tokens: 32, 64 or 128 rows
                 const int rows = it.n / CG, cls = rows <= 32 ? 0 : rows <= 64 ? 1 : 2;
                 const int b_row = it.row0 + (int)rank * rows;
-                const bool two = NT / CG > 128 && rows > 128;
-                const uint32_t bytes = (FMT ? 0u : (uint32_t)kABytes) + ((32u * kBK * 2) << (two ? 3 : cls));
+                const uint32_t bytes = (FMT ? 0u : (uint32_t)kABytes) + ((32u * kBK * 2) << cls);
                 auto load_a = [&](int kb, uint32_t dst, uint32_t bar) {
-                    if (FMT)
-                        return;
                     if (PHASE == 1)
                         tma_load_4d(dst, map_w, kb * kBK, 0, 0, (slot * p.F + it.m0) / 8, bar);
                     else
@@ -638,8 +653,6 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 };
                 auto load_b = [&](int kb, uint32_t dst, uint32_t bar) {
                     tma_load_2d(dst, map_b + cls, kb * kBK, b_row, bar);
-                    if (two)
-                        tma_load_2d(dst + 128 * kBK * 2, map_b + cls, kb * kBK, b_row + 128, bar);
                 };
                 int kb0 = it.k0;
                 if (CG == 1 && !waited) {
@@ -673,7 +686,9 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                         const uint32_t bar = cluster_addr(full0 + 8 * s, 0);
                         if (rank == 0)
                             mbar_expect(full0 + 8 * s, 2 * bytes);
-                        if (PHASE == 1)
+                        if (FMT == 1)
+                            ;            // (the weights come from the expanding warps)
+                        else if (PHASE == 1)
                             tma_load_4d_pair(a_dst, map_w, kb * kBK, 0, 0, (slot * p.F + it.m0) / 8, bar);
                         else
                             tma_load_4d_pair(a_dst, map_w, 0, kb * kBK, it.m0 / 64, slot, bar);
@@ -690,54 +705,68 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         }
     } else if (warp == 1) {
         // ============================================================ MMA issuer (of a pair: the even CTA's)
-        if (lane == 0 && rank == 0) {
-            uint32_t n = 0, item = 0;
+        // The whole warp goes through the loop and one lane issues: values that are the same in all lanes stay in uniform
+        // registers, where the tensor-core instructions want them.
+        if (rank == 0) {
+            uint32_t s = 0, parity = 0, item = 0;
             auto items = walk();
-            for (; !*abort_flag && items.next(it); ++item) {
-                const uint32_t idesc = instr_desc_bf16(CG * 128, it.n, PHASE == 2);
-                const uint32_t acc = item & 1u;
-                if (item >= 2 && !mbar_wait(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag))
+            const uint32_t ring_d = (ring_s & 0x3FFFFu) >> 4;
+            const uint64_t a_hi = (PHASE == 1 ? smem_desc_sw128(0) : smem_desc_sw128_mmajor(0)), b_hi = smem_desc_sw128(0);
+            for (;; ++item) {
+                const bool more = !*abort_flag && items.next(it);
+                if (!__all_sync(0xffffffffu, more))
                     break;
+                const int k0 = __shfl_sync(0xffffffffu, it.k0, 0), k1 = __shfl_sync(0xffffffffu, it.k1, 0);
+                const uint32_t idesc = instr_desc_bf16(CG * 128, __shfl_sync(0xffffffffu, it.n, 0), PHASE == 2);
+                const uint32_t acc = item & 1u;
                 // a tile whose first parts other CTAs computed starts from their sums
-                const bool merge = CG == 1 && it.k0 > 0 && it.k1 == kblocks;
-                if (merge && !mbar_wait(tinit, 0, abort_flag))
+                const bool merge = kSplit && k0 > 0 && k1 == kblocks;
+                bool ok = item < 2 || mbar_wait(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag);
+                if (merge)
+                    ok = ok && mbar_wait(tinit, 0, abort_flag);
+                if (!__all_sync(0xffffffffu, ok))
                     break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d_tmem = tmem_base + acc * NT;
-                bool ok = true;
-                for (int kb = it.k0; kb < it.k1; ++kb, ++n) {
-                    const uint32_t s = n % kStages;
-                    if (!mbar_wait(full0 + 8 * s, (n / kStages) & 1u, abort_flag)) {
-                        ok = false;
+                uint32_t accumulate = merge ? 1u : 0u;
+                for (int kb = k0; kb < k1; ++kb) {
+                    ok = mbar_wait(full0 + 8 * s, parity, abort_flag);
+                    if (!__all_sync(0xffffffffu, ok))
                         break;
-                    }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a_addr = ring_s + s * kStageBytes, b_addr = a_addr + kABytes;
-                    const uint64_t a_desc = PHASE == 1 ? smem_desc_sw128(a_addr) : smem_desc_sw128_mmajor(a_addr);
-                    const uint64_t b_desc = smem_desc_sw128(b_addr);
+                    const uint64_t a_desc = a_hi | (ring_d + s * (kStageBytes >> 4));
+                    const uint64_t b_desc = b_hi | (ring_d + s * (kStageBytes >> 4) + (kABytes >> 4));
                     // 16 K elements: 32 bytes along a K-major row (2 descriptor units), 16 rows of 128 bytes
                     // in an M-major box (128 units)
                     constexpr int kAStep = PHASE == 1 ? 2 : 128;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < kBK / 16; ++ks) {
+                        for (int ks = 0; ks < kBK / 16; ++ks) {
+                            if (CG == 1)
+                                umma_bf16(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, ks ? 1u : accumulate);
+                            else
+                                umma_bf16_pair(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, ks ? 1u : accumulate);
+                        }
+                        // the stage is free once these MMAs have read it
                         if (CG == 1)
-                            umma_bf16(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, merge || kb != it.k0 || ks != 0);
+                            umma_commit(empty0 + 8 * s);
                         else
-                            umma_bf16_pair(d_tmem, a_desc + kAStep * ks, b_desc + 2 * ks, idesc, merge || kb != it.k0 || ks != 0);
+                            umma_commit_pair(empty0 + 8 * s);
+                        // the accumulator is complete
+                        if (kb + 1 == k1) {
+                            if (CG == 1)
+                                umma_commit(tfull0 + 8 * acc);
+                            else
+                                umma_commit_pair(tfull0 + 8 * acc);
+                        }
                     }
-                    // the stage is free once these MMAs have read it
-                    if (CG == 1)
-                        umma_commit(empty0 + 8 * s);
-                    else
-                        umma_commit_pair(empty0 + 8 * s);
+                    __syncwarp();
+                    accumulate = 1u;
+                    if (++s == (uint32_t)kStages) {
+                        s = 0;
+                        parity ^= 1u;
+                    }
                 }
-                if (!ok)
-                    break;
-                // the accumulator is complete
-                if (CG == 1)
-                    umma_commit(tfull0 + 8 * acc);
-                else
-                    umma_commit_pair(tfull0 + 8 * acc);
             }
         }
     } else if (warp < 2 + kEpilogueWarps) {
@@ -751,10 +780,10 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         // sums of the CTAs with the earlier parts of a tile ([token][row] of fp32 per CTA, and a word per CTA and
         // quarter that says they are there) into the accumulator that the tile will use
         auto preload = [&](const GemmItem &nx, uint32_t acc) {
-            if constexpr (CG == 1) {
+            if constexpr (kSplit) {
                 const unsigned long long others = items.partners();
                 for (unsigned long long m = others; m; m &= m - 1) {
-                    const unsigned *flag = p.flags + (blockIdx.x - __ffsll((long long)m)) * kEpilogueWarps + (warp - 2);
+                    const unsigned *flag = p.flags + (blockIdx.x - CG * __ffsll((long long)m)) * kEpilogueWarps + (warp - 2);
                     const long long c0 = clock64();
                     for (;;) {
                         unsigned v;
@@ -777,7 +806,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     for (int i = 63 - __clzll((long long)others); i >= 0; --i) {
                         if (!((others >> i) & 1ull))
                             continue;
-                        const float *src = p.partial + ((size_t)(blockIdx.x - 1 - i) * p.part_tokens + c) * 128 + quarter * 32 + lane;
+                        const float *src = p.partial + ((size_t)(blockIdx.x - CG * (1 + i)) * p.part_tokens + c) * 128 + quarter * 32 + lane;
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
                             sum[j] += __ldcg(src + j * 128);      // (tokens that do not exist: whatever is there)
@@ -787,20 +816,24 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
-                if (lane == 0)
-                    mbar_arrive(tinit);
+                if (lane == 0) {
+                    if (CG == 1 || rank == 0)
+                        mbar_arrive(tinit);
+                    else
+                        mbar_arrive_cluster(cluster_addr(tinit, 0));
+                }
             }
         };
         GemmItem nx;
         bool more = items.next(nx);
-        if (more && CG == 1 && nx.k0 > 0 && nx.k1 == kblocks)
+        if (more && kSplit && nx.k0 > 0 && nx.k1 == kblocks)
             preload(nx, 0);
         for (; !*abort_flag && more; ++item) {
             it = nx;
             const uint32_t acc = item & 1u;
             more = items.next(nx);
             // (the other accumulator was drained before this item; a part that this CTA owes another goes out first)
-            const bool owed = CG == 1 && it.k1 < kblocks, merge_next = CG == 1 && more && nx.k0 > 0 && nx.k1 == kblocks;
+            const bool owed = kSplit && it.k1 < kblocks, merge_next = kSplit && more && nx.k0 > 0 && nx.k1 == kblocks;
             if (merge_next && !owed)
                 preload(nx, acc ^ 1u);
             if (!mbar_wait(tfull0 + 8 * acc, (item >> 1) & 1u, abort_flag))
@@ -966,8 +999,12 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the tensor cores read what was just stored
                 __syncwarp();
-                if (lane == 0)
-                    mbar_arrive(full0 + 8 * s);
+                if (lane == 0) {
+                    if (rank == 0)
+                        mbar_arrive(full0 + 8 * s);
+                    else
+                        mbar_arrive_cluster(cluster_addr(full0 + 8 * s, 0));
+                }
                 }
                 if (lane == 0)
                     mbar_arrive(rempty0 + 8 * rs);
@@ -1161,33 +1198,33 @@ cudaError_t launch_after(cudaStream_t stream, void (*kernel)(Params...), dim3 gr
     return e;
 }
 
-constexpr size_t gemm_smem(int cg, int fmt)
+constexpr size_t gemm_smem(int fmt)
 {
-    return (size_t)gemm_stages(cg, fmt) * gemm_stage_bytes(cg, fmt) + (fmt ? kRawStages * kRawBytes : 0) + 1024;
+    return (size_t)gemm_stages(fmt) * kStageBytes + (fmt ? kRawStages * kRawBytes : 0) + 1024;
 }
 
 template <int PHASE, int CG, int FMT>
 cudaError_t gemm_launch(cudaStream_t stream, int n_sms, const GemmParams &p)
 {
-    return launch_after(stream, ffn_gemm_kernel<PHASE, CG, FMT>, dim3(n_sms / CG * CG), gemm_threads(FMT), gemm_smem(CG, FMT), CG, p);
+    return launch_after(stream, ffn_gemm_kernel<PHASE, CG, FMT>, dim3(n_sms / CG * CG), gemm_threads(FMT), gemm_smem(FMT), CG, p);
 }
 
 template <int PHASE, int CG, int FMT>
 cudaError_t gemm_configure()
 {
-    return cudaFuncSetAttribute(ffn_gemm_kernel<PHASE, CG, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(CG, FMT));
+    return cudaFuncSetAttribute(ffn_gemm_kernel<PHASE, CG, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(FMT));
 }
 
 }  // namespace
 
-int ffn_gemm_part_tokens(int fmt) { return gemm_tokens(1, fmt); }
+int ffn_gemm_part_tokens(int fmt) { return gemm_tokens(fmt ? 2 : 1); }
 
 bool ffn_gemm_supported(int d, int F) { return d % 256 == 0 && F % kUnitRows == 0; }
 
 cudaError_t ffn_gemm_configure()
 {
     const cudaError_t e[6] = {gemm_configure<1, 1, 0>(), gemm_configure<2, 1, 0>(), gemm_configure<1, 2, 0>(),
-                              gemm_configure<2, 2, 0>(), gemm_configure<1, 1, 1>(), gemm_configure<2, 1, 1>()};
+                              gemm_configure<2, 2, 0>(), gemm_configure<1, 2, 1>(), gemm_configure<2, 2, 1>()};
     for (cudaError_t r : e)
         if (r != cudaSuccess)
             return r;
@@ -1207,7 +1244,7 @@ cudaError_t launch_gather_rows(cudaStream_t stream, int n_sms, const GatherParam
 cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, int fmt, const GemmParams &p)
 {
     if (fmt == 1)
-        return phase == 1 ? gemm_launch<1, 1, 1>(stream, n_sms, p) : gemm_launch<2, 1, 1>(stream, n_sms, p);
+        return phase == 1 ? gemm_launch<1, 2, 1>(stream, n_sms, p) : gemm_launch<2, 2, 1>(stream, n_sms, p);
     if (pairs)
         return phase == 1 ? gemm_launch<1, 2, 0>(stream, n_sms, p) : gemm_launch<2, 2, 0>(stream, n_sms, p);
     return phase == 1 ? gemm_launch<1, 1, 0>(stream, n_sms, p) : gemm_launch<2, 1, 0>(stream, n_sms, p);

@@ -133,22 +133,22 @@ __device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// Tiled TMA loads: box at the given coordinates (innermost first) of the tensor map into shared memory.  The _pair
-// forms are those of a CTA pair, whose completion may be counted on the peer CTA's barrier (bar is an address in
-// the cluster's shared window).
+// Tiled TMA loads: box at the given coordinates (innermost first) of the tensor map into shared memory.  The forms of a
+// CTA pair (CG = 2) may count their completion on the peer CTA's barrier (bar is an address in the
+// cluster's shared window).
+template <int CG>
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar)
 {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
-        : "memory");
+    if (CG == 1)
+        asm volatile(
+            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+            ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
+            : "memory");
+    else
+        asm volatile(
+            "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+            ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
+            : "memory");
 }
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar)
 {
@@ -157,19 +157,19 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
 }
+template <int CG>
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, int w, uint32_t bar)
 {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap *map, int x, int y, int z, int w, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
-        : "memory");
+    if (CG == 1)
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+            ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+            : "memory");
+    else
+        asm volatile(
+            "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+            ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+            : "memory");
 }
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, int w, int v, uint32_t bar)
 {
@@ -631,77 +631,80 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     GemmItem it;
 
     if (warp == 0) {
-        // ============================================================ TMA producer
-        if (lane == 0) {
-            const CUtensorMap *map_b = p.maps + (PHASE == 1 ? kMapXs0 : kMapHs0);
-            uint32_t n = 0;
-            bool waited = false;
-            auto items = walk();
-            while (!*abort_flag && items.next(it)) {
-                // the weights of the slots, or of the shared expert
-                const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
-                const int slot = it.slot >= 0 ? it.slot : 0;
-                // the smallest box that holds this CTA's share of the tokens: 32, 64 or 128 rows
-                const int rows = it.n / CG, cls = rows <= 32 ? 0 : rows <= 64 ? 1 : 2;
-                const int b_row = it.row0 + (int)rank * rows;
-                const uint32_t bytes = (FMT ? 0u : (uint32_t)kABytes) + ((32u * kBK * 2) << cls);
-                auto load_a = [&](int kb, uint32_t dst, uint32_t bar) {
-                    if (PHASE == 1)
-                        tma_load_4d(dst, map_w, kb * kBK, 0, 0, (slot * p.F + it.m0) / 8, bar);
-                    else
-                        tma_load_4d(dst, map_w, 0, kb * kBK, it.m0 / 64, slot, bar);
-                };
-                auto load_b = [&](int kb, uint32_t dst, uint32_t bar) {
-                    tma_load_2d(dst, map_b + cls, kb * kBK, b_row, bar);
-                };
-                int kb0 = it.k0;
-                if (CG == 1 && !waited) {
-                    // the first stages' weights are on their way while the kernel ahead finishes
-                    const int pre = min(it.k1 - it.k0, kStages);
+        // ============================================================ TMA producer (the whole warp, one lane issues)
+        const CUtensorMap *map_b = p.maps + (PHASE == 1 ? kMapXs0 : kMapHs0);
+        // of a pair, the bytes of both CTAs are expected and counted on the even CTA's barriers
+        const uint32_t full_b = CG == 1 ? full0 : cluster_addr(full0, 0);
+        uint32_t s = 0, parity = 1, n = 0;
+        bool waited = false;
+        auto items = walk();
+        for (;;) {
+            const bool more = !*abort_flag && items.next(it);
+            if (!__all_sync(0xffffffffu, more))
+                break;
+            const int k0 = __shfl_sync(0xffffffffu, it.k0, 0), k1 = __shfl_sync(0xffffffffu, it.k1, 0);
+            const int m0 = __shfl_sync(0xffffffffu, it.m0, 0), item_slot = __shfl_sync(0xffffffffu, it.slot, 0);
+            // the weights of the slots, or of the shared expert
+            const CUtensorMap *map_w = p.maps + (item_slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - item_slot)) + (PHASE - 1);
+            const int slot = item_slot >= 0 ? item_slot : 0;
+            // the smallest box that holds this CTA's share of the tokens: 32, 64 or 128 rows
+            const int rows = __shfl_sync(0xffffffffu, it.n, 0) / CG, cls = rows <= 32 ? 0 : rows <= 64 ? 1 : 2;
+            const int b_row = __shfl_sync(0xffffffffu, it.row0, 0) + (int)rank * rows;
+            const uint32_t bytes = CG * ((FMT ? 0u : (uint32_t)kABytes) + ((32u * kBK * 2) << cls));
+            auto load_a = [&](int kb, uint32_t dst, uint32_t bar) {
+                if (FMT == 1)
+                    return;                 // (the weights come from the expanding warps)
+                if (PHASE == 1)
+                    tma_load_4d<CG>(dst, map_w, kb * kBK, 0, 0, (slot * p.F + m0) / 8, bar);
+                else
+                    tma_load_4d<CG>(dst, map_w, 0, kb * kBK, m0 / 64, slot, bar);
+            };
+            auto load_b = [&](int kb, uint32_t dst, uint32_t bar) { tma_load_2d<CG>(dst, map_b + cls, kb * kBK, b_row, bar); };
+            int kb = k0;
+            if (!waited) {
+                // single CTAs: the first stages' weights are on their way while the kernel ahead finishes
+                const int pre = CG == 1 ? min(k1 - k0, kStages) : 0;
+                if (CG == 1 && elect_one())
                     for (int i = 0; i < pre; ++i) {
                         mbar_expect(full0 + 8 * i, bytes);
-                        load_a(it.k0 + i, ring_s + i * kStageBytes, full0 + 8 * i);
+                        load_a(k0 + i, ring_s + i * kStageBytes, full0 + 8 * i);
                     }
-                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                __syncwarp();
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                if (CG == 1 && elect_one())
                     for (int i = 0; i < pre; ++i)
-                        load_b(it.k0 + i, ring_s + i * kStageBytes + kABytes, full0 + 8 * i);
-                    n = pre;
-                    kb0 += pre;
-                } else if (!waited) {
-                    asm volatile("griddepcontrol.wait;" ::: "memory");
-                }
+                        load_b(k0 + i, ring_s + i * kStageBytes + kABytes, full0 + 8 * i);
+                __syncwarp();
+                kb += pre;
+                n = pre;
+                s = pre % kStages;
+                parity ^= pre / kStages;
                 waited = true;
-                for (int kb = kb0; kb < it.k1; ++kb, ++n) {
-                    const uint32_t s = n % kStages;
-                    if (n >= (uint32_t)kStages && !mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag))
-                        break;
-                    const uint32_t a_dst = ring_s + s * kStageBytes, b_dst = a_dst + kABytes;
-                    if (CG == 1) {
-                        const uint32_t bar = full0 + 8 * s;
-                        mbar_expect(bar, bytes);
-                        load_a(kb, a_dst, bar);
-                        load_b(kb, b_dst, bar);
-                    } else {
-                        // the bytes of both CTAs are expected, once, on the even CTA's barrier
-                        const uint32_t bar = cluster_addr(full0 + 8 * s, 0);
-                        if (rank == 0)
-                            mbar_expect(full0 + 8 * s, 2 * bytes);
-                        if (FMT == 1)
-                            ;            // (the weights come from the expanding warps)
-                        else if (PHASE == 1)
-                            tma_load_4d_pair(a_dst, map_w, kb * kBK, 0, 0, (slot * p.F + it.m0) / 8, bar);
-                        else
-                            tma_load_4d_pair(a_dst, map_w, 0, kb * kBK, it.m0 / 64, slot, bar);
-                        tma_load_2d_pair(b_dst, map_b + cls, kb * kBK, b_row, bar);
-                    }
+            }
+            for (; kb < k1; ++kb, ++n) {
+                // (a fresh barrier counts as being past its odd phase)
+                const bool ok = mbar_wait(empty0 + 8 * s, parity, abort_flag);
+                if (!__all_sync(0xffffffffu, ok))
+                    break;
+                if (elect_one()) {
+                    const uint32_t a_dst = ring_s + s * kStageBytes, bar = full_b + 8 * s;
+                    if (CG == 1 || rank == 0)
+                        mbar_expect(full0 + 8 * s, bytes);
+                    load_a(kb, a_dst, bar);
+                    load_b(kb, a_dst + kABytes, bar);
+                }
+                __syncwarp();
+                if (++s == (uint32_t)kStages) {
+                    s = 0;
+                    parity ^= 1u;
                 }
             }
-            if (CG == 2) {
-                // The MMA thread's commits arrive on this CTA's barriers from outside: wait for the last
-                // ones so that none is still under way when the CTA ends.
-                for (uint32_t j = n > (uint32_t)kStages ? n - kStages : 0; j < n && !*abort_flag; ++j)
-                    mbar_wait(empty0 + 8 * (j % kStages), (j / kStages) & 1u, abort_flag);
-            }
+        }
+        if (CG == 2) {
+            // The MMA thread's commits arrive on this CTA's barriers from outside: wait for the last
+            // ones so that none is still under way when the CTA ends.
+            for (uint32_t j = n > (uint32_t)kStages ? n - kStages : 0; j < n && !*abort_flag; ++j)
+                mbar_wait(empty0 + 8 * (j % kStages), (j / kStages) & 1u, abort_flag);
         }
     } else if (warp == 1) {
         // ============================================================ MMA issuer (of a pair: the even CTA's)

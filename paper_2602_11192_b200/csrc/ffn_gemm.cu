@@ -74,9 +74,10 @@ constexpr int kABytes = 128 * kBK * 2;     // weight tile of a stage: 128 rows
 constexpr int kRawBytes = 16384;           // 4-bit slots: codes of one fetch (GEMM 1: 256 columns of 128 rows; GEMM 2: 128 rows f of 256 columns)
 constexpr int kRawStages = 3;
 constexpr int kEpilogueWarps = 8;          // two per 32 accumulator rows, each with every other 16 tokens
+constexpr int kExpandGroups = 4;           // 4-bit slots: groups of four warps that expand k-blocks in turn
 constexpr size_t kGemmSmem = 227 * 1024 - 4096;      // dynamic shared memory of a CTA (the static part is below 3 KB)
 // threads, tokens of a chunk at most, number of ring stages for CG CTAs per operation and slot format FMT
-__host__ __device__ constexpr int gemm_threads(int fmt) { return fmt ? 608 : 320; }
+__host__ __device__ constexpr int gemm_threads(int fmt) { return 32 * (2 + kEpilogueWarps + (fmt ? 4 * kExpandGroups + 1 : 0)); }
 __host__ __device__ constexpr int gemm_tokens(int cg) { return cg == 2 ? 256 : 128; }
 constexpr int kStageBytes = kABytes + 128 * kBK * 2;      // a CTA stages 128 tokens in both forms
 __host__ __device__ constexpr int gemm_stages(int fmt)
@@ -542,7 +543,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         if (FMT)
             for (int i = 0; i < kRawStages; ++i) {
                 mbar_init(rfull0 + 8 * i, 1);
-                mbar_init(rempty0 + 8 * i, 8);
+                mbar_init(rempty0 + 8 * i, 4 * kExpandGroups);
             }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -921,8 +922,8 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     mbar_arrive_cluster(cluster_addr(tempty0 + 8 * acc, 0));
             }
         }
-    } else if (FMT == 1 && warp < 18) {
-        // ============================================================ expansion of 4-bit codes (warps 10..17)
+    } else if (FMT == 1 && warp < 2 + kEpilogueWarps + 4 * kExpandGroups) {
+        // ============================================================ expansion of 4-bit codes (warps 10..25)
         // Two groups of four warps take the k-blocks in turn: what a k-block takes is latency (waits, the fence before the
         // tensor cores may read), which the other group's k-block covers.  (Eight warps on every k-block: 0.6 us each, as
         // with four.)
@@ -943,12 +944,12 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     return f_row < p.F && kb < kblocks ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base) + kb) : 0u;
                 return kb * kBK + f_row < p.F ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base + (size_t)kb * kBK * ub)) : 0u;
             };
-            uint32_t sc = scale_of(it.k0 + group);
+            uint32_t sc = scale_of(it.k0 + group);      // (runs begin at multiples of 4 k-blocks)
             bool ok = true;
             for (int kr = it.k0; kr < it.k1 && ok; kr += kRawBlocks, ++rn) {
                 const uint32_t rs = rn % kRawStages;
                 ok = mbar_wait(rfull0 + 8 * rs, (rn / kRawStages) & 1u, abort_flag);
-                for (int sub = group; sub < kRawBlocks && kr + sub < it.k1 && ok; sub += 2) {
+                for (int sub = (group - kr) & (kExpandGroups - 1); sub < kRawBlocks && kr + sub < it.k1 && ok; sub += kExpandGroups) {
                 const int kb = kr + sub;
                 const uint32_t n = n0 + (uint32_t)(kb - it.k0), s = n % kStages;
                 if (n >= (uint32_t)kStages)
@@ -956,7 +957,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 if (!ok)
                     break;
                 const uint32_t ss = sc * 0x10001u;
-                sc = scale_of(kb + 2);
+                sc = scale_of(kb + kExpandGroups);
                 const uint32_t raw = raw_s + rs * kRawBytes, a_dst = ring_s + s * kStageBytes + row * 128;
                 const uint32_t x = (uint32_t)(row & 7);      // = f mod 8 in both phases
                 if (PHASE == 1) {
@@ -1014,7 +1015,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
             }
             n0 += (uint32_t)(it.k1 - it.k0);
         }
-    } else if (FMT == 1 && warp == 18) {
+    } else if (FMT == 1 && warp == 2 + kEpilogueWarps + 4 * kExpandGroups) {
         // ============================================================ fetch of 4-bit codes
         if (lane == 0) {
             uint32_t rn = 0;

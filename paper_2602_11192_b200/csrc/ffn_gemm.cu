@@ -800,22 +800,39 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 }
                 __syncwarp();
                 const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * NT;
+                // (64 tokens a time, so that two chunks' loads are in flight; with 4-bit slots registers do for one)
+                constexpr int kAhead = FMT ? 1 : 2;
 #pragma unroll 1
-                for (int c = c_first; c < nx.n; c += 32) {
-                    float sum[16];
+                for (int c = c_first; c < nx.n; c += 32 * kAhead) {
+                    float sum[kAhead][16];
 #pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        sum[j] = 0.0f;
+                    for (int h = 0; h < kAhead; ++h)
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            sum[h][j] = 0.0f;
                     // (in ascending order of the CTAs, which is that of the k-blocks)
                     for (int i = 63 - __clzll((long long)others); i >= 0; --i) {
                         if (!((others >> i) & 1ull))
                             continue;
                         const float *src = p.partial + ((size_t)(blockIdx.x - CG * (1 + i)) * p.part_tokens + c) * 128 + quarter * 32 + lane;
+                        float o[kAhead][16];
 #pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            sum[j] += __ldcg(src + j * 128);      // (tokens that do not exist: whatever is there)
+                        for (int h = 0; h < kAhead; ++h)
+                            if (c + 32 * h < nx.n)
+#pragma unroll
+                                for (int j = 0; j < 16; ++j)
+                                    o[h][j] = __ldcg(src + (32 * h + j) * 128);      // (tokens that do not exist: whatever is there)
+#pragma unroll
+                        for (int h = 0; h < kAhead; ++h)
+                            if (c + 32 * h < nx.n)
+#pragma unroll
+                                for (int j = 0; j < 16; ++j)
+                                    sum[h][j] += o[h][j];
                     }
-                    tmem_st16(t_row + c, sum);
+#pragma unroll
+                    for (int h = 0; h < kAhead; ++h)
+                        if (c + 32 * h < nx.n)
+                            tmem_st16(t_row + c + 32 * h, sum[h]);
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

@@ -22,7 +22,7 @@
  *  - Environment switches, read once per process (for measurements and tests; none changes results):
  *    MELINOE_MOE_NO_PDL          launch the decode kernels without programmatic stream serialisation;
  *    MELINOE_MOE_HOST_COPIES     every expert transfer is a cudaMemcpyAsync issued by the host;
- *    MELINOE_MOE_GEMM_SINGLE     the prefill GEMM never pairs CTAs (tcgen05 cta_group::1 only).
+ *    MELINOE_MOE_GEMM_SINGLE     the prefill GEMM of bf16 slots never pairs CTAs (tcgen05 cta_group::1 only).
  */
 #ifndef MELINOE_MOE_H_
 #define MELINOE_MOE_H_

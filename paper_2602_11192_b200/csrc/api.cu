@@ -183,9 +183,6 @@ struct melinoe_moe {
     // grouped-GEMM path (calls of more than 8 tokens): gathered activations, h, tensor maps
     bool gemm_ok = false, last_used_gemm = false;
     uint16_t *xs = nullptr, *hs = nullptr;
-    float *partial = nullptr;              // GEMM tiles computed in parts: see GemmParams
-    unsigned *part_flags = nullptr, gemm_seq = 0;
-    int part_tokens = 0;
     CUtensorMap *maps_dev = nullptr;
     CUtensorMap maps_host[kMapCount];
     const void *shared_ptrs[kMaxShared] = {nullptr};
@@ -271,11 +268,7 @@ void free_scratch(melinoe_moe *h)
     cudaFree(h->stage_out);
     cudaFree(h->xs);
     cudaFree(h->hs);
-    cudaFree(h->partial);
-    cudaFree(h->part_flags);
     h->xs = h->hs = nullptr;
-    h->partial = nullptr;
-    h->part_flags = nullptr;
     o = Scratch{};
     h->last = Scratch{};
     h->zbuf = nullptr;
@@ -352,11 +345,6 @@ int ensure_capacity(melinoe_moe *h, int T)
         CU_TRY(cudaMalloc(&h->zbuf, sorted * h->d * sizeof(float)));
         CU_TRY(cudaMalloc(&h->xs, sorted * h->d * 2));
         CU_TRY(cudaMalloc(&h->hs, sorted * h->F * 2));
-        h->part_tokens = (cap + 31) / 32 * 32 < ffn_gemm_part_tokens(h->fmt) ? (cap + 31) / 32 * 32 : ffn_gemm_part_tokens(h->fmt);
-        CU_TRY(cudaMalloc(&h->partial, (size_t)h->n_sms * 128 * h->part_tokens * sizeof(float)));
-        CU_TRY(cudaMalloc(&h->part_flags, (size_t)h->n_sms * 8 * sizeof(unsigned)));
-        CU_TRY(cudaMemset(h->part_flags, 0, (size_t)h->n_sms * 8 * sizeof(unsigned)));
-        h->gemm_seq = 0;
         if (!encode_activation_maps(&h->maps_host[kMapXs0], h->xs, h->d, sorted) ||
             !encode_activation_maps(&h->maps_host[kMapHs0], h->hs, h->F, sorted))
             return MELINOE_ERR_CUDA;
@@ -1023,9 +1011,6 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     gp.slot_stride = h->slot_stride;
     gp.shared_blobs = h->shared_dev;
     gp.unit_bytes = (int)(h->expert_bytes / (size_t)h->F);
-    gp.partial = h->partial;
-    gp.flags = h->part_flags;
-    gp.part_tokens = h->part_tokens;
     auto launch_group = [&](int g) -> int {
         TimedPair tp{nullptr, nullptr};
         if (h->timing) {
@@ -1036,13 +1021,11 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         }
         if (use_gemm) {
             gp.group = g;
-            // CTA pairs take twice the tokens per weight tile: worth it where the arithmetic, not reading the weights, is
-            // the work; MELINOE_MOE_GEMM_SINGLE in the environment keeps the single-CTA form
+            // CTA pairs, for every size (see ffn_gemm.cu); MELINOE_MOE_GEMM_SINGLE in the environment keeps bf16 slots on
+            // single CTAs
             static const bool single_only = std::getenv("MELINOE_MOE_GEMM_SINGLE") != nullptr;
-            const bool pairs = !single_only && h->fmt == 0 && (long long)T * h->k >= 128ll * h->E;
-            gp.seq = ++h->gemm_seq;
+            const bool pairs = h->fmt != 0 || !single_only;
             CU_TRY(launch_ffn_gemm(s, 1, h->n_sms, pairs, h->fmt, gp));
-            gp.seq = ++h->gemm_seq;
             CU_TRY(launch_ffn_gemm(s, 2, h->n_sms, pairs, h->fmt, gp));
         } else {
             for (int c = 0; c < n_chunks; ++c) {

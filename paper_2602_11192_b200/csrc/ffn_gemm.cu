@@ -29,7 +29,7 @@
 //             d_ff is out of bounds there and reads as zero, so d_ff may end inside a stage.
 // The slots' experts are addressed through one tensor map per view, because the slots are contiguous.
 //
-// 4-bit slots (template parameter FMT = 1): TMA brings the codes into a ring of its own, and eight warps expand
+// 4-bit slots (template parameter FMT = 1): TMA brings the codes into a ring of its own, and sixteen warps expand
 // them into the weight tile of a stage (the arithmetic of the decode kernel: 15 instructions per 8
 // weights) in front of the tensor cores, so that HBM carries 4-bit data only and no bf16 copy of an expert
 // exists.  In GEMM 1 the expansion leaves elements j and j + 4 of eight side by side; a sum over K does not
@@ -37,15 +37,15 @@
 //
 // One persistent CTA per SM, warp-specialised: warp 0 issues TMA loads into a ring of stages, warp 1
 // issues the MMAs (one elected thread) and commits them to mbarriers, warps 2..9 drain
-// the accumulator (tcgen05.ld, 32 rows per warp) and write the tile; with 4-bit slots warps 10..17 expand and
-// warp 18 fetches codes.  Two accumulators alternate so the epilogue of a tile overlaps the MMAs of the next.
+// the accumulator (tcgen05.ld, 32 rows per warp) and write the tile; with 4-bit slots warps 10..25 expand and
+// warp 26 fetches codes.  Two accumulators alternate so the epilogue of a tile overlaps the MMAs of the next.
 // Work items are (request, weight tile, token chunk) triples of the launch's compute group, dealt
-// round-robin to CTA pairs, and cut into equal runs of k-blocks for single CTAs (GemmWalk, GemmSplit).
+// round-robin to the CTA pairs (GemmWalk).
 //
 // Ragged N: a chunk's box may run past its expert's last row; those columns are computed on whatever
 // the next rows hold (or zeros past the end of the buffer) and never stored.
 //
-// CTA pairs (template parameter CG = 2, used where the experts have enough tokens): two CTAs of a
+// CTA pairs (template parameter CG = 2, the form in use; CG = 1 stays selectable): two CTAs of a
 // cluster on neighbouring SMs take two adjacent weight tiles of the same expert and chunk and run them
 // as ONE tensor-core operation of M = 256 (tcgen05.mma.cta_group::2, issued by the even CTA).  Each
 // CTA stages its own 128 weight rows but only HALF of the tokens; the tensor cores of both SMs read both
@@ -288,15 +288,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&r)[16])
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-        ::"r"(taddr), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "f"(r[8]), "f"(r[9]),
-          "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15])
-        : "memory");
-}
 // to nearest even, as the low half
 __device__ __forceinline__ uint16_t bf16_bits(float v)
 {
@@ -349,18 +340,19 @@ struct GemmItem {
     int n_live;    // tokens that exist
     int m0;        // first hidden unit (GEMM 1) or output column (GEMM 2) of this CTA's weight tile
     int slot;      // cache slot of the expert, or -1 - index of the shared expert
-    int k0, k1;    // k-blocks of this piece of the tile
 };
 
-// The items of one CTA pair, in order: every n_ctas-th, the chunks of one weight tile adjacent, so that pairs
-// working side by side share it in L2.
-template <int NT, int kMTile>
+// The items of one CTA pair (or single CTA), in order: every n_units-th, the chunks of one weight tile adjacent, so that
+// pairs working side by side share it in L2.  (Equal runs of k-blocks for each, with tiles computed in parts
+// where a run's border cuts them, were slower once the MMA warp kept up: 128 tokens over some 20 experts 74 against
+// 66 us a layer, 4096 tokens over 16 experts 1735 against 1330.)
+template <int CG, int NT, int kMTile>
 struct GemmWalk {
     const int4 *rec;         // first row, tokens, slot (shared expert s: -1 - s), tokens of a chunk
     const int *item0;        // first item of every request
-    int q, w, step, total, rank, kblocks;
-    __device__ GemmWalk(const int4 *rec_, const int *item0_, const int *, int n_reqs, int unit, int n_ctas, int rank_, int kblocks_)
-        : rec(rec_), item0(item0_), q(0), w(unit), step(n_ctas), total(item0_[n_reqs]), rank(rank_), kblocks(kblocks_)
+    int q, w, step, total, rank;
+    __device__ GemmWalk(const int4 *rec_, const int *item0_, int n_reqs, int unit, int n_units, int rank_)
+        : rec(rec_), item0(item0_), q(0), w(unit), step(n_units), total(item0_[n_reqs]), rank(rank_)
     {
     }
     __device__ bool next(GemmItem &it)
@@ -371,130 +363,14 @@ struct GemmWalk {
             ++q;
         const int4 r = rec[q];
         const int local = w - item0[q], n = (r.y + NT - 1) / NT, c = local % n;
-        it.m0 = (local / n * 2 + rank) * kMTile;
-        it.row0 = r.x + c * r.w;
-        it.n_live = min(r.w, r.y - c * r.w);
-        it.n = (it.n_live + 31) / 32 * 32;
-        it.slot = r.z;
-        it.k0 = 0;
-        it.k1 = kblocks;
-        w += step;
-        return true;
-    }
-};
-
-// The pieces of one single CTA.  With few tokens per expert there are few rounds of tiles (or less than one), and the last
-// round would leave most of the chip idle; so the tiles are laid end to end, each as long as its k-blocks (in quads
-// of 4, the unit in which 4-bit codes are fetched) times what one costs, and every CTA takes an equal run.  A tile that a
-// run's border cuts is computed in parts: the CTA with its last k-blocks starts its accumulator from the others' fp32 sums,
-// added up in their order (its epilogue warps put them there while the tile before is computed).  A CTA does
-// the first part of the tile that it shares with its successor before everything else, and the
-// last part of the tile that it shares with its predecessors last, so that it finds their sums ready; it only ever
-// waits for CTAs of lower index, which never wait before they have delivered.
-// (Dealing out rows of weights instead was slower than whole tiles: a short tile's k-blocks take as long as a
-// whole one's.)
-// A k-block's cost: reading the weights (16-bit), which tokens hardly add to, or expanding them.
-__device__ __forceinline__ int gemm_item_cost(int chunk, int fmt)
-{
-    return fmt ? 20 + (chunk + 31) / 32 + (chunk <= 64 ? 2 : chunk <= 128 ? 4 : 8) : 16 + (chunk + 31) / 32;
-}
-template <int CG, int NT, int kMTile, int FMT>
-struct GemmSplit {
-    const int4 *rec;
-    const int *item0, *cost0;      // first item of every request, and its place on the line of costs
-    int n_reqs, kblocks, quads, units, unit, rank;
-    int w_lo, q_lo, w_hi, q_hi, cur, step;
-    __device__ GemmSplit(const int4 *rec_, const int *item0_, const int *cost0_, int n_reqs_, int unit_, int n_units, int rank_, int kblocks_)
-        : rec(rec_), item0(item0_), cost0(cost0_), n_reqs(n_reqs_), kblocks(kblocks_), quads((kblocks_ + 3) / 4), unit(unit_), rank(rank_), step(0)
-    {
-        // no more CTAs than there are tiles, or pieces of two quads
-        const int items = item0[n_reqs];
-        units = min(n_units, max(items, items * quads / 2));
-        locate(unit, w_lo, q_lo);
-        locate(unit + 1, w_hi, q_hi);
-        cur = w_lo + (q_lo > 0 ? 1 : 0);
-    }
-    // where the run of CTA u begins: tile and quad
-    __device__ void locate(int u, int &w, int &quad) const
-    {
-        const int total = cost0[n_reqs];
-        const int at = u >= units ? total : (int)((long long)u * total / units);
-        if (at >= total) {
-            w = item0[n_reqs];
-            quad = 0;
-            return;
-        }
-        int r = 0;
-        for (int s = 64; s; s >>= 1)
-            if (r + s < n_reqs && cost0[r + s] <= at)
-                r += s;
-        const int c = gemm_item_cost(rec[r].w, FMT), local = at - cost0[r];
-        w = item0[r] + local / (c * quads);
-        quad = local % (c * quads) / c;
-    }
-    __device__ bool fill(GemmItem &it, int w, int qa, int qb) const
-    {
-        int q = 0;
-        for (int s = 64; s; s >>= 1)
-            if (q + s < n_reqs && item0[q + s] <= w)
-                q += s;
-        const int4 r = rec[q];
-        const int local = w - item0[q], n = (r.y + NT - 1) / NT, c = local % n;
         it.m0 = (local / n * CG + rank) * kMTile;
         it.row0 = r.x + c * r.w;
         it.n_live = min(r.w, r.y - c * r.w);
         it.n = (it.n_live + 16 * CG - 1) / (16 * CG) * (16 * CG);
         it.slot = r.z;
-        it.k0 = 4 * qa;
-        it.k1 = min(4 * qb, kblocks);
+        w += step;
         return true;
     }
-    __device__ bool next(GemmItem &it)
-    {
-        if (step == 0) {
-            step = 1;
-            if (w_hi != w_lo && q_hi > 0)
-                return fill(it, w_hi, 0, q_hi);
-        }
-        if (step == 1) {
-            if (cur < w_hi)
-                return fill(it, cur++, 0, quads);
-            step = 2;
-        }
-        if (step == 2) {
-            step = 3;
-            if (w_lo == w_hi)
-                return q_lo < q_hi && fill(it, w_lo, q_lo, q_hi);
-            if (q_lo > 0)
-                return fill(it, w_lo, q_lo, quads);
-        }
-        return false;
-    }
-    // the CTAs with the earlier parts of tile w_lo: bit i = CTA unit - 1 - i
-    __device__ unsigned long long partners() const
-    {
-        unsigned long long m = 0;
-        int wb = w_lo, qb = q_lo;
-        for (int i = 0; i < 64 && unit - 1 - i >= 0; ++i) {
-            int wa, qa;
-            locate(unit - 1 - i, wa, qa);
-            if (wa != wb || qa != qb)
-                m |= 1ull << i;
-            if (wa < w_lo || qa == 0)
-                break;
-            wb = wa;
-            qb = qa;
-        }
-        return m;
-    }
-};
-template <int CG, int NT, int kMTile, int FMT>
-struct GemmItems {
-    using type = GemmSplit<CG, NT, kMTile, FMT>;
-};
-template <int NT, int kMTile>
-struct GemmItems<2, NT, kMTile, 0> {
-    using type = GemmWalk<NT, kMTile>;
 };
 
 // PHASE 1: h = SiLU(Xs W_g^T) * (Xs W_u^T) -> hs (bf16).  PHASE 2: z = hs W_d^T -> zs (fp32).
@@ -503,14 +379,14 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
 {
     static_assert(FMT == 0 || CG == 2, "4-bit slots: CTA pairs");
     constexpr int kStages = gemm_stages(FMT), NT = gemm_tokens(CG);
-    constexpr bool kSplit = CG == 1 || FMT == 1;             // tiles may be computed in parts
+    static_assert(FMT == 0 || kExpandGroups <= kStages, "a group's wait for its stage has to be for the last use of it");
     constexpr int kMTile = PHASE == 1 ? 64 : 128;            // hidden units, or output columns, of one CTA's tile
     constexpr int kRawBlocks = PHASE == 1 ? 4 : 2;           // k-blocks of one fetch of codes
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ uint64_t s_bars[2 * kStages + 5 + 2 * kRawStages];
+    __shared__ uint64_t s_bars[2 * kStages + 4 + 2 * kRawStages];
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
-    __shared__ int s_tile0[kMaxReq + 1], s_cost0[kMaxReq + 1], s_nreq;
+    __shared__ int s_tile0[kMaxReq + 1], s_nreq;
     __shared__ int4 s_rec[kMaxReq];                          // see GemmWalk
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -520,7 +396,6 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     const uint32_t ring_s = smem_u32(ring), raw_s = ring_s + kStages * kStageBytes;
     const uint32_t full0 = smem_u32(s_bars), empty0 = full0 + 8 * kStages;
     const uint32_t tfull0 = empty0 + 8 * kStages, tempty0 = tfull0 + 16, rfull0 = tempty0 + 16, rempty0 = rfull0 + 8 * kRawStages;
-    const uint32_t tinit = rempty0 + 8 * kRawStages;
     volatile int *abort_flag = &s_abort;
     // rank within the CTA pair; the even CTA issues the MMAs, owns the "stage full" barriers and counts
     // the drained accumulators of both
@@ -539,7 +414,6 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
             mbar_init(tfull0 + 8 * i, 1);
             mbar_init(tempty0 + 8 * i, kEpilogueWarps * CG);
         }
-        mbar_init(tinit, kEpilogueWarps * CG);
         if (FMT)
             for (int i = 0; i < kRawStages; ++i) {
                 mbar_init(rfull0 + 8 * i, 1);
@@ -561,7 +435,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     const int kblocks = (K + kBK - 1) / kBK;
     if (warp == 0) {
         const int n_req_total = plan->n_req + p.n_shared;
-        int n = 0, tiles = 0, costs = 0;
+        int n = 0, tiles = 0;
         for (int r0 = 0; r0 < n_req_total; r0 += 32) {
             const int r = r0 + lane;
             bool on = false;
@@ -577,27 +451,22 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 items = on ? chunks * m_tiles : 0;
             }
             const unsigned m = __ballot_sync(0xffffffffu, on);
-            const int cost = kSplit ? items * gemm_item_cost(rec.w, FMT) * ((kblocks + 3) / 4) : 0;
-            int inc = items, inc_c = cost;
+            int inc = items;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, inc, o), c = __shfl_up_sync(0xffffffffu, inc_c, o);
+                const int v = __shfl_up_sync(0xffffffffu, inc, o);
                 inc += lane >= o ? v : 0;
-                inc_c += lane >= o ? c : 0;
             }
             if (on) {
                 const int at = n + __popc(m & ((1u << lane) - 1u));
                 s_rec[at] = rec;
                 s_tile0[at] = tiles + inc - items;
-                s_cost0[at] = costs + inc_c - cost;
             }
             n += __popc(m);
             tiles += __shfl_sync(0xffffffffu, inc, 31);
-            costs += __shfl_sync(0xffffffffu, inc_c, 31);
         }
         if (lane == 0) {
             s_tile0[n] = tiles;
-            s_cost0[n] = costs;
             s_nreq = n;
         }
     }
@@ -627,8 +496,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = s_tmem_base;
 
-    using Items = typename GemmItems<CG, NT, kMTile, FMT>::type;
-    auto walk = [&] { return Items(s_rec, s_tile0, s_cost0, n_reqs, unit, n_units, (int)rank, kblocks); };
+    auto walk = [&] { return GemmWalk<CG, NT, kMTile>(s_rec, s_tile0, n_reqs, unit, n_units, (int)rank); };
     GemmItem it;
 
     if (warp == 0) {
@@ -637,13 +505,11 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         // of a pair, the bytes of both CTAs are expected and counted on the even CTA's barriers
         const uint32_t full_b = CG == 1 ? full0 : cluster_addr(full0, 0);
         uint32_t s = 0, parity = 1, n = 0;
-        bool waited = false;
         auto items = walk();
         for (;;) {
             const bool more = !*abort_flag && items.next(it);
             if (!__all_sync(0xffffffffu, more))
                 break;
-            const int k0 = __shfl_sync(0xffffffffu, it.k0, 0), k1 = __shfl_sync(0xffffffffu, it.k1, 0);
             const int m0 = __shfl_sync(0xffffffffu, it.m0, 0), item_slot = __shfl_sync(0xffffffffu, it.slot, 0);
             // the weights of the slots, or of the shared expert
             const CUtensorMap *map_w = p.maps + (item_slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - item_slot)) + (PHASE - 1);
@@ -661,28 +527,28 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     tma_load_4d<CG>(dst, map_w, 0, kb * kBK, m0 / 64, slot, bar);
             };
             auto load_b = [&](int kb, uint32_t dst, uint32_t bar) { tma_load_2d<CG>(dst, map_b + cls, kb * kBK, b_row, bar); };
-            int kb = k0;
-            if (!waited) {
-                // single CTAs: the first stages' weights are on their way while the kernel ahead finishes
-                const int pre = CG == 1 ? min(k1 - k0, kStages) : 0;
-                if (CG == 1 && elect_one())
+            int kb = 0;
+            if (n == 0) {
+                // the first stages' weights are on their way while the kernel ahead finishes
+                const int pre = min(kblocks, kStages);
+                if (elect_one())
                     for (int i = 0; i < pre; ++i) {
-                        mbar_expect(full0 + 8 * i, bytes);
-                        load_a(k0 + i, ring_s + i * kStageBytes, full0 + 8 * i);
+                        if (CG == 1 || rank == 0)
+                            mbar_expect(full0 + 8 * i, bytes);
+                        load_a(i, ring_s + i * kStageBytes, full_b + 8 * i);
                     }
                 __syncwarp();
                 asm volatile("griddepcontrol.wait;" ::: "memory");
-                if (CG == 1 && elect_one())
+                if (elect_one())
                     for (int i = 0; i < pre; ++i)
-                        load_b(k0 + i, ring_s + i * kStageBytes + kABytes, full0 + 8 * i);
+                        load_b(i, ring_s + i * kStageBytes + kABytes, full_b + 8 * i);
                 __syncwarp();
-                kb += pre;
+                kb = pre;
                 n = pre;
                 s = pre % kStages;
                 parity ^= pre / kStages;
-                waited = true;
             }
-            for (; kb < k1; ++kb, ++n) {
+            for (; kb < kblocks; ++kb, ++n) {
                 // (a fresh barrier counts as being past its odd phase)
                 const bool ok = mbar_wait(empty0 + 8 * s, parity, abort_flag);
                 if (!__all_sync(0xffffffffu, ok))
@@ -720,20 +586,15 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 const bool more = !*abort_flag && items.next(it);
                 if (!__all_sync(0xffffffffu, more))
                     break;
-                const int k0 = __shfl_sync(0xffffffffu, it.k0, 0), k1 = __shfl_sync(0xffffffffu, it.k1, 0);
                 const uint32_t idesc = instr_desc_bf16(CG * 128, __shfl_sync(0xffffffffu, it.n, 0), PHASE == 2);
                 const uint32_t acc = item & 1u;
-                // a tile whose first parts other CTAs computed starts from their sums
-                const bool merge = kSplit && k0 > 0 && k1 == kblocks;
                 bool ok = item < 2 || mbar_wait(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag);
-                if (merge)
-                    ok = ok && mbar_wait(tinit, 0, abort_flag);
                 if (!__all_sync(0xffffffffu, ok))
                     break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d_tmem = tmem_base + acc * NT;
-                uint32_t accumulate = merge ? 1u : 0u;
-                for (int kb = k0; kb < k1; ++kb) {
+                uint32_t accumulate = 0;
+                for (int kb = 0; kb < kblocks; ++kb) {
                     ok = mbar_wait(full0 + 8 * s, parity, abort_flag);
                     if (!__all_sync(0xffffffffu, ok))
                         break;
@@ -757,7 +618,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                         else
                             umma_commit_pair(empty0 + 8 * s);
                         // the accumulator is complete
-                        if (kb + 1 == k1) {
+                        if (kb + 1 == kblocks) {
                             if (CG == 1)
                                 umma_commit(tfull0 + 8 * acc);
                             else
@@ -781,106 +642,13 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         const int c_first = (warp - 2) / 4 * 16;             // its chunks of 16 tokens: c_first, c_first + 32, ..
         uint32_t item = 0;
         auto items = walk();
-        // sums of the CTAs with the earlier parts of a tile ([token][row] of fp32 per CTA, and a word per CTA and
-        // quarter that says they are there) into the accumulator that the tile will use
-        auto preload = [&](const GemmItem &nx, uint32_t acc) {
-            if constexpr (kSplit) {
-                const unsigned long long others = items.partners();
-                for (unsigned long long m = others; m; m &= m - 1) {
-                    const unsigned *flag = p.flags + (blockIdx.x - CG * __ffsll((long long)m)) * kEpilogueWarps + (warp - 2);
-                    const long long c0 = clock64();
-                    for (;;) {
-                        unsigned v;
-                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-                        if (v == p.seq || *abort_flag)
-                            break;
-                        if (clock64() - c0 > kGemmWaitCycles)
-                            *abort_flag = 1;
-                    }
-                }
-                __syncwarp();
-                const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * NT;
-                // (64 tokens a time, so that two chunks' loads are in flight; with 4-bit slots registers do for one)
-                constexpr int kAhead = FMT ? 1 : 2;
-#pragma unroll 1
-                for (int c = c_first; c < nx.n; c += 32 * kAhead) {
-                    float sum[kAhead][16];
-#pragma unroll
-                    for (int h = 0; h < kAhead; ++h)
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            sum[h][j] = 0.0f;
-                    // (in ascending order of the CTAs, which is that of the k-blocks)
-                    for (int i = 63 - __clzll((long long)others); i >= 0; --i) {
-                        if (!((others >> i) & 1ull))
-                            continue;
-                        const float *src = p.partial + ((size_t)(blockIdx.x - CG * (1 + i)) * p.part_tokens + c) * 128 + quarter * 32 + lane;
-                        float o[kAhead][16];
-#pragma unroll
-                        for (int h = 0; h < kAhead; ++h)
-                            if (c + 32 * h < nx.n)
-#pragma unroll
-                                for (int j = 0; j < 16; ++j)
-                                    o[h][j] = __ldcg(src + (32 * h + j) * 128);      // (tokens that do not exist: whatever is there)
-#pragma unroll
-                        for (int h = 0; h < kAhead; ++h)
-                            if (c + 32 * h < nx.n)
-#pragma unroll
-                                for (int j = 0; j < 16; ++j)
-                                    sum[h][j] += o[h][j];
-                    }
-#pragma unroll
-                    for (int h = 0; h < kAhead; ++h)
-                        if (c + 32 * h < nx.n)
-                            tmem_st16(t_row + c + 32 * h, sum[h]);
-                }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    if (CG == 1 || rank == 0)
-                        mbar_arrive(tinit);
-                    else
-                        mbar_arrive_cluster(cluster_addr(tinit, 0));
-                }
-            }
-        };
-        GemmItem nx;
-        bool more = items.next(nx);
-        if (more && kSplit && nx.k0 > 0 && nx.k1 == kblocks)
-            preload(nx, 0);
-        for (; !*abort_flag && more; ++item) {
-            it = nx;
+        for (; !*abort_flag && items.next(it); ++item) {
             const uint32_t acc = item & 1u;
-            more = items.next(nx);
-            // (the other accumulator was drained before this item; a part that this CTA owes another goes out first)
-            const bool owed = kSplit && it.k1 < kblocks, merge_next = kSplit && more && nx.k0 > 0 && nx.k1 == kblocks;
-            if (merge_next && !owed)
-                preload(nx, acc ^ 1u);
             if (!mbar_wait(tfull0 + 8 * acc, (item >> 1) & 1u, abort_flag))
                 break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * NT;
-            if (owed) {
-                // an earlier part of a tile, for the CTA that finishes it
-                float *dst = p.partial + (size_t)blockIdx.x * p.part_tokens * 128 + quarter * 32 + lane;
-#pragma unroll 1
-                for (int c = c_first; c < it.n; c += 32) {
-                    float v[16];
-                    tmem_ld16(t_row + c, v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        __stcg(dst + (c + j) * 128, v[j]);
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    __threadfence();
-                    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.flags + blockIdx.x * kEpilogueWarps + (warp - 2)), "r"(p.seq) : "memory");
-                }
-                __syncwarp();
-                if (merge_next)
-                    preload(nx, acc ^ 1u);
-            } else if (PHASE == 1) {
+            if (PHASE == 1) {
                 // lanes 0..7 hold g of eight hidden units, 8..15 u of the same ones, 16..31 those of the next eight.  Of two
                 // neighbouring tokens the g lane finishes the first and the u lane the second.
                 const int f = it.m0 + quarter * 16 + (lane >> 4) * 8 + (lane & 7);
@@ -941,9 +709,10 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         }
     } else if (FMT == 1 && warp < 2 + kEpilogueWarps + 4 * kExpandGroups) {
         // ============================================================ expansion of 4-bit codes (warps 10..25)
-        // Two groups of four warps take the k-blocks in turn: what a k-block takes is latency (waits, the fence before the
-        // tensor cores may read), which the other group's k-block covers.  (Eight warps on every k-block: 0.6 us each, as
-        // with four.)
+        // Groups of four warps take the k-blocks in turn, counted over all items (so that a group is never two uses of
+        // a stage ahead, which a barrier's parity could not tell): what a k-block takes is latency, 1350 cycles of waits, arithmetic
+        // and the fence before the tensor cores may read, which the other groups' k-blocks cover.  (512 tokens,
+        // us a pass: two groups 140, four 127.)
         const int row = ((warp - 10) & 3) * 32 + lane, group = (warp - 10) >> 2;     // row of the weight tile, or (column group, f) of GEMM 2's
         const size_t ub = (size_t)p.unit_bytes, scales = 3 * (size_t)(p.d / 2);
         uint32_t n0 = 0, rn = 0;
@@ -961,14 +730,14 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     return f_row < p.F && kb < kblocks ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base) + kb) : 0u;
                 return kb * kBK + f_row < p.F ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base + (size_t)kb * kBK * ub)) : 0u;
             };
-            uint32_t sc = scale_of(it.k0 + group);      // (runs begin at multiples of 4 k-blocks)
+            uint32_t sc = scale_of((group - (int)n0) & (kExpandGroups - 1));
             bool ok = true;
-            for (int kr = it.k0; kr < it.k1 && ok; kr += kRawBlocks, ++rn) {
+            for (int kr = 0; kr < kblocks && ok; kr += kRawBlocks, ++rn) {
                 const uint32_t rs = rn % kRawStages;
                 ok = mbar_wait(rfull0 + 8 * rs, (rn / kRawStages) & 1u, abort_flag);
-                for (int sub = (group - kr) & (kExpandGroups - 1); sub < kRawBlocks && kr + sub < it.k1 && ok; sub += kExpandGroups) {
+                for (int sub = (group - (int)n0 - kr) & (kExpandGroups - 1); sub < kRawBlocks && kr + sub < kblocks && ok; sub += kExpandGroups) {
                 const int kb = kr + sub;
-                const uint32_t n = n0 + (uint32_t)(kb - it.k0), s = n % kStages;
+                const uint32_t n = n0 + (uint32_t)kb, s = n % kStages;
                 if (n >= (uint32_t)kStages)
                     ok = mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag);
                 if (!ok)
@@ -1030,7 +799,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                 if (lane == 0)
                     mbar_arrive(rempty0 + 8 * rs);
             }
-            n0 += (uint32_t)(it.k1 - it.k0);
+            n0 += (uint32_t)kblocks;
         }
     } else if (FMT == 1 && warp == 2 + kEpilogueWarps + 4 * kExpandGroups) {
         // ============================================================ fetch of 4-bit codes
@@ -1040,7 +809,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
             while (!*abort_flag && items.next(it)) {
                 const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (PHASE - 1);
                 const int slot = it.slot >= 0 ? it.slot : 0;
-                for (int kb = it.k0; kb < it.k1; kb += kRawBlocks, ++rn) {
+                for (int kb = 0; kb < kblocks; kb += kRawBlocks, ++rn) {
                     const uint32_t rs = rn % kRawStages;
                     if (rn >= (uint32_t)kRawStages && !mbar_wait(rempty0 + 8 * rs, ((rn / kRawStages) - 1u) & 1u, abort_flag))
                         break;
@@ -1237,8 +1006,6 @@ cudaError_t gemm_configure()
 }
 
 }  // namespace
-
-int ffn_gemm_part_tokens(int fmt) { return gemm_tokens(fmt ? 2 : 1); }
 
 bool ffn_gemm_supported(int d, int F) { return d % 256 == 0 && F % kUnitRows == 0; }
 

@@ -166,15 +166,7 @@ struct GemmParams {
     size_t slot_stride;
     const char *const *shared_blobs;
     int unit_bytes;
-    // tiles computed in parts by several CTAs: [CTA][part_tokens][128] fp32 sums, eight words per CTA, and what the
-    // words of this launch say
-    float *partial;
-    unsigned *flags;
-    unsigned seq;
-    int part_tokens;
 };
-// tokens of a chunk at most, of the forms that compute tiles in parts
-int ffn_gemm_part_tokens(int fmt);
 bool ffn_gemm_supported(int d, int F);
 cudaError_t ffn_gemm_configure();
 // Token lists (perm, inv_pos, tok_of_sorted) of a call planned by the general kernel and, unless xs is null, the

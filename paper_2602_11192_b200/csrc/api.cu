@@ -603,6 +603,7 @@ static int create_layer(int d, int F, int E, int k, int C, int fmt, melinoe_moe_
     // grouped GEMM for calls of many tokens: one tensor map per view covers every slot (bf16 blobs are multiples of
     // 1 KiB, so their slots are contiguous)
     std::memset(h->maps_host, 0, sizeof(h->maps_host));
+    CR(router_configure());
     if (ffn_gemm_supported(d, F) && (fmt == 1 || h->slot_stride == h->expert_bytes) && ffn_gemm_configure() == cudaSuccess) {
         CR(cudaMalloc(&h->maps_dev, sizeof(h->maps_host)));
         if (encode_weight_maps(&h->maps_host[kMapSlots0], h->slots, d, F, C, h->slot_stride, fmt)) {

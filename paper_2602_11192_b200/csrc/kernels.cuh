@@ -20,6 +20,7 @@ struct RouterShape {
 };
 RouterShape router_shape(int T, int E, int n_sms);
 // block_counts [n_blocks][kMaxExperts]
+cudaError_t router_configure();
 cudaError_t launch_router(cudaStream_t stream, const RouterShape &shape, const uint16_t *x, const uint16_t *w_r,
                           const float *bias, const int32_t *token_seq, int T, int d, int E, int k,
                           int32_t *idx, float *gate, float *logits_out, int32_t *block_counts);

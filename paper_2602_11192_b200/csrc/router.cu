@@ -37,7 +37,20 @@ __device__ __forceinline__ void fma2(uint64_t &acc, uint64_t a, uint64_t b)
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
-// TT tokens x EE experts per warp, CH pieces of 256 columns loaded ahead of their arithmetic.
+constexpr int kStages = 4;                 // staged form: pieces of 256 columns in the ring
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+
+// TT tokens x EE experts per warp, CH pieces of 256 columns loaded ahead of their arithmetic; CH = 0: the block's rows of
+// both operands go through a ring in shared memory.
 template <int TT, int EE, int CH>
 __global__ void __launch_bounds__(512)
 router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ w_r,
@@ -71,8 +84,28 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
         for (int e = 0; e < EE / 2; ++e)
             acc[t][e] = 0ull;
     // (the router matrix does not change while calls are queued; everything else may be the work of the kernel ahead)
+    // staged form: this warp's rows of a piece, those of the router matrix or those of the tokens
+    const int w_rows = n_eg * EE, stage_bytes = (w_rows + tokens_per_block) * 512;
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_logit + tokens_per_block * kMaxExperts);
+    auto fetch = [&](int c, bool tokens) {
+        const uint32_t dst = ring + (c % kStages) * stage_bytes + lane * 16;
+        const int n = tokens ? tokens_per_block : w_rows;
+        for (int r = warp; r < n; r += n_warps) {
+            const uint16_t *row = tokens ? x + (size_t)min(b0 + r, T - 1) * d : w_r + (size_t)min(r, E - 1) * d;
+            copy16(dst + (tokens ? w_rows + r : r) * 512, row + c * 256 + lane * 8);
+        }
+    };
+    if (CH == 0)
+        for (int c = 0; c < kStages - 1 && c < n_chunks; ++c)
+            fetch(c, false);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (CH == 0)
+        for (int c = 0; c < kStages - 1; ++c) {
+            if (c < n_chunks)
+                fetch(c, true);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
     // top-k below: warp w serves token w of the block first; its bias is on the way meanwhile
     float bias0 = 0.0f, bias1 = 0.0f;
     auto load_bias = [&](int t) {
@@ -83,12 +116,59 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
     if (bias && warp < n_tok)
         load_bias(warp);
 
-    if (tl < n_tok) {
-#pragma unroll 1
-        for (int c0 = 0; c0 < n_chunks; c0 += CH) {
-            uint4 xv[CH][TT], wv[CH][EE];
+    auto multiply = [&](const uint4(&xv)[TT], const uint4(&wv)[EE]) {
 #pragma unroll
-            for (int c = 0; c < CH; ++c)
+        for (int r = 0; r < 4; ++r) {
+            auto word = [r](const uint4 &v) { return r == 0 ? v.x : r == 1 ? v.y : r == 2 ? v.z : v.w; };
+            uint64_t wl[EE / 2], wh[EE / 2];
+#pragma unroll
+            for (int e = 0; e < EE / 2; ++e) {
+                const uint32_t a = word(wv[2 * e]), b = word(wv[2 * e + 1]);
+                wl[e] = pack2(bf16lo(a), bf16lo(b));
+                wh[e] = pack2(bf16hi(a), bf16hi(b));
+            }
+#pragma unroll
+            for (int t = 0; t < TT; ++t) {
+                const uint32_t v = word(xv[t]);
+                const uint64_t xl = pack2(bf16lo(v), bf16lo(v)), xh = pack2(bf16hi(v), bf16hi(v));
+#pragma unroll
+                for (int e = 0; e < EE / 2; ++e)
+                    fma2(acc[t][e], xl, wl[e]);
+#pragma unroll
+                for (int e = 0; e < EE / 2; ++e)
+                    fma2(acc[t][e], xh, wh[e]);
+            }
+        }
+    };
+    if (CH == 0) {
+#pragma unroll 1
+        for (int c = 0; c < n_chunks; ++c) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+            __syncthreads();
+            // (every warp has read the stage that is filled now)
+            if (c + kStages - 1 < n_chunks) {
+                fetch(c + kStages - 1, false);
+                fetch(c + kStages - 1, true);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            const uint32_t src = ring + (c % kStages) * stage_bytes + lane * 16;
+            uint4 xv[TT], wv[EE];
+#pragma unroll
+            for (int t = 0; t < TT; ++t)
+                xv[t] = lds128(src + (w_rows + tl + t) * 512);
+#pragma unroll
+            for (int e = 0; e < EE; ++e)
+                wv[e] = lds128(src + (e0 + e) * 512);
+            multiply(xv, wv);
+        }
+    }
+    if (tl < n_tok) {
+        constexpr int kAhead = CH ? CH : 1;
+#pragma unroll 1
+        for (int c0 = 0; CH != 0 && c0 < n_chunks; c0 += kAhead) {
+            uint4 xv[kAhead][TT], wv[kAhead][EE];
+#pragma unroll
+            for (int c = 0; c < kAhead; ++c)
                 if (c0 + c < n_chunks) {
 #pragma unroll
                     for (int t = 0; t < TT; ++t)
@@ -98,31 +178,9 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
                         wv[c][e] = __ldg(wrow[e] + (c0 + c) * 32);
                 }
 #pragma unroll
-            for (int c = 0; c < CH; ++c)
-                if (c0 + c < n_chunks) {
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        auto word = [r](const uint4 &v) { return r == 0 ? v.x : r == 1 ? v.y : r == 2 ? v.z : v.w; };
-                        uint64_t wl[EE / 2], wh[EE / 2];
-#pragma unroll
-                        for (int e = 0; e < EE / 2; ++e) {
-                            const uint32_t a = word(wv[c][2 * e]), b = word(wv[c][2 * e + 1]);
-                            wl[e] = pack2(bf16lo(a), bf16lo(b));
-                            wh[e] = pack2(bf16hi(a), bf16hi(b));
-                        }
-#pragma unroll
-                        for (int t = 0; t < TT; ++t) {
-                            const uint32_t v = word(xv[c][t]);
-                            const uint64_t xl = pack2(bf16lo(v), bf16lo(v)), xh = pack2(bf16hi(v), bf16hi(v));
-#pragma unroll
-                            for (int e = 0; e < EE / 2; ++e)
-                                fma2(acc[t][e], xl, wl[e]);
-#pragma unroll
-                            for (int e = 0; e < EE / 2; ++e)
-                                fma2(acc[t][e], xh, wh[e]);
-                        }
-                    }
-                }
+            for (int c = 0; c < kAhead; ++c)
+                if (c0 + c < n_chunks)
+                    multiply(xv[c], wv[c]);
         }
         // the butterfly over the lanes: while more than one value is left, the lower lanes of a stride take the first half
         // of them and the upper lanes the second
@@ -228,7 +286,8 @@ cudaError_t router_launch(cudaStream_t stream, const RouterShape &sh, const uint
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(sh.n_blocks);
     lc.blockDim = dim3(32 * sh.n_eg * (sh.tokens_per_block / TT));
-    lc.dynamicSmemBytes = (size_t)sh.tokens_per_block * kMaxExperts * sizeof(float);
+    lc.dynamicSmemBytes = (size_t)sh.tokens_per_block * kMaxExperts * sizeof(float) +
+                          (CH == 0 ? (size_t)kStages * (sh.n_eg * EE + sh.tokens_per_block) * 512 : 0);
     lc.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -241,19 +300,27 @@ cudaError_t router_launch(cudaStream_t stream, const RouterShape &sh, const uint
 
 }  // namespace
 
-// One token per warp while that gives no more than four blocks per SM, two up to eight, else four; more token
-// groups per block (at most 16 warps) once there are blocks for every SM.
+// One token per warp while that gives no more than two blocks per SM, two up to four, else four (the staged form); more
+// token groups per block (at most 16 warps) once there are blocks for every SM, and of the staged form, of which an SM
+// holds one, so many that the blocks fit in one round.
 RouterShape router_shape(int T, int E, int n_sms)
 {
     RouterShape s;
     s.tokens_per_warp = T <= 2 * n_sms ? 1 : T <= 4 * n_sms ? 2 : 4;
     const int ee = s.tokens_per_warp == 4 ? 8 : 4;
     s.n_eg = (E + ee - 1) / ee;
-    int tg = T / (s.tokens_per_warp * n_sms);
+    int tg = (T + (s.tokens_per_warp == 4 ? 4 * n_sms - 1 : 0)) / (s.tokens_per_warp * n_sms);
     tg = tg < 1 ? 1 : tg > 16 / s.n_eg ? 16 / s.n_eg : tg;
     s.tokens_per_block = tg * s.tokens_per_warp;
     s.n_blocks = (T + s.tokens_per_block - 1) / s.tokens_per_block;
     return s;
+}
+
+// the staged form's ring: at most 8 expert groups of 8 rows beside 2 groups of 4 tokens, or one beside 16
+cudaError_t router_configure()
+{
+    return cudaFuncSetAttribute(router_topk_kernel<4, 8, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                64 * kMaxExperts * (int)sizeof(float) + kStages * 72 * 512);
 }
 
 cudaError_t launch_router(cudaStream_t stream, const RouterShape &sh, const uint16_t *x, const uint16_t *w_r,
@@ -266,7 +333,7 @@ cudaError_t launch_router(cudaStream_t stream, const RouterShape &sh, const uint
     else if (sh.tokens_per_warp == 2)
         e = router_launch<2, 4, 2>(stream, sh, x, w_r, bias, token_seq, T, d, E, k, idx, gate, logits_out, block_counts);
     else
-        e = router_launch<4, 8, 1>(stream, sh, x, w_r, bias, token_seq, T, d, E, k, idx, gate, logits_out, block_counts);
+        e = router_launch<4, 8, 0>(stream, sh, x, w_r, bias, token_seq, T, d, E, k, idx, gate, logits_out, block_counts);
     count_launch();
     return e;
 }

@@ -11,12 +11,13 @@
 //
 // A warp holds TT tokens x EE experts in registers; a block is n_eg expert groups x TG token groups of warps, so
 // every block reads the whole router matrix once.  What bounds it: for a few hundred tokens the latency of those
-// reads (TT = 1 or 2, EE = 4: many warps, CH pieces of 256 columns in flight), for thousands the issue slots: 4 x 8
-// gives 256 multiply-adds per 12 loads and 128 conversions, and fma.rn.f32x2 (two experts at a time, each rounded
-// on its own: the same bits) halves what the multiply-adds take of the issue slots.  The butterfly folds
+// reads (TT = 1 or 2, EE = 4: many warps, CH pieces of 256 columns in flight), for thousands the FMA pipe and the issue
+// slots: 4 x 8 gives 256 multiply-adds per 12 loads and 128 conversions, and fma.rn.f32x2 (two experts at a time, each rounded
+// on its own: the same bits) halves what the multiply-adds take of the issue slots; an SM holds only 16 such warps,
+// so their operands go through a ring in shared memory (cp.async) instead of waiting for the loads.  The butterfly folds
 // TT * EE values at once by exchanging halves: 31 shuffles for 32 values instead of 160.  The bias is added by
-// the warp that selects, a lane per expert.  Measured (d 2048, 64 experts): 128 tokens 16.7 -> 8.4 us, 512 tokens
-// 38 -> 18 us, 8192 tokens 193 -> 101 us; 4096 tokens, d 4096, 16 experts 119 -> 48 us.
+// the warp that selects, a lane per expert.  Measured (d 2048, 64 experts): 128 tokens 16.7 -> 8 us, 512 tokens
+// 38 -> 17 us, 8192 tokens 193 -> 93 us (FMA pipe half busy); 4096 tokens, d 4096, 16 experts 119 -> 26 us.
 #include "kernels.cuh"
 
 namespace melinoe {
@@ -35,6 +36,17 @@ __device__ __forceinline__ uint64_t pack2(float lo, float hi)
 __device__ __forceinline__ void fma2(uint64_t &acc, uint64_t a, uint64_t b)
 {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+// Unsigned numbers (none of them 0) in the order of floats, both zeros alike, and back.
+__device__ __forceinline__ unsigned order_key(float v)
+{
+    const unsigned b = __float_as_uint(v + 0.0f);
+    return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ float key_value(unsigned key)
+{
+    return __uint_as_float(key & 0x80000000u ? key & 0x7fffffffu : ~key);
 }
 
 constexpr int kStages = 4;                 // staged form: pieces of 256 columns in the ring
@@ -60,8 +72,6 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
 {
     extern __shared__ __align__(16) float s_logit[];        // [tokens_per_block][kMaxExperts]
     __shared__ int32_t s_count[kMaxExperts];
-    __shared__ float s_sel[16][32];
-    __shared__ int32_t s_sel_idx[16][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const int b0 = blockIdx.x * tokens_per_block;            // the block's first token
     const int n_tok = min(tokens_per_block, T - b0);
@@ -89,11 +99,13 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
     const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_logit + tokens_per_block * kMaxExperts);
     auto fetch = [&](int c, bool tokens) {
         const uint32_t dst = ring + (c % kStages) * stage_bytes + lane * 16;
-        const int n = tokens ? tokens_per_block : w_rows;
-        for (int r = warp; r < n; r += n_warps) {
-            const uint16_t *row = tokens ? x + (size_t)min(b0 + r, T - 1) * d : w_r + (size_t)min(r, E - 1) * d;
-            copy16(dst + (tokens ? w_rows + r : r) * 512, row + c * 256 + lane * 8);
-        }
+        const int at = c * 256 + lane * 8;
+        if (tokens)
+            for (int r = warp; r < tokens_per_block; r += n_warps)
+                copy16(dst + (w_rows + r) * 512, x + (size_t)min(b0 + r, T - 1) * d + at);
+        else
+            for (int r = warp; r < w_rows; r += n_warps)
+                copy16(dst + r * 512, w_r + (min(r, E - 1) * d + at));
     };
     if (CH == 0)
         for (int c = 0; c < kStages - 1 && c < n_chunks; ++c)
@@ -216,52 +228,36 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
 
     // top-k: a warp per token.  Lane l holds experts l and l + 32.
     for (int t = warp; t < n_tok; t += n_warps) {
-        const float NEG = -__int_as_float(0x7f800000);  // -inf
-        float *row = s_logit + t * kMaxExperts;
+        const float *row = s_logit + t * kMaxExperts;
         if (bias && t != warp)
             load_bias(t);
-        float v0 = NEG, v1 = NEG;
+        float v0 = 0.0f, v1 = 0.0f;
         if (lane < E)
             v0 = bias ? __fadd_rn(row[lane], bias0) : row[lane];
         if (lane + 32 < E)
             v1 = bias ? __fadd_rn(row[lane + 32], bias1) : row[lane + 32];
-        row[lane] = v0;
-        row[lane + 32] = v1;
         if (lane < E)
             logits_out[(size_t)(b0 + t) * E + lane] = v0;
         if (lane + 32 < E)
             logits_out[(size_t)(b0 + t) * E + lane + 32] = v1;
-        __syncwarp();
-        // an element's rank is the number of elements that beat it (greater, or equal with a lower
-        // index); the k elements of rank below k are the selection, in order
-        int r0 = 0, r1 = 0;
-#pragma unroll
-        for (int i = 0; i < kMaxExperts / 4; ++i) {
-            if (4 * i >= E)
-                break;
-            const float4 o4 = reinterpret_cast<const float4 *>(row)[i];
-            const float ov[4] = {o4.x, o4.y, o4.z, o4.w};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int e = 4 * i + c;
-                r0 += (ov[c] > v0) || (ov[c] == v0 && e < lane);
-                r1 += (ov[c] > v1) || (ov[c] == v1 && e < lane + 32);
-            }
+        // k times the greatest of what is left, the lowest index among equals.  (Counting for every element those that
+        // beat it took 770 instructions a token whatever k; this takes about 12 per selected expert.)
+        unsigned key0 = lane < E ? order_key(v0) : 0u, key1 = lane + 32 < E ? order_key(v1) : 0u;
+        float my_sel = 0.0f, top = 0.0f;
+        int my_idx = 0;
+        for (int j = 0; j < k; ++j) {
+            const unsigned best = __reduce_max_sync(0xffffffffu, max(key0, key1));
+            const unsigned at0 = __ballot_sync(0xffffffffu, key0 == best), at1 = __ballot_sync(0xffffffffu, key1 == best);
+            const int e = at0 ? __ffs(at0) - 1 : 31 + __ffs(at1);
+            const float value = key_value(best);
+            top = j ? top : value;
+            my_sel = lane == j ? value : my_sel;
+            my_idx = lane == j ? e : my_idx;
+            key0 = e == lane ? 0u : key0;
+            key1 = e == lane + 32 ? 0u : key1;
         }
-        if (lane < E && r0 < k) {
-            s_sel[warp][r0] = v0;
-            s_sel_idx[warp][r0] = lane;
-            atomicAdd(&s_count[lane], 1);
-        }
-        if (lane + 32 < E && r1 < k) {
-            s_sel[warp][r1] = v1;
-            s_sel_idx[warp][r1] = lane + 32;
-            atomicAdd(&s_count[lane + 32], 1);
-        }
-        __syncwarp();
-        const float top = s_sel[warp][0];
-        const float my_sel = lane < k ? s_sel[warp][lane] : 0.0f;
-        const int my_idx = lane < k ? s_sel_idx[warp][lane] : 0;
+        if (lane < k)
+            atomicAdd(&s_count[my_idx], 1);
         float ev = lane < k ? expf(my_sel - top) : 0.0f;
         float sum = ev;
 #pragma unroll
@@ -271,7 +267,6 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
             idx[(size_t)(b0 + t) * k + lane] = my_idx;
             gate[(size_t)(b0 + t) * k + lane] = ev / sum;
         }
-        __syncwarp();
     }
     __syncthreads();
     for (int i = threadIdx.x; i < kMaxExperts; i += blockDim.x)

@@ -562,29 +562,116 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
         asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const DevPlan *plan = p.plan;
-    if (tid == 0) {
+    // One token: if every expert is resident, the requests' records come without that word and say themselves that they
+    // are there (one round trip instead of two, and no fence in the planner); otherwise as for more tokens.
+    const int n_one = XT == 0 && p.fast && Tc == 1 ? p.k + p.n_shared : 0;
+    bool got = true;
+    if (tid < max(n_one, 1)) {
+        got = false;
         const long long t0 = clock64();
-        for (;;) {
+        for (unsigned i = 0;; ++i) {
+            if (n_one) {
+                unsigned long long src, tag;
+                asm volatile(
+                    "{\n\t.reg .b128 v;\n\t"
+                    "ld.acquire.gpu.global.b128 v, [%2];\n\t"
+                    "mov.b128 {%0, %1}, v;\n\t}"
+                    : "=l"(src), "=l"(tag)
+                    : "l"(&plan->one[tid])
+                    : "memory");
+                if ((unsigned)(tag >> 32) == p.call_seq) {
+                    FastReq r = {};
+                    r.src = reinterpret_cast<const char *>(src);
+                    r.gate[0] = __uint_as_float((unsigned)tag);
+                    s_req[tid] = r;
+                    got = true;
+                    break;
+                }
+                if (i & 3u)             // (the word comes instead only where experts are fetched, which takes far longer)
+                    continue;
+            }
             unsigned long long v;
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&plan->ready) : "memory");
-            s_ready = v;
-            if ((unsigned)v == p.call_seq)
+            if ((unsigned)v == p.call_seq) {
+                s_ready = v;
                 break;
+            }
             if (clock64() - t0 > kWaitLimitCycles) {
                 s_abort = 1;
                 break;
             }
         }
     }
-    __syncthreads();
+    const bool quick = __syncthreads_and(got) != 0 && n_one > 0;
+
+    // the producer's place: copies issued, ring stage of the next one and parity of its being free, rows left of this CTA's
+    // share, request and row of the next one
+    struct Feed {
+        uint32_t n, st, ph;
+        int left, a, f0;
+        __device__ void begin(int rows, int F, int G)
+        {
+            const int lo = (int)((long long)blockIdx.x * rows / G), hi = (int)((long long)(blockIdx.x + 1) * rows / G);
+            n = st = 0;
+            ph = 1;
+            left = hi - lo;
+            a = lo / F;
+            f0 = lo % F;
+        }
+    } feed;
+    feed.n = 0;
+    auto issue = [&] {
+        const int m = min(min(TR, F - feed.f0), feed.left);
+        const uint32_t bytes = (uint32_t)m * RB;
+        mbar_expect(full0 + 8 * feed.st, bytes);
+        bulk_g2s(ring_s + feed.st * STAGE, s_req[feed.a].src + (size_t)feed.f0 * RB, bytes, full0 + 8 * feed.st);
+        ++feed.n;
+        if (++feed.st == (uint32_t)S) {
+            feed.st = 0;
+            feed.ph ^= 1u;
+        }
+        feed.left -= m;
+        feed.f0 += m;
+        if (feed.f0 == F) {
+            feed.f0 = 0;
+            ++feed.a;
+        }
+    };
 
     // ---- everything the launch needs to know, in one round trip to memory
-    if (p.fast) {
+    if (quick) {
+        if (tid == kThreads - 1) {
+            s_hdr[0] = MELINOE_OK;
+            s_hdr[1] = 1;
+            s_hdr[2] = 0;
+            s_hdr[3] = n_one;
+            s_nact = n_one;
+        }
+        // the first copies go out while the others stage the hidden state
+        if (warp == NW && lane == 0) {
+            feed.begin(n_one * F, F, G);
+            while (feed.left > 0 && feed.n < (uint32_t)S)
+                issue();
+        }
+    } else if (p.fast) {
         // the plan word says how many requests there are; their records come as the loops below want them
         const unsigned hdr = (unsigned)(s_ready >> 32);
         const int n = min((int)(hdr & 0xffu), kMaxReq);
-        if (tid < 4 * n)
-            reinterpret_cast<uint4 *>(s_req)[tid] = __ldcg(reinterpret_cast<const uint4 *>(plan->fast) + tid);
+        if (warp == NW) {
+            bool lost = s_abort != 0 || ((hdr >> 8) & 0xffu) != MELINOE_OK;
+            for (int i = lane; i < 4 * n; i += 32) {
+                const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(plan->fast) + i);
+                reinterpret_cast<uint4 *>(s_req)[i] = v;
+                lost = lost || (i % 4 == 0 && (v.x | v.y) == 0u);       // no pointer: cannot be read from here
+            }
+            lost = __any_sync(0xffffffffu, lost);
+            __syncwarp();
+            if (XT == 0 && lane == 0) {
+                feed.begin(lost ? 0 : n * F, F, G);
+                while (feed.left > 0 && feed.n < (uint32_t)S)
+                    issue();
+            }
+        }
         if (tid == kThreads - 1) {
             s_hdr[0] = (int)((hdr >> 8) & 0xffu);
             s_hdr[1] = 1;
@@ -745,32 +832,18 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
     if (warp == NW) {
         // =================================================================== producer
         if (lane == 0) {
-            uint32_t n = 0, st = 0, ph = 1;         // copies issued; ring stage of the next one, parity of its being free
-            int left = q_hi - q_lo, a = q_lo / F, f0 = q_lo % F;
-            while (left > 0) {
-                const int m = min(min(TR, F - f0), left);
-                if (n >= (uint32_t)S && !mbar_wait(empty0 + 8 * st, ph, abort_flag))
+            if (XT != 0 || !p.fast)
+                feed.begin(rows, F, G);
+            while (feed.left > 0) {
+                if (feed.n >= (uint32_t)S && !mbar_wait(empty0 + 8 * feed.st, feed.ph, abort_flag))
                     break;
-                const uint32_t bytes = (uint32_t)m * RB;
-                mbar_expect(full0 + 8 * st, bytes);
-                bulk_g2s(ring_s + st * STAGE, s_req[a].src + (size_t)f0 * RB, bytes, full0 + 8 * st);
-                ++n;
-                if (++st == (uint32_t)S) {
-                    st = 0;
-                    ph ^= 1u;
-                }
-                left -= m;
-                f0 += m;
-                if (f0 == F) {
-                    f0 = 0;
-                    ++a;
-                }
+                issue();
             }
             if (*abort_flag) {
                 // a wait ran out: give the copies still in flight a bounded time to land before this
                 // CTA's shared memory goes away
                 const long long t0 = clock64();
-                for (uint32_t j = n > (uint32_t)S ? n - S : 0; j < n; ++j)
+                for (uint32_t j = feed.n > (uint32_t)S ? feed.n - S : 0; j < feed.n; ++j)
                     while (!mbar_try(full0 + 8 * (j % S), (j / S) & 1u) && clock64() - t0 < kWaitLimitCycles) {
                     }
             }

@@ -68,6 +68,13 @@ struct __align__(64) FastReq {
     int32_t expert, reserved;
     float gate[kTokPerVr];       // its gate for every token of the call; 0 = not routed to it
 };
+// A request of a one-token call whose experts are all resident: all that the FFN launch needs of it, in one 16-byte
+// piece that is stored and loaded as a whole and says itself which call it belongs to.
+struct __align__(16) OneReq {
+    const char *src;
+    float gate;
+    uint32_t seq;
+};
 // What the word that announces a plan says beside the call's sequence number (low half): requests of the decode
 // launch, status, whether one of them is deferred.
 __host__ __device__ inline uint64_t ready_word(uint32_t seq, int n_fast, int status, bool deferred)
@@ -94,6 +101,7 @@ struct DevPlan {
     ReqRec req[kMaxReq];
     DecReq dreq[kMaxReq];                     // group 0 (hits, then shared experts), then the misses by wave
     FastReq fast[kMaxReq];
+    OneReq one[kMaxReq];                      // in the order of fast[]; written instead of it, and of `ready`
 };
 
 // The miss queue of a call: what the host needs in order to issue the transfers, written by

@@ -103,6 +103,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     __shared__ int32_t s_live_occ[kMaxExperts];
     __shared__ unsigned long long s_live_stamp[kMaxExperts];
     __shared__ float s_cntf[kMaxExperts];
+    __shared__ float s_gate[kMaxExperts];                        // one token: its gate for every expert
     __shared__ int32_t s_grp_of[kMaxExperts];
     __shared__ int32_t s_grp_first[kMaxGroups + 1];              // first miss of a wave
     __shared__ int32_t s_idx[kMaxPairs];
@@ -342,6 +343,10 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
 #pragma unroll
             for (int m = 16; m >= 1; m >>= 1)
                 sum += __shfl_xor_sync(0xffffffffu, sum, m);
+            if (p.fast && T == 1) {
+                s_gate[e0] = on0 ? expf(v0 - top) / sum : 0.0f;
+                s_gate[e1] = on1 ? expf(v1 - top) / sum : 0.0f;
+            }
             if (p.fast) {
                 // the gates of every needed expert for this token, at the expert's place in the launch's order
                 if ((need >> e0) & 1ull)
@@ -462,7 +467,8 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         *reinterpret_cast<ulonglong2 *>(&f->src) = make_ulonglong2((unsigned long long)src, (unsigned long long)wb);
         *reinterpret_cast<ulonglong2 *>(&f->deferred) = make_ulonglong2((unsigned long long)deferred, (unsigned long long)(unsigned)e);
     };
-    if (p.fast) {
+    const bool one = p.fast && T == 1 && n_miss == 0 && ok;     // see OneReq
+    if (p.fast && !one) {
         if ((hit_mask >> e0) & 1ull)
             write_fast(rank_below(need, e0), e0, slot_ptr(soe0), nullptr, nullptr);
         if ((hit_mask >> e1) & 1ull)
@@ -477,6 +483,24 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     // whoever acquires the word sees them all.)
     auto announce = [&] {
         asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+        if (one) {
+            // no fence, and no second round trip for whoever waits: every record speaks for itself
+            auto put = [&](int at, const char *src, float gate) {
+                asm volatile(
+                    "{\n\t.reg .b128 v;\n\t"
+                    "mov.b128 v, {%1, %2};\n\t"
+                    "st.relaxed.gpu.global.b128 [%0], v;\n\t}"
+                    ::"l"(&plan->one[at]), "l"(src), "l"((unsigned long long)__float_as_uint(gate) | (unsigned long long)p.call_seq << 32)
+                    : "memory");
+            };
+            if ((need >> e0) & 1ull)
+                put(rank_below(need, e0), slot_ptr(soe0), s_gate[e0]);
+            if ((need >> e1) & 1ull)
+                put(rank_below(need, e1), slot_ptr(soe1), s_gate[e1]);
+            for (int s = lane; s < p.n_shared; s += 32)
+                put(n_req + s, p.shared_blobs[s], 1.0f);
+            return;
+        }
         const bool any = __any_sync(0xffffffffu, deferred);
         if (lane == 0)
             asm volatile("st.release.gpu.global.u64 [%0], %1;"

@@ -68,6 +68,17 @@ def test_decode_router_over_its_token_groups_and_sequences(d, E, k, n_seq):
     P.close()
 
 
+@pytest.mark.parametrize("store,d,E,k,n_shared", [("bf16", 512, 64, 32, 3), ("q4slots", 512, 9, 1, 0), ("bf16", 256, 1, 1, 0), ("bf16", 4096, 5, 4, 1)])
+def test_one_token_calls_take_their_requests_from_records_of_their_own(store, d, E, k, n_shared):
+    """One-token calls, fetching (announced by the plan's word) and then all resident (announced by the records, of
+    which a warp's lanes are too few for 32 experts and 3 shared ones), between calls of two tokens."""
+    P = _pair(d, 24, E, k, E, seed=95 + E, n_shared=n_shared, store=store)
+    P.set_bias(_bias(95, E, 0.3, 2), None)
+    for step, T in enumerate((1, 1, 2, 1, 1, 1, 2, 1)):
+        P.step(gen.hidden_states(95 + E, 0, "decode", step % 3, T, d))
+    P.close()
+
+
 def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory():
     """d_model 4096 with 5 to 8 tokens per call: the decode kernel writes the hidden states' tensor-core
     operands into tensor memory once and reads them from there (the shared memory goes to taller weight

@@ -54,10 +54,12 @@
 // CTAs at once (commit with cluster multicast); the odd CTA's epilogue warps report to the even CTA's
 // barrier.  Each CTA drains its own accumulator rows.
 //
-// Measured, the form with the tokens on the M side -> this one (GEMM 1, GEMM 2, us): 8192 token-expert pairs, 16
-// experts, d 4096, d_ff 6400: 771, 395 -> 698, 353 (1224 TFLOP/s); 65536 pairs, d 2048, d_ff 1408: 631, 433 -> 571, 314
-// (1280 TFLOP/s); 1024 pairs over some 20 experts, d 2048, d_ff 1024, where reading the weights is the work: 51, 30 ->
-// 43, 26.  4-bit slots, 4096 pairs, d 2048, d_ff 1024: 99 and 73, where 64 launches of the decode kernel took 2900.
+// What bounds it: the tensor cores under the power cap from some 250 tokens per expert on (457 cycles per k-block at 1.34
+// GHz), reading the weights below some 150, the expansion with 4-bit slots.  Measured, the form with the tokens on the M side
+// and single CTAs for few tokens -> this one (GEMM 1, GEMM 2, us): 8192 token-expert pairs, 16 experts, d 4096, d_ff
+// 6400: 771, 395 -> 601, 311; 65536 pairs, d 2048, d_ff 1408: 631, 433 -> 506, 295 (single launches; 1266 and 1312
+// TFLOP/s in a steady stream); 1024 pairs over some 20 experts, d 2048, d_ff 1024: 51, 30 -> 40, 24.  4-bit slots, 4096
+// pairs, d 2048, d_ff 1024: 55, 38, where 64 launches of the decode kernel took 2600.
 //
 // Every wait is bounded; on a timeout the CTA raises its abort flag, every role leaves its
 // loops, tensor memory is freed and the error word tells the host.

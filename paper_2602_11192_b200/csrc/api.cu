@@ -878,7 +878,7 @@ int launch_decode(melinoe_moe *h, cudaStream_t s, const Scratch &sc, const void 
     dp.write_back = 1;
     dp.wait_prior = behind_planner ? 0 : 1;     // directly behind the fused planner: its plan word says enough
     dp.fmt = h->fmt;
-    dp.fast = behind_planner && group < 0 ? 1 : 0;
+    dp.fast = behind_planner ? 1 : 0;
     CU_TRY(launch_ffn_decode(s, h->cfg, geo, dp));
     return MELINOE_OK;
 }
@@ -934,7 +934,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     const bool small = route_plan_small_supported(T, h->k, h->d);
     // everything on the device (see below): not for calls that may need more distinct experts than there are slots
     const bool pull = h->pull_ok && T <= kTokPerVr && ((long long)T * h->k <= h->C || h->E <= h->C);
-    pp.fast = small && pull;
+    pp.fast = !small ? 0 : pull ? 1 : 2;
     // calls of more than 8 tokens go through the grouped GEMM
     const bool use_gemm = h->gemm_ok && T > kTokPerVr && h->xs != nullptr && sc.idx == h->own.idx;
     if (small) {

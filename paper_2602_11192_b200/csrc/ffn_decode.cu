@@ -545,11 +545,6 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
     }
     if (tid == 1)
         s_deferred = 0;
-    if (!p.fast)
-        for (int i = tid; i < kMaxReq; i += kThreads) {
-            tab.match[i] = 0u;
-            tab.of_expert[i] = -1;
-        }
     // Nothing above reads what an earlier kernel wrote.  With programmatic stream serialisation this
     // CTA may be running while the kernel ahead of it in the stream (the planner) still is.  It does
     // not wait for that grid to drain (which costs microseconds) but for the word the planner writes
@@ -603,6 +598,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
         }
     }
     const bool quick = __syncthreads_and(got) != 0 && n_one > 0;
+    const bool fast = quick || (p.fast && (p.group < 0 || ((s_ready >> 32) & 0xffu) != 0));
 
     // the producer's place: copies issued, ring stage of the next one and parity of its being free, rows left of this CTA's
     // share, request and row of the next one
@@ -653,7 +649,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
             while (feed.left > 0 && feed.n < (uint32_t)S)
                 issue();
         }
-    } else if (p.fast) {
+    } else if (fast) {
         // the plan word says how many requests there are; their records come as the loops below want them
         const unsigned hdr = (unsigned)(s_ready >> 32);
         const int n = min((int)(hdr & 0xffu), kMaxReq);
@@ -692,13 +688,17 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
             s_hdr[3] = plan->group_vr_begin[p.group + 1];
         }
     }
-    if (!p.fast && tid < kMaxReq) {
+    for (int i = tid; !fast && i < kMaxReq; i += kThreads) {
+        tab.match[i] = 0u;
+        tab.of_expert[i] = -1;
+    }
+    if (!fast && tid < kMaxReq) {
         const uint4 *src = reinterpret_cast<const uint4 *>(plan->dreq + tid);
         uint4 *dst = reinterpret_cast<uint4 *>(tab.raw + tid);
         dst[0] = src[0];
         dst[1] = src[1];
     }
-    for (int i = tid; !p.fast && i < Tc * p.k; i += kThreads) {
+    for (int i = tid; !fast && i < Tc * p.k; i += kThreads) {
         tab.idx[i] = p.idx[(size_t)tok0 * p.k + i];
         tab.gw[i] = p.gate[(size_t)tok0 * p.k + i];
     }
@@ -736,7 +736,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
-    if (!p.fast) {
+    if (!fast) {
         // gate of every (request, token): the token's gate for that expert if the router chose it
         for (int i = tid; i < nrq * kTokPerVr; i += kThreads) {
             const int r = i / kTokPerVr, t = i % kTokPerVr;
@@ -832,7 +832,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
     if (warp == NW) {
         // =================================================================== producer
         if (lane == 0) {
-            if (XT != 0 || !p.fast)
+            if (XT != 0 || !fast)
                 feed.begin(rows, F, G);
             while (feed.left > 0) {
                 if (feed.n >= (uint32_t)S && !mbar_wait(empty0 + 8 * feed.st, feed.ph, abort_flag))

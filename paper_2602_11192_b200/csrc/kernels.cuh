@@ -42,7 +42,8 @@ struct PlanParams {
     uint32_t call_seq;        // written to the miss queue's seq word when the record is complete
     uint32_t prev_seq;        // sequence number of the call planned before this one
     int *err;                 // device error word (0 = ok)
-    int fast;                 // fused planner: the call is served by one decode launch that fetches the missed experts itself
+    int fast;                 // fused planner: 1 = the call is served by one decode launch that fetches the missed experts itself,
+                              // 2 = by one launch per compute group, the first of which is queued already
     int policy;               // MELINOE_POLICY_LRU or MELINOE_POLICY_COUNT
     float gamma;              // decay of the count policy
     melinoe_moe_stats *stats; // may be null
@@ -118,7 +119,8 @@ struct DecParams {
     int wait_prior;                  // the kernel ahead in the stream is another launch of the same call (it uses the
                                      // same accumulator): wait for that grid to finish before anything else
     int fmt;                         // 0: bf16 blobs, 1: 4-bit blobs
-    int fast;                        // the launch's requests are plan->fast (planned by the fused planner for this launch)
+    int fast;                        // directly behind the fused planner: the launch's requests are plan->fast or plan->one; those of
+                                     // group 0 only if the plan's word says so, or plan->one does
 };
 // The counters of DecParams::sync, a cache line each: where the CTAs end together, sixteen counters in one line cost a
 // short launch about a microsecond.

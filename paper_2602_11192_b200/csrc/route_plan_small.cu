@@ -467,8 +467,11 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         *reinterpret_cast<ulonglong2 *>(&f->src) = make_ulonglong2((unsigned long long)src, (unsigned long long)wb);
         *reinterpret_cast<ulonglong2 *>(&f->deferred) = make_ulonglong2((unsigned long long)deferred, (unsigned long long)(unsigned)e);
     };
-    const bool one = p.fast && T == 1 && n_miss == 0 && ok;     // see OneReq
-    if (p.fast && !one) {
+    // Calls whose transfers the host issues are computed group by group; one without misses is a single group, which takes
+    // its requests as if it were not.
+    const bool fast = p.fast == 1 || (p.fast == 2 && n_miss == 0);
+    const bool one = fast && T == 1 && n_miss == 0 && ok;       // see OneReq
+    if (fast && !one) {
         if ((hit_mask >> e0) & 1ull)
             write_fast(rank_below(need, e0), e0, slot_ptr(soe0), nullptr, nullptr);
         if ((hit_mask >> e1) & 1ull)
@@ -504,12 +507,19 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         const bool any = __any_sync(0xffffffffu, deferred);
         if (lane == 0)
             asm volatile("st.release.gpu.global.u64 [%0], %1;"
-                         ::"l"(&plan->ready), "l"(ready_word(p.call_seq, p.fast && ok ? ndr : 0, status, any))
+                         ::"l"(&plan->ready), "l"(ready_word(p.call_seq, fast && ok ? ndr : 0, status, any))
                          : "memory");
     };
-    const bool early = p.fast && n_miss == 0;
+    const bool early = fast && n_miss == 0;
+    auto tell_host = [&] {
+        const HostPlanHeader hdr{n_miss, n_groups, status, p.call_seq};
+        store16_host(&p.hplan->hdr, &hdr);
+    };
     if (early)
         announce();
+    // (the host, too, may go on: there is nothing to transfer)
+    if (early && p.fast == 2 && lane == 0)
+        tell_host();
 
     if (by_count) {
         // Definition C.1: one time step per call, count <- gamma * count + request
@@ -566,7 +576,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         const char *host = p.host_blobs ? p.host_blobs[e] : nullptr;
         plan->dreq[n_hits + p.n_shared + i] =
             DecReq{slot_ptr(slot), host, e, kDecMiss | (stays ? kDecStays : 0) | (hazard ? kDecHazard : 0), group, 0};
-        if (p.fast) {
+        if (fast) {
             write_fast(rank_below(need, e), e, host, stays && !hazard ? slot_ptr(slot) : nullptr, hazard ? slot_ptr(slot) : nullptr);
             deferred |= hazard;
         }
@@ -656,7 +666,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             }
         }
     }
-    if (p.fast && !early)
+    if (fast && !early)
         announce();
 
     // ---- the hits' records and stamps; under LRU, the misses' records and what they change in the cache
@@ -733,14 +743,14 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     }
     // the planning is complete now, with the token lists' records; a call computed group by group is announced
     asm volatile("bar.sync 4, 64;" ::: "memory");
-    if (!p.fast)
+    if (!fast)
         announce();
     if (lane == 0)
         planning_complete(p);
     // What may live in host memory goes out last, so that no fence above has to wait for the host link:
     // the statistics, and the miss queue for calls whose transfers the host issues.
     __syncwarp();
-    if (!p.fast)
+    if (!fast)
         for (int i = lane; i < n_miss; i += 32)
             store16_host(&p.hplan->miss[i], &s_hm[i]);
     if (lane == 0) {
@@ -758,10 +768,8 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             st.call_no = call_no;
             *p.stats = st;
         }
-        if (!p.fast) {
-            const HostPlanHeader hdr{n_miss, n_groups, status, p.call_seq};
-            store16_host(&p.hplan->hdr, &hdr);
-        }
+        if (!fast)
+            tell_host();
         if (p.trace_rec) {
             melinoe_moe_trace_header th;
             th.call_no = call_no;

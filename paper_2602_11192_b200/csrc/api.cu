@@ -183,6 +183,7 @@ struct melinoe_moe {
     // grouped-GEMM path (calls of more than 8 tokens): gathered activations, h, tensor maps
     bool gemm_ok = false, last_used_gemm = false;
     uint16_t *xs = nullptr, *hs = nullptr;
+    float *row_gate = nullptr;             // 4-bit slots
     CUtensorMap *maps_dev = nullptr;
     CUtensorMap maps_host[kMapCount];
     const void *shared_ptrs[kMaxShared] = {nullptr};
@@ -268,7 +269,9 @@ void free_scratch(melinoe_moe *h)
     cudaFree(h->stage_out);
     cudaFree(h->xs);
     cudaFree(h->hs);
+    cudaFree(h->row_gate);
     h->xs = h->hs = nullptr;
+    h->row_gate = nullptr;
     o = Scratch{};
     h->last = Scratch{};
     h->zbuf = nullptr;
@@ -345,6 +348,8 @@ int ensure_capacity(melinoe_moe *h, int T)
         CU_TRY(cudaMalloc(&h->zbuf, sorted * h->d * sizeof(float)));
         CU_TRY(cudaMalloc(&h->xs, sorted * h->d * 2));
         CU_TRY(cudaMalloc(&h->hs, sorted * h->F * 2));
+        if (h->fmt == 1)
+            CU_TRY(cudaMalloc(&h->row_gate, sorted * sizeof(float)));
         if (!encode_activation_maps(&h->maps_host[kMapXs0], h->xs, h->d, sorted) ||
             !encode_activation_maps(&h->maps_host[kMapHs0], h->hs, h->F, sorted))
             return MELINOE_ERR_CUDA;
@@ -953,11 +958,13 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         ga.plan = h->plan;
         ga.x = static_cast<const uint16_t *>(hidden_dev);
         ga.idx = sc.idx;
+        ga.gate = sc.gate;
         ga.block_base = sc.block_counts;
         ga.perm = sc.perm;
         ga.inv_pos = sc.inv_pos;
         ga.tok_of_sorted = sc.tok_of_sorted;
         ga.xs = use_gemm ? h->xs : nullptr;
+        ga.row_gate = use_gemm ? h->row_gate : nullptr;
         ga.T = T;
         ga.d = h->d;
         ga.E = h->E;
@@ -1002,6 +1009,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     gp.plan = h->plan;
     gp.maps = h->maps_dev;
     gp.hs = h->hs;
+    gp.row_gate = h->row_gate;
     gp.zs = h->zbuf;
     gp.err = h->err_word;
     gp.d = h->d;
@@ -1162,7 +1170,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     }
 
     if (use_gemm)
-        CU_TRY(launch_combine_rows(s, h->plan, sc.gate, sc.inv_pos, h->zbuf, static_cast<uint16_t *>(out_dev), T, h->d,
+        CU_TRY(launch_combine_rows(s, h->plan, h->row_gate ? nullptr : sc.gate, sc.inv_pos, h->zbuf, static_cast<uint16_t *>(out_dev), T, h->d,
                                    h->k, h->n_shared, h->n_sms));
     CU_TRY(cudaEventRecord(h->ev_last, s));
     h->has_last = true;

@@ -8,6 +8,8 @@
 //             stores it as bf16.
 //   GEMM 2    per expert: Z^T = W_d * H_e^T (K = d_ff), fp32.
 //   combine   y_t = sum_j gate[t][j] * Z[pos(t, j)] (+ shared experts), rank order, one rounding.
+// With 4-bit slots the gate goes into h before its rounding, as in the decode kernel, and the combine adds the rows up: a token
+// gets the same result from a long call as from a short one, but for the order of fp32 sums (3.2e-3 apart otherwise).
 //
 // The weights are the M side of the tensor-core operation and the tokens its N side.  An expert's weights
 // come in whole tiles of 128 rows (64 hidden units of W_g and W_u, or 128 output columns), but its
@@ -642,10 +644,18 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
         // 256 tokens longer than the products of the next tile), hence eight, and no predicates on whole chunks.
         const int quarter = warp & 3;                        // the 32 accumulator rows this warp may read
         const int c_first = (warp - 2) / 4 * 16;             // its chunks of 16 tokens: c_first, c_first + 32, ..
+        constexpr bool kGated = FMT == 1 && PHASE == 1;
+        if (kGated)          // (the rows' gates are the gather's)
+            asm volatile("griddepcontrol.wait;" ::: "memory");
         uint32_t item = 0;
         auto items = walk();
         for (; !*abort_flag && items.next(it); ++item) {
             const uint32_t acc = item & 1u;
+            // 4-bit slots: lanes l and l + 16 hold the gate of the chunk's token l, the next chunk's is on its way
+            auto gate_of = [&](int c) {
+                return c + (lane & 15) < it.n_live ? __ldcg(p.row_gate + it.row0 + c + (lane & 15)) : 0.0f;
+            };
+            float next_gate = kGated ? gate_of(c_first) : 0.0f;
             if (!mbar_wait(tfull0 + 8 * acc, (item >> 1) & 1u, abort_flag))
                 break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -662,13 +672,19 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
 #pragma unroll 1
                 for (int c = c_first; c < it.n_live; c += 32, dst += 16 * step) {
                     float v[16];
+                    const float gate = next_gate;
+                    if (kGated)
+                        next_gate = gate_of(c + 32);
                     tmem_ld16(t_row + c, v);
                     uint16_t h[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const float o = __shfl_xor_sync(0xffffffffu, is_u ? v[2 * j] : v[2 * j + 1], 8);
                         const float g = is_u ? o : v[2 * j], u = is_u ? v[2 * j + 1] : o;
-                        h[j] = bf16_bits(__fdividef(g, 1.0f + __expf(-g)) * u);
+                        float hv = __fdividef(g, 1.0f + __expf(-g)) * u;
+                        if (kGated)
+                            hv *= __shfl_sync(0xffffffffu, gate, 2 * j + (is_u ? 1 : 0));
+                        h[j] = bf16_bits(hv);
                     }
                     if (c + 14 < left) {
 #pragma unroll
@@ -879,6 +895,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(GatherParams p)
                 pos = s_run[e] + r;
                 s_pos[i] = pos;
                 if (first) {
+                    if (p.row_gate)
+                        p.row_gate[pos] = p.gate[q];
                     p.perm[pos] = q;
                     p.inv_pos[q] = pos;
                     p.tok_of_sorted[pos] = t0 + i / k;
@@ -890,8 +908,12 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(GatherParams p)
             __syncwarp();
         }
     }
-    for (int i = tid; blockIdx.y == 0 && i < n * p.n_shared; i += 256)
-        p.tok_of_sorted[n_pairs + i / n * p.T + t0 + i % n] = t0 + i % n;
+    for (int i = tid; blockIdx.y == 0 && i < n * p.n_shared; i += 256) {
+        const int pos = n_pairs + i / n * p.T + t0 + i % n;
+        p.tok_of_sorted[pos] = t0 + i % n;
+        if (p.row_gate)
+            p.row_gate[pos] = 1.0f;
+    }
     if (p.xs == nullptr)
         return;
     __syncthreads();
@@ -911,8 +933,10 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(GatherParams p)
     }
 }
 
-// y_t = sum_j gate[t][j] * Z[inv_pos[t*k+j]] + sum_s Z[T*k + s*T + t], fp32 in rank order, bf16 out.  Memory-bound:
-// full occupancy (32 registers a thread), the rows of four experts at a time in flight; work is (token, 1024 columns).
+// y_t = sum_j gate[t][j] * Z[inv_pos[t*k+j]] + sum_s Z[T*k + s*T + t], fp32 in rank order, bf16 out (GATED = false: the
+// rows of Z are weighted already).  Memory-bound: full occupancy (32 registers a thread), the rows of four experts at a
+// time in flight; work is (token, 1024 columns).
+template <bool GATED>
 __global__ void __launch_bounds__(256, 8) combine_rows_kernel(const DevPlan *plan, const float *__restrict__ gate,
                                                               const int32_t *__restrict__ inv_pos, const float *__restrict__ zs,
                                                               uint16_t *out, int T, int d, int k, int n_shared)
@@ -922,7 +946,7 @@ __global__ void __launch_bounds__(256, 8) combine_rows_kernel(const DevPlan *pla
     const bool ok = plan->status == MELINOE_OK;
     for (int t = blockIdx.x; t < T; t += gridDim.x) {
         const int32_t *pos = inv_pos + t * k;
-        const float *gt = gate + t * k;
+        auto gate_of = [&](int j) { return GATED ? gate[t * k + j] : 1.0f; };
         for (int c = (blockIdx.y * 256 + threadIdx.x) * 4; c < d; c += gridDim.y * 1024) {
             float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
             if (ok) {
@@ -937,19 +961,19 @@ __global__ void __launch_bounds__(256, 8) combine_rows_kernel(const DevPlan *pla
                 int j = 0;
                 for (; j + 4 <= k; j += 4) {
                     const float4 z0 = row(pos[j]), z1 = row(pos[j + 1]), z2 = row(pos[j + 2]), z3 = row(pos[j + 3]);
-                    add(gt[j], z0);
-                    add(gt[j + 1], z1);
-                    add(gt[j + 2], z2);
-                    add(gt[j + 3], z3);
+                    add(gate_of(j), z0);
+                    add(gate_of(j + 1), z1);
+                    add(gate_of(j + 2), z2);
+                    add(gate_of(j + 3), z3);
                 }
                 if (j + 2 <= k) {
                     const float4 z0 = row(pos[j]), z1 = row(pos[j + 1]);
-                    add(gt[j], z0);
-                    add(gt[j + 1], z1);
+                    add(gate_of(j), z0);
+                    add(gate_of(j + 1), z1);
                     j += 2;
                 }
                 if (j < k)
-                    add(gt[j], row(pos[j]));
+                    add(gate_of(j), row(pos[j]));
                 for (int s = 0; s < n_shared; ++s)
                     add(1.0f, row(T * k + s * T + t));
             }
@@ -1045,7 +1069,8 @@ cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const 
 {
     // a whole row per block once that fills the GPU
     const int x = T < 8 * n_sms ? T : 8 * n_sms, y = T < 4 * n_sms ? (d + 1023) / 1024 : 1;
-    return launch_after(stream, combine_rows_kernel, dim3(x, y), 256, 0, 1, plan, gate, inv_pos, zs, out, T, d, k, n_shared);
+    return launch_after(stream, gate ? combine_rows_kernel<true> : combine_rows_kernel<false>, dim3(x, y), 256, 0, 1, plan, gate, inv_pos,
+                        zs, out, T, d, k, n_shared);
 }
 
 }  // namespace melinoe

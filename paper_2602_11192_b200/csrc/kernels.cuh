@@ -160,7 +160,8 @@ enum {
 struct GemmParams {
     const DevPlan *plan;
     const CUtensorMap *maps;         // device array of kMapCount tensor maps
-    uint16_t *hs;                    // h, [sorted rows][F] bf16
+    uint16_t *hs;                    // h, [sorted rows][F] bf16; with 4-bit slots times the row's gate
+    const float *row_gate;           // 4-bit slots: gate of every sorted row (GatherParams::row_gate)
     float *zs;                       // expert outputs, [sorted rows][d] fp32
     int *err;
     int group, d, F, E, n_shared;
@@ -172,21 +173,24 @@ struct GemmParams {
 };
 bool ffn_gemm_supported(int d, int F);
 cudaError_t ffn_gemm_configure();
-// Token lists (perm, inv_pos, tok_of_sorted) of a call planned by the general kernel and, unless xs is null, the
-// gathered activations, in the blocks the router worked in.
+// Token lists (perm, inv_pos, tok_of_sorted) of a call planned by the general kernel and, unless they are null, the
+// gathered activations and the rows' gates, in the blocks the router worked in.
 struct GatherParams {
     const DevPlan *plan;
     const uint16_t *x;               // hidden [T][d]
     const int32_t *idx;              // [T][k]
+    const float *gate;               // [T][k]
     const int32_t *block_base;       // PlanParams::block_counts after the planning kernel
     int32_t *perm, *inv_pos, *tok_of_sorted;
     uint16_t *xs;
+    float *row_gate;                 // the gate of the pair at every sorted position, 1 for a shared expert's rows
     int T, d, E, k, n_shared, tokens_per_block, n_blocks;
     int permute;                     // store elements j and j + 4 of every eight side by side (the order in which 4-bit codes expand)
 };
 cudaError_t launch_gather_rows(cudaStream_t stream, int n_sms, const GatherParams &p);
 // pairs: CTA pairs (bf16 slots only); fmt: what the slots hold, 0 = bf16 blobs, 1 = 4-bit blobs
 cudaError_t launch_ffn_gemm(cudaStream_t stream, int phase, int n_sms, bool pairs, int fmt, const GemmParams &p);
+// gate null: the rows are weighted already
 cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const float *gate, const int32_t *inv_pos,
                                 const float *zs, uint16_t *out, int T, int d, int k, int n_shared, int n_sms);
 

@@ -527,6 +527,22 @@ def test_q4_slots_match_the_oracle(d, F, E, k, C, n_shared):
         MoELayer(1536, 64, 8, 2, 4, slots="q4")
 
 
+@pytest.mark.parametrize("d,F,E,k,n_shared,T", [(512, 72, 6, 2, 1, 40), (2048, 264, 5, 4, 0, 72), (1024, 64, 3, 3, 2, 300)])
+def test_4bit_tokens_get_the_same_result_from_long_and_short_calls(d, F, E, k, n_shared, T):
+    """A prompt through the grouped GEMM against the same tokens in decode calls of 8: both round gate * h to bf16, so
+    only fp32 sums of the tensor cores differ in their order.  Where such sums differ by delta of themselves, a share of
+    delta / 2^-8 of the roundings of h and y falls the other way, by 2^-8 of a value: sqrt(2^-8 * delta) in the 2-norm, 1e-3
+    for delta = 2^-12 (twice the 4.9e-4 measured at d_model 2048); rounding h without its gate would be 3.2e-3."""
+    P = _pair(d, F, E, k, E, seed=700 + d // 256, n_shared=n_shared, store="q4slots")
+    P.set_bias(_bias(24, E, 0.5, 1), None)
+    x = gen.hidden_states(701, 0, "prefill", 0, T, d)
+    long_call = gen.bf16_bits_to_f32(P.gpu.forward_np(x)["out_bits"]).astype(np.float64)
+    short = np.concatenate([gen.bf16_bits_to_f32(P.gpu.forward_np(x[i:i + 8])["out_bits"]) for i in range(0, T, 8)]).astype(np.float64)
+    err = np.linalg.norm(long_call - short) / np.linalg.norm(short)
+    assert err <= 1e-3, err
+    P.close()
+
+
 def test_parity_without_programmatic_launch():
     """The decode kernels are launched with programmatic stream serialisation by default; the
     same parity must hold with the attribute switched off (the switch is read once per process,

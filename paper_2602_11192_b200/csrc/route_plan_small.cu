@@ -141,15 +141,15 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     // (long past when this kernel waits for the call before to end)
     if (cta_rank == 0 && warp <= 1)
         wait_for_previous_planning(p);
-    // The launch may have been made with programmatic stream serialisation: this block can then be
-    // running before the kernel ahead of it in the stream has finished.  Nothing before this point
-    // reads what that kernel may have written; wait for it here (returns at once in an ordinary
-    // launch).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool by_count = p.policy == MELINOE_POLICY_COUNT;
     // The dot products run twice: first on whatever the hidden states' memory holds, while the kernel ahead ends, so that
     // the pass that counts finds its instructions in the caches (2.3 -> 1.5 us for one token of d_model 2048; the
     // same for the planning below, or for the FFN kernel while it waits, costs registers and gains nothing).
+    // With programmatic stream serialisation this block can be running before the kernel ahead of it in the stream
+    // has finished.  What that kernel may be writing (hidden states, sequences, biases) is only loaded and dropped by the
+    // first pass: no branch, no result and no address beyond its arrays comes from it.  The second pass waits for
+    // that kernel (in an ordinary launch the wait returns at once).
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
     if (pass == 1)
@@ -183,7 +183,9 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
                 const float of_seq = lane < n_seq ? __uint_as_float(ld_now(bias + (size_t)lane * E + e_mine)) : 0.0f;
                 my_bias = __shfl_sync(0xffffffffu, of_seq, q & 31);
             } else if (lane < mine) {
-                my_bias = __uint_as_float(ld_now(bias + (size_t)q * E + e_mine));
+                // (the first pass may find anything in token_seq: kept inside the table, one instruction; loading it in the second
+                // pass only costs a layer of one-token calls 0.3 us)
+                my_bias = __uint_as_float(ld_now(bias + (size_t)min((unsigned)q, (unsigned)n_seq - 1u) * E + e_mine));
             }
         }
         float a = 0.0f, b = 0.0f, my_logit = 0.0f;

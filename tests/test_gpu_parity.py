@@ -68,6 +68,35 @@ def test_decode_router_over_its_token_groups_and_sequences(d, E, k, n_seq):
     P.close()
 
 
+@pytest.mark.parametrize("T", [1, 4, 8])
+def test_decode_router_takes_sequences_that_the_kernel_ahead_writes(T):
+    """token_seq is the output of the kernel directly ahead (a prompt through experts of zeros), over what was no valid
+    sequence before, with more sequences than a warp has lanes: the router may be running by then, and must not have
+    looked a bias up with what it found."""
+    import torch
+    from paper_2602_11192_b200.runner import current_stream_ptr, to_dev_bf16
+    d, E, k, n_seq = 512, 12, 2, 40
+    A, P = _pair(d, 16, E, k, E, seed=97), _pair(d, 16, E, k, E, seed=98)
+    A.gpu.store.zero_()
+    bias = _bias(97, E, 0.5, n_seq)
+    bias_dev, seq = torch.from_numpy(bias).cuda(), torch.empty((9, d // 2), dtype=torch.int32, device="cuda")
+    P.gpu.layer.set_router_bias(bias_dev, seq, n_seq)
+    x = [gen.hidden_states(98, 0, "decode", i, T, d) for i in range(4)]
+    xd, xa = [to_dev_bf16(v) for v in x], to_dev_bf16(gen.hidden_states(97, 0, "prefill", 0, 9, d))
+    out = torch.empty((T, d), dtype=torch.int16, device="cuda")
+    for step in range(4):
+        seq.fill_(0x7FFFFFF0 if step % 2 else -5)
+        A.gpu.layer.forward(current_stream_ptr(), xa, 9, seq)
+        P.gpu.layer.forward(current_stream_ptr(), xd[step], T, out)
+        torch.cuda.synchronize()
+        assert int(seq.abs().max()) == 0
+        idx, _, logits = oracle.route(x[step], P.w_r, k, bias, np.zeros(T, np.int32))
+        assert np.array_equal(P.gpu.layer.last_logits(T).view(np.uint32), logits.view(np.uint32))
+        assert np.array_equal(P.gpu.layer.last_routing(T)[0], idx)
+    A.close()
+    P.close()
+
+
 @pytest.mark.parametrize("store,d,E,k,n_shared", [("bf16", 512, 64, 32, 3), ("q4slots", 512, 9, 1, 0), ("bf16", 256, 1, 1, 0), ("bf16", 4096, 5, 4, 1)])
 def test_one_token_calls_take_their_requests_from_records_of_their_own(store, d, E, k, n_shared):
     """One-token calls, fetching (announced by the plan's word) and then all resident (announced by the records, of

@@ -219,7 +219,7 @@ struct melinoe_moe {
     cudaEvent_t ev_arrive = nullptr;    // copy stream: a wave's transfers have landed
     std::vector<cudaEvent_t> ev_group;  // compute stream: FFN group g of the current call is done
     bool has_last = false;
-    uint32_t call_seq = 0, planned_seq = 0;   // the latest call, and the latest whose planning kernel was queued
+    uint32_t call_seq = 0;
     int last_T = 0;
     std::atomic<int> sticky{0};
 
@@ -922,8 +922,6 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     pp.hplan = h->hplan;
     pp.gmax = gmax;
     pp.call_seq = h->call_seq;
-    pp.prev_seq = h->planned_seq;
-    pp.err = h->err_word;
     pp.policy = h->policy;
     pp.gamma = h->gamma;
     pp.stats = stats_dev;
@@ -945,7 +943,6 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     if (small) {
         CU_TRY(launch_route_plan_small(s, static_cast<const uint16_t *>(hidden_dev), h->w_router, h->bias, h->token_seq,
                                        h->n_seq, h->d, sc.idx, sc.gate, sc.logits, pp));
-        h->planned_seq = h->call_seq;
     } else {
         const RouterShape sh = router_shape(T, h->E, h->n_sms);
         pp.block_counts = sc.block_counts;
@@ -953,7 +950,6 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         CU_TRY(launch_router(s, sh, static_cast<const uint16_t *>(hidden_dev), h->w_router, h->bias, h->token_seq, T, h->d,
                              h->E, h->k, sc.idx, sc.gate, sc.logits, sc.block_counts));
         CU_TRY(launch_plan(s, pp));
-        h->planned_seq = h->call_seq;
         GatherParams ga;
         ga.plan = h->plan;
         ga.x = static_cast<const uint16_t *>(hidden_dev);

@@ -553,8 +553,13 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
     // routing, plan) is in memory once the word is there.  A programmatically launched grid never
     // starts before every CTA of the grid ahead of it is running, and the planner waits for nobody
     // behind it, so the wait ends; it is bounded all the same.
+    // This grid must not end before the planner's either, which is still writing cache state, token lists and
+    // statistics when it announces the plan: whatever comes behind this kernel (the next planner, a preload, a copy of
+    // the statistics) is ordered behind both by this kernel's end alone.  The producer's thread waits for it when its
+    // last copy is on the way, where the wait costs nothing.
+    auto planner_ended = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
     if (p.wait_prior)
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        planner_ended();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const DevPlan *plan = p.plan;
     // One token: if every expert is resident, the requests' records come without that word and say themselves that they
@@ -726,6 +731,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
         // the counters advance once per CTA and launch, whatever happens
         if (tid < NW && atomicAdd(p.sync + tid * kSyncPitch, 1u) == (unsigned)(G - 1))
             p.sync[tid * kSyncPitch] = 0u;
+        planner_ended();
         return;
     }
     if (XT) {
@@ -847,6 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
                     while (!mbar_try(full0 + 8 * (j % S), (j / S) & 1u) && clock64() - t0 < kWaitLimitCycles) {
                     }
             }
+            planner_ended();
         }
     } else {
         // =================================================================== consumers

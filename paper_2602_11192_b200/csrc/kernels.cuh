@@ -40,8 +40,6 @@ struct PlanParams {
     HostPlan *hplan;          // page-locked host memory (device-visible address)
     uint32_t gmax;            // compute groups the caller has room for
     uint32_t call_seq;        // written to the miss queue's seq word when the record is complete
-    uint32_t prev_seq;        // sequence number of the call planned before this one
-    int *err;                 // device error word (0 = ok)
     int fast;                 // fused planner: 1 = the call is served by one decode launch that fetches the missed experts itself,
                               // 2 = by one launch per compute group, the first of which is queued already
     int policy;               // MELINOE_POLICY_LRU or MELINOE_POLICY_COUNT
@@ -70,27 +68,6 @@ __host__ __device__ inline TraceLayout trace_layout(int n_experts, int top_k, in
     return t;
 }
 cudaError_t launch_plan(cudaStream_t stream, const PlanParams &p);
-#ifdef __CUDACC__
-// Waits (bounded, about 2 s) until the planning of the call before is complete: see DevPlan::done.
-__device__ __forceinline__ void wait_for_previous_planning(const PlanParams &p)
-{
-    const long long t0 = clock64();
-    for (;;) {
-        uint32_t v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&p.plan->done) : "memory");
-        if (v == p.prev_seq)
-            return;
-        if (clock64() - t0 > 4000000000ll) {
-            atomicExch(p.err, MELINOE_ERR_TIMEOUT);
-            return;
-        }
-    }
-}
-__device__ __forceinline__ void planning_complete(const PlanParams &p)
-{
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&p.plan->done), "r"(p.call_seq) : "memory");
-}
-#endif
 
 // ---- router and planning in one kernel (one thread-block cluster), for calls of at most 8 tokens
 bool route_plan_small_supported(int T, int k, int d);

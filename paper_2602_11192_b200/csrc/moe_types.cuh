@@ -90,10 +90,6 @@ struct DevPlan {
     // planner's grid to drain.  A decode call whose FFN launch fetches the missed experts itself needs fast[] alone: it is
     // announced as soon as that is complete, the rest of the plan follows (before the planner's grid ends).
     uint64_t ready;
-    // Sequence number of the call whose planning is complete, cache state included; the next call's planner looks at
-    // it (the grid ahead of that planner in the stream is the FFN kernel's, whose end does not say that this one has ended).
-    uint32_t done;
-    uint32_t pad_;
     int32_t group_vr_begin[kMaxGroups + 1];   // first entry of dreq[] of every compute group
     int32_t counts[kMaxReq];
     int32_t offsets[kMaxReq + 1];

@@ -50,7 +50,6 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
 
     // ---- load persistent cache state, clear tables.  The router, which may still be running (programmatic launch), lets
     // this kernel start only once everything ahead of it is complete.
-    wait_for_previous_planning(p);
     {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(p.cache);
         uint32_t *dst = reinterpret_cast<uint32_t *>(&s_cache);
@@ -456,7 +455,6 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p)
     if (tid == 0) {
         __threadfence();
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&plan->ready), "l"(ready_word(p.call_seq, 0, 0, false)) : "memory");
-        planning_complete(p);
     }
 }
 

@@ -138,9 +138,6 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     DevCache *cache = p.cache;
     if (cta_rank == 0 && tid < 12)       // into L2, whatever of it is not there yet
         prefetch_l2(reinterpret_cast<const char *>(cache) + min(tid * 128, (int)sizeof(DevCache) - 4));
-    // (long past when this kernel waits for the call before to end)
-    if (cta_rank == 0 && warp <= 1)
-        wait_for_previous_planning(p);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool by_count = p.policy == MELINOE_POLICY_COUNT;
     // The dot products run twice: first on whatever the hidden states' memory holds, while the kernel ahead ends, so that
@@ -747,8 +744,6 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     asm volatile("bar.sync 4, 64;" ::: "memory");
     if (!fast)
         announce();
-    if (lane == 0)
-        planning_complete(p);
     // What may live in host memory goes out last, so that no fence above has to wait for the host link:
     // the statistics, and the miss queue for calls whose transfers the host issues.
     __syncwarp();

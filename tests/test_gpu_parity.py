@@ -108,6 +108,53 @@ def test_one_token_calls_take_their_requests_from_records_of_their_own(store, d,
     P.close()
 
 
+@pytest.mark.parametrize("policy", ["lru", "count"])
+def test_what_follows_a_decode_call_sees_all_that_its_planner_wrote(policy):
+    """The smallest layer, whose FFN kernel takes hardly longer than the rest of the planning it overlaps.  The kernel
+    directly behind it (programmatically launched: another layer's call that takes the statistics as its hidden state)
+    reads the statistics of this very call; preloads queued behind calls, with nothing waiting in between, leave the
+    cache as the oracle has it."""
+    import torch
+    from paper_2602_11192_b200.runner import current_stream_ptr, to_dev_bf16
+    d, F, E, k, C = 256, 8, 12, 2, 6
+    P, R = _pair(d, F, E, k, C, seed=101), _pair(d, F, E, k, E, seed=102)
+    P.set_policy(policy, 0.9 if policy == "count" else 0.0)
+    # (whole numbers as bf16 patterns are denormal: the reader's router scales them up)
+    R.gpu.set_router(np.full((E, d), 0x4E80, np.uint16))
+    s = current_stream_ptr()
+    out = torch.empty((1, d), dtype=torch.int16, device="cuda")
+    xs = [gen.hidden_states(101, 0, "decode", i, 1, d) for i in range(40)]
+    xd = [to_dev_bf16(x) for x in xs]
+    rec = torch.zeros(d // 2, dtype=torch.int32, device="cuda")      # a hidden state that begins with a statistics record
+    for i, x in enumerate(xs):
+        P.gpu.layer.forward(s, xd[i], 1, out, rec)
+        R.gpu.layer.forward(s, rec, 1, out)
+        torch.cuda.synchronize()
+        seen = R.gpu.layer.last_logits(1).copy()
+        R.gpu.layer.forward(s, rec, 1, out)
+        torch.cuda.synchronize()
+        assert np.array_equal(seen.view(np.uint32), R.gpu.layer.last_logits(1).view(np.uint32)), "call %d" % i
+        assert int(rec[10]) == i + 1                                 # call_no
+        P.cache.call(oracle.route(x, P.w_r, k, None, None)[0])
+    rs = np.random.default_rng(101)
+    for rnd in range(10):
+        for i, x in enumerate(xs[:8]):
+            P.gpu.layer.forward(s, xd[i], 1, out, rec)
+            ids = rs.permutation(E)[:2].astype(np.int32)
+            P.gpu.layer.preload(ids)
+            P.cache.call(oracle.route(x, P.w_r, k, None, None)[0])
+            P.cache.preload(ids.tolist())
+        P.gpu.layer.forward(s, xd[8], 1, out, rec)
+        P.cache.call(oracle.route(xs[8], P.w_r, k, None, None)[0])
+        torch.cuda.synchronize()
+        eos, _, tot = P.cache.state()
+        eos_g, tot_g = P.gpu.layer.cache_state()
+        assert np.array_equal(eos_g, eos) and tot_g == tot
+        assert np.array_equal(P.gpu.layer.cache_counts(E).view(np.uint32), P.cache.counts().view(np.uint32))
+    P.close()
+    R.close()
+
+
 def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory():
     """d_model 4096 with 5 to 8 tokens per call: the decode kernel writes the hidden states' tensor-core
     operands into tensor memory once and reads them from there (the shared memory goes to taller weight

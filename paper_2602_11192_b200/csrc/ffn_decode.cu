@@ -547,10 +547,10 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
         s_deferred = 0;
     // Nothing above reads what an earlier kernel wrote.  With programmatic stream serialisation this
     // CTA may be running while the kernel ahead of it in the stream (the planner) still is.  It does
-    // not wait for that grid to drain (which costs microseconds) but for the word the planner writes
-    // last, behind a device-wide fence, when the call's plan is complete.  The planner itself has
-    // waited for everything ahead of it in the stream, so whatever this kernel reads (hidden states,
-    // routing, plan) is in memory once the word is there.  A programmatically launched grid never
+    // not wait for that grid to drain (which costs microseconds) but acquires what the planner releases when the records
+    // that this launch reads are complete: the plan's word, or for one token the records themselves.  The planner itself
+    // has waited for everything ahead of it in the stream, so whatever else this kernel reads (hidden states, resident
+    // weights) is in memory then.  A programmatically launched grid never
     // starts before every CTA of the grid ahead of it is running, and the planner waits for nobody
     // behind it, so the wait ends; it is bounded all the same.
     // This grid must not end before the planner's either, which is still writing cache state, token lists and
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const DevPlan *plan = p.plan;
     // One token: if every expert is resident, the requests' records come without that word and say themselves that they
-    // are there (one round trip instead of two, and no fence in the planner); otherwise as for more tokens.
+    // are there (one round trip instead of two); otherwise as for more tokens.
     const int n_one = XT == 0 && p.fast && Tc == 1 ? p.k + p.n_shared : 0;
     bool got = true;
     if (tid < max(n_one, 1)) {

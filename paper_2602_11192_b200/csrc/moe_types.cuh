@@ -85,10 +85,12 @@ __host__ __device__ inline uint64_t ready_word(uint32_t seq, int n_fast, int sta
 // Per-call plan written by the planning kernel, read by the FFN and combine kernels.
 struct DevPlan {
     int32_t n_tokens, n_req, n_hits, n_miss, n_evict, n_groups, n_dreq, status;
-    // Announces the plan: ready_word(), written behind a device-wide fence by the planning kernel.  The decode FFN
-    // kernel, which may have been scheduled while the planner was still running, waits for it instead of waiting for the
-    // planner's grid to drain.  A decode call whose FFN launch fetches the missed experts itself needs fast[] alone: it is
-    // announced as soon as that is complete, the rest of the plan follows (before the planner's grid ends).
+    // Announces the plan: ready_word(), stored with release semantics by the planning kernel.  The decode FFN
+    // kernel, which may have been scheduled while the planner was still running, acquires it instead of waiting for the
+    // planner's grid to drain.  A call that one decode launch serves (the launch fetches the missed experts itself, or
+    // there are none) needs fast[] alone: it is announced as soon as that is complete; cache state, lists, inspection records and
+    // statistics follow before the planner's grid ends, which the FFN kernel's grid waits for before it ends itself.
+    // One token without misses: one[] takes the place of both.
     uint64_t ready;
     int32_t group_vr_begin[kMaxGroups + 1];   // first entry of dreq[] of every compute group
     int32_t counts[kMaxReq];
@@ -97,7 +99,7 @@ struct DevPlan {
     ReqRec req[kMaxReq];
     DecReq dreq[kMaxReq];                     // group 0 (hits, then shared experts), then the misses by wave
     FastReq fast[kMaxReq];
-    OneReq one[kMaxReq];                      // in the order of fast[]; written instead of it, and of `ready`
+    OneReq one[kMaxReq];                      // in the order of fast[]
 };
 
 // The miss queue of a call: what the host needs in order to issue the transfers, written by

@@ -281,6 +281,10 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     if (cta_rank != 0)
         return;
+    // One token: the fence of the records that announce the plan (see `put` below), in front of all of them and here, where
+    // this warp waits for the others' logits anyway.
+    if (warp == 0 && p.fast && T == 1)
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
     // ================================================================ top-k
@@ -486,7 +490,9 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     auto announce = [&] {
         asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
         if (one) {
-            // no fence, and no second round trip for whoever waits: every record speaks for itself
+            // No second round trip for whoever waits: every record speaks for itself.  What is announced beside it is what was
+            // complete when this grid's wait for the grid ahead returned (hidden state, slots, the FFN kernel's accumulator
+            // and counters): the fence that these lanes executed since makes each of these stores a release of it.
             auto put = [&](int at, const char *src, float gate) {
                 asm volatile(
                     "{\n\t.reg .b128 v;\n\t"

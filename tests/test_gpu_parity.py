@@ -155,6 +155,41 @@ def test_what_follows_a_decode_call_sees_all_that_its_planner_wrote(policy):
     R.close()
 
 
+@pytest.mark.parametrize("d,F", [(256, 8), (2048, 64)])
+def test_one_token_calls_in_a_chain_read_what_the_call_ahead_wrote(d, F):
+    """Layers whose hidden state is the output of the layer ahead, in two buffers that take turns (so every SM has held
+    older contents of the same addresses), all resident: queued back to back, the bits of calls that are waited for."""
+    import torch
+    from paper_2602_11192_b200.runner import current_stream_ptr, to_dev_bf16
+    E, k, n_layers = 8, 2, 5
+    Ps = [_pair(d, F, E, k, E, seed=110 + l) for l in range(n_layers)]
+    s = current_stream_ptr()
+    for l, P in enumerate(Ps):
+        P.gpu.layer.preload(np.arange(E, dtype=np.int32))
+        P.set_bias(_bias(110 + l, E, 0.5, 1), None)
+    buf = torch.empty((2, d), dtype=torch.int16, device="cuda")
+    xs = torch.stack([to_dev_bf16(gen.hidden_states(110, 0, "decode", i, 1, d))[0] for i in range(20)])
+
+    def chain(wait):
+        outs = torch.empty((len(xs), n_layers, d), dtype=torch.int16, device="cuda")
+        for i in range(len(xs)):
+            buf[0].copy_(xs[i])
+            for l, P in enumerate(Ps):
+                P.gpu.layer.forward(s, buf[l % 2], 1, buf[(l + 1) % 2])
+                if wait:
+                    torch.cuda.synchronize()
+                    outs[i, l].copy_(buf[(l + 1) % 2])
+            outs[i, -1].copy_(buf[n_layers % 2])
+        torch.cuda.synchronize()
+        return outs.cpu().numpy()
+
+    want = chain(True)
+    for _ in range(5):
+        assert np.array_equal(chain(False)[:, -1], want[:, -1])
+    for P in Ps:
+        P.close()
+
+
 def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory():
     """d_model 4096 with 5 to 8 tokens per call: the decode kernel writes the hidden states' tensor-core
     operands into tensor memory once and reads them from there (the shared memory goes to taller weight

@@ -105,16 +105,32 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// The same where threads of the other CTA of a pair arrive, too: acquires at the scope of the cluster.
+__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag)
 {
-    if (mbar_try(bar, parity))
+    auto reached = [&] { return CLUSTER ? mbar_try_cluster(bar, parity) : mbar_try(bar, parity); };
+    if (reached())
         return true;
     if (*abort_flag)
         return false;
     const long long t0 = clock64();
     for (;;) {
         for (int i = 0; i < 64; ++i)
-            if (mbar_try(bar, parity))
+            if (reached())
                 return true;
         if (*abort_flag)
             return false;
@@ -190,12 +206,12 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// Arrival on the peer CTA's barrier.  What it reports is in this SM (expanded weights, behind a proxy fence; accumulators
-// drained or filled, behind tcgen05.wait), so nothing has to be made visible through memory: with release semantics
-// of cluster scope each arrival took its warp 1100 cycles.
+// Arrival on the peer CTA's barrier, a release at the scope of the cluster: what it reports (expanded weights in this CTA's
+// shared memory, an accumulator that may be overwritten) is used by an operation that a thread of the peer issues.  It
+// takes its warp some 1100 cycles.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar)
 {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 // One lane of a converged warp.
 __device__ __forceinline__ bool elect_one()
@@ -592,14 +608,14 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
                     break;
                 const uint32_t idesc = instr_desc_bf16(CG * 128, __shfl_sync(0xffffffffu, it.n, 0), PHASE == 2);
                 const uint32_t acc = item & 1u;
-                bool ok = item < 2 || mbar_wait(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag);
+                bool ok = item < 2 || mbar_wait<CG == 2>(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag);
                 if (!__all_sync(0xffffffffu, ok))
                     break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d_tmem = tmem_base + acc * NT;
                 uint32_t accumulate = 0;
                 for (int kb = 0; kb < kblocks; ++kb) {
-                    ok = mbar_wait(full0 + 8 * s, parity, abort_flag);
+                    ok = mbar_wait<FMT == 1>(full0 + 8 * s, parity, abort_flag);
                     if (!__all_sync(0xffffffffu, ok))
                         break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -728,9 +744,11 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(GemmPara
     } else if (FMT == 1 && warp < 2 + kEpilogueWarps + 4 * kExpandGroups) {
         // ============================================================ expansion of 4-bit codes (warps 10..25)
         // Groups of four warps take the k-blocks in turn, counted over all items (so that a group is never two uses of
-        // a stage ahead, which a barrier's parity could not tell): what a k-block takes is latency, 1350 cycles of waits, arithmetic
-        // and the fence before the tensor cores may read, which the other groups' k-blocks cover.  (512 tokens,
-        // us a pass: two groups 140, four 127.)
+        // a stage ahead, which a barrier's parity could not tell): what a k-block takes is latency, waits, arithmetic and
+        // the fence before the tensor cores may read, which the other groups' k-blocks cover.  (512 tokens, us a
+        // pass: two groups 140, four 127.)  In the odd CTA the arrival that makes the weights visible to the MMA thread of
+        // the even one adds to it (512 tokens 114 -> 137 us, 8192 tokens 1084 -> 1218; a relaying warp, one arrival
+        // per k-block by the group's warps in turn, or more stages do not make it less).
         const int row = ((warp - 10) & 3) * 32 + lane, group = (warp - 10) >> 2;     // row of the weight tile, or (column group, f) of GEMM 2's
         const size_t ub = (size_t)p.unit_bytes, scales = 3 * (size_t)(p.d / 2);
         uint32_t n0 = 0, rn = 0;

@@ -654,6 +654,19 @@ def test_4bit_tokens_get_the_same_result_from_long_and_short_calls(d, F, E, k, n
     P.close()
 
 
+@pytest.mark.parametrize("T", [24, 300])
+def test_4bit_prompts_give_the_same_bits_every_time(T):
+    """Weight tiles that one CTA of a pair expands and the other's thread multiplies, many per CTA: a tile that was read
+    before it was complete would change some output."""
+    d, F, E, k = 2048, 1408, 12, 4
+    P = _pair(d, F, E, k, E, seed=66, store="q4slots")
+    x = gen.hidden_states(66, 0, "prefill", 0, T, d)
+    res, _ = P.step(x, tokens=[0, T // 2, T - 1])
+    for _ in range(30):
+        assert np.array_equal(P.gpu.forward_np(x)["out_bits"], res["out_bits"])
+    P.close()
+
+
 def test_parity_without_programmatic_launch():
     """The decode kernels are launched with programmatic stream serialisation by default; the
     same parity must hold with the attribute switched off (the switch is read once per process,

@@ -786,6 +786,26 @@ def test_trace_miss_proxies_at_the_edges_of_their_batches(T, K, E, gamma, sizes)
         assert abs(soft[j] - so.mean()) <= 1e-10 * max(1.0, abs(so.mean())), (c, soft[j], so.mean())
 
 
+@pytest.mark.parametrize("n_layers,E,n", [(1, 64, 57), (3, 5, 700)])
+def test_trace_miss_proxies_of_no_tokens_are_zero(n_layers, E, n):
+    """A trace without tokens: no misses and a mean of 0 for every configuration, whatever an earlier kernel left in
+    shared memory (a trace of many tokens is evaluated ahead of each); a configuration that names nothing is marked."""
+    from paper_2602_11192_b200 import binding as B
+    from paper_2602_11192_b200.runner import current_stream_ptr
+    import torch
+    cfg = (B.ProxyConfig * (n + 1))(*[B.ProxyConfig(i % n_layers, 1 + i % E, 0.9) for i in range(n)], B.ProxyConfig(n_layers, 1, 0.9))
+    cfg_dev = torch.frombuffer(bytearray(bytes(cfg)), dtype=torch.uint8).cuda()
+    trace = (torch.arange(n_layers * 600 * 2, dtype=torch.int32, device="cuda") % E).contiguous()
+    soft = torch.empty(n + 1, dtype=torch.float64, device="cuda")
+    hard = torch.empty(n + 1, dtype=torch.int64, device="cuda")
+    for _ in range(10):
+        B.melinoe_trace_miss_proxies(current_stream_ptr(), trace, n_layers, 600, 2, E, cfg_dev, n + 1, soft, hard)
+        soft.fill_(7.0)
+        B.melinoe_trace_miss_proxies(current_stream_ptr(), trace, n_layers, 0, 2, E, cfg_dev, n + 1, soft, hard)
+        assert not bool(soft[:n].any()) and not bool(hard[:n].any())
+        assert bool(torch.isnan(soft[n])) and int(hard[n]) == -1
+
+
 def test_argument_and_state_errors():
     import torch
     from paper_2602_11192_b200 import MoELayer, MelinoeError, melinoe_moe_expert_bytes

@@ -93,7 +93,6 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
 #pragma unroll
         for (int e = 0; e < EE / 2; ++e)
             acc[t][e] = 0ull;
-    // (the router matrix does not change while calls are queued; everything else may be the work of the kernel ahead)
     // staged form: this warp's rows of a piece, those of the router matrix or those of the tokens
     const int w_rows = n_eg * EE, stage_bytes = (w_rows + tokens_per_block) * 512;
     const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_logit + tokens_per_block * kMaxExperts);
@@ -107,15 +106,15 @@ router_topk_kernel(const uint16_t *__restrict__ x, const uint16_t *__restrict__ 
             for (int r = warp; r < w_rows; r += n_warps)
                 copy16(dst + r * 512, w_r + (min(r, E - 1) * d + at));
     };
-    if (CH == 0)
-        for (int c = 0; c < kStages - 1 && c < n_chunks; ++c)
-            fetch(c, false);
+    // (all operands, the router matrix too, may be the work of the kernel ahead)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (CH == 0)
         for (int c = 0; c < kStages - 1; ++c) {
-            if (c < n_chunks)
+            if (c < n_chunks) {
+                fetch(c, false);
                 fetch(c, true);
+            }
             asm volatile("cp.async.commit_group;" ::: "memory");
         }
     // top-k below: warp w serves token w of the block first; its bias is on the way meanwhile

@@ -356,6 +356,30 @@ def test_router_and_token_lists_at_the_edges_of_their_tiles(E, k, Ts):
     P.close()
 
 
+@pytest.mark.parametrize("T,d,E,k", [(9, 512, 12, 2), (400, 512, 12, 2), (600, 4096, 64, 32), (1500, 2048, 64, 32)])
+def test_prompts_read_a_router_matrix_that_the_kernel_ahead_writes(T, d, E, k):
+    """Only decode calls may read the router matrix before the work ahead of them has finished: here it is the output of
+    the kernel directly ahead of a prompt, which may be running by then."""
+    import torch
+    from paper_2602_11192_b200.runner import current_stream_ptr, to_dev_bf16
+    A, P = _pair(d, 16, E, k, E, seed=121), _pair(d, 16, E, 2, E, seed=122)
+    A.gpu.layer.preload(np.arange(E, dtype=np.int32))
+    w = torch.zeros((E, d), dtype=torch.int16, device="cuda")
+    P.gpu.layer.set_router(w)
+    x = gen.hidden_states(122, 0, "prefill", 0, T, d)
+    xd, out = to_dev_bf16(x), torch.empty((T, d), dtype=torch.int16, device="cuda")
+    for step in range(4):
+        xa = to_dev_bf16(gen.hidden_states(121, 0, "prefill", step, E, d))
+        A.gpu.layer.forward(current_stream_ptr(), xa, E, w)
+        P.gpu.layer.forward(current_stream_ptr(), xd, T, out)
+        torch.cuda.synchronize()
+        idx, _, logits = oracle.route(x, w.cpu().numpy().view(np.uint16), 2, None, None)
+        assert np.array_equal(P.gpu.layer.last_logits(T).view(np.uint32), logits.view(np.uint32))
+        assert np.array_equal(P.gpu.layer.last_routing(T)[0], idx)
+    A.close()
+    P.close()
+
+
 def test_prefill_router_breaks_ties_towards_the_lowest_expert_id():
     """More than 8 tokens go through the general router kernel: with a zero router matrix the logits are
     the bias alone, and a bias with equal entries makes ties that must go to the lowest ids (Eq. 1 with

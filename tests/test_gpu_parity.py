@@ -97,6 +97,51 @@ def test_decode_router_takes_sequences_that_the_kernel_ahead_writes(T):
     P.close()
 
 
+@pytest.mark.parametrize("T,E,k,C", [(1, 64, 8, 64), (1, 40, 3, 5), (3, 12, 2, 6), (8, 33, 8, 33), (8, 16, 2, 4), (20, 12, 2, 6)])
+def test_hidden_states_and_biases_that_are_not_finite(T, E, k, C):
+    """One token's hidden state holds NaNs (all its logits are NaN: the lowest ids are taken, once each), another's experts
+    are masked with a bias of -inf but for k - 1 of them, a third's are all +inf: every token has k distinct experts, the
+    call's requests are no more than its pairs, and the other tokens' results are the oracle's."""
+    d = 512
+    P = _pair(d, 16, E, k, C, seed=130 + E)
+    bias = np.zeros((3, E), np.float32)
+    bias[1, :] = -np.inf
+    bias[1, E - (k - 1):] = 0.0
+    bias[2, :] = np.inf
+    for step in range(3):
+        x = gen.hidden_states(130 + E, 0, "decode", step, T, d)
+        bad = step % T
+        x[bad, ::7] = 0x7FC1 if step != 1 else 0xFFFF
+        seq = np.zeros(T, np.int32)
+        if T > 2:
+            seq[(bad + 1) % T], seq[(bad + 2) % T] = 1, 2
+        P.set_bias(bias, seq)
+        res = P.gpu.forward_np(x)
+        idx, _ = P.gpu.layer.last_routing(T)
+        assert idx.min() >= 0 and idx.max() < E and all(len(set(r)) == k for r in idx.tolist())
+        assert idx[bad].tolist() == list(range(k))
+        good = [t for t in range(T) if t != bad and seq[t] != 2]
+        if T > 2:
+            assert sorted(idx[(bad + 1) % T].tolist()) == [0] + list(range(E - (k - 1), E))
+            assert idx[(bad + 2) % T].tolist() == list(range(k))
+        st = res["stats"]
+        assert st["status"] == 0 and st["n_distinct"] == len(np.unique(idx)) == st["hits"] + st["misses"]
+        cnt, off, perm = P.gpu.layer.last_gather(T)
+        assert np.array_equal(cnt, np.bincount(idx.reshape(-1), minlength=E)) and sorted(perm.tolist()) == list(range(T * k))
+        if good:
+            sub_bias, sub_seq = bias, seq[good]
+            idx_o, gate_o, _ = oracle.route(x[good], P.w_r, k, sub_bias, sub_seq)
+            assert np.array_equal(idx[good], idx_o)
+            y = oracle.ffn_combine(x[good], idx_o, gate_o, P.weights, P.F, 0)
+            from parity_util import rel_err_per_token
+            assert rel_err_per_token(res["out_bits"][good], y).max() <= 8e-3
+    # and the cache is in order: every resident expert in one slot
+    eos, _ = P.gpu.layer.cache_state()
+    held = [e for e in eos.tolist() if e >= 0]
+    assert len(set(held)) == len(held)
+    P.close()
+
+
 @pytest.mark.parametrize("store,d,E,k,n_shared", [("bf16", 512, 64, 32, 3), ("q4slots", 512, 9, 1, 0), ("bf16", 256, 1, 1, 0), ("bf16", 4096, 5, 4, 1)])
 def test_one_token_calls_take_their_requests_from_records_of_their_own(store, d, E, k, n_shared):
     """One-token calls, fetching (announced by the plan's word) and then all resident (announced by the records, of

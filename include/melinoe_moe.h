@@ -20,7 +20,7 @@
  *    the host and all of its transfers and kernels are queued.  It never waits for transfers or
  *    compute.
  *  - Environment switches, read once per process (for measurements and tests; none changes results):
- *    MELINOE_MOE_NO_PDL          launch the decode kernels without programmatic stream serialisation;
+ *    MELINOE_MOE_NO_PDL          launch the kernels of forward calls without programmatic stream serialisation;
  *    MELINOE_MOE_HOST_COPIES     every expert transfer is a cudaMemcpyAsync issued by the host;
  *    MELINOE_MOE_GEMM_SINGLE     the prefill GEMM of bf16 slots never pairs CTAs (tcgen05 cta_group::1 only).
  */

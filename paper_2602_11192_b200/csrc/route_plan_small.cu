@@ -715,6 +715,15 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             s_hm[i] = HostMiss{e, slot, (int16_t)group, (int16_t)dep, p.call_seq};
         }
     }
+    // What the host waits for goes to it at once: queuing the transfers takes longer than announcing and computing group 0, behind
+    // a fence that covers these stores too.
+    if (!fast) {
+        __syncwarp();
+        for (int i = lane; i < n_miss; i += 32)
+            store16_host(&p.hplan->miss[i], &s_hm[i]);
+        if (lane == 0)
+            tell_host();
+    }
     const int n_evict = by_count ? n_evict_seq : __popcll(ballot64(ev_flag[0], ev_flag[1]));
     // shared experts: always resident, group 0, behind the hits
     for (int s = lane; s < p.n_shared; s += 32) {
@@ -750,12 +759,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     asm volatile("bar.sync 4, 64;" ::: "memory");
     if (!fast)
         announce();
-    // What may live in host memory goes out last, so that no fence above has to wait for the host link:
-    // the statistics, and the miss queue for calls whose transfers the host issues.
-    __syncwarp();
-    if (!fast)
-        for (int i = lane; i < n_miss; i += 32)
-            store16_host(&p.hplan->miss[i], &s_hm[i]);
+    // The statistics, which may live in host memory, go out last, so that no fence above has to wait for the host link.
     if (lane == 0) {
         if (p.stats) {
             melinoe_moe_stats st;
@@ -771,8 +775,6 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             st.call_no = call_no;
             *p.stats = st;
         }
-        if (!fast)
-            tell_host();
         if (p.trace_rec) {
             melinoe_moe_trace_header th;
             th.call_no = call_no;

@@ -373,7 +373,7 @@ def test_prefill_grouped_gemm(d, F, E, k, C, n_shared, Ts):
     ("q4slots", 512, 200, 3, 3, 1, (9, 16, 129)),      # the same of 4-bit codes, with a shared expert
     ("q4slots", 1024, 264, 4, 2, 0, (70,)),            # codes of a column group in both halves of their 128 bytes
     ("q4slots", 4096, 136, 2, 1, 0, (20,)),
-    ("bf16", 2048, 1416, 2, 1, 1, (9, 140)),           # tiles computed in parts by many CTAs, the last part of GEMM 2 three k-blocks
+    ("bf16", 2048, 1416, 2, 1, 1, (9, 140)),           # d_ff of 22 tiles and an eighth of one; GEMM 2 of 23 k-blocks, the last an eighth
     ("q4slots", 2048, 1416, 2, 1, 1, (9, 300)),        # the same of 4-bit codes; chunks of up to 256 tokens
     ("q4slots", 512, 64, 2, 2, 0, (256, 257)),         # one and two chunks; GEMM 2 of a single k-block
 ])
@@ -777,6 +777,32 @@ def test_parity_with_every_transfer_issued_by_the_host():
            "for step, T in enumerate((1, 2, 1, 8, 2, 1, 12, 1)):\n"
            "    P.step(gen.hidden_states(62, 0, 'decode', step, T, 512))\n"
            "P.close()\n", {"MELINOE_MOE_HOST_COPIES": "1"})
+
+
+@pytest.mark.parametrize("policy,T", [("lru", 1), ("count", 1), ("lru", 3)])
+def test_host_issued_transfers_of_calls_queued_back_to_back(policy, T):
+    """A 4-bit store feeding bf16 slots: the host queues the copies of a call while its planner is still writing the cache
+    state, and then the next call.  Bits and cache are those of calls that are waited for."""
+    import torch
+    from paper_2602_11192_b200.runner import current_stream_ptr, to_dev_bf16
+    d, F, E, k, C, n = 512, 40, 16, 2, 4, 40
+    P = _pair(d, F, E, k, C, seed=64, store="q4")
+    P.set_policy(policy, 0.9 if policy == "count" else 0.0)
+    xs = [gen.hidden_states(64, 0, "decode", i, T, d) for i in range(n)]
+    want = [P.step(x)[0]["out_bits"].copy() for x in xs]
+    P.reset()
+    xd, out = [to_dev_bf16(x) for x in xs], torch.empty((n, T, d), dtype=torch.int16, device="cuda")
+    for i in range(n):
+        P.gpu.layer.forward(current_stream_ptr(), xd[i], T, out[i])
+        P.cache.call(oracle.route(xs[i], P.w_r, k)[0])
+    torch.cuda.synchronize()
+    got = out.cpu().numpy().view(np.uint16)
+    for i in range(n):
+        assert np.array_equal(got[i], want[i]), i
+    eos, _, tot = P.cache.state()
+    eos_g, tot_g = P.gpu.layer.cache_state()
+    assert np.array_equal(eos_g, eos) and tot_g == tot and tot["misses"] > n // 4
+    P.close()
 
 
 def test_parity_of_the_single_cta_gemm_on_a_call_of_many_tokens():

@@ -13,20 +13,6 @@ void count_launch();
 // Programmatic stream serialisation for the decode kernels (on unless MELINOE_MOE_NO_PDL is set in the environment).
 bool pdl_enabled();
 
-#ifdef __CUDACC__
-// Unsigned numbers (none of them 0) in the order of floats, both zeros alike, and back.  A NaN (the sum
-// makes every one the same) is above all: the order is total, whatever the logits are.
-__device__ __forceinline__ unsigned order_key(float v)
-{
-    const unsigned b = __float_as_uint(v + 0.0f);
-    return b & 0x80000000u ? ~b : b | 0x80000000u;
-}
-__device__ __forceinline__ float key_value(unsigned key)
-{
-    return __uint_as_float(key & 0x80000000u ? key & 0x7fffffffu : ~key);
-}
-#endif
-
 // ---- router (Eq. 1): logits, top-k, gates, and per block how many of its tokens chose each expert
 struct RouterShape {
     int tokens_per_warp, n_eg;       // tokens and expert groups of a warp's tile

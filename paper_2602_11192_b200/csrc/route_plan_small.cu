@@ -95,7 +95,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
                         int32_t *__restrict__ idx_out, float *__restrict__ gate_out, float *logits_out,
                         PlanParams p)
 {
-    __shared__ __align__(16) unsigned s_logit[kMaxT][kMaxExperts];     // as order keys
+    __shared__ __align__(16) float s_logit[kMaxT][kMaxExperts];
     __shared__ int32_t s_cnt[2][kMaxExperts];                    // pairs of an expert among pairs 0..31 / 32..63
     __shared__ int32_t s_tok[kMaxPairs];                         // token of a pair
     __shared__ int32_t s_rank[kMaxT][kMaxExperts];               // rank of an expert among a token's logits
@@ -241,7 +241,9 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
                          : "=r"(remote)
                          : "r"((uint32_t)__cvta_generic_to_shared(&s_logit[t][e_mine])), "r"(0));
-            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(order_key(my_logit)) : "memory");
+            // (a NaN counts as +inf from here on, see below)
+            asm volatile("st.shared::cluster.f32 [%0], %1;"
+                         ::"r"(remote), "f"(my_logit == my_logit ? my_logit : __int_as_float(0x7f800000)) : "memory");
             logits_out[(size_t)t * E + e_mine] = my_logit;
         }
     }
@@ -291,21 +293,23 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
     // An element's rank is the number of elements that beat it (greater, or equal with a lower
     // index).  The eight warps share the count (warp w compares against elements 8w .. 8w + 7 of
     // every token) and add their parts up in shared memory.  The ranks are used as places, so they have to be a permutation
-    // whatever the logits are: keys of a total order are compared, not floats (a NaN would be beaten by nothing).
+    // whatever the logits are, and a NaN would be beaten by nothing: it has become +inf, whose gates are NaN all the same.
+    // (Keys of a total order in place of the floats: a tiny layer 11.3 -> 11.5 us.)
+    const float NEG = -__int_as_float(0x7f800000);  // -inf
     if (8 * warp < E)
         for (int t = 0; t < T; ++t) {
-            const unsigned v0 = lane < E ? s_logit[t][lane] : 0u;
-            const unsigned v1 = lane + 32 < E ? s_logit[t][lane + 32] : 0u;
+            const float v0 = lane < E ? s_logit[t][lane] : NEG;
+            const float v1 = lane + 32 < E ? s_logit[t][lane + 32] : NEG;
             int r0 = 0, r1 = 0;
-            const uint4 *row = reinterpret_cast<const uint4 *>(s_logit[t]) + 2 * warp;
+            const float4 *row = reinterpret_cast<const float4 *>(s_logit[t]) + 2 * warp;
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                const uint4 o4 = row[i];
-                const unsigned ov[4] = {o4.x, o4.y, o4.z, o4.w};
+                const float4 o4 = row[i];
+                const float ov[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const int e = 8 * warp + 4 * i + c;
-                    const unsigned o = e < E ? ov[c] : 0u;     // the row's tail beyond E was never written
+                    const float o = e < E ? ov[c] : NEG;     // the row's tail beyond E was never written
                     r0 += (o > v0) || (o == v0 && e < lane);
                     r1 += (o > v1) || (o == v1 && e < lane + 32);
                 }
@@ -329,7 +333,7 @@ route_plan_small_kernel(const uint16_t *__restrict__ x, const uint16_t *__restri
         // ============================================================ selection and gates (Eq. 1), beside the planner
         for (int t = warp - 1; t < T; t += kWarpsPerBlock - 1) {
             const int r0 = s_rank[t][e0], r1 = s_rank[t][e1];
-            const float v0 = key_value(s_logit[t][e0]), v1 = key_value(s_logit[t][e1]);
+            const float v0 = s_logit[t][e0], v1 = s_logit[t][e1];
             const bool on0 = e0 < E && r0 < k, on1 = e1 < E && r1 < k;
             if (on0) {
                 s_sel[t][r0] = v0;

@@ -38,6 +38,18 @@ __device__ __forceinline__ void fma2(uint64_t &acc, uint64_t a, uint64_t b)
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
+// Unsigned numbers (none of them 0) in the order of floats, both zeros alike, and back.  A NaN (the sum
+// makes every one the same) is above all: the order is total, whatever the logits are.
+__device__ __forceinline__ unsigned order_key(float v)
+{
+    const unsigned b = __float_as_uint(v + 0.0f);
+    return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ float key_value(unsigned key)
+{
+    return __uint_as_float(key & 0x80000000u ? key & 0x7fffffffu : ~key);
+}
+
 constexpr int kStages = 4;                 // staged form: pieces of 256 columns in the ring
 __device__ __forceinline__ void copy16(uint32_t dst, const void *src)
 {

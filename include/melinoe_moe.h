@@ -458,6 +458,10 @@ int melinoe_moe_last_call_used_gemm(melinoe_moe_t *h);
  * partly queued call can be exercised without any fault on the device.  0 switches it off. */
 int melinoe_debug_fail_host_copy(int nth);
 
+/* Test hook: queues the gather of a long call, alone, for a plan that nobody announces.  Its bounded wait (about 2 s)
+ * runs out, the kernel ends, and the handle reports TIMEOUT until the cache is reset. */
+int melinoe_debug_gather_without_plan(melinoe_moe_t *h, void *cuda_stream);
+
 /* Number of kernels this library has launched in this process (all handles). */
 int64_t melinoe_launch_count(void);
 

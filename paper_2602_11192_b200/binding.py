@@ -26,6 +26,7 @@ EXPORTED_SYMBOLS = [
     "melinoe_moe_last_call_used_gemm", "melinoe_moe_set_policy", "melinoe_moe_cache_counts", "melinoe_moe_expert_bytes_q4",
     "melinoe_moe_pack_expert_q4", "melinoe_moe_register_host_experts_q4", "melinoe_trace_miss_proxies", "melinoe_launch_count",
     "melinoe_last_cuda_error", "melinoe_strerror", "melinoe_moe_ffn_launch_times_ms", "melinoe_debug_fail_host_copy",
+    "melinoe_debug_gather_without_plan",
     "melinoe_moe_preload_pooled",
 ]
 
@@ -103,6 +104,7 @@ def lib():
     L.melinoe_moe_transfer_time_ms.argtypes = [vp, C.POINTER(C.c_double), C.POINTER(C.c_uint64)]
     L.melinoe_moe_ffn_launch_times_ms.argtypes = [vp, vp, i32, C.POINTER(i32)]
     L.melinoe_debug_fail_host_copy.argtypes = [i32]
+    L.melinoe_debug_gather_without_plan.argtypes = [vp, vp]
     L.melinoe_moe_set_trace.argtypes = [vp, vp, sz, i32]
     L.melinoe_moe_trace_count.argtypes = [vp]
     L.melinoe_moe_trace_count.restype = C.c_int64

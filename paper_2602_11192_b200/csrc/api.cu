@@ -965,6 +965,7 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         pr.lists = by_index ? 1 : 0;
         pr.row_gate = use_gemm ? h->row_gate : nullptr;
         pr.counters = use_gemm ? h->counters : nullptr;
+        pr.err = h->err_word;
         CU_TRY(launch_router(s, sh, static_cast<const uint16_t *>(hidden_dev), h->w_router, h->bias, h->token_seq, T, h->d,
                              h->E, h->k, sc.idx, sc.gate, sc.logits, sc.block_counts));
         CU_TRY(launch_plan(s, pp, pr));
@@ -1708,6 +1709,27 @@ int melinoe_moe_last_call_used_gemm(melinoe_moe_t *h) { return h && h->last_used
 int melinoe_debug_fail_host_copy(int nth)
 {
     g_fail_copy_in.store(nth > 0 ? nth : 0);
+    return MELINOE_OK;
+}
+
+int melinoe_debug_gather_without_plan(melinoe_moe_t *h, void *cuda_stream)
+{
+    if (!h)
+        return MELINOE_ERR_INVALID;
+    // (one token, no rows to copy: the kernel reads the plan's word and, as it never matches, nothing else)
+    PlanParams pp = {};
+    pp.T = 1;
+    pp.k = h->k;
+    pp.E = h->E;
+    pp.plan = h->plan;
+    pp.call_seq = h->call_seq + 0x80000000u;
+    pp.n_blocks = 1;
+    PromptParams pr = {};
+    pr.tokens_per_block = 1;
+    pr.err = h->err_word;
+    CU_TRY(launch_gather_rows(static_cast<cudaStream_t>(cuda_stream), h->n_sms, pp, pr, nullptr, nullptr, h->d, false));
+    CU_TRY(cudaEventRecord(h->ev_last, static_cast<cudaStream_t>(cuda_stream)));
+    h->has_last = true;
     return MELINOE_OK;
 }
 

@@ -554,14 +554,15 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
     if (warp == 0) {
         uint32_t hdr = 0;
         bool ok = true;
-        if (lane == 0)
+        if (lane == 0) {
             ok = wait_for_ready(plan, p.call_seq, &hdr);
+            if (!ok)
+                s_abort = 1;
+        }
         __syncwarp();
         hdr = __shfl_sync(0xffffffffu, hdr, 0);
         ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-        if (hdr == 0xffffffffu && lane == 0)
-            s_abort = 1;
-        const int n_req_total = ok ? (int)(hdr & 0xffu) : 0;
+        const int n_req_total = ok && plan_accepted(hdr) ? (int)(hdr & 0xffu) : 0;
         if (rank == 0 && n_req_total > 0)
             ahead = claim();
         int n = 0, sum = 0;

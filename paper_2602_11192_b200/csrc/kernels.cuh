@@ -67,6 +67,7 @@ struct PromptParams {
     int lists;                // the planning kernel makes the token lists, too (each of the router's blocks had one token)
     float *row_gate;          // null, or the gate of the pair at every sorted position, 1 for a shared expert's rows
     GemmCounters *counters;   // null, or the grouped GEMM's
+    int *err;                 // device error word (0 = ok)
 };
 // Layout of one request-trace record for a layer of n_experts experts and top_k, max_tokens tokens.
 struct TraceLayout {

@@ -109,23 +109,23 @@ struct GemmCounters {
     int32_t done[kMaxReq];
 };
 
-// Waits, by one thread and bounded (about 2 s), until the plan of call `seq` is announced; the word's high half says the
-// rest (ready_word), all ones if the wait ran out.  False: that, or the call was refused.
+// Whether the plan of call `seq` is announced; the word's high half says the rest (ready_word).
+__device__ inline bool plan_announced(const DevPlan *plan, uint32_t seq, uint32_t *hdr)
+{
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&plan->ready) : "memory");
+    *hdr = (uint32_t)(v >> 32);
+    return (uint32_t)v == seq;
+}
+__device__ inline bool plan_accepted(uint32_t hdr) { return ((hdr >> 8) & 0xffu) == 0; }
+// Waits, by one thread and bounded (about 2 s), until the plan of call `seq` is announced.  False: the wait ran out.
 __device__ inline bool wait_for_ready(const DevPlan *plan, uint32_t seq, uint32_t *hdr)
 {
     const long long t0 = clock64();
-    for (;;) {
-        unsigned long long v;
-        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&plan->ready) : "memory");
-        if ((uint32_t)v == seq) {
-            *hdr = (uint32_t)(v >> 32);
-            return ((v >> 40) & 0xffu) == 0;
-        }
-        if (clock64() - t0 > 4000000000ll) {
-            *hdr = 0xffffffffu;
+    while (!plan_announced(plan, seq, hdr))
+        if (clock64() - t0 > 4000000000ll)
             return false;
-        }
-    }
+    return true;
 }
 
 // The miss queue of a call: what the host needs in order to issue the transfers, written by

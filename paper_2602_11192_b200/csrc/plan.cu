@@ -498,7 +498,16 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(PlanParams p, PromptPa
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
         uint32_t hdr;
-        s_ok = wait_for_ready(p.plan, p.call_seq, &hdr);
+        bool known = wait_for_ready(p.plan, p.call_seq, &hdr);
+        if (!known) {
+            // The wait ran out: the planner may have been held up, but behind its end the word stands.  If it does not even
+            // then, the call has failed, and says so: the kernels behind must not pass for good what the last call's lists give.
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            known = plan_announced(p.plan, p.call_seq, &hdr);
+            if (!known)
+                atomicExch(q.err, MELINOE_ERR_TIMEOUT);
+        }
+        s_ok = known && plan_accepted(hdr);
     }
     __syncthreads();
     // (what comes behind this grid is behind the planning kernel's, too)

@@ -546,6 +546,25 @@ def test_a_failed_host_copy_leaves_the_handle_usable():
     P.close()
 
 
+def test_a_gather_whose_plan_never_comes_reports_it():
+    """The gather of a long call waits for the plan's word, bounded.  With a word that nobody sets the wait runs out, the
+    kernel ends and the handle says so, instead of leaving the lists and rows of the call before to be computed with."""
+    import torch
+    from paper_2602_11192_b200 import MelinoeError, lib
+    from paper_2602_11192_b200.runner import current_stream_ptr
+    P = _pair(512, 128, 8, 2, 8, seed=84)
+    x = gen.hidden_states(84, 0, "prefill", 0, 70, 512)
+    P.step(x, tokens=[0, 69])
+    assert lib().melinoe_debug_gather_without_plan(P.gpu.layer._h, current_stream_ptr()) == 0
+    torch.cuda.synchronize()
+    with pytest.raises(MelinoeError) as ei:
+        P.gpu.layer.cache_state()
+    assert ei.value.status == 5
+    P.reset()
+    P.step(x, tokens=[0, 69])
+    P.close()
+
+
 def test_request_trace_records_calls_without_synchronising():
     """The request trace: 24 calls (decode-sized ones through the fused planner, two larger ones through the
     general planner) are queued back to back with no synchronisation in between; afterwards the ring holds

@@ -482,11 +482,15 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanParams p, Prompt
 // Token lists and Xs[pos] = hidden[token of pos].  A block takes the tokens that one block of the router took: a pair's
 // position is its expert's offset, plus the pairs of that expert in the blocks before (both from the planning kernel),
 // plus those before it in this block.  A token's row is read once and written k times (and once per shared
-// expert).  PERMUTE: elements (0,4) (1,5) (2,6) (3,7) of every eight, the order in which 4-bit codes expand.
+// expert).  early: the GEMM may come while this one waits for the plan.  4-bit slots want that, as their codes are fetched and expanded
+// meanwhile (60 tokens, d 4096, d_ff 6400, 8 experts, 2 per token: 192 us a pass, 190 early), but not where its CTAs would take the SMs that a
+// block per token or more is still working on (d 2048, d_ff 1024, 64 experts, 8 per token, 400 tokens: 209 early, 206); bf16 slots
+// lose by it always (80 tokens 145.6 and 144.9, 800 tokens 183.9 and 183.2; d 512, d_ff 2048, 800 tokens 56.9 and 56.3).  PERMUTE: elements (0,4) (1,5) (2,6) (3,7) of every eight, the order in which 4-bit codes expand.
 constexpr int kGatherMaxPairs = 512;       // pairs of one router block at most (see router_shape)
 
 template <bool PERMUTE>
-__global__ void __launch_bounds__(256) gather_rows_kernel(PlanParams p, PromptParams q, const uint16_t *__restrict__ x, uint16_t *__restrict__ xs, int d)
+__global__ void __launch_bounds__(256) gather_rows_kernel(PlanParams p, PromptParams q, const uint16_t *__restrict__ x, uint16_t *__restrict__ xs, int d,
+                                                          int early)
 {
     __shared__ int32_t s_run[kMaxExperts];
     __shared__ int32_t s_pos[kGatherMaxPairs];
@@ -494,8 +498,9 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(PlanParams p, PromptPa
     const int tid = threadIdx.x, lane = tid & 31;
     const int t0 = blockIdx.x * q.tokens_per_block, n = min(q.tokens_per_block, p.T - t0);
     const int k = p.k, n_pairs = p.T * k;
+    if (early)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // The planning kernel, which may still be running, has waited for the router and all before it.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
         uint32_t hdr;
         bool known = wait_for_ready(p.plan, p.call_seq, &hdr);
@@ -510,6 +515,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(PlanParams p, PromptPa
         s_ok = known && plan_accepted(hdr);
     }
     __syncthreads();
+    if (!early)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // (what comes behind this grid is behind the planning kernel's, too)
     auto leave = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
     if (!s_ok)
@@ -581,6 +588,7 @@ cudaError_t launch_gather_rows(cudaStream_t stream, int n_sms, const PlanParams 
     // four blocks per SM, no more than one per 256 pieces to copy
     const int pieces = (q.tokens_per_block * (d / 8) + 255) / 256, want = (4 * n_sms + p.n_blocks - 1) / p.n_blocks;
     const int parts = xs == nullptr || want < 1 ? 1 : want < pieces ? want : pieces;
+    const int early = permute && p.n_blocks * parts <= n_sms ? 1 : 0;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(p.n_blocks, parts);
     lc.blockDim = dim3(256);
@@ -590,7 +598,7 @@ cudaError_t launch_gather_rows(cudaStream_t stream, int n_sms, const PlanParams 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = pdl_enabled() ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&lc, permute ? gather_rows_kernel<true> : gather_rows_kernel<false>, p, q, x, xs, d);
+    const cudaError_t e = cudaLaunchKernelEx(&lc, permute ? gather_rows_kernel<true> : gather_rows_kernel<false>, p, q, x, xs, d, early);
     count_launch();
     return e;
 }

@@ -1031,14 +1031,8 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
         }
         if (use_gemm) {
             gp.group = g;
-            // CTA pairs for bf16 slots (see ffn_gemm.cu; MELINOE_MOE_GEMM_SINGLE in the environment keeps them on single CTAs).
-            // 4-bit slots: single CTAs while an expert has few tokens.  They expand the codes without waiting for a peer's
-            // stores to be seen, but take chunks of 128 tokens instead of 256 and expand a tile again for each.  (d 2048, d_ff
-            // 1024, 64 experts, 8 per token, us a pass, pairs and single CTAs: 16 tokens 67 and 55, 64 tokens 78 and 67, 200 tokens
-            // 101 and 95, 512 tokens 129 and 132, 2048 tokens 327 and 383.)
             static const bool single_only = std::getenv("MELINOE_MOE_GEMM_SINGLE") != nullptr;
-            const bool pairs = h->fmt != 0 ? (long long)T * h->k > 32ll * h->E : !single_only;
-            CU_TRY(launch_ffn_gemm(s, h->n_sms, pairs, h->fmt, gp));
+            CU_TRY(launch_ffn_gemm(s, h->n_sms, h->fmt, single_only, gp, T, h->k));
         } else {
             for (int c = 0; c < n_chunks; ++c) {
                 int rc = launch_decode(h, s, sc, hidden_dev, out_dev, T, g, c, small && g == 0 && c == 0);

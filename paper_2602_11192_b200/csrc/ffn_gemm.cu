@@ -42,8 +42,9 @@
 // issues the MMAs (one elected thread) and commits them to mbarriers, warps 2..9 drain
 // the accumulator (tcgen05.ld, 32 rows per warp) and write the tile, warp 10 loads activations; with 4-bit slots warp 0 loads those,
 // warps 10..25 expand and warp 26 fetches codes.  Two accumulators alternate so the epilogue of a tile overlaps the MMAs of the next.
-// One launch does both GEMMs of a compute group; its work items are (GEMM, request, weight tile, token chunk), handed out
-// to the CTA pairs as they run out of work (GemmWalk, ffn_gemm_kernel).
+// Work items are (GEMM, request, weight tile, token chunk).  One launch does both GEMMs of a compute group and hands its items out to
+// the CTA pairs as they run out of work, or each GEMM has a launch of its own, whose items are dealt out beforehand (GemmWalk,
+// ffn_gemm_kernel; which: launch_ffn_gemm).
 //
 // Ragged N: a chunk's box may run past its expert's last row; those columns are computed on whatever
 // the next rows hold (or zeros past the end of the buffer) and never stored.
@@ -415,10 +416,10 @@ struct TokenBox {
     __device__ uint32_t bytes(bool indexed) const { return indexed ? (uint32_t)rows * kBK * 2 : (32u * kBK * 2) << cls; }
 };
 
-// The items of a launch in one order: all of GEMM 1, then all of GEMM 2, by request, weight tile, chunk of tokens (the chunks
-// of a tile side by side, so that pairs working at the same time share it in L2).  A CTA pair takes the next one whenever it
-// is about to run out of work, so a unit's items come in this order too.
-template <int CG, int NT>
+// The items of both GEMMs in one order: all of GEMM 1, then all of GEMM 2, by request, weight tile, chunk of tokens (the chunks
+// of a tile side by side, so that pairs working at the same time share it in L2).  A unit's items come in this order, too, whether a
+// CTA pair takes the next one whenever it is about to run out of work (PHASE 0) or has every n-th of one GEMM's.
+template <int CG, int PHASE>
 struct GemmWalk {
     const int4 *rec;         // first row, tokens, slot (shared expert s: -1 - s), tokens of a chunk
     const int *chunk0;       // chunks of the requests before each
@@ -429,27 +430,32 @@ struct GemmWalk {
           phase(1), rank(rank_)
     {
         total1 = chunk0_[n_reqs] * m1;
-        total = total1 + chunk0_[n_reqs] * m2;
+        total = PHASE == 1 ? total1 : total1 + chunk0_[n_reqs] * m2;
+    }
+    // PHASE 1, 2: item i of this unit
+    __device__ int dealt(uint32_t i) const
+    {
+        return (PHASE == 2 ? total1 : 0) + (int)blockIdx.x / CG + (int)i * ((int)gridDim.x / CG);
     }
     // item w, which is never before the one asked for last
     __device__ bool at(int w, GemmItem &it)
     {
         if (w >= total)
             return false;
-        if (w >= total1) {
+        if (PHASE != 1 && w >= total1) {
             if (phase == 1)
                 q = 0;
             phase = 2;
             w -= total1;
         }
-        const int m = phase == 1 ? m1 : m2;
+        const int ph = PHASE ? PHASE : phase, m = ph == 1 ? m1 : m2;
         while (chunk0[q + 1] * m <= w)
             ++q;
         const int4 r = rec[q];
         const int n = chunk0[q + 1] - chunk0[q], local = w - chunk0[q] * m, tile = local / n, c = local - tile * n;
-        it.phase = phase;
-        it.m0 = (tile * CG + rank) * (phase == 1 ? 64 : 128);
-        it.kblocks = phase == 1 ? k1 : k2;
+        it.phase = ph;
+        it.m0 = (tile * CG + rank) * (ph == 1 ? 64 : 128);
+        it.kblocks = ph == 1 ? k1 : k2;
         it.row0 = r.x + c * r.w;
         it.n_live = min(r.w, r.y - c * r.w);
         it.n = (it.n_live + 16 * CG - 1) / (16 * CG) * (16 * CG);
@@ -461,7 +467,7 @@ struct GemmWalk {
 
 // GEMM 1: h = SiLU(Xs W_g^T) * (Xs W_u^T) -> hs (bf16).  GEMM 2: z = hs W_d^T -> zs (fp32).
 //
-// One launch does both.  As two launches, each ended with a round of items that did not fill the GPU (a prompt of 128 tokens
+// PHASE 0: one launch does both.  As two launches, each ended with a round of items that did not fill the GPU (a prompt of 128 tokens
 // over some 20 experts has 160 items for 74 pairs in both: 3 rounds for 2.16) and the second began with an empty pipeline; and
 // items of unequal sizes were dealt out beforehand.  Now a pair fetches its next item's number from a counter
 // in global memory (the loading warp of the even CTA, a few stages before its loads run out; it hands the
@@ -469,7 +475,13 @@ struct GemmWalk {
 // items wait until as many epilogue warps as GEMM 1 has for it have counted themselves out.  That wait ends whatever else is on
 // the GPU: GEMM 2's items are handed out after all of GEMM 1's, so what it waits for is in the hands of CTAs
 // that are running, and GEMM 1 waits for nobody.
-template <int CG, int FMT>
+//
+// PHASE 1, 2: that GEMM alone, a unit's items known from the start; GEMM 2 loads weights ahead of the end of GEMM 1's grid.  PHASE 0
+// has a price: the round trip to the counter and the number's way to the odd CTA before the first load (2 us a launch), and a
+// release per item and epilogue warp, which waits for the stores of h, before the next tile is drained.  Reductions of 4 to 12
+// k-blocks (d up to 768) do not cover it (4000 tokens, d 512, d_ff 8192, 8 experts, 2 per token, 4-bit slots: 297 us a pass, 262 in two
+// launches; of the difference 16 us are the releases, 7 the numbers, the rest loops over a phase that the compiler knows).
+template <int CG, int FMT, int PHASE>
 __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __grid_constant__ GemmParams p)
 {
     constexpr int kStages = gemm_stages(FMT), NT = gemm_tokens(CG);
@@ -563,7 +575,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
         hdr = __shfl_sync(0xffffffffu, hdr, 0);
         ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
         const int n_req_total = ok && plan_accepted(hdr) ? (int)(hdr & 0xffu) : 0;
-        if (rank == 0 && n_req_total > 0)
+        if (PHASE == 0 && rank == 0 && n_req_total > 0)
             ahead = claim();
         int n = 0, sum = 0;
         constexpr int kRounds = (kMaxReq + 31) / 32;
@@ -609,12 +621,14 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
     __syncthreads();
     const int n_reqs = s_nreq;
 
-    GemmWalk<CG, NT> walk(s_rec, s_chunk0, n_reqs, p.d, p.F, (int)rank);
+    GemmWalk<CG, PHASE> walk(s_rec, s_chunk0, n_reqs, p.d, p.F, (int)rank);
     GemmItem it;
     // of a pair, the bytes of both CTAs are expected and counted on the even CTA's barriers
     const uint32_t full_b = CG == 1 ? full0 : cluster_addr(full0, 0);
-    // Item number i of this unit, for the whole warp; false behind the last one.
+    // Item i of this unit, for the whole warp; false behind the last one.
     auto next = [&](uint32_t i) -> bool {
+        if (PHASE)
+            return __all_sync(0xffffffffu, !*abort_flag) && walk.at(walk.dealt(i), it);
         const uint32_t slot = i % kItemRing;
         const bool ok = !*abort_flag && mbar_wait<CG == 2>(ifull0 + 8 * slot, (i / kItemRing) & 1u, abort_flag);
         if (!__all_sync(0xffffffffu, ok))
@@ -631,10 +645,11 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
         return more;
     };
 
-    // The warps that load activations: those of GEMM 2 are complete once GEMM 1's epilogue warps of the request have counted themselves out.
+    // The warps that load activations: those of GEMM 2 are complete once GEMM 1's epilogue warps of the request have counted themselves
+    // out, or, if it had a launch of its own, once that has ended.
     int h_of = -1;                                           // the request that was waited for last
     auto wait_for_h = [&]() -> bool {
-        if (it.phase == 1 || it.q == h_of)
+        if (PHASE || it.phase == 1 || it.q == h_of)
             return true;
         h_of = it.q;
         const int *done = &p.counters->done[s_req[it.q]];
@@ -693,11 +708,11 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
             }
             __syncwarp();
         };
-        if (rank == 0)
+        if (PHASE == 0 && rank == 0)
             publish(0, ahead);
         // (the odd CTA: the number of an item, which arrives by st.async, is expected two items ahead)
         auto expect_number = [&](uint32_t i) {
-            if (CG == 2 && rank == 1 && lane == 0)
+            if (PHASE == 0 && CG == 2 && rank == 1 && lane == 0)
                 mbar_expect(ifull0 + 8 * (i % kItemRing), 4);
         };
         expect_number(0);
@@ -706,13 +721,13 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
             asm volatile("griddepcontrol.wait;" ::: "memory");
         uint32_t s = 0, parity = 1, n = 0;                   // stage of the next k-block, parity of its being free; k-blocks so far
         for (uint32_t i = 0;; ++i) {
-            const bool more = rank == 0 ? !*abort_flag && walk.at(__shfl_sync(0xffffffffu, ahead, 0), it) : next(i);
+            const bool more = PHASE == 0 && rank == 0 ? !*abort_flag && walk.at(__shfl_sync(0xffffffffu, ahead, 0), it) : next(i);
             if (!__all_sync(0xffffffffu, more))
                 break;
             expect_number(i + 2);
             const int kblocks = __shfl_sync(0xffffffffu, it.kblocks, 0), m0 = __shfl_sync(0xffffffffu, it.m0, 0);
             const int slot_ = __shfl_sync(0xffffffffu, it.slot, 0), slot = slot_ >= 0 ? slot_ : 0;
-            const int phase = __shfl_sync(0xffffffffu, it.phase, 0);
+            const int phase = PHASE ? PHASE : __shfl_sync(0xffffffffu, it.phase, 0);
             // the weights of the slots, or of the shared expert
             const CUtensorMap *map_w = p.maps + (slot_ >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - slot_)) + (phase - 1);
             const TokenBox box(it, CG, (int)rank);
@@ -722,7 +737,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
             if (FMT == 1 && !wait_for_h())
                 break;
             auto run = [&](auto phase_, int kb, int kb_end) -> bool {
-                constexpr int PHASE = decltype(phase_)::value;
+                constexpr int kPhase = decltype(phase_)::value;
                 const int row = (slot * p.F + m0) / 8, col = m0 / 64;
                 n += (uint32_t)(kb_end - kb);
                 for (; kb < kb_end; ++kb) {
@@ -735,7 +750,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
                         const uint32_t dst = ring_s + s * kStageBytes;
                         if (FMT == 1)
                             tma_load_2d<CG>(dst + kABytes, map_b, kb * kBK, box.row, full_b + 8 * s);
-                        else if (PHASE == 1)
+                        else if (kPhase == 1)
                             tma_load_4d<CG>(dst, map_w, kb * kBK, 0, 0, row, full_b + 8 * s);
                         else
                             tma_load_4d<CG>(dst, map_w, 0, kb * kBK, col, slot, full_b + 8 * s);
@@ -750,7 +765,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
             };
             auto part = [&](int kb, int kb_end) { return phase == 1 ? run(Const<1>(), kb, kb_end) : run(Const<2>(), kb, kb_end); };
             const int ask = max(kblocks - (FMT ? kAskAhead4 : kAskAhead), 0), tell = min(ask + 2, kblocks);
-            if (rank == 0) {
+            if (PHASE == 0 && rank == 0) {
                 if (!part(0, ask))
                     break;
                 ahead = claim();
@@ -771,7 +786,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
         }
     } else if (FMT == 0 && warp == 2 + kEpilogueWarps) {
         // ============================================================ loads of the activations
-        if (!p.by_index)
+        if (PHASE == 2 || !p.by_index)
             asm volatile("griddepcontrol.wait;" ::: "memory");
         uint32_t s = 0, parity = 1;
         for (uint32_t i = 0; next(i); ++i) {
@@ -779,7 +794,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
                 break;
             const int kblocks = __shfl_sync(0xffffffffu, it.kblocks, 0);
             const TokenBox box(it, CG, (int)rank);
-            const bool first = __shfl_sync(0xffffffffu, it.phase, 0) == 1;
+            const bool first = PHASE ? PHASE == 1 : __shfl_sync(0xffffffffu, it.phase, 0) == 1;
             const CUtensorMap *map_b = p.maps + (first ? kMapXs0 : kMapHs0) + box.cls;
             auto run = [&](auto indexed) -> bool {
                 for (int kb = 0; kb < kblocks; ++kb) {
@@ -814,7 +829,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
             for (uint32_t item = 0;; ++item) {
                 if (!next(item))
                     break;
-                const int phase = __shfl_sync(0xffffffffu, it.phase, 0), kblocks = __shfl_sync(0xffffffffu, it.kblocks, 0);
+                const int phase = PHASE ? PHASE : __shfl_sync(0xffffffffu, it.phase, 0), kblocks = __shfl_sync(0xffffffffu, it.kblocks, 0);
                 const uint32_t idesc = instr_desc_bf16(CG * 128, __shfl_sync(0xffffffffu, it.n, 0), phase == 2);
                 const uint32_t acc = item & 1u;
                 bool ok = item < 2 || mbar_wait<CG == 2>(tempty0 + 8 * acc, ((item >> 1) - 1u) & 1u, abort_flag);
@@ -880,7 +895,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
             asm volatile("griddepcontrol.wait;" ::: "memory");
         for (uint32_t item = 0; next(item); ++item) {
             const uint32_t acc = item & 1u;
-            const bool first = it.phase == 1;
+            const bool first = PHASE ? PHASE == 1 : it.phase == 1;
             // 4-bit slots: lanes l and l + 16 hold the gate of the chunk's token l, the next chunk's is on its way
             auto gate_of = [&](int c) {
                 return first && c + (lane & 15) < it.n_live ? __ldcg(p.row_gate + it.row0 + c + (lane & 15)) : 0.0f;
@@ -941,7 +956,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
                 drained();
                 // this warp's part of h is written: GEMM 2 of the request, in whichever CTA, counts these
                 __syncwarp();
-                if (lane == 0)
+                if (PHASE == 0 && lane == 0)
                     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(&p.counters->done[s_req[it.q]]) : "memory");
             } else {
                 float *dst = p.zs + (size_t)(it.row0 + c_first) * p.d + it.m0 + quarter * 32 + lane;
@@ -979,16 +994,16 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
             const char *blob = it.slot >= 0 ? p.slots + (size_t)it.slot * p.slot_stride : p.shared_blobs[-1 - it.slot];
             const int kblocks = it.kblocks;
             auto expand = [&](auto phase_) {
-            constexpr int PHASE = decltype(phase_)::value;
-            constexpr int kRawBlocks = PHASE == 1 ? 4 : 2;           // k-blocks of one fetch of codes
+            constexpr int kPhase = decltype(phase_)::value;
+            constexpr int kRawBlocks = kPhase == 1 ? 4 : 2;           // k-blocks of one fetch of codes
             // GEMM 1: rows of eight g, eight u, ..; GEMM 2: rows f, 64 of the first column group, 64 of the second
-            const int f_row = PHASE == 1 ? it.m0 + (row >> 4) * 8 + (row & 7) : (row & 63);
+            const int f_row = kPhase == 1 ? it.m0 + (row >> 4) * 8 + (row & 7) : (row & 63);
             const int part = (row >> 3) & 1, cg = row >> 6;
-            const char *sc_base = PHASE == 1 ? blob + (size_t)f_row * ub + scales + (size_t)part * (p.d / 32)
+            const char *sc_base = kPhase == 1 ? blob + (size_t)f_row * ub + scales + (size_t)part * (p.d / 32)
                                              : blob + (size_t)f_row * ub + scales + 2 * (size_t)(p.d / 32) + (size_t)(it.m0 / 64 + cg) * 2;
             // the scale of the next k-block is in flight while this one is expanded
             auto scale_of = [&](int kb) -> uint32_t {
-                if (PHASE == 1)
+                if (kPhase == 1)
                     return f_row < p.F && kb < kblocks ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base) + kb) : 0u;
                 return kb * kBK + f_row < p.F ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base + (size_t)kb * kBK * ub)) : 0u;
             };
@@ -1007,7 +1022,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
                 const uint32_t ss = sc * 0x10001u;
                 const uint32_t raw = raw_s + rs * kRawBytes, a_dst = ring_s + s * kStageBytes + row * 128;
                 const uint32_t x = (uint32_t)(row & 7);      // = f mod 8 in both phases
-                if (PHASE == 1) {
+                if (kPhase == 1) {
                     // 64 columns = pieces 2 sub, 2 sub + 1 of this row's 128 bytes of codes -> eight pieces of bf16
                     const uint32_t src = raw + row * 128;
 #pragma unroll
@@ -1062,7 +1077,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
                     mbar_arrive(rempty0 + 8 * rs);
             }
             };
-            if (it.phase == 1)
+            if (PHASE ? PHASE == 1 : it.phase == 1)
                 expand(Const<1>());
             else
                 expand(Const<2>());
@@ -1072,9 +1087,10 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
         // ============================================================ fetch of 4-bit codes
         uint32_t rn = 0;
         for (uint32_t item = 0; next(item); ++item) {
-            const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (it.phase - 1);
+            const int phase = PHASE ? PHASE : it.phase;
+            const CUtensorMap *map_w = p.maps + (it.slot >= 0 ? kMapSlots0 : kMapShared0 + 2 * (-1 - it.slot)) + (phase - 1);
             const int slot = it.slot >= 0 ? it.slot : 0;
-            for (int kb = 0; kb < it.kblocks; kb += it.phase == 1 ? 4 : 2, ++rn) {
+            for (int kb = 0; kb < it.kblocks; kb += phase == 1 ? 4 : 2, ++rn) {
                 const uint32_t rs = rn % kRawStages;
                 const bool ok = rn < (uint32_t)kRawStages || mbar_wait(rempty0 + 8 * rs, ((rn / kRawStages) - 1u) & 1u, abort_flag);
                 if (!__all_sync(0xffffffffu, ok))
@@ -1082,7 +1098,7 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
                 if (lane == 0) {
                     const uint32_t dst = raw_s + rs * kRawBytes, bar = rfull0 + 8 * rs;
                     mbar_expect(bar, kRawBytes);
-                    if (it.phase == 2)
+                    if (phase == 2)
                         tma_load_3d(dst, map_w, it.m0 / 256 * 128, kb * kBK, slot, bar);
                     else
                         tma_load_5d(dst, map_w, kb * 32, 0, 0, it.m0 / 8, slot, bar);
@@ -1211,16 +1227,27 @@ constexpr size_t gemm_smem(int fmt)
     return (size_t)gemm_stages(fmt) * kStageBytes + (fmt ? kRawStages * kRawBytes : 0) + 1024;
 }
 
-template <int CG, int FMT>
+template <int CG, int FMT, int PHASE>
 cudaError_t gemm_launch(cudaStream_t stream, int n_sms, const GemmParams &p)
 {
-    return launch_after(stream, ffn_gemm_kernel<CG, FMT>, dim3(n_sms / CG * CG), gemm_threads(FMT), gemm_smem(FMT), CG, p);
+    return launch_after(stream, ffn_gemm_kernel<CG, FMT, PHASE>, dim3(n_sms / CG * CG), gemm_threads(FMT), gemm_smem(FMT), CG, p);
 }
 
-template <int CG, int FMT>
+template <int FMT>
+cudaError_t gemm_launch(cudaStream_t stream, int n_sms, int ctas, bool apart, const GemmParams &p)
+{
+    if (ctas == 1)
+        return gemm_launch<1, FMT, 0>(stream, n_sms, p);
+    if (!apart)
+        return gemm_launch<2, FMT, 0>(stream, n_sms, p);
+    const cudaError_t e = gemm_launch<2, FMT, 1>(stream, n_sms, p);
+    return e != cudaSuccess ? e : gemm_launch<2, FMT, 2>(stream, n_sms, p);
+}
+
+template <int CG, int FMT, int PHASE>
 cudaError_t gemm_configure()
 {
-    return cudaFuncSetAttribute(ffn_gemm_kernel<CG, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(FMT));
+    return cudaFuncSetAttribute(ffn_gemm_kernel<CG, FMT, PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(FMT));
 }
 
 }  // namespace
@@ -1229,18 +1256,30 @@ bool ffn_gemm_supported(int d, int F) { return d % 256 == 0 && F % kUnitRows == 
 
 cudaError_t ffn_gemm_configure()
 {
-    const cudaError_t e[4] = {gemm_configure<1, 0>(), gemm_configure<1, 1>(), gemm_configure<2, 0>(), gemm_configure<2, 1>()};
+    const cudaError_t e[] = {gemm_configure<1, 0, 0>(), gemm_configure<1, 1, 0>(), gemm_configure<2, 0, 0>(), gemm_configure<2, 1, 0>(),
+                             gemm_configure<2, 0, 1>(), gemm_configure<2, 0, 2>(), gemm_configure<2, 1, 1>(), gemm_configure<2, 1, 2>()};
     for (cudaError_t r : e)
         if (r != cudaSuccess)
             return r;
     return cudaSuccess;
 }
 
-cudaError_t launch_ffn_gemm(cudaStream_t stream, int n_sms, bool pairs, int fmt, const GemmParams &p)
+cudaError_t launch_ffn_gemm(cudaStream_t stream, int n_sms, int fmt, bool single_only, const GemmParams &p, int T, int k)
 {
-    if (fmt == 1)
-        return pairs ? gemm_launch<2, 1>(stream, n_sms, p) : gemm_launch<1, 1>(stream, n_sms, p);
-    return pairs ? gemm_launch<2, 0>(stream, n_sms, p) : gemm_launch<1, 0>(stream, n_sms, p);
+    const long long pairs_of_all = (long long)T * k;     // (token, expert) pairs
+    // CTA pairs for bf16 slots (MELINOE_MOE_GEMM_SINGLE in the environment keeps them on single CTAs).  4-bit slots: single CTAs while
+    // an expert has few tokens.  They expand the codes without waiting for a peer's stores to be seen, but take chunks of 128
+    // tokens instead of 256 and expand a tile again for each.  (d 2048, d_ff 1024, 64 experts, 8 per token, us a pass, pairs and single
+    // CTAs: 16 tokens 67 and 55, 64 tokens 78 and 67, 200 tokens 101 and 95, 512 tokens 129 and 132, 2048 tokens 327 and 383.)
+    const int ctas = fmt != 0 ? (pairs_of_all > 32ll * p.E ? 2 : 1) : single_only ? 1 : 2;
+    // A launch for each GEMM where GEMM 1's reductions are short and its tiles many: there the way from one item to the next counts
+    // (see ffn_gemm_kernel) and a last round that is not full does not.  us a pass, one launch and two (experts, per token, tokens):
+    // bf16, d 512, d_ff 512 (32, 4, 400) 35.2 and 35.9, d_ff 1024 51.7 and 46.4; d 256, d_ff 4096 (8, 2, 800) 61.6 and 58.0; d 768,
+    // d_ff 768 (32, 4, 400) 52.8 and 50.4; d 1024 (8, 2, 400), d_ff 4096 71.3 and 69.8, d_ff 8192 109.8 and 106.5, d_ff 1024 (32, 4, 400)
+    // 65.1 and 66.7; d 4096, d_ff 1024 (16, 2, 400) 103 and 109.  4-bit, d 512, d_ff 8192 (8, 2, 2000) 201 and 183; d 1024, d_ff 6144
+    // (8, 2), 400 tokens 119.0 and 113.8, 2000 tokens, two chunks for an expert, 225.8 and 234.2; d 2048, d_ff 8384 (8, 2, 160) 190.8 and 187.9.
+    const bool apart = p.F > 512 && (p.d < 1024 || (pairs_of_all <= 256ll * p.E && (fmt != 0 ? 2 * p.F >= 5 * p.d : p.d == 1024 && p.F >= 6 * p.d)));
+    return fmt != 0 ? gemm_launch<1>(stream, n_sms, ctas, apart, p) : gemm_launch<0>(stream, n_sms, ctas, apart, p);
 }
 
 cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const float *gate, const int32_t *inv_pos,

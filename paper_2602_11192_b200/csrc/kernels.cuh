@@ -181,8 +181,9 @@ cudaError_t ffn_gemm_configure();
 // and j + 4 of every eight side by side (the order in which 4-bit codes expand).
 cudaError_t launch_gather_rows(cudaStream_t stream, int n_sms, const PlanParams &p, const PromptParams &q, const uint16_t *x, uint16_t *xs, int d,
                                bool permute);
-// Both GEMMs of a compute group.  pairs: CTA pairs; fmt: what the slots hold, 0 = bf16 blobs, 1 = 4-bit blobs
-cudaError_t launch_ffn_gemm(cudaStream_t stream, int n_sms, bool pairs, int fmt, const GemmParams &p);
+// Both GEMMs of a compute group, in one launch or two, by CTA pairs or single CTAs (single_only: bf16 slots, too).  fmt: what the slots
+// hold, 0 = bf16 blobs, 1 = 4-bit blobs; T, k: of the call
+cudaError_t launch_ffn_gemm(cudaStream_t stream, int n_sms, int fmt, bool single_only, const GemmParams &p, int T, int k);
 // gate null: the rows are weighted already
 cudaError_t launch_combine_rows(cudaStream_t stream, const DevPlan *plan, const float *gate, const int32_t *inv_pos,
                                 const float *zs, uint16_t *out, int T, int d, int k, int n_shared, int n_sms);

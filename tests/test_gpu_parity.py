@@ -374,6 +374,7 @@ def test_prefill_then_decode_with_waves():
     (512, 256, 4, 2, 4, 0, (600, 385, 40)),      # many tokens per expert, ragged
     (1024, 384, 4, 2, 2, 1, (700,)),             # many tokens per expert with a shared expert and miss waves
     (256, 256, 2, 2, 2, 0, (1100, 520)),         # every token to both experts: nine m-tiles (CTA pairs, the last one half empty)
+    (512, 1032, 6, 3, 3, 1, (130, 64)),          # a launch for each GEMM of a wave
 ])
 def test_prefill_grouped_gemm(d, F, E, k, C, n_shared, Ts):
     """Calls of more than 8 tokens run the tensor-core grouped GEMM (d_ff a multiple of 128)."""
@@ -408,6 +409,11 @@ def test_prefill_grouped_gemm(d, F, E, k, C, n_shared, Ts):
     ("q4slots", 512, 64, 2, 2, 0, (256, 257)),         # one and two chunks; GEMM 2 of a single k-block
     ("bf16", 512, 200, 3, 3, 1, (32, 64, 65)),         # rows fetched by index up to 64 tokens, copied from 65 on
     ("q4slots", 512, 72, 6, 2, 0, (96, 97)),           # single CTAs up to 32 pairs per expert, pairs of CTAs beyond
+    ("bf16", 256, 520, 5, 2, 1, (9, 64, 65, 700)),     # a launch for each GEMM; rows by index and copied
+    ("bf16", 768, 1160, 3, 2, 0, (70, 300)),
+    ("q4slots", 512, 1416, 4, 2, 1, (64, 65, 513)),    # one launch of single CTAs, then two of pairs
+    ("bf16", 1024, 6144, 2, 1, 0, (512, 513)),         # two launches up to 256 pairs per expert, one beyond
+    ("q4slots", 1024, 2560, 2, 1, 0, (512, 513)),
 ])
 def test_grouped_gemm_at_the_edges_of_its_tiles(store, d, F, E, k, n_shared, Ts):
     """Token counts around the steps of the tensor-core operation's N and d_ff that ends inside weight tiles and
@@ -419,13 +425,13 @@ def test_grouped_gemm_at_the_edges_of_its_tiles(store, d, F, E, k, n_shared, Ts)
     P.close()
 
 
-@pytest.mark.parametrize("T", [20, 200])
-def test_prompts_of_two_layers_on_two_streams(T):
-    """GEMM 2's items wait for GEMM 1's of whichever CTA has them: with two layers' launches competing for the SMs, queued
-    back to back on a stream each, both give the bits that they give alone."""
+@pytest.mark.parametrize("T,d", [(20, 1024), (200, 1024), (200, 512)])
+def test_prompts_of_two_layers_on_two_streams(T, d):
+    """GEMM 2's items wait for GEMM 1's of whichever CTA has them, or its launch for GEMM 1's: with two layers' launches competing
+    for the SMs, queued back to back on a stream each, both give the bits that they give alone."""
     import torch
     from paper_2602_11192_b200.runner import to_dev_bf16
-    d, F, E, k = 1024, 1024, 16, 4
+    F, E, k = 1024, 16, 4
     Ps = [_pair(d, F, E, k, E, seed=520 + l) for l in range(2)]
     streams = [torch.cuda.Stream() for _ in Ps]
     xs = [to_dev_bf16(gen.hidden_states(520 + l, 0, "prefill", 0, T, d)) for l in range(2)]

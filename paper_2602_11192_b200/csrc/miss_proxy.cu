@@ -191,12 +191,14 @@ __global__ void __launch_bounds__(kProxyThreads, 7) miss_proxy_kernel(const int3
         }
         __syncthreads();
         if (t0 == 0) {
-            // the tokens this block ranks, and the warps that do it: one where many configurations share the work
+            // The tokens this block ranks, and the warps that do it: one where many configurations share the work.  Every n-th
+            // block ranks only where that leaves 16 or more of the group (512 tokens, us, every third or fourth block of any group
+            // and this: 400 groups of 3 sizes 174 and 154, 160 of 4 105 and 72, 64 of 14 53.3 and 50.4).
             const int G = s_group[0][1] + s_group[1][1] + s_group[2][1] + s_group[3][1];
             const int o = s_group[0][0] + s_group[1][0] + s_group[2][0] + s_group[3][0];
-            const int n_rank_warps = G >= 16 * share ? 1 : 2;
-            if (role - 2 < n_rank_warps && o % share == 0) {
-                const long long parts = (long long)((G + share - 1) / share) * n_rank_warps, part = (long long)(o / share) * n_rank_warps + (role - 2);
+            const int n_rank_warps = G >= 16 ? 1 : 2, every = max(1, min(share, G / 16));
+            if (role - 2 < n_rank_warps && o % every == 0) {
+                const long long parts = (long long)((G + every - 1) / every) * n_rank_warps, part = (long long)(o / every) * n_rank_warps + (role - 2);
                 rank_lo = (int)(part * T / parts);
                 rank_hi = (int)((part + 1) * T / parts);
             }
@@ -386,7 +388,8 @@ cudaError_t launch_miss_proxies(cudaStream_t stream, const int32_t *idx, int n_l
     clear_totals_kernel<<<n_clear < 64 ? n_clear : 64, 256, 0, stream>>>(reinterpret_cast<unsigned long long *>(hard_total), n_cfg);
     count_launch();
     // Every block ranks while the GPU is not full; beyond two blocks per SM the replays that this takes cost more than the ranking
-    // of more tokens by fewer blocks (912 configurations: 47.7 us with every block, 43.3 with every third, 43.3 with every sixth).
+    // of more tokens by fewer blocks (912 configurations in groups of 57: 46.2 us with every block, 43.4 with every third), as long as
+    // enough blocks of a group are left to rank (see the kernel).
     const int want = n_cfg / (2 * n_sms), share = want < 1 ? 1 : want < 4 ? want : 4;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(n_cfg);

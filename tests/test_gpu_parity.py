@@ -970,6 +970,34 @@ def test_trace_miss_proxies_at_the_edges_of_their_batches(T, K, E, gamma, sizes)
         assert abs(soft[j] - so.mean()) <= 1e-10 * max(1.0, abs(so.mean())), (c, soft[j], so.mean())
 
 
+@pytest.mark.parametrize("total", [600, 1200])
+def test_trace_miss_proxies_of_groups_of_all_sizes(total):
+    """Many configurations, so that not every block ranks, in groups (of a layer and gamma) of 15, 16, 31, 32, 48 and 57 sizes and
+    of one to three, in an order that mixes them: hard misses exact, soft proxy to fp64 rounding."""
+    from paper_2602_11192_b200 import binding as B
+    from paper_2602_11192_b200.runner import current_stream_ptr
+    import torch
+    rs = np.random.default_rng(total)
+    T, K, E, L = 90, 2, 64, 12
+    trace = np.stack([np.stack([rs.choice(E, size=K, replace=False) for _ in range(T)]) for _ in range(L)]).astype(np.int32)
+    cfgs = [(l, c, 0.9) for l, n in enumerate((15, 16, 31, 32, 48, 57)) for c in range(K, K + n)]
+    for i in range(total):
+        if len(cfgs) >= total:
+            break
+        cfgs += [(i % L, c, 0.5 + i / (4.0 * total)) for c in (3, 16, 40)[:1 + i % 3]]
+    cfgs = [cfgs[i] for i in rs.permutation(len(cfgs))]
+    n = len(cfgs)
+    cfg_dev = torch.frombuffer(bytearray(bytes((B.ProxyConfig * n)(*[B.ProxyConfig(*c) for c in cfgs]))), dtype=torch.uint8).cuda()
+    soft = torch.zeros(n, dtype=torch.float64, device="cuda")
+    hard = torch.full((n,), 7, dtype=torch.int64, device="cuda")
+    B.melinoe_trace_miss_proxies(current_stream_ptr(), torch.from_numpy(trace).cuda(), L, T, K, E, cfg_dev, n, soft, hard)
+    soft, hard = soft.cpu().numpy(), hard.cpu().numpy()
+    for j, (l, c, gamma) in enumerate(cfgs):
+        so, ho = oracle.miss_proxies(trace[l], E, c, gamma)
+        assert hard[j] == int(ho.sum()), (l, c, gamma, hard[j], int(ho.sum()))
+        assert abs(soft[j] - so.mean()) <= 1e-10 * max(1.0, abs(so.mean())), (l, c, gamma, soft[j], so.mean())
+
+
 @pytest.mark.parametrize("n_layers,E,n", [(1, 64, 57), (3, 5, 700)])
 def test_trace_miss_proxies_of_no_tokens_are_zero(n_layers, E, n):
     """A trace without tokens: no misses and a mean of 0 for every configuration, whatever an earlier kernel left in

@@ -1390,7 +1390,8 @@ cudaError_t ffn_decode_geometry(const DecLaunchCfg &cfg, int d, int F, int token
     size_t n = avail / geo->stage_bytes;
     if (n > (size_t)kMaxStages)
         n = kMaxStages;
-    n -= n % decode_groups(d, tokens, fmt, min_req * F / cfg.grid);      // a stage belongs to one group
+    geo->groups = decode_groups(d, tokens, fmt, min_req * F / cfg.grid);
+    n -= n % geo->groups;            // a stage belongs to one group
     geo->n_stages = (int)n;
     geo->smem_bytes = n * geo->stage_bytes + fixed;
     return cudaSuccess;
@@ -1415,7 +1416,7 @@ cudaError_t launch_ffn_decode(cudaStream_t stream, const DecLaunchCfg &cfg, cons
     }
     lc.attrs = attr;
     lc.numAttrs = na;
-    const int mt = p.d / (16 * NW), ng = decode_groups(p.d, geo.tokens, p.fmt, (p.k + p.n_shared) * p.F / cfg.grid);
+    const int mt = p.d / (16 * NW), ng = geo.groups;
     auto launch = [&](auto kernel) { return cudaLaunchKernelEx(&lc, kernel, p, geo); };
     cudaError_t e;
     if (p.fmt == 0) {

@@ -1382,9 +1382,10 @@ cudaError_t ffn_decode_geometry(const DecLaunchCfg &cfg, int d, int F, int token
     // four rows or less, at which the per-tile work of the warps, not HBM, sets the pace.  Where that makes tiles higher, their operand
     // fragments go to tensor memory instead (d_ff 4096, 2 experts out of 16 per token, 4 layers, us: d 3584, 8 tokens, 3 -> 5 rows 811 -> 675; d 3072,
     // 8 tokens, 4 -> 5 rows 596 -> 563; d 4096, 3 tokens, 3 -> 4 rows 355 -> 293 (2 layers of d_ff 6400); from 5 rows on it loses: d 2560, 8 tokens,
-    // 5 -> 7 rows 491 -> 506).
-    const int with_rows = tile(bufs + rows);
-    geo->x_tmem = fmt == 0 && d >= 3072 && tokens > 1 && with_rows <= 4 && tile(bufs) > with_rows ? 1 : 0;
+    // 5 -> 7 rows 491 -> 506), as far as that makes a CTA's share a tile less: the set-up takes about a microsecond (d 4096, 2 experts out of 8, 4 layers,
+    // without and with: 4 tokens, d_ff 256, 3 rows of a CTA, 128 and 134, d_ff 1024, 14 rows, 202 and 195; 8 tokens 179 and 183, 272 and 259).
+    const int with_rows = tile(bufs + rows), more_rows = tile(bufs), share = min_req * F / cfg.grid;
+    geo->x_tmem = fmt == 0 && d >= 3072 && tokens > 1 && with_rows <= 4 && share * (more_rows - with_rows) >= with_rows * more_rows ? 1 : 0;
     const size_t fixed = bufs + (geo->x_tmem ? 0 : rows);
     const int tr = tile(fixed);
     if (tr == 0)

@@ -235,13 +235,14 @@ def test_one_token_calls_in_a_chain_read_what_the_call_ahead_wrote(d, F):
         P.close()
 
 
-def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory():
-    """d_model 4096 with 5 to 8 tokens per call: the decode kernel writes the hidden states' tensor-core
-    operands into tensor memory once and reads them from there (the shared memory goes to taller weight
-    tiles).  Calls whose missed experts the kernel fetches itself (token-expert pairs <= slots), with a
+@pytest.mark.parametrize("F", [48, 600])
+def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory(F):
+    """d_model 4096 with 5 to 8 tokens per call: where that saves an SM a tile (d_ff 600: twelve rows of three experts), the decode
+    kernel writes the hidden states' tensor-core operands into tensor memory once and reads them from there (the shared memory goes
+    to taller weight tiles).  Calls whose missed experts the kernel fetches itself (token-expert pairs <= slots), with a
     shared expert, between calls of fewer tokens that take the shared-memory form; then the same bits
     again from a warm cache (the sum over the SMs is exact, so residency must not change the output)."""
-    d, F, E, k, C = 4096, 48, 20, 2, 16
+    d, E, k, C = 4096, 20, 2, 16
     P = _pair(d, F, E, k, C, seed=77, n_shared=1)
     P.set_bias(_bias(9, E, 0.5, 4), None)
     outs = {}
@@ -263,7 +264,9 @@ def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory()
     ("bf16", 512, 3608, 1, 0, 4), ("bf16", 768, 1200, 2, 1, 2),      # d_ff that ends inside a tile; missed experts stored by either group
     ("bf16", 1024, 1768, 2, 0, 2),
     ("bf16", 1280, 72, 2, 0, 3), ("bf16", 1792, 1768, 1, 1, 4),      # one group, widths of their own
-    ("bf16", 2304, 72, 2, 0, 2), ("bf16", 3840, 48, 2, 1, 4),        # token operands in tensor memory from some number of tokens on
+    ("bf16", 2304, 72, 2, 0, 2), ("bf16", 3840, 48, 2, 1, 4),
+    ("bf16", 3072, 1480, 2, 0, 4), ("bf16", 3328, 1480, 2, 0, 3),    # token operands in tensor memory from some number of tokens on
+    ("bf16", 3584, 1480, 2, 0, 4), ("bf16", 3840, 888, 1, 1, 2), ("bf16", 4096, 888, 1, 1, 4),
     ("q4slots", 512, 1768, 2, 0, 3), ("q4slots", 512, 64, 2, 0, 3),  # 4-bit slots: two groups and one
     ("q4slots", 1024, 1768, 2, 0, 2), ("q4slots", 1024, 72, 2, 1, 3),
     ("q4slots", 2048, 1768, 2, 0, 4), ("q4slots", 4096, 72, 2, 0, 3),

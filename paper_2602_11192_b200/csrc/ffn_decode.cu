@@ -237,6 +237,8 @@ constexpr int NW = 16;                           // consumer warps
 //     108.8 and 108.3; d 256, d_ff 512, 8 tokens 173 and 152); four from twice as many on (d 256, 14 rows 80.9 with two, 82.6 with four);
 //   - where a warp's output columns of two would not fit its 96 registers: 4-bit slots of d_model 4096, and of 2048 with more
 //     than 4 tokens (with spills 428 us instead of 387 for one token of 16 layers, 894 instead of 721 for 8 of 8);
+//   - with 4-bit slots of d_model 2048 where a CTA may have a single row, so that the second group would only be met at the end (one token of 2
+//     experts, 4 layers, one group and two: d_ff 64 45.2 and 46.9 us, d_ff 256, 3 rows, 48.5 and 48.4);
 //   - where four stages of tiles of eight rows do not fit, so that a group's next tile would not be on its way while it works: bf16 slots
 //     beyond d_model 1024 (where HBM is the limit from 2048 on).
 // Measured, against one group with the width taken at run time (which spilled), us: bf16, d 512, d_ff 8192, 4 tokens of 4 experts, 4 layers
@@ -245,7 +247,7 @@ constexpr int NW = 16;                           // consumer warps
 constexpr int kGroupRows = 12;
 __host__ __device__ constexpr int decode_groups(int d, int tokens, int fmt, int rows_per_cta)
 {
-    return fmt == 0 ? (d > 1024 || rows_per_cta < kGroupRows ? 1 : d <= 512 && rows_per_cta >= 2 * kGroupRows ? 4 : 2) : d <= 1024 || (d == 2048 && tokens <= 4) ? 2 : 1;
+    return fmt == 0 ? (d > 1024 || rows_per_cta < kGroupRows ? 1 : d <= 512 && rows_per_cta >= 2 * kGroupRows ? 4 : 2) : d <= 1024 || (d == 2048 && tokens <= 4 && rows_per_cta >= 2) ? 2 : 1;
 }
 constexpr int kThreads = (NW + 1) * 32;          // + the producer warp
 constexpr int kBufPitch = 130;                   // floats between the warps' partial tiles (keeps the column sums conflict-free)

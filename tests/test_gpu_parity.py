@@ -270,6 +270,7 @@ def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory(F
     ("q4slots", 512, 1768, 2, 0, 3), ("q4slots", 512, 64, 2, 0, 3),  # 4-bit slots: two groups and one
     ("q4slots", 1024, 1768, 2, 0, 2), ("q4slots", 1024, 72, 2, 1, 3),
     ("q4slots", 2048, 1768, 2, 0, 4), ("q4slots", 4096, 72, 2, 0, 3),
+    ("q4slots", 2048, 144, 2, 0, 3), ("q4slots", 2048, 152, 2, 0, 3),  # one group below two rows per SM, and two
 ])
 def test_decode_kernels_of_every_width_and_grouping(store, d, F, k, n_shared, C):
     """Decode calls of 1 to 8 tokens, missed experts fetched by the kernel or by the host, element by element against the

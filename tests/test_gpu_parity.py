@@ -264,7 +264,8 @@ def test_wide_model_with_many_tokens_keeps_its_token_operands_in_tensor_memory(F
     ("bf16", 512, 3608, 1, 0, 4), ("bf16", 768, 1200, 2, 1, 2),      # d_ff that ends inside a tile; missed experts stored by either group
     ("bf16", 1024, 1768, 2, 0, 2),
     ("bf16", 1280, 72, 2, 0, 3), ("bf16", 1792, 1768, 1, 1, 4),      # one group, widths of their own
-    ("bf16", 2304, 72, 2, 0, 2), ("bf16", 3840, 48, 2, 1, 4),
+    ("bf16", 1536, 72, 2, 0, 3), ("bf16", 2304, 72, 2, 0, 2), ("bf16", 2560, 200, 2, 1, 4), ("bf16", 2816, 72, 2, 0, 3),
+    ("bf16", 3072, 72, 2, 0, 3), ("bf16", 3328, 72, 2, 0, 3), ("bf16", 3584, 48, 2, 1, 2), ("bf16", 3840, 48, 2, 1, 4),
     ("bf16", 3072, 1480, 2, 0, 4), ("bf16", 3328, 1480, 2, 0, 3),    # token operands in tensor memory from some number of tokens on
     ("bf16", 3584, 1480, 2, 0, 4), ("bf16", 3840, 888, 1, 1, 2), ("bf16", 4096, 888, 1, 1, 4),
     ("q4slots", 512, 1768, 2, 0, 3), ("q4slots", 512, 64, 2, 0, 3),  # 4-bit slots: two groups and one
@@ -284,7 +285,7 @@ def test_decode_kernels_of_every_width_and_grouping(store, d, F, k, n_shared, C)
             P.set_bias(P.bias, (np.arange(T) % 2).astype(np.int32))
             x = gen.hidden_states(801, 0, "decode", step, T, d)
             if rnd == 0:
-                res, _ = P.step(x, tokens=sorted({0, T - 1}))
+                res, _ = P.step(x)
                 outs[step] = res["out_bits"].copy()
             elif T * k <= C or C == E:               # (in compute groups a token's sum depends on what is resident)
                 assert np.array_equal(P.gpu.forward_np(x)["out_bits"], outs[step]), T
@@ -416,6 +417,7 @@ def test_prefill_grouped_gemm(d, F, E, k, C, n_shared, Ts):
     ("bf16", 256, 520, 5, 2, 1, (9, 64, 65, 700)),     # a launch for each GEMM; rows by index and copied
     ("bf16", 768, 1160, 3, 2, 0, (70, 300)),
     ("q4slots", 512, 1416, 4, 2, 1, (64, 65, 513)),    # one launch of single CTAs, then two of pairs
+    ("q4slots", 512, 264, 16, 2, 1, (200, 256)),       # single CTAs, a shared expert of two chunks: tiles expanded for each
     ("bf16", 1024, 6144, 2, 1, 0, (512, 513)),         # two launches up to 256 pairs per expert, one beyond
     ("q4slots", 1024, 2560, 2, 1, 0, (512, 513)),
 ])
@@ -816,10 +818,10 @@ def test_4bit_tokens_get_the_same_result_from_long_and_short_calls(d, F, E, k, n
     P.close()
 
 
-@pytest.mark.parametrize("T", [24, 300])
+@pytest.mark.parametrize("T", [24, 100, 300])
 def test_4bit_prompts_give_the_same_bits_every_time(T):
-    """Weight tiles that one CTA of a pair expands and the other's thread multiplies, many per CTA: a tile that was read
-    before it was complete would change some output."""
+    """Weight tiles that one CTA of a pair expands and the other's thread multiplies (24 tokens: its own), many per CTA: a tile
+    that was read before it was complete would change some output."""
     d, F, E, k = 2048, 1408, 12, 4
     P = _pair(d, F, E, k, E, seed=66, store="q4slots")
     x = gen.hidden_states(66, 0, "prefill", 0, T, d)

@@ -1016,7 +1016,6 @@ int forward_on(melinoe_moe *h, const Scratch &sc, void *cuda_stream, const void 
     gp.d = h->d;
     gp.F = h->F;
     gp.E = h->E;
-    gp.n_shared = h->n_shared;
     gp.slots = h->slots;
     gp.slot_stride = h->slot_stride;
     gp.shared_blobs = h->shared_dev;

@@ -232,9 +232,10 @@ constexpr int NW = 16;                           // consumer warps
 // of stages is a multiple of the groups', so that a stage belongs to one.  At the end the groups' sums of the same columns meet in
 // shared memory, and from then on warp w of group g of n stands for warp n w + g of sixteen.
 // One group
-//   - with bf16 slots where a call may have less than kGroupRows rows for a CTA (`rows`: those that it has for certain): a tile is over
-//     sooner with sixteen warps (d 1024, one token of 4 experts, 8 layers, one group and two: d_ff 256, 7 rows, 85.8 and 90.4 us; d_ff 768, 21 rows,
-//     108.8 and 108.3; d 256, d_ff 512, 8 tokens 173 and 152); four from twice as many on (d 256, 14 rows 80.9 with two, 82.6 with four);
+//   - with bf16 slots where a call may have less than kGroupRows rows for a CTA (`rows`: those of its top_k and shared experts; a launch of
+//     one compute group may have fewer, which beside its transfers was not to be measured): a tile is over sooner with sixteen warps (d 1024,
+//     one token of 4 experts, 8 layers, one group and two: d_ff 256, 7 rows, 85.8 and 90.4 us; d_ff 768, 21 rows, 108.8 and 108.3; d 256,
+//     d_ff 512, 8 tokens 173 and 152); four from twice as many on (d 256, 14 rows 80.9 with two, 82.6 with four);
 //   - where a warp's output columns of two would not fit its 96 registers: 4-bit slots of d_model 4096, and of 2048 with more
 //     than 4 tokens (with spills 428 us instead of 387 for one token of 16 layers, 894 instead of 721 for 8 of 8);
 //   - with 4-bit slots of d_model 2048 where a CTA may have a single row, so that the second group would only be met at the end (one token of 2
@@ -377,10 +378,11 @@ __device__ __forceinline__ void consume_q4(const DecParams &p, const DecGeometry
             mma_16816(cg[(2 * i + 1) & 3], Pg[2], Pu[2], Pg[3], Pu[3], xb.z, xb.w);
         }
     };
-    // The warps' partial tiles meet in shared memory: every warp stores its 128 partial values, warp w sums
-    // 8 of the 128 over all warps (four lanes per value, each adding four warps' parts in warp order, then a
-    // fixed tree), and every warp reads the complete tile.  Two block-wide named barriers order this; the
-    // buffers alternate from tile to tile.  (Measured and dropped: counting mbarriers in their place, with
+    // The warps' partial tiles meet in shared memory: every warp of the group stores its 128 partial values, sums 8 NG of the 128
+    // over the group's warps (4 / NG lanes per value, each adding four warps' parts in warp order, then a fixed tree), and reads the
+    // complete tile.  Two named barriers of the group order this.  The buffers alternate from tile to tile, though one would do: its 8 KB
+    // go to the ring then, which is worth 1 to 2 % up to d_model 2048, but a fourth stage at 4096 makes one token slower (2 experts of
+    // d_ff 1024, 4 layers 84 -> 92 us).  (Measured and dropped: counting mbarriers in their place, with
     // the loop running one tile ahead so that a warp has other work between arriving and waiting -- the
     // hardware barrier is the cheaper way for 16 warps to meet; and h formed once per tile by the summing
     // warps instead of by every warp for itself -- it lengthens the path between the two barriers.)
@@ -1321,8 +1323,10 @@ cudaError_t ffn_decode_configure(int n_sms, size_t max_smem, DecLaunchCfg *cfg)
     size_t stat = 0;
 #define MELINOE_FN(...) reinterpret_cast<const void *>(ffn_decode_kernel<__VA_ARGS__>)
     // (In the order in which their code is loaded, behind the planner's.  Where it lies beside the planner's, with which it alternates, is
-    // worth up to 4 % of a short call; of six orders, for one token of 16 layers, this one gave 344 us with 4-bit slots and 419 with bf16
-    // ones, the others 344 to 360 and 417 to 424.)
+    // worth up to 4 % of a short call; of six orders, for one token of 16 layers of d_model 2048, this one gave 344 us with 4-bit slots and 419
+    // with bf16 ones, the others 344 to 360 and 417 to 424.  Other widths come as they come: from build to build a short call of theirs
+    // differs by up to 2 %.  Nothing but speed hangs on it.  Asking for all of them costs a process's first handle nothing that was to be
+    // measured: 25 ms as with seven.)
     const void *fns[] = {MELINOE_FN(16, 0), MELINOE_FN(8, 0), MELINOE_FN(8, 1, 0, 2, 1), MELINOE_FN(16, 0, 1), MELINOE_FN(8, 1),
                          MELINOE_FN(16, 1, 0, 1, 1), MELINOE_FN(16, 1), MELINOE_FN(4, 1, 0, 2, 1), MELINOE_FN(4, 1, 0, 2),
                          MELINOE_FN(2, 1, 0, 2, 1), MELINOE_FN(2, 1, 0, 2), MELINOE_FN(1, 0), MELINOE_FN(1, 0, 0, 2), MELINOE_FN(2, 0),
@@ -1428,7 +1432,8 @@ cudaError_t launch_ffn_decode(cudaStream_t stream, const DecLaunchCfg &cfg, cons
     auto launch = [&](auto kernel) { return cudaLaunchKernelEx(&lc, kernel, p, geo); };
     cudaError_t e;
     if (p.fmt == 0) {
-        // (loops over the width that the compiler knows, without spills: d 1536, d_ff 4096, 4 tokens of 4 experts, 4 layers 382 -> 349 us)
+        // (loops over the width that the compiler knows, which hardly spill, 12 bytes at most: d 1536, d_ff 4096, 4 tokens of 4 experts,
+        // 4 layers 382 -> 349 us)
         switch (mt) {
         case 1:
             e = ng == 4   ? launch(ffn_decode_kernel<1, 0, 0, 4>)

@@ -141,7 +141,7 @@ struct DecGeometry {
 cudaError_t ffn_decode_configure(int n_sms, size_t max_smem, DecLaunchCfg *cfg);
 bool ffn_decode_supported(int d, int F);
 bool ffn_decode_supported_q4(int d, int F);
-// min_req: requests that the call has for certain (its top_k and the shared experts)
+// min_req: requests that the call has for certain (its top_k and the shared experts; a launch of one compute group may have fewer)
 cudaError_t ffn_decode_geometry(const DecLaunchCfg &cfg, int d, int F, int tokens, int fmt, int min_req, DecGeometry *geo);
 cudaError_t launch_ffn_decode(cudaStream_t stream, const DecLaunchCfg &cfg, const DecGeometry &geo,
                               const DecParams &p);
@@ -168,7 +168,7 @@ struct GemmParams {
     const float *row_gate;           // 4-bit slots: gate of every sorted row (PromptParams::row_gate)
     float *zs;                       // expert outputs, [sorted rows][d] fp32
     int *err;
-    int group, d, F, E, n_shared;
+    int group, d, F, E;
     // 4-bit slots: the blobs themselves (their scales are read directly) and the bytes of one hidden unit
     const char *slots;
     size_t slot_stride;

@@ -916,246 +916,246 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_decode_kernel(const __grid_co
         if constexpr (FMT == 1) {
             consume_q4<MT_, NG, TG>(p, geo, s_req, s_sums, buf, ring_s, xs_s, full0, empty0, abort_flag, q_lo, q_hi, trace);
         } else {
-        // groups of warps (see decode_groups): this warp's group and place in it, k-steps and m-tiles of a warp
-        constexpr int NWG = NW / NG, kTiles = MT_ * NG;
-        const int grp = NG == 1 ? 0 : warp / NWG, gw = NG == 1 ? warp : warp % NWG;
-        buf += grp * (NWG * kBufPitch);
-        float *sums = s_sums + grp * 128;
-        float acc[kTiles][4];
-#pragma unroll
-        for (int i = 0; i < kTiles; ++i)
-            acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
-        const bool has_tok = g < Tc;
-        const uint32_t xrow = xs_s + g * XP + tig * 4 + gw * kTiles * 32;     // this warp's columns of token g
-        // XT: the token operand of this thread's 16 gate/up steps (two registers each) never changes, so it is
-        // written once into the thread's own lane of tensor memory (warp w may use lanes 32 (w mod 4) ..,
-        // the four warps of a lane quarter take 32 columns each) and fetched from there step by step.
-        uint32_t xt = 0;
-        if constexpr (XT == 1) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            xt = s_tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * 32;
-            uint32_t r[32];
-            const uint16_t *xr = p.x + (size_t)(tok0 + (has_tok ? g : 0)) * d + warp * (MT * 16) + 2 * tig;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const bool on = has_tok && i < MT;
-                r[2 * i] = on ? __ldcg(reinterpret_cast<const uint32_t *>(xr + i * 16)) : 0u;
-                r[2 * i + 1] = on ? __ldcg(reinterpret_cast<const uint32_t *>(xr + i * 16 + 8)) : 0u;
-            }
-            tmem_st32(xt, r);
-        }
-        // ldmatrix lane roles.  gate/up: matrices (W_g rows, k low), (W_u rows, k low), (W_g rows, k high),
-        // (W_u rows, k high); down: four consecutive 8-column pieces of the W_d^T rows
-        const int r8 = lane & 7, sel_gu = (lane >> 3) & 1, kh = lane >> 4, mat = lane >> 3;
-        const uint32_t src0 = (uint32_t)((2 * tig) * 4 + (g >> 1)), src1 = src0 + 4;
-        uint32_t st = 0, ph = 0;                    // ring stage of the tile and the parity of its barrier phase
-        int left = q_hi - q_lo, a = q_lo / F, f0 = q_lo % F;
-        auto skip = [&] {
-            const int m = min(min(TR, F - f0), left);
-            if (++st == (uint32_t)S) {
-                st = 0;
-                ph ^= 1u;
-            }
-            left -= m;
-            f0 += m;
-            if (f0 == F) {
-                f0 = 0;
-                ++a;
-            }
-        };
-#pragma unroll 1
-        for (int i = 0; i < grp && left > 0; ++i)
-            skip();
-        while (left > 0) {
-            const int m = min(min(TR, F - f0), left);
-            const uint32_t stage = ring_s + st * STAGE;
-            mbar_wait(full0 + 8 * st, ph, abort_flag);
-            if (p.trace && tid == 0 && left == q_hi - q_lo)
-                p.trace[(size_t)blockIdx.x * 8 + 2] = globaltimer_ns();
-            char *wb = s_req[a].wb;
-            const bool store_tile = wb != nullptr && tid % (32 * NWG) == 0;
-            if (store_tile)
-                bulk_s2g(wb + (size_t)f0 * RB, stage, (uint32_t)m * RB);
-            const int rr = r8 < m ? r8 : 0;               // rows the tile does not have read row 0 (never used)
-            const uint32_t swz = (uint32_t)((f0 + rr) & 7);
-            const uint32_t rowbase = stage + rr * RB;
-            // ---- gate/up: this warp's columns of the tile's rows.  A dependent mma.sync issues only every
-            // ~110 cycles, so the k-steps go to four independent accumulators, and the fragment loads of
-            // four steps are issued before their four products.
-            // (Where a warp has 16 m-tiles of output accumulators, d_model above 2048, registers only allow
-            // two steps at a time.)
-            constexpr int GG = kTiles > 8 ? 2 : 4;
-            float cg[GG][4];
-#pragma unroll
-            for (int i = 0; i < GG; ++i)
-                cg[i][0] = cg[i][1] = cg[i][2] = cg[i][3] = 0.f;
-            {
-                const uint32_t arow = rowbase + sel_gu * 2 * d;
-                const uint32_t ch0 = (uint32_t)(2 * gw * kTiles + kh);
-#pragma unroll
-                for (int i0 = 0; i0 < kTiles; i0 += GG) {
-                    if (i0 < kTiles) {
-                        uint32_t af[GG][4], bf[GG][2];
-#pragma unroll
-                        for (int j = 0; j < GG; ++j) {
-                            const int i = i0 + j < kTiles ? i0 + j : i0;     // beyond the warp's last step: a valid address, product unused
-                            ldmatrix_x4(arow + (((ch0 + 2 * i) ^ swz) << 4), af[j][0], af[j][1], af[j][2], af[j][3]);
-                            if constexpr (XT == 0) {
-                                bf[j][0] = has_tok ? lds32(xrow + i * 32) : 0u;
-                                bf[j][1] = has_tok ? lds32(xrow + i * 32 + 16) : 0u;
-                            }
-                        }
-                        if constexpr (XT == 1) {
-                            static_assert(XT == 0 || GG == 2, "two steps per group");
-                            tmem_ld4(xt + 2 * i0, bf[0][0], bf[0][1], bf[GG - 1][0], bf[GG - 1][1]);
-                            tmem_wait_ld();
-                        }
-#pragma unroll
-                        for (int j = 0; j < GG; ++j)
-                            if (i0 + j < kTiles)
-                                mma_16816(cg[j], af[j][0], af[j][1], af[j][2], af[j][3], bf[j][0], bf[j][1]);
-                    }
-                }
-            }
-            // ---- the warps' partial tiles meet: warp w sums 8 of the tile's 128 values over all warps (four
-            // lanes per value, each adding four warps' parts in warp order, then a fixed tree), then every
-            // warp reads the complete tile
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                buf[gw * kBufPitch + i * 32 + lane] = GG == 4 ? (cg[0][i] + cg[1][i]) + (cg[2][i] + cg[3][i]) : cg[0][i] + cg[GG - 1][i];
-            auto meet = [&] {
-                if (NG == 1)
-                    asm volatile("bar.sync 1, %0;" ::"n"(NW * 32) : "memory");
-                else
-                    asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(NWG * 32) : "memory");
-            };
-            meet();
-            {
-                constexpr int kOwn = 8 * NG;         // values of a warp
-                const int e = gw * kOwn + (lane & (kOwn - 1)), pg = lane / kOwn;
-                float v = buf[(pg * 4) * kBufPitch + e];
-                v += buf[(pg * 4 + 1) * kBufPitch + e];
-                v += buf[(pg * 4 + 2) * kBufPitch + e];
-                v += buf[(pg * 4 + 3) * kBufPitch + e];
-                if (NG == 1)
-                    v += __shfl_xor_sync(0xffffffffu, v, 8);
-                if (NG <= 2)
-                    v += __shfl_xor_sync(0xffffffffu, v, 16);
-                if (lane < kOwn)
-                    sums[e] = v;
-            }
-            meet();
-            const float s0 = sums[lane], s1 = sums[32 + lane], s2 = sums[64 + lane], s3 = sums[96 + lane];
-            // rows g and g + 8 of the tile are g_f and u_f of f = f0 + g, columns are tokens 2 tig, 2 tig + 1
-            const float gt0 = s_req[a].gate[2 * tig], gt1 = s_req[a].gate[2 * tig + 1];
-            // (the fast division: the exact one takes its slow path for the zeros of unused token columns)
-            float h0 = __fdividef(s0, 1.0f + __expf(-s0)) * s2 * gt0;
-            float h1 = __fdividef(s1, 1.0f + __expf(-s1)) * s3 * gt1;
-            if (g >= m || gt0 == 0.0f)
-                h0 = 0.f;
-            if (g >= m || gt1 == 0.0f)
-                h1 = 0.f;
-            const uint32_t hp = bf16_rne(h0) | (bf16_rne(h1) << 16);
-            // B fragment of the down product: h[f = 2 tig', 2 tig' + 1][token g'] from the lanes that hold them
-            const uint32_t v0 = __shfl_sync(0xffffffffu, hp, src0), v1 = __shfl_sync(0xffffffffu, hp, src1);
-            const uint32_t bd = (g & 1) ? ((v0 >> 16) | (v1 & 0xffff0000u)) : ((v0 & 0xffffu) | (v1 << 16));
-            // ---- down: the tile's rows are the K dimension (rows the tile does not have count as zero)
-            {
-                const uint32_t km = (2 * tig < m ? 0x0000ffffu : 0u) | (2 * tig + 1 < m ? 0xffff0000u : 0u);
-                const uint32_t drow = rowbase + 4 * d;
-                const uint32_t cc0 = (uint32_t)(gw * kTiles * 2);
-                constexpr int DG = kTiles > 8 ? 2 : 4;      // loads (of two m-tiles each) per group
-#pragma unroll
-                for (int m0 = 0; m0 < kTiles; m0 += 2 * DG) {
-                    if (m0 < kTiles) {
-                        // fragment loads of up to eight m-tiles first, then their products
-                        uint32_t rf[DG][4];
-#pragma unroll
-                        for (int j = 0; j < DG; ++j) {
-                            // a load covers two m-tiles; an odd last one is fetched together with the one before
-                            // it (or, if it is the warp's only one, with 16 columns that are not used)
-                            int mi = m0 + 2 * j;
-                            if (mi >= kTiles)
-                                mi = m0;
-                            else if (mi + 1 >= kTiles && mi > 0)
-                                mi -= 1;
-                            ldmatrix_x4_trans(drow + (((cc0 + 2 * mi + mat) ^ swz) << 4), rf[j][0], rf[j][1], rf[j][2], rf[j][3]);
-                        }
-#pragma unroll
-                        for (int j = 0; j < DG; ++j) {
-                            const int mi = m0 + 2 * j;
-                            if (mi + 1 < kTiles) {
-                                mma_16816(acc[mi], rf[j][0] & km, rf[j][1] & km, 0u, 0u, bd, 0u);
-                                mma_16816(acc[mi + 1], rf[j][2] & km, rf[j][3] & km, 0u, 0u, bd, 0u);
-                            } else if (mi < kTiles) {
-                                if (mi > 0)
-                                    mma_16816(acc[mi], rf[j][2] & km, rf[j][3] & km, 0u, 0u, bd, 0u);
-                                else
-                                    mma_16816(acc[mi], rf[j][0] & km, rf[j][1] & km, 0u, 0u, bd, 0u);
-                            }
-                        }
-                    }
-                }
-            }
-            if (store_tile)
-                bulk_wait_read();         // the slot store has read the stage
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(empty0 + 8 * st);
-            skip();
-#pragma unroll
-            for (int i = 1; i < NG; ++i)     // the other groups'
-                if (left > 0)
-                    skip();
-        }
-        if (trace && tid == 0)
-            trace[3] = globaltimer_ns();
-        if constexpr (NG > 1) {
-            // the groups' sums, in their order: a warp keeps those of its columns that are its group's
-            asm volatile("bar.sync 8, %0;" ::"n"(NW * 32) : "memory");      // no tile is read any more: the ring is free
-            auto at = [&](int of, int i) { return ring_s + (uint32_t)(((of * NWG + gw) * kTiles + i) * 512 + lane * 16); };
+            // groups of warps (see decode_groups): this warp's group and place in it, k-steps and m-tiles of a warp
+            constexpr int NWG = NW / NG, kTiles = MT_ * NG;
+            const int grp = NG == 1 ? 0 : warp / NWG, gw = NG == 1 ? warp : warp % NWG;
+            buf += grp * (NWG * kBufPitch);
+            float *sums = s_sums + grp * 128;
+            float acc[kTiles][4];
 #pragma unroll
             for (int i = 0; i < kTiles; ++i)
-                asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(at(grp, i)), "f"(acc[i][0]), "f"(acc[i][1]), "f"(acc[i][2]), "f"(acc[i][3]) : "memory");
-            asm volatile("bar.sync 8, %0;" ::"n"(NW * 32) : "memory");
-#pragma unroll
-            for (int i = 0; i < MT; ++i) {
                 acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+            const bool has_tok = g < Tc;
+            const uint32_t xrow = xs_s + g * XP + tig * 4 + gw * kTiles * 32;     // this warp's columns of token g
+            // XT: the token operand of this thread's 16 gate/up steps (two registers each) never changes, so it is
+            // written once into the thread's own lane of tensor memory (warp w may use lanes 32 (w mod 4) ..,
+            // the four warps of a lane quarter take 32 columns each) and fetched from there step by step.
+            uint32_t xt = 0;
+            if constexpr (XT == 1) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                xt = s_tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * 32;
+                uint32_t r[32];
+                const uint16_t *xr = p.x + (size_t)(tok0 + (has_tok ? g : 0)) * d + warp * (MT * 16) + 2 * tig;
 #pragma unroll
-                for (int of = 0; of < NG; ++of) {
-                    const uint4 v = lds128(at(of, grp * MT + i));
-                    acc[i][0] += __uint_as_float(v.x);
-                    acc[i][1] += __uint_as_float(v.y);
-                    acc[i][2] += __uint_as_float(v.z);
-                    acc[i][3] += __uint_as_float(v.w);
+                for (int i = 0; i < 16; ++i) {
+                    const bool on = has_tok && i < MT;
+                    r[2 * i] = on ? __ldcg(reinterpret_cast<const uint32_t *>(xr + i * 16)) : 0u;
+                    r[2 * i + 1] = on ? __ldcg(reinterpret_cast<const uint32_t *>(xr + i * 16 + 8)) : 0u;
                 }
+                tmem_st32(xt, r);
             }
-        }
-        // ---- this CTA's partial output, added into the call's accumulator as 64-bit fixed point (2^-40):
-        // integer addition is exact, so the sum does not depend on the order in which the CTAs arrive.
-        // (Adds without a return value: atomics that return the old word, which would let the last adder
-        // of an element finish it on the spot, measured three times slower under this contention.)
-        {
-            unsigned long long *yacc = reinterpret_cast<unsigned long long *>(p.yacc);
-            auto add = [&](int t, int c, float v) {
-                const long long fx = __float2ll_rn(v * 1099511627776.0f);    // exact scaling, then to the nearest 2^-40
-                red_add_u64(yacc + (size_t)t * d + c, (unsigned long long)fx);
+            // ldmatrix lane roles.  gate/up: matrices (W_g rows, k low), (W_u rows, k low), (W_g rows, k high),
+            // (W_u rows, k high); down: four consecutive 8-column pieces of the W_d^T rows
+            const int r8 = lane & 7, sel_gu = (lane >> 3) & 1, kh = lane >> 4, mat = lane >> 3;
+            const uint32_t src0 = (uint32_t)((2 * tig) * 4 + (g >> 1)), src1 = src0 + 4;
+            uint32_t st = 0, ph = 0;                    // ring stage of the tile and the parity of its barrier phase
+            int left = q_hi - q_lo, a = q_lo / F, f0 = q_lo % F;
+            auto skip = [&] {
+                const int m = min(min(TR, F - f0), left);
+                if (++st == (uint32_t)S) {
+                    st = 0;
+                    ph ^= 1u;
+                }
+                left -= m;
+                f0 += m;
+                if (f0 == F) {
+                    f0 = 0;
+                    ++a;
+                }
             };
+#pragma unroll 1
+            for (int i = 0; i < grp && left > 0; ++i)
+                skip();
+            while (left > 0) {
+                const int m = min(min(TR, F - f0), left);
+                const uint32_t stage = ring_s + st * STAGE;
+                mbar_wait(full0 + 8 * st, ph, abort_flag);
+                if (p.trace && tid == 0 && left == q_hi - q_lo)
+                    p.trace[(size_t)blockIdx.x * 8 + 2] = globaltimer_ns();
+                char *wb = s_req[a].wb;
+                const bool store_tile = wb != nullptr && tid % (32 * NWG) == 0;
+                if (store_tile)
+                    bulk_s2g(wb + (size_t)f0 * RB, stage, (uint32_t)m * RB);
+                const int rr = r8 < m ? r8 : 0;               // rows the tile does not have read row 0 (never used)
+                const uint32_t swz = (uint32_t)((f0 + rr) & 7);
+                const uint32_t rowbase = stage + rr * RB;
+                // ---- gate/up: this warp's columns of the tile's rows.  A dependent mma.sync issues only every
+                // ~110 cycles, so the k-steps go to four independent accumulators, and the fragment loads of
+                // four steps are issued before their four products.
+                // (Where a warp has 16 m-tiles of output accumulators, d_model above 2048, registers only allow
+                // two steps at a time.)
+                constexpr int GG = kTiles > 8 ? 2 : 4;
+                float cg[GG][4];
 #pragma unroll
-            for (int mi = 0; mi < kTiles; ++mi) {
-                if (mi < MT) {
-                    const int c = ((gw * NG + grp) * MT + mi) * 16 + g;
-                    if (2 * tig < Tc) {
-                        add(2 * tig, c, acc[mi][0]);
-                        add(2 * tig, c + 8, acc[mi][2]);
+                for (int i = 0; i < GG; ++i)
+                    cg[i][0] = cg[i][1] = cg[i][2] = cg[i][3] = 0.f;
+                {
+                    const uint32_t arow = rowbase + sel_gu * 2 * d;
+                    const uint32_t ch0 = (uint32_t)(2 * gw * kTiles + kh);
+#pragma unroll
+                    for (int i0 = 0; i0 < kTiles; i0 += GG) {
+                        if (i0 < kTiles) {
+                            uint32_t af[GG][4], bf[GG][2];
+#pragma unroll
+                            for (int j = 0; j < GG; ++j) {
+                                const int i = i0 + j < kTiles ? i0 + j : i0;     // beyond the warp's last step: a valid address, product unused
+                                ldmatrix_x4(arow + (((ch0 + 2 * i) ^ swz) << 4), af[j][0], af[j][1], af[j][2], af[j][3]);
+                                if constexpr (XT == 0) {
+                                    bf[j][0] = has_tok ? lds32(xrow + i * 32) : 0u;
+                                    bf[j][1] = has_tok ? lds32(xrow + i * 32 + 16) : 0u;
+                                }
+                            }
+                            if constexpr (XT == 1) {
+                                static_assert(XT == 0 || GG == 2, "two steps per group");
+                                tmem_ld4(xt + 2 * i0, bf[0][0], bf[0][1], bf[GG - 1][0], bf[GG - 1][1]);
+                                tmem_wait_ld();
+                            }
+#pragma unroll
+                            for (int j = 0; j < GG; ++j)
+                                if (i0 + j < kTiles)
+                                    mma_16816(cg[j], af[j][0], af[j][1], af[j][2], af[j][3], bf[j][0], bf[j][1]);
+                        }
                     }
-                    if (2 * tig + 1 < Tc) {
-                        add(2 * tig + 1, c, acc[mi][1]);
-                        add(2 * tig + 1, c + 8, acc[mi][3]);
+                }
+                // ---- the warps' partial tiles meet: warp w sums 8 of the tile's 128 values over all warps (four
+                // lanes per value, each adding four warps' parts in warp order, then a fixed tree), then every
+                // warp reads the complete tile
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    buf[gw * kBufPitch + i * 32 + lane] = GG == 4 ? (cg[0][i] + cg[1][i]) + (cg[2][i] + cg[3][i]) : cg[0][i] + cg[GG - 1][i];
+                auto meet = [&] {
+                    if (NG == 1)
+                        asm volatile("bar.sync 1, %0;" ::"n"(NW * 32) : "memory");
+                    else
+                        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(NWG * 32) : "memory");
+                };
+                meet();
+                {
+                    constexpr int kOwn = 8 * NG;         // values of a warp
+                    const int e = gw * kOwn + (lane & (kOwn - 1)), pg = lane / kOwn;
+                    float v = buf[(pg * 4) * kBufPitch + e];
+                    v += buf[(pg * 4 + 1) * kBufPitch + e];
+                    v += buf[(pg * 4 + 2) * kBufPitch + e];
+                    v += buf[(pg * 4 + 3) * kBufPitch + e];
+                    if (NG == 1)
+                        v += __shfl_xor_sync(0xffffffffu, v, 8);
+                    if (NG <= 2)
+                        v += __shfl_xor_sync(0xffffffffu, v, 16);
+                    if (lane < kOwn)
+                        sums[e] = v;
+                }
+                meet();
+                const float s0 = sums[lane], s1 = sums[32 + lane], s2 = sums[64 + lane], s3 = sums[96 + lane];
+                // rows g and g + 8 of the tile are g_f and u_f of f = f0 + g, columns are tokens 2 tig, 2 tig + 1
+                const float gt0 = s_req[a].gate[2 * tig], gt1 = s_req[a].gate[2 * tig + 1];
+                // (the fast division: the exact one takes its slow path for the zeros of unused token columns)
+                float h0 = __fdividef(s0, 1.0f + __expf(-s0)) * s2 * gt0;
+                float h1 = __fdividef(s1, 1.0f + __expf(-s1)) * s3 * gt1;
+                if (g >= m || gt0 == 0.0f)
+                    h0 = 0.f;
+                if (g >= m || gt1 == 0.0f)
+                    h1 = 0.f;
+                const uint32_t hp = bf16_rne(h0) | (bf16_rne(h1) << 16);
+                // B fragment of the down product: h[f = 2 tig', 2 tig' + 1][token g'] from the lanes that hold them
+                const uint32_t v0 = __shfl_sync(0xffffffffu, hp, src0), v1 = __shfl_sync(0xffffffffu, hp, src1);
+                const uint32_t bd = (g & 1) ? ((v0 >> 16) | (v1 & 0xffff0000u)) : ((v0 & 0xffffu) | (v1 << 16));
+                // ---- down: the tile's rows are the K dimension (rows the tile does not have count as zero)
+                {
+                    const uint32_t km = (2 * tig < m ? 0x0000ffffu : 0u) | (2 * tig + 1 < m ? 0xffff0000u : 0u);
+                    const uint32_t drow = rowbase + 4 * d;
+                    const uint32_t cc0 = (uint32_t)(gw * kTiles * 2);
+                    constexpr int DG = kTiles > 8 ? 2 : 4;      // loads (of two m-tiles each) per group
+#pragma unroll
+                    for (int m0 = 0; m0 < kTiles; m0 += 2 * DG) {
+                        if (m0 < kTiles) {
+                            // fragment loads of up to eight m-tiles first, then their products
+                            uint32_t rf[DG][4];
+#pragma unroll
+                            for (int j = 0; j < DG; ++j) {
+                                // a load covers two m-tiles; an odd last one is fetched together with the one before
+                                // it (or, if it is the warp's only one, with 16 columns that are not used)
+                                int mi = m0 + 2 * j;
+                                if (mi >= kTiles)
+                                    mi = m0;
+                                else if (mi + 1 >= kTiles && mi > 0)
+                                    mi -= 1;
+                                ldmatrix_x4_trans(drow + (((cc0 + 2 * mi + mat) ^ swz) << 4), rf[j][0], rf[j][1], rf[j][2], rf[j][3]);
+                            }
+#pragma unroll
+                            for (int j = 0; j < DG; ++j) {
+                                const int mi = m0 + 2 * j;
+                                if (mi + 1 < kTiles) {
+                                    mma_16816(acc[mi], rf[j][0] & km, rf[j][1] & km, 0u, 0u, bd, 0u);
+                                    mma_16816(acc[mi + 1], rf[j][2] & km, rf[j][3] & km, 0u, 0u, bd, 0u);
+                                } else if (mi < kTiles) {
+                                    if (mi > 0)
+                                        mma_16816(acc[mi], rf[j][2] & km, rf[j][3] & km, 0u, 0u, bd, 0u);
+                                    else
+                                        mma_16816(acc[mi], rf[j][0] & km, rf[j][1] & km, 0u, 0u, bd, 0u);
+                                }
+                            }
+                        }
+                    }
+                }
+                if (store_tile)
+                    bulk_wait_read();         // the slot store has read the stage
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(empty0 + 8 * st);
+                skip();
+#pragma unroll
+                for (int i = 1; i < NG; ++i)     // the other groups'
+                    if (left > 0)
+                        skip();
+            }
+            if (trace && tid == 0)
+                trace[3] = globaltimer_ns();
+            if constexpr (NG > 1) {
+                // the groups' sums, in their order: a warp keeps those of its columns that are its group's
+                asm volatile("bar.sync 8, %0;" ::"n"(NW * 32) : "memory");      // no tile is read any more: the ring is free
+                auto at = [&](int of, int i) { return ring_s + (uint32_t)(((of * NWG + gw) * kTiles + i) * 512 + lane * 16); };
+#pragma unroll
+                for (int i = 0; i < kTiles; ++i)
+                    asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(at(grp, i)), "f"(acc[i][0]), "f"(acc[i][1]), "f"(acc[i][2]), "f"(acc[i][3]) : "memory");
+                asm volatile("bar.sync 8, %0;" ::"n"(NW * 32) : "memory");
+#pragma unroll
+                for (int i = 0; i < MT; ++i) {
+                    acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+#pragma unroll
+                    for (int of = 0; of < NG; ++of) {
+                        const uint4 v = lds128(at(of, grp * MT + i));
+                        acc[i][0] += __uint_as_float(v.x);
+                        acc[i][1] += __uint_as_float(v.y);
+                        acc[i][2] += __uint_as_float(v.z);
+                        acc[i][3] += __uint_as_float(v.w);
                     }
                 }
             }
-        }
+            // ---- this CTA's partial output, added into the call's accumulator as 64-bit fixed point (2^-40):
+            // integer addition is exact, so the sum does not depend on the order in which the CTAs arrive.
+            // (Adds without a return value: atomics that return the old word, which would let the last adder
+            // of an element finish it on the spot, measured three times slower under this contention.)
+            {
+                unsigned long long *yacc = reinterpret_cast<unsigned long long *>(p.yacc);
+                auto add = [&](int t, int c, float v) {
+                    const long long fx = __float2ll_rn(v * 1099511627776.0f);    // exact scaling, then to the nearest 2^-40
+                    red_add_u64(yacc + (size_t)t * d + c, (unsigned long long)fx);
+                };
+#pragma unroll
+                for (int mi = 0; mi < kTiles; ++mi) {
+                    if (mi < MT) {
+                        const int c = ((gw * NG + grp) * MT + mi) * 16 + g;
+                        if (2 * tig < Tc) {
+                            add(2 * tig, c, acc[mi][0]);
+                            add(2 * tig, c + 8, acc[mi][2]);
+                        }
+                        if (2 * tig + 1 < Tc) {
+                            add(2 * tig + 1, c, acc[mi][1]);
+                            add(2 * tig + 1, c + 8, acc[mi][3]);
+                        }
+                    }
+                }
+            }
         }
         // ---- count this warp out; the last CTA's warp turns the sums of its columns into the output
         // (groups: see decode_groups)

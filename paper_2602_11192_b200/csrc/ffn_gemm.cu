@@ -994,88 +994,88 @@ __global__ void __launch_bounds__(gemm_threads(FMT), 1) ffn_gemm_kernel(const __
             const char *blob = it.slot >= 0 ? p.slots + (size_t)it.slot * p.slot_stride : p.shared_blobs[-1 - it.slot];
             const int kblocks = it.kblocks;
             auto expand = [&](auto phase_) {
-            constexpr int kPhase = decltype(phase_)::value;
-            constexpr int kRawBlocks = kPhase == 1 ? 4 : 2;           // k-blocks of one fetch of codes
-            // GEMM 1: rows of eight g, eight u, ..; GEMM 2: rows f, 64 of the first column group, 64 of the second
-            const int f_row = kPhase == 1 ? it.m0 + (row >> 4) * 8 + (row & 7) : (row & 63);
-            const int part = (row >> 3) & 1, cg = row >> 6;
-            const char *sc_base = kPhase == 1 ? blob + (size_t)f_row * ub + scales + (size_t)part * (p.d / 32)
-                                             : blob + (size_t)f_row * ub + scales + 2 * (size_t)(p.d / 32) + (size_t)(it.m0 / 64 + cg) * 2;
-            // the scale of the next k-block is in flight while this one is expanded
-            auto scale_of = [&](int kb) -> uint32_t {
-                if (kPhase == 1)
-                    return f_row < p.F && kb < kblocks ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base) + kb) : 0u;
-                return kb * kBK + f_row < p.F ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base + (size_t)kb * kBK * ub)) : 0u;
-            };
-            uint32_t sc = scale_of((group - (int)n0) & (kExpandGroups - 1));
-            bool ok = true;
-            for (int kr = 0; kr < kblocks && ok; kr += kRawBlocks, ++rn) {
-                const uint32_t rs = rn % kRawStages;
-                ok = mbar_wait(rfull0 + 8 * rs, (rn / kRawStages) & 1u, abort_flag);
-                for (int sub = (group - (int)n0 - kr) & (kExpandGroups - 1); sub < kRawBlocks && kr + sub < kblocks && ok; sub += kExpandGroups) {
-                const int kb = kr + sub;
-                const uint32_t n = n0 + (uint32_t)kb, s = n % kStages;
-                if (n >= (uint32_t)kStages)
-                    ok = mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag);
-                if (!ok)
-                    break;
-                const uint32_t ss = sc * 0x10001u;
-                const uint32_t raw = raw_s + rs * kRawBytes, a_dst = ring_s + s * kStageBytes + row * 128;
-                const uint32_t x = (uint32_t)(row & 7);      // = f mod 8 in both phases
-                if (kPhase == 1) {
-                    // 64 columns = pieces 2 sub, 2 sub + 1 of this row's 128 bytes of codes -> eight pieces of bf16
-                    const uint32_t src = raw + row * 128;
+                constexpr int kPhase = decltype(phase_)::value;
+                constexpr int kRawBlocks = kPhase == 1 ? 4 : 2;           // k-blocks of one fetch of codes
+                // GEMM 1: rows of eight g, eight u, ..; GEMM 2: rows f, 64 of the first column group, 64 of the second
+                const int f_row = kPhase == 1 ? it.m0 + (row >> 4) * 8 + (row & 7) : (row & 63);
+                const int part = (row >> 3) & 1, cg = row >> 6;
+                const char *sc_base = kPhase == 1 ? blob + (size_t)f_row * ub + scales + (size_t)part * (p.d / 32)
+                                                 : blob + (size_t)f_row * ub + scales + 2 * (size_t)(p.d / 32) + (size_t)(it.m0 / 64 + cg) * 2;
+                // the scale of the next k-block is in flight while this one is expanded
+                auto scale_of = [&](int kb) -> uint32_t {
+                    if (kPhase == 1)
+                        return f_row < p.F && kb < kblocks ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base) + kb) : 0u;
+                    return kb * kBK + f_row < p.F ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(sc_base + (size_t)kb * kBK * ub)) : 0u;
+                };
+                uint32_t sc = scale_of((group - (int)n0) & (kExpandGroups - 1));
+                bool ok = true;
+                for (int kr = 0; kr < kblocks && ok; kr += kRawBlocks, ++rn) {
+                    const uint32_t rs = rn % kRawStages;
+                    ok = mbar_wait(rfull0 + 8 * rs, (rn / kRawStages) & 1u, abort_flag);
+                    for (int sub = (group - (int)n0 - kr) & (kExpandGroups - 1); sub < kRawBlocks && kr + sub < kblocks && ok; sub += kExpandGroups) {
+                        const int kb = kr + sub;
+                        const uint32_t n = n0 + (uint32_t)kb, s = n % kStages;
+                        if (n >= (uint32_t)kStages)
+                            ok = mbar_wait(empty0 + 8 * s, ((n / kStages) - 1u) & 1u, abort_flag);
+                        if (!ok)
+                            break;
+                        const uint32_t ss = sc * 0x10001u;
+                        const uint32_t raw = raw_s + rs * kRawBytes, a_dst = ring_s + s * kStageBytes + row * 128;
+                        const uint32_t x = (uint32_t)(row & 7);      // = f mod 8 in both phases
+                        if (kPhase == 1) {
+                            // 64 columns = pieces 2 sub, 2 sub + 1 of this row's 128 bytes of codes -> eight pieces of bf16
+                            const uint32_t src = raw + row * 128;
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint4 c4 = lds128(src + (((2 * sub + h) ^ x) << 4));
-                        const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
+                            for (int h = 0; h < 2; ++h) {
+                                const uint4 c4 = lds128(src + (((2 * sub + h) ^ x) << 4));
+                                const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            uint32_t P[4];
-                            expand8(cw[i], ss, P);
-                            sts128(a_dst + (((4 * h + i) ^ x) << 4), P[0], P[1], P[2], P[3]);
-                        }
-                    }
-                } else {
-                    // one f, one group of 64 columns; nibble q of word w is column 8 q + w
-                    const uint32_t src = raw + (sub * 64 + (row & 63)) * 128;
-                    const uint32_t pc0 = (uint32_t)((it.m0 / 32) & 7) + 2u * cg;      // first piece of the group in its 128 bytes
-                    const uint4 ca = lds128(src + ((pc0 ^ x) << 4)), cb = lds128(src + (((pc0 + 1) ^ x) << 4));
-                    // (half of the nibbles at a time, to save registers)
+                                for (int i = 0; i < 4; ++i) {
+                                    uint32_t P[4];
+                                    expand8(cw[i], ss, P);
+                                    sts128(a_dst + (((4 * h + i) ^ x) << 4), P[0], P[1], P[2], P[3]);
+                                }
+                            }
+                        } else {
+                            // one f, one group of 64 columns; nibble q of word w is column 8 q + w
+                            const uint32_t src = raw + (sub * 64 + (row & 63)) * 128;
+                            const uint32_t pc0 = (uint32_t)((it.m0 / 32) & 7) + 2u * cg;      // first piece of the group in its 128 bytes
+                            const uint4 ca = lds128(src + ((pc0 ^ x) << 4)), cb = lds128(src + (((pc0 + 1) ^ x) << 4));
+                            // (half of the nibbles at a time, to save registers)
 #pragma unroll
-                    for (int side = 0; side < 2; ++side) {
-                        const uint32_t cw[8] = {ca.x >> (8 * side), ca.y >> (8 * side), ca.z >> (8 * side), ca.w >> (8 * side),
-                                                cb.x >> (8 * side), cb.y >> (8 * side), cb.z >> (8 * side), cb.w >> (8 * side)};
-                        uint32_t o[4][4];
+                            for (int side = 0; side < 2; ++side) {
+                                const uint32_t cw[8] = {ca.x >> (8 * side), ca.y >> (8 * side), ca.z >> (8 * side), ca.w >> (8 * side),
+                                                        cb.x >> (8 * side), cb.y >> (8 * side), cb.z >> (8 * side), cb.w >> (8 * side)};
+                                uint32_t o[4][4];
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            uint32_t P[2], Q[2];
-                            expand4(cw[2 * i], ss, P);
-                            expand4(cw[2 * i + 1], ss, Q);
+                                for (int i = 0; i < 4; ++i) {
+                                    uint32_t P[2], Q[2];
+                                    expand4(cw[2 * i], ss, P);
+                                    expand4(cw[2 * i + 1], ss, Q);
 #pragma unroll
-                            for (int q = 0; q < 2; ++q) {
-                                o[q][i] = __byte_perm(P[q], Q[q], 0x5410);
-                                o[q + 2][i] = __byte_perm(P[q], Q[q], 0x7632);
+                                    for (int q = 0; q < 2; ++q) {
+                                        o[q][i] = __byte_perm(P[q], Q[q], 0x5410);
+                                        o[q + 2][i] = __byte_perm(P[q], Q[q], 0x7632);
+                                    }
+                                }
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    sts128(a_dst + ((((q & 1) + 2 * side + 4 * (q >> 1)) ^ x) << 4), o[q][0], o[q][1], o[q][2], o[q][3]);
                             }
                         }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            sts128(a_dst + ((((q & 1) + 2 * side + 4 * (q >> 1)) ^ x) << 4), o[q][0], o[q][1], o[q][2], o[q][3]);
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the tensor cores read what was just stored
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (rank == 0)
+                                mbar_arrive(full0 + 8 * s);
+                            else
+                                mbar_arrive_cluster(cluster_addr(full0 + 8 * s, 0));
+                        }
+                        sc = scale_of(kb + kExpandGroups);       // (in front of the arrival, that would wait for it)
                     }
+                    if (lane == 0)
+                        mbar_arrive(rempty0 + 8 * rs);
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the tensor cores read what was just stored
-                __syncwarp();
-                if (lane == 0) {
-                    if (rank == 0)
-                        mbar_arrive(full0 + 8 * s);
-                    else
-                        mbar_arrive_cluster(cluster_addr(full0 + 8 * s, 0));
-                }
-                sc = scale_of(kb + kExpandGroups);       // (in front of the arrival, that would wait for it)
-                }
-                if (lane == 0)
-                    mbar_arrive(rempty0 + 8 * rs);
-            }
             };
             if (PHASE ? PHASE == 1 : it.phase == 1)
                 expand(Const<1>());

@@ -440,9 +440,9 @@ def shape_record(torch, M, gen, name, n_layers, K, W, hbm_peak, link_peak, peaks
         rec["prefill_gemm"] = {"tokens": T, "token_expert_pairs_per_layer": pairs, "tflops": tf,
                                "frac_of_bf16_burst": tf / peaks.get("bf16_tflops", 1590.0),
                                "frac_of_bf16_sustained": tf / peaks.get("bf16_tflops_sustained", 1400.0),
-                               "gemm_launch_pairs": n, "gemm_ms_per_layer": ms_sum / n_layers,
-                               "note": "flops = 6 d_model d_ff per (token, expert) pair; time = CUDA events around the two "
-                                       "GEMM launches of every compute group, transfers excluded"}
+                               "gemm_compute_groups": n, "gemm_ms_per_layer": ms_sum / n_layers,
+                               "note": "flops = 6 d_model d_ff per (token, expert) pair; time = CUDA events around both "
+                                       "GEMMs of every compute group, transfers excluded"}
     R.close()
     # the same shape with every expert resident: the decode kernel in its HBM-bound regime
     Ra = Runner(torch, M, gen, cfg, alpha, cfg.n_experts, n_layers, K, W, store=store)

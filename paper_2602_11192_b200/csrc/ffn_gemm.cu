@@ -62,7 +62,7 @@
 // stream), reading the weights below some 150 (6 TB/s), the expansion with 4-bit slots.  A pass of a layer, two launches of the GEMMs ->
 // one, with the front end as it is now (us): 16 tokens, d 2048, d_ff 1024, 64 experts, 8 per token 61 -> 55; 128 tokens 72 -> 66;
 // 4096 tokens, d 4096, d_ff 6400, 16 experts, 2 per token 1295 -> 1246; 8192 tokens, d 2048, d_ff 1408, 66 experts
-// 1225 -> 1227; 4-bit slots of the first shape, 16 tokens 70 -> 52, 512 tokens 137 -> 129.
+// 1225 -> 1227; 4-bit slots of the first shape, 16 tokens 70 -> 52, 512 tokens 128 -> 123.
 //
 // Every wait is bounded; on a timeout the CTA raises its abort flag, every role leaves its
 // loops, tensor memory is freed and the error word tells the host.
